@@ -529,30 +529,32 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
         workers_sync<kPfWorkers>();  // the row's four slice maxima
         const float M = sg * fmaxf(fmaxf(smax[rl], smax[kPfRows + rl]),
                                    fmaxf(smax[2 * kPfRows + rl], smax[3 * kPfRows + rl]));
-        if (M > c_ref + 8.f) {  // the same decision on the row's four threads
-          if (c_ref != -INFINITY) {
-            // O holds this job's earlier tiles: rescale this thread's 32
-            // channels once the previous tile's value product is done
-            if (!wait_pv(kk - 1)) {
-              failed = true;
-              *abort_flag = 1;
-            } else {
-              tc_fence_after();
-              const float f = fast_exp2(c_ref - M);
-              float z[16];
-              uint32_t zw[16];
+        const bool move = M > c_ref + 8.f;  // the same decision on the row's four threads
+        const bool resc = move && c_ref != -INFINITY;
+        if (__any_sync(0xffffffffu, resc)) {
+          // O holds this job's earlier tiles: rescale this thread's 32
+          // channels once the previous tile's value product is done.  Lanes
+          // are rows and the TMEM accesses are warp-wide (.sync.aligned), so
+          // the whole warp takes part, rows that do not move with factor 1.
+          if (!__all_sync(0xffffffffu, wait_pv(kk - 1))) {
+            failed = true;
+            *abort_flag = 1;
+          } else {
+            tc_fence_after();
+            const float f = resc ? fast_exp2(c_ref - M) : 1.f;
+            float z[16];
+            uint32_t zw[16];
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                tmem_ld16(t_o + 32 * slice + 16 * h + lane_off, z);
+            for (int h = 0; h < 2; ++h) {
+              tmem_ld16(t_o + 32 * slice + 16 * h + lane_off, z);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) zw[i] = __float_as_uint(z[i] * f);
-                tmem_st16_nw(t_o + 32 * slice + 16 * h + lane_off, zw);
-              }
-              l_run *= f;
+              for (int i = 0; i < 16; ++i) zw[i] = __float_as_uint(z[i] * f);
+              tmem_st16_nw(t_o + 32 * slice + 16 * h + lane_off, zw);
             }
+            l_run *= f;
           }
-          c_ref = M;
         }
+        if (move) c_ref = M;
         // P of this row over the slice's 16 positions, hi and lo halves
         float x0[8], x1[8];
         if (nv >= 16) {

@@ -90,6 +90,27 @@ def test_prefill_long_chunk_many_tiles(fmt):
     assert_close(f32(out), _expected(q, st, lens, 0.09), what=f"{_fid(fmt)} long chunk")
 
 
+@pytest.mark.parametrize("fmt", [FORMATS[0], FORMATS[2]], ids=_fid)
+def test_prefill_row_maxima_rise(fmt):
+    # keys grow along the context by a factor of its own per KV head, so that
+    # some rows of a warp move their reference maximum (by far more than 8,
+    # at several tiles) and others of the same warp do not
+    B, Hkv, G, T, n_q = 2, 2, 5, 512, 70
+    c = _cache(B, G * Hkv, Hkv, T, [fmt])
+    g = torch.Generator().manual_seed(3)
+    grow = 1.0 + torch.arange(T)[None, :, None, None] / 64.0 * torch.tensor([1.0, 0.25])[None, None, :, None]
+    K = (torch.randn((B, T, Hkv, 128), generator=g) * grow).to(torch.bfloat16)
+    V = torch.randn((B, T, Hkv, 128), generator=g).to(torch.bfloat16)
+    c.append(0, K.cuda(), V.cuda())
+    st = oracle_state(f32(K), f32(V), np.array([T] * B), fmt)
+    q = _queries(B, n_q, G * Hkv, seed=5, dtype=torch.bfloat16)
+    q[:, ::3] *= 0.05
+    sigma = 1.0 / math.sqrt(128)
+    out = c.prefill(0, q.cuda(), sigma)
+    assert_close(f32(out), _expected(q, st, np.array([T] * B), sigma), what=f"{_fid(fmt)} rising maxima")
+    assert c.device_error() == 0
+
+
 def test_prefill_one_query_is_decode_and_inheritor_reads_anchor():
     B, Hkv, G, T = 2, 4, 5, 600
     fmt = dict(bits=4, group=32, key_axis="token")
