@@ -60,33 +60,89 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-// more than 16 splits: the same, with the split loop not unrolled
-__global__ void __launch_bounds__(128)
-    splitk_merge_kernel_n(const float *P, int S, int n_rows, int dim,
-                          float *__restrict__ out) {
+// More than 16 splits (few units over a long context): one CTA per row, warp
+// w takes splits w, w + 8, ..., lane L channels L + 32 j.  A thread issues
+// the loads of its first 8 splits (maxima, sums, accumulators: every split up
+// to 64) before it uses any, so this merge too is one memory round trip; the
+// warps' maxima and then their sums meet in shared memory.  Bound by that
+// latency: a serial loop over the splits (a dependent load and exponential
+// each) took 32.1 us for 57 splits of 40 rows of 128; the whole decode step
+// around it (one sequence of 32769 int8 positions) went 40.3 -> 33.4 us.
+constexpr int kWideWarps = 8, kWideRound = 8;
+__global__ void __launch_bounds__(32 * kWideWarps)
+    splitk_merge_wide(const float *P, int S, int n_rows, int dim, float *__restrict__ out) {
   pdl_wait();
   pdl_trigger();
-  const int width = dim >= 128 ? 128 : dim;  // threads per row
-  const int rpc = 128 / width, r_in = (int)threadIdx.x / width;
-  const int row = blockIdx.x * rpc + r_in;
-  if (r_in >= rpc || row >= n_rows) return;
-  const int ch0 = (int)threadIdx.x % width;
+  __shared__ float s_m[kWideWarps], s_l[kWideWarps], s_a[kWideWarps][128];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = blockIdx.x;
   const size_t RS = (size_t)dim + 2;
   const size_t SS = (size_t)n_rows * RS;
   const float *pr = P + (size_t)row * RS;
+  float m[kWideRound], l[kWideRound], x[kWideRound][4];
+  auto load_acc = [&](int ch0) {
+#pragma unroll
+    for (int i = 0; i < kWideRound; ++i) {
+      const int s = warp + kWideWarps * i;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int ch = ch0 + lane + 32 * j;
+        x[i][j] = s < S && ch < dim ? pr[s * SS + ch] : 0.f;
+      }
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < kWideRound; ++i) {
+    const int s = warp + kWideWarps * i;
+    m[i] = s < S ? pr[s * SS + dim] : -INFINITY;
+    l[i] = s < S ? pr[s * SS + dim + 1] : 0.f;
+  }
+  load_acc(0);
   float M = -INFINITY;
-  for (int s = 0; s < S; ++s) M = fmaxf(M, pr[s * SS + dim]);
-  for (int ch = ch0; ch < dim; ch += 128) {
-    float L = 0.f, A = 0.f;
+#pragma unroll
+  for (int i = 0; i < kWideRound; ++i) M = fmaxf(M, m[i]);
+  for (int s = warp + kWideWarps * kWideRound; s < S; s += kWideWarps) M = fmaxf(M, pr[s * SS + dim]);
+  if (lane == 0) s_m[warp] = M;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kWideWarps; ++w) M = fmaxf(M, s_m[w]);
+  for (int ch0 = 0; ch0 < dim; ch0 += 128) {
+    if (ch0 > 0) load_acc(ch0);
+    float L = 0.f, A[4] = {0.f, 0.f, 0.f, 0.f};
     if (M != -INFINITY) {
-      for (int s = 0; s < S; ++s) {
+#pragma unroll
+      for (int i = 0; i < kWideRound; ++i) {
+        const float w = m[i] == -INFINITY ? 0.f : exp2f(m[i] - M);
+        L = fmaf(w, l[i], L);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) A[j] = fmaf(w, x[i][j], A[j]);
+      }
+      for (int s = warp + kWideWarps * kWideRound; s < S; s += kWideWarps) {
         const float ms = pr[s * SS + dim];
         const float w = ms == -INFINITY ? 0.f : exp2f(ms - M);
         L = fmaf(w, pr[s * SS + dim + 1], L);
-        A = fmaf(w, pr[s * SS + ch], A);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int ch = ch0 + lane + 32 * j;
+          if (ch < dim) A[j] = fmaf(w, pr[s * SS + ch], A[j]);
+        }
       }
     }
-    out[(size_t)row * dim + ch] = (L > 0.f) ? A / L : 0.f;
+    if (lane == 0) s_l[warp] = L;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s_a[warp][lane + 32 * j] = A[j];
+    __syncthreads();
+    const int ch = ch0 + (int)threadIdx.x;
+    if (threadIdx.x < 128 && ch < dim) {
+      float a = 0.f, ls = 0.f;
+#pragma unroll
+      for (int w = 0; w < kWideWarps; ++w) {
+        a += s_a[w][threadIdx.x];
+        ls += s_l[w];
+      }
+      out[(size_t)row * dim + ch] = ls > 0.f ? a / ls : 0.f;
+    }
+    __syncthreads();
   }
 }
 
@@ -116,7 +172,7 @@ cudaError_t launch_splitk_merge(const float *partials, int n_splits, int n_rows,
   else if (n_splits <= 16)
     return launch_pdl(splitk_merge_kernel<16>, grid, dim3(128), 0, st, partials, n_splits, n_rows, dim, out);
   else
-    return launch_pdl(splitk_merge_kernel_n, grid, dim3(128), 0, st, partials, n_splits, n_rows, dim, out);
+    return launch_pdl(splitk_merge_wide, n_rows, dim3(32 * kWideWarps), 0, st, partials, n_splits, n_rows, dim, out);
 }
 
 }  // namespace kvk

@@ -192,7 +192,7 @@ def test_partials_and_reduce_equal_decode():
 
 
 @pytest.mark.parametrize("S,dim", [(1, 128), (5, 128), (8, 64), (9, 96), (16, 130), (17, 512),
-                                   (40, 128), (64, 32)])
+                                   (40, 128), (64, 32), (65, 64), (200, 300)])
 def test_splitk_reduce_matches_log_sum_exp(S, dim):
     """The merge against the log-sum-exp identity in fp64, with empty splits
     (m = -inf, l = 0) and rows whose splits are all empty."""
