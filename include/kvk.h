@@ -276,17 +276,23 @@ kvk_status kvk_prefill_attention(kvk_cache *cache, int32_t layer, const void *q,
  * sequence b, at position len_b - n_q + i, attends to positions 0 .. itself
  * with the absorbed query of each head (Appendix C.2, as
  * kvk_decode_attention_mla: q_lat = W_UK[h][:, :d]^T q_nope, scores
- * sigma (q_lat . c[:d] + q_pe . k^R), output W_UV[h][:, :d] o_lat).  Each
- * query row runs the decode path over its own causal prefix (one CTA per
- * row, or per pair of consecutive rows of a sequence for bf16 latents of
- * width >= 256 when n_q is even).  Queries before position 0 give zeros.
+ * sigma (q_lat . c[:d] + q_pe . k^R), output W_UV[h][:, :d] o_lat).  Short
+ * chunks run the decode path per query row over its own causal prefix (one
+ * CTA per row, or per pair of consecutive rows of a sequence for bf16 latents
+ * of width >= 256 when n_q is even).  Longer ones form each head's keys
+ * W_UK[h][:, :d] c and values W_UV[h][:, :d] c once and attend over them (the
+ * same algebra); where the line lies depends on the cache's batch, width and
+ * precision.  Queries before position 0 give zeros.
  *  q_nope:  device bf16 [B, n_q, H, head_dim]; q_pe: bf16 [B, n_q, H, rope]
  *           (post-RoPE);
  *  w_uk, w_uv: device bf16 [H, head_dim, latent] as for decode;
  *  out:     device float32 [B, n_q, H, head_dim];
  *  scratch: device, 256-byte aligned, at least kvk_prefill_scratch_size
- *           bytes (which answers for MLA layers too): the rows' absorbed
- *           queries and latent partials;
+ *           bytes (which answers for MLA layers too, and never less for a
+ *           larger n_q): the rows' absorbed queries and latent partials, or
+ *           the formed keys and values (1 KB per position and head, heads and
+ *           sequences in groups of at most 2 GiB) and a job counter.  A
+ *           buffer that holds only the former serves every chunk by rows;
  * all 16-byte aligned.  Errors: INVALID_ARG (not an MLA cache, n_q outside
  * [1, max_ctx], null or misaligned pointers, scale not finite and positive,
  * scratch too small). */

@@ -137,12 +137,22 @@ struct PfArgs {
   float sig_log2;      // softmax scale * log2(e)
   float *out;          // [B, n_q, Hq, D]
   int *counter;        // the job counter, zeroed by the launch
-  uint8_t *tiles;      // [B * Hkv][cap / 64] expanded tiles of prefill_tile_bytes(bits)
+  uint8_t *tiles;      // [B * Hkv] units of prefill_unit_bytes(bits, cap): expanded tiles
   int32_t *err;
+  // MLA chunks over formed keys and values (units = heads: v.B sequences from
+  // b0 on, v.Hkv heads from h0 on, G = 1; of v only lens, B, Hkv and cap are
+  // read): the positional queries and the positional keys' tiles
+  const void *q_pe = nullptr;   // bf16 [B, n_q, Hq, 64]
+  const uint8_t *kr = nullptr;  // [v.B][tiles of 128 positions] of kr_bytes: hi box, lo box if quantised
+  int kr_bytes = 0;             // 0: GQA
+  int b0 = 0, h0 = 0;
 };
 cudaError_t launch_gqa_prefill(const PfArgs &a, cudaStream_t st);
+// the attention over tiles that launch_mla_form wrote (prefill.cu)
+cudaError_t launch_mla_prefill_formed(const PfArgs &a, cudaStream_t st);
 bool prefill_plan_fits(const PfArgs &a);
-size_t prefill_tile_bytes(int bits);
+// expanded tiles of one unit (a KV head of a sequence of capacity cap)
+size_t prefill_unit_bytes(int bits, int64_t cap);
 constexpr int kEvictTile = 128;
 constexpr int kEvictStatSub = 4;  // statistics entries per tile and row, at most
 // Whether the evictor scores on the tensor cores (head_dim 128, at most 256
@@ -175,6 +185,21 @@ struct MlaDecodeArgs {
   uint32_t wait_limit = 1u << 22;  // polls of a bounded wait in the tile loop before it gives up
 };
 cudaError_t launch_mla_decode(const MlaDecodeArgs &a, cudaStream_t st);
+// Keys and values of heads h0 .. h0 + nh - 1 of sequences b0 .. b0 + nb - 1
+// formed from an MLA anchor's latents (mla_form.cu), as pre-fill tiles.
+struct MlaFormArgs {
+  MlaView v;
+  int b0, nb, h0, nh;
+  int n_t;             // 128-position tiles per sequence
+  const float *wsum;   // [H][256] column sums of the weights (grouped codes), else null
+  uint8_t *tiles;      // [nb][nh][n_t] tiles of 128 KB (layout: prefill.cu)
+  uint8_t *kr;         // [nb][n_t] tiles of kr_bytes (16 KB hi; quantised latents + 16 KB lo)
+  int kr_bytes;
+  int32_t *err;
+};
+cudaError_t launch_mla_wsum(const void *w_uk, const void *w_uv, int H, int r, int W, float *wsum, cudaStream_t st);
+cudaError_t launch_mla_form(const MlaFormArgs &a, const void *w_uk, const void *w_uv, int H, int r, int sms,
+                            cudaStream_t st);
 // the same for an anchor of quantised latents (mla_q.cu; one CTA per SM)
 cudaError_t launch_mla_decode_q(const MlaDecodeArgs &a, cudaStream_t st);
 // Encodes the decode kernel's tensor map of an MLA anchor into `out` (128

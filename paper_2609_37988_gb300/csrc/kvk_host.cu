@@ -183,6 +183,7 @@ struct kvk_cache {
   int sm_count;
   int device;
   std::vector<int> ctas;  // per layer, decode CTAs per SM (0 = not queried)
+  std::vector<int> formed_from;  // per MLA anchor, the shortest chunk over formed keys (mla_formed_from)
   uint32_t wait_limit = KVK_WAIT_LIMIT_DEFAULT;  // decode tile-loop waits (kvk_set_wait_limit)
   int schedule = KVK_SCHEDULE_AUTO;              // decode partition (kvk_set_decode_schedule)
   int run_ctas = 0;                              // CTAs of a run-schedule decode (0: whole waves)
@@ -401,6 +402,43 @@ bool plan_runs(kvk_cache *c, int a, RunPlan *p) {
   return true;
 }
 
+// The shortest chunk of layer `a` that attends over formed keys and values;
+// shorter ones run the absorbed decode per row.  Both costs in ns per cached
+// position, measured (4 x 4096, 1 x 8192 and 8 x 1024 positions, 8-128
+// queries, every width; e.g. bf16 d = 512, 4 x 4096, absorbed / formed us: 48
+// queries 162 / 163, 64 170 / 162, 96 309 / 163; d = 64: 128 92 / 134, 1 x
+// 8192 d = 512: 8 266 / 203):
+//  absorbed: a wave of resident CTAs (one row each, or two at d >= 256 over
+//            bf16 latents) takes `full` (`half` if at most half of it is
+//            there), plus about 10 us;
+//  formed:   a wave of jobs (128 rows of one head) 14.8, the forming itself
+//            `form` per sequence, plus about 15 us.
+// The answer is one more than the longest chunk (of up to 1024 queries) that
+// the absorbed path serves faster; at least 16 (a handful of queries is not
+// worth the formed tiles' memory), never where one head's tiles pass 2 GiB.
+int mla_formed_from(const kvk_cache *c, int a) {
+  const kvk_layer_cfg &L = c->cfg[a];
+  const int w = L.width == 512 ? 0 : L.width == 256 ? 1 : L.width == 128 ? 2 : 3;
+  static const double kHalf[4] = {36.0, 14.5, 10.0, 8.5}, kFull[4] = {41.0, 18.5, 15.6, 12.0};
+  static const double kQuant[4] = {37.0, 18.5, 10.5, 10.0};
+  static const double kForm[4] = {5.1, 3.9, 3.5, 3.3}, kFormQ[4] = {3.5, 2.5, 1.8, 1.5};
+  if (c->lay[a].cap > (1 << 21)) return INT32_MAX;
+  const double B = c->desc.max_batch, H = c->desc.n_q_heads, T = c->desc.max_ctx, sms = c->sm_count;
+  for (int n = std::min(1024, c->desc.max_ctx); n >= 1; --n) {
+    const double rows = B * n;
+    double absorbed;
+    if (L.bits != 16) {
+      absorbed = kQuant[w] * std::ceil(rows / sms);
+    } else {
+      const double slots = w >= 2 || n % 2 == 0 ? 2.0 * sms : sms;
+      absorbed = rows <= slots / 2 ? kHalf[w] : kFull[w] * std::ceil(rows / slots);
+    }
+    const double jobs = B * H * ((n + 127) / 128);
+    const double formed = 14.8 * std::ceil(jobs / sms) + B * (kForm[w] + (L.bits != 16 ? kFormQ[w] : 0.0));
+    if (absorbed * T + 10e3 < formed * T + 15e3) return std::max(16, n + 1);
+  }
+  return 16;
+}
 }  // namespace
 
 extern "C" {
@@ -475,6 +513,7 @@ kvk_status kvk_cache_create(const kvk_model_desc *desc, const kvk_layer_cfg *cfg
   c->len_hi.assign(desc->n_layers, 0);
   c->kept_on.assign(desc->n_layers, 0);
   c->ctas.assign(desc->n_layers, 0);
+  c->formed_from.assign(desc->n_layers, 0);
   int last = 0;
   for (int l = 0; l < desc->n_layers; ++l) {
     if (!cfg[l].inherit) {
@@ -499,6 +538,7 @@ kvk_status kvk_cache_create(const kvk_model_desc *desc, const kvk_layer_cfg *cfg
   for (int l = 0; l < desc->n_layers; ++l) {
     if (cfg[l].inherit) continue;
     if (desc->kind == KVK_KIND_MLA) {
+      c->formed_from[l] = mla_formed_from(c, l);
       if (cfg[l].bits != 16) continue;  // quantised tiles use bulk copies
       e = mla_make_tmap(c->tmap[l].bytes, c->mla_view(l));
     } else {
@@ -791,7 +831,7 @@ PrefillScratch prefill_scratch(const kvk_cache *c, int32_t layer, int32_t n_q) {
   p.counters = 0;
   p.tiles = 1024;
   const size_t units = (size_t)c->desc.max_batch * c->desc.n_kv_heads;
-  p.total = p.tiles + units * (size_t)(c->lay[a].cap / 64) * prefill_tile_bytes(c->cfg[a].bits);
+  p.total = p.tiles + units * prefill_unit_bytes(c->cfg[a].bits, c->lay[a].cap);
   return p;
 }
 }  // namespace
@@ -812,6 +852,29 @@ MlaPrefillScratch mla_prefill_scratch(const kvk_cache *c, int32_t layer, int32_t
   p.total = p.partial + rows * (W + 2) * 4;
   return p;
 }
+// MLA chunks over formed keys and values (mla_form.cu): the job counter, the
+// weights' column sums, then the positional keys' tiles and the formed tiles
+// of one group of nb sequences x nh heads (at most 2 GiB of tiles, or one
+// head of one sequence; the groups run one after another in the same space).
+struct MlaFormedScratch {
+  size_t wsum, kr, tiles, total;
+  int nb, nh, kr_bytes;
+};
+MlaFormedScratch mla_formed_scratch(const kvk_cache *c, int32_t layer) {
+  const int a = c->src[layer];
+  const long long B = c->desc.max_batch, H = c->desc.n_q_heads, n_t = (c->lay[a].cap + 127) / 128;
+  const long long unit = n_t * 131072;
+  const long long fit = std::max(1LL, (2LL << 30) / unit);
+  MlaFormedScratch p;
+  p.nh = (int)std::min(H, fit);
+  p.nb = (int)std::max(1LL, std::min(B, fit / p.nh));
+  p.kr_bytes = c->cfg[a].bits == 16 ? 16384 : 32768;
+  p.wsum = 1024;
+  p.kr = p.wsum + (size_t)align256(H * 256 * 4);
+  p.tiles = p.kr + (size_t)p.nb * n_t * p.kr_bytes;
+  p.total = p.tiles + (size_t)p.nb * p.nh * unit;
+  return p;
+}
 kvk_status check_prefill_mla(const kvk_cache *c, int32_t layer, int32_t n_q) {
   kvk_status s = check_layer_index(c, layer);
   if (s) return s;
@@ -827,7 +890,11 @@ kvk_status kvk_prefill_scratch_size(const kvk_cache *c, int32_t layer, int32_t n
     kvk_status s = check_prefill_mla(c, layer, n_q);
     if (s) return s;
     if (!bytes) return fail(KVK_ERR_INVALID_ARG, "null output");
-    *bytes = mla_prefill_scratch(c, layer, n_q).total;
+    // never less for more queries: a buffer sized for the longest chunk
+    // serves every shorter one
+    const int from = c->formed_from[c->src[layer]];
+    *bytes = mla_prefill_scratch(c, layer, std::min(n_q, from)).total;
+    if (n_q >= from) *bytes = std::max(*bytes, mla_formed_scratch(c, layer).total);
     return KVK_OK;
   }
   kvk_status s = check_prefill(c, layer, n_q);
@@ -1094,10 +1161,62 @@ kvk_status kvk_prefill_attention_mla(kvk_cache *c, int32_t layer, const void *q_
   if (!std::isfinite(softmax_scale) || !(softmax_scale > 0.f))
     return fail(KVK_ERR_INVALID_ARG, "softmax scale must be finite and positive");
   const MlaPrefillScratch ps = mla_prefill_scratch(c, layer, n_q);
-  if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 255u) || scratch_bytes < ps.total)
-    return fail(KVK_ERR_INVALID_ARG, "scratch null, not 256-byte aligned or smaller than %zu bytes",
-                ps.total);
+  const MlaFormedScratch fs = mla_formed_scratch(c, layer);
+  const bool formed = n_q >= c->formed_from[c->src[layer]] && scratch_bytes >= fs.total;
+  if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 255u) || (!formed && scratch_bytes < ps.total)) {
+    size_t need = 0;
+    kvk_prefill_scratch_size(c, layer, n_q, &need);
+    return fail(KVK_ERR_INVALID_ARG, "scratch null, not 256-byte aligned or smaller than %zu bytes", need);
+  }
   const int a = c->src[layer];
+  if (formed) {
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    uint8_t *sc = static_cast<uint8_t *>(scratch);
+    const MlaView mv = c->mla_view(a);
+    const int H = c->desc.n_q_heads, r = c->desc.latent_dim;
+    MlaFormArgs f;
+    f.v = mv;
+    f.n_t = (int)((mv.cap + 127) / 128);
+    const bool offsets = mv.bits != 16 && mv.scheme != kSchemeSym;
+    f.wsum = offsets ? reinterpret_cast<float *>(sc + fs.wsum) : nullptr;
+    f.tiles = sc + fs.tiles;
+    f.kr = sc + fs.kr;
+    f.kr_bytes = fs.kr_bytes;
+    f.err = c->err();
+    PfArgs p;
+    p.v = GqaView{};
+    p.v.lens = mv.lens;
+    p.v.cap = mv.cap;
+    p.v.bits = 16;
+    p.v.rec_bytes = 16;
+    p.q = q_nope;
+    p.q_f32 = 0;
+    p.Hq = H;
+    p.G = 1;
+    p.n_q = n_q;
+    p.sig_log2 = softmax_scale * 1.4426950408889634f;
+    p.out = out;
+    p.counter = reinterpret_cast<int *>(sc);
+    p.tiles = f.tiles;
+    p.err = c->err();
+    p.q_pe = q_pe;
+    p.kr = f.kr;
+    p.kr_bytes = fs.kr_bytes;
+    cudaError_t e = cudaSuccess;
+    if (offsets) e = launch_mla_wsum(w_uk, w_uv, H, r, mv.width, reinterpret_cast<float *>(sc + fs.wsum), st);
+    for (int b0 = 0; b0 < mv.B && e == cudaSuccess; b0 += fs.nb)
+      for (int h0 = 0; h0 < H && e == cudaSuccess; h0 += fs.nh) {
+        f.b0 = p.b0 = b0;
+        f.h0 = p.h0 = h0;
+        f.nb = p.v.B = std::min(fs.nb, mv.B - b0);
+        f.nh = p.v.Hkv = std::min(fs.nh, H - h0);
+        e = cudaMemsetAsync(p.counter, 0, sizeof(int), st);
+        if (e == cudaSuccess) e = launch_mla_form(f, w_uk, w_uv, H, r, c->sm_count, st);
+        if (e == cudaSuccess) e = launch_mla_prefill_formed(p, st);
+      }
+    if (e != cudaSuccess) return cuda_fail(e, "MLA pre-fill launch");
+    return KVK_OK;
+  }
   MlaDecodeArgs args;
   args.v = c->mla_view(a);
   args.v.n_q = n_q;  // query row b n_q + i: query i of sequence b over its causal prefix

@@ -9,27 +9,42 @@
 // head h of the KV head's group; query i sits at position len - n_q + i and
 // sees positions 0 .. len - n_q + i.  A job is 128 consecutive rows of one
 // unit.  Two launches:
-//  * expand: every 64-position tile of the cache is dequantised once into
-//    the layout the products read (bf16 hi and lo halves, K-major
-//    128-byte-swizzled boxes), in caller scratch;
+//  * expand: the cache is dequantised once into the layout the products read
+//    (bf16 hi and lo halves, 128-byte-swizzled boxes of 64 channels), in
+//    caller scratch, tiles of 128 positions;
 //  * attention, one pass over the tiles: per tile, S = Q K^T (TMEM lane =
 //    row) with x = sigma log2(e) <q, k>; each row's maximum over the tile
 //    (its four slices' maxima through shared memory) against the row's
 //    reference m, which moves only when a score rises more than 8 above it
 //    (O and the row's sums then rescaled by 2^(m_old - m_new) in place);
 //    P = 2^(x - m) (zero past the row's limit, at most 2^8) as bf16 hi and
-//    lo pairs into TMEM, O += P V (P the A operand from TMEM, the value
-//    tile an MN-major B operand); after the job's last tile O (TMEM lane =
-//    row) is divided by the row's sum of P and written out.
-// The attention kernel runs one persistent CTA per SM: a copy warp
-// brings each job's tiles in with bulk copies, three MMA warps issue the
-// tcgen05 products (one thread issues at most one product per ~45 cycles:
-// the scores of even and of odd tiles, and the value products, are three
-// streams), 16 worker warps stage the query rows into TMEM (the A operand
-// of the score products) and run the epilogues.  Products are hi*hi +
-// hi*lo + lo*hi (no lo part for bf16 caches or bf16 queries), fp32
-// accumulation in TMEM.  Jobs are handed out from a counter in bands of
-// units whose tiles stay in L2, the longest row blocks first.
+//    lo pairs into TMEM in place of the scores, O += P V (P the A operand
+//    from TMEM, the values an MN-major B operand); after the job's last tile
+//    O (TMEM lane = row) is divided by the row's sum of P and written out.
+// The attention kernel runs one persistent CTA per SM: two copy warps bring
+// each job's keys and values in with bulk copies, one MMA warp issues the
+// score products and one the value products, 16 worker warps stage the query
+// rows and run the epilogues.  Products are hi*hi + hi*lo + lo*hi (no lo
+// part for bf16 caches or bf16 queries), fp32 accumulation in TMEM.  Jobs
+// are handed out from a counter in bands of units whose tiles stay in L2,
+// the longest row blocks first.
+//
+// Why tiles of 128 positions: a score product of N = 64 with its A operand
+// in TMEM took 77-90 cycles (a clock64 trace of the 64-position version: 16
+// of them 1450 cycles, 12 value products 800 alone) against 64 for N = 128,
+// and the two products of a tile then cost 2560 cycles per 128 positions
+// (16 + 24 at 64), under which the epilogue (about 1500) hides.
+//
+// MLA chunks run the same attention kernel over keys and values formed per
+// head (mla_form.cu): units are heads (G = 1), and the score products go on
+// over the 64 positional channels, whose keys (one tile per sequence, shared
+// by the heads) come through a ring of their own.  Their query rows sit in
+// shared memory and the freed TMEM columns hold a second accumulator, for
+// the products with a lo half: a tensor-core accumulation rounds towards
+// zero, so each one costs its accumulator about 2^-25 of its value in one
+// direction, and three per k-step into one accumulator left 1.3e-5 of the
+// result over 3584 positions where the absorbed path has 5.6e-6 (the lo
+// products' own sum is 2^-8 of the result).
 #include <math.h>
 
 #include <algorithm>
@@ -44,25 +59,43 @@ namespace kvk {
 namespace {
 
 constexpr int kPfWorkers = 512;
-constexpr int kPfThreads = kPfWorkers + 128;  // + three MMA warps and the copy warp
+constexpr int kPfThreads = kPfWorkers + 128;  // + two MMA warps and two copy warps
 constexpr int kPfRows = 128;                 // rows per job
-constexpr int kPfT = 64;                     // positions per tile
-constexpr int kPfBox = kPfT * 128;           // one 64-channel box of a tile (8 KB)
-constexpr int kPfMaxStages = 6;              // key (and value) stages at most
-constexpr int kPfBarBytes = 320;             // barriers and the CTA's shared words
+constexpr int kPfT = 128;                    // positions per tile
+constexpr int kPfBox = 64 * 128;             // 64 channels x 64 positions (8 KB)
+constexpr int kPfMaxStages = 8;              // key (and value) units at most
+constexpr int kPfBarBytes = 448;             // barriers and the CTA's shared words
 
+// A tile in scratch: two key units, one per 64 channels ([hi | lo], 128
+// positions x 128 bytes each), then two value units, one per 64 positions
+// ([hi | lo], two boxes of 64 channels each); no lo halves for bf16 caches.
 struct PfPlan {
-  int n_rb, n_jobs, grid, n_t64;
+  int n_rb, n_jobs, grid, n_t;  // n_t: tiles per unit in scratch
   int q_lo, k_lo, fmt, gshift;
   int kpc;            // keys with per-channel groups (codes + group plane + residual)
   int ks16, nrec;
   uint32_t nc_magic;  // expand: ceil(2^32 / nrec), e / nrec = umulhi(e, nc_magic)
   int b_stride;       // expand: staged record stride (odd multiple of 16 bytes)
-  int kbytes, tbytes; // a tile's keys (hi, lo); the whole tile (keys, values)
-  int ns;             // key stages of the attention kernels
-  int nv;             // value stages (output pass)
+  int ub, tbytes;     // a unit; the whole tile (two key and two value units)
+  int krb;            // positional keys of a tile (MLA; else 0)
+  int nk, nv, nr;     // key and value units and positional tiles in shared memory
   int band;           // units per band of the job order
-  int off_v, off_red, off_bar, smem, smem_x;  // key stages at offset 0
+  int off_v, off_r, off_q, off_red, off_bar, smem, smem_x;  // key units at offset 0
+};
+
+// A place in a ring of n units and the parity of its current round (units
+// are counted without dividing: a division takes a lone thread hundreds of
+// cycles).  A full barrier is awaited at parity `ph`, a free one at ph ^ 1
+// (which holds at once in the first round).
+struct PfRing {
+  int s = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next(int n) {
+    if (++s == n) {
+      s = 0;
+      ph ^= 1;
+    }
+  }
 };
 
 // Tiles a job reads: positions up to that of the job's last row.
@@ -71,27 +104,29 @@ __device__ __forceinline__ int pf_tiles(int len, int n_q, int G, int r_last) {
   return p_max >= 0 ? p_max / kPfT + 1 : 0;
 }
 
-// Expand: the keys and values of one 64-position tile of one unit, staged
-// raw (rotations undone), dequantised per (position, channel quarter) into
-// [K hi | K lo | V hi | V lo] (8 KB boxes; no lo halves for bf16 caches)
-// and stored for every job of the unit to copy.  Positions past the length
-// are zero.
+// Expand: the keys and values of 64 positions (half a tile) of one unit,
+// staged raw (rotations undone), dequantised per (position, channel quarter)
+// into [K hi | K lo | V hi | V lo] (8 KB boxes; no lo halves for bf16
+// caches) and stored in the tile's units for every job of the unit to copy.
+// Positions past the length are zero, to the end of the last tile.
 __global__ void __launch_bounds__(kPfWorkers) prefill_expand_kernel(const PfArgs a, const PfPlan p) {
   extern __shared__ uint8_t pf_raw[];
   uint8_t *sm = pf_raw + ((1024u - (smem_u32(pf_raw) & 1023u)) & 1023u);
   const GqaView &v = a.v;
-  const int tile = blockIdx.x, unit = blockIdx.y, tid = threadIdx.x;
+  constexpr int T = 64;
+  const int unit = blockIdx.y, tid = threadIdx.x;
   pdl_wait();
   const int len = v.lens[unit / v.Hkv];
-  const int t0 = tile * kPfT;
-  if (t0 >= len) {
+  const int t0 = blockIdx.x * T;
+  if (t0 >= (len + kPfT - 1) / kPfT * kPfT) {
     pdl_trigger();
     return;
   }
-  uint8_t *stg = sm + p.tbytes;
+  const int kbytes = p.ub;  // 64 positions of both key units
+  uint8_t *stg = sm + 2 * kbytes;
   const uint8_t *base = v.rec + (size_t)unit * v.cap * v.rec_bytes;
   const bool sym = p.fmt >= kFmtS8, bf = p.fmt == kFmtBf16;
-  for (int e = tid; e < kPfT * p.nrec; e += kPfWorkers) {
+  for (int e = tid; e < T * p.nrec; e += kPfWorkers) {
     const int pos = (int)__umulhi((uint32_t)e, p.nc_magic), c = e - pos * p.nrec;
     const int t = t0 + pos;
     const bool ok = t < len;
@@ -102,21 +137,21 @@ __global__ void __launch_bounds__(kPfWorkers) prefill_expand_kernel(const PfArgs
       so = p.ks16 + ((c - p.ks16 + v_rot(t, v.rec_bytes, p.ks16)) & (p.ks16 - 1));
     else
       so = c;
-    cp_async16(stg + pos * p.b_stride + 16 * c, base + (size_t)(ok ? t : t0) * v.rec_bytes + 16 * so, ok);
+    cp_async16(stg + pos * p.b_stride + 16 * c, base + (size_t)(ok ? t : 0) * v.rec_bytes + 16 * so, ok);
   }
   if (sym)
-    for (int pos = tid; pos < kPfT; pos += kPfWorkers) {
+    for (int pos = tid; pos < T; pos += kPfWorkers) {
       const int t = t0 + pos;
       const bool ok = t < len;
-      cp_async4(stg + pos * p.b_stride + v.rec_bytes, v.scales + (size_t)unit * v.cap + (ok ? t : t0), ok);
+      cp_async4(stg + pos * p.b_stride + v.rec_bytes, v.scales + (size_t)unit * v.cap + (ok ? t : 0), ok);
     }
   // per-channel keys: the (scale, zero) rows of the tile's complete groups
-  // of positions (kPfT >> gshift groups of 128 channels; rows of the open
+  // of positions (T >> gshift groups of 128 channels; rows of the open
   // group are zero and unused: those positions come from the residual)
   const int g0 = t0 >> p.gshift, full = (len >> p.gshift) << p.gshift;
-  float2 *mrows = reinterpret_cast<float2 *>(stg + kPfT * p.b_stride);
+  float2 *mrows = reinterpret_cast<float2 *>(stg + T * p.b_stride);
   if (p.kpc) {
-    const int ng = kPfT >> p.gshift;
+    const int ng = T >> p.gshift;
     for (int i = tid; i < ng * 128 * 8 / 16; i += kPfWorkers) {
       const int gi = i / 64, c = i - gi * 64;  // 64 chunks of 16 bytes per row
       const bool ok = ((g0 + gi) << p.gshift) < full;
@@ -128,7 +163,7 @@ __global__ void __launch_bounds__(kPfWorkers) prefill_expand_kernel(const PfArgs
   cp_async_wait<0>();
   __syncthreads();
   // threads [0, 256): key quarters; [256, 512): value quarters
-  const int pidx = tid & (kPfT - 1), part = tid / kPfT;
+  const int pidx = tid & (T - 1), part = tid / T;
   const uint8_t *bundle = stg + pidx * p.b_stride;
   const int ks = 16 * p.ks16;
   const int mb = (p.nrec * 16 - 2 * ks) / 2;  // grouped: one metadata block
@@ -167,7 +202,7 @@ __global__ void __launch_bounds__(kPfWorkers) prefill_expand_kernel(const PfArgs
     }
   } else {
     const int qc = part - 4;
-    uint8_t *vh = sm + p.kbytes, *vl = vh + 2 * kPfBox;
+    uint8_t *vh = sm + kbytes, *vl = vh + 2 * kPfBox;
     const uint8_t *vsec = bundle + ks, *vmeta = bundle + 2 * ks + (p.kpc ? 0 : mb);
     const float svs =
         sym ? __uint_as_float(*reinterpret_cast<const uint32_t *>(bundle + v.rec_bytes) & 0xFFFF0000u) : 0.f;
@@ -181,61 +216,86 @@ __global__ void __launch_bounds__(kPfWorkers) prefill_expand_kernel(const PfArgs
     }
   }
   __syncthreads();
-  uint4 *dst = reinterpret_cast<uint4 *>(a.tiles + ((size_t)unit * p.n_t64 + tile) * p.tbytes);
+  // shared: keys [hi box 0 | hi box 1 | lo box 0 | lo box 1], then values the
+  // same; key box b goes to unit b, half (hi, lo) h, rows 64 (half tile) on
+  uint8_t *dst = a.tiles + ((size_t)unit * p.n_t + (blockIdx.x >> 1)) * p.tbytes;
+  const int hf = blockIdx.x & 1;
+  constexpr int B16 = kPfBox / 16;
   const uint4 *src = reinterpret_cast<const uint4 *>(sm);
-  for (int i = tid; i < p.tbytes / 16; i += kPfWorkers) dst[i] = src[i];
+  for (int i = tid; i < kbytes / 16; i += kPfWorkers) {
+    const int x = i / B16, b = x & 1, h = x >> 1;
+    reinterpret_cast<uint4 *>(dst + b * p.ub + h * 2 * kPfBox + hf * kPfBox)[i - x * B16] = src[i];
+  }
+  uint4 *dv = reinterpret_cast<uint4 *>(dst + (2 + hf) * p.ub);
+  for (int i = tid; i < p.ub / 16; i += kPfWorkers) dv[i] = src[kbytes / 16 + i];
   pdl_trigger();
 }
 
-// S = Q K^T of one tile into TMEM columns d0.., Q (bf16 pairs, hi then lo
-// 64 columns on) from TMEM at t_q, the keys (hi, then lo 2 boxes on) K-major
-// in shared memory at kh: 16 channels per k-step.
+// S (+)= Q K^T of one key unit (64 channels) into TMEM columns d0.., 128
+// positions: Q (bf16 pairs) from TMEM at t_q, its lo halves 64 columns on;
+// the keys (hi, then lo 16 KB on) K-major in shared memory at k.
 template <bool KLO, bool QLO>
-__device__ __forceinline__ void pf_issue_scores(uint32_t d0, uint32_t t_q, uint32_t kh) {
+__device__ __forceinline__ void pf_issue_scores(uint32_t d0, uint32_t t_q, uint32_t k, bool acc) {
   constexpr uint32_t id = umma_idesc(128, kPfT, false, false);
   constexpr uint32_t hi = umma_desc_hi_sw128(1024);
-  const uint32_t lo_h = umma_desc_lo(kh, 16), lo_l = lo_h + (2 * kPfBox >> 4);
+  const uint32_t lo_h = umma_desc_lo(k, 16), lo_l = lo_h + (2 * kPfBox >> 4);
 #pragma unroll
-  for (int ks = 0; ks < 8; ++ks) {
-    const uint32_t ko = ((ks >> 2) * kPfBox + (ks & 3) * 32) >> 4;
-    umma_f16_ts_w(d0, t_q + 8 * ks, lo_h + ko, hi, id, ks > 0);
-    if (KLO) umma_f16_ts_w(d0, t_q + 8 * ks, lo_l + ko, hi, id, true);
-    if (QLO) umma_f16_ts_w(d0, t_q + 64 + 8 * ks, lo_h + ko, hi, id, true);
+  for (int ks = 0; ks < 4; ++ks) {
+    umma_f16_ts_w(d0, t_q + 8 * ks, lo_h + 2 * ks, hi, id, acc || ks > 0);
+    if (KLO) umma_f16_ts_w(d0, t_q + 8 * ks, lo_l + 2 * ks, hi, id, true);
+    if (QLO) umma_f16_ts_w(d0, t_q + 64 + 8 * ks, lo_h + 2 * ks, hi, id, true);
   }
 }
-// O += P V of one tile: P (bf16 pairs, hi then lo 32 columns on) from TMEM
-// at pa, the values (hi, then lo 2 boxes on) MN-major in shared memory at vh
-// (64-channel boxes kPfBox apart), 16 positions per k-step.
+// The same with Q's 64 channels K-major in shared memory at q (128 rows).
 template <bool KLO>
-__device__ __forceinline__ void pf_issue_values(uint32_t t_o, uint32_t pa, uint32_t vh, bool acc) {
+__device__ __forceinline__ void pf_issue_scores_ss(uint32_t d0, uint32_t q, uint32_t k, bool acc) {
+  constexpr uint32_t id = umma_idesc(128, kPfT, false, false);
+  const uint64_t da = umma_desc(q, 16, 1024, 2), dh = umma_desc(k, 16, 1024, 2);
+#pragma unroll
+  for (int ks = 0; ks < 4; ++ks) {
+    umma_f16(d0, da + (uint64_t)(2 * ks), dh + (uint64_t)(2 * ks), id, acc || ks > 0);
+    if (KLO) umma_f16(d0, da + (uint64_t)(2 * ks), dh + (uint64_t)((2 * kPfBox >> 4) + 2 * ks), id, true);
+  }
+}
+// O += P V of one value unit (64 positions): P (bf16 pairs, hi then lo 64
+// columns on) from TMEM at pa, the values (hi, then lo 2 boxes on) MN-major
+// in shared memory at vh (64-channel boxes kPfBox apart), 16 positions per
+// k-step; the products with a lo half into t_ol (t_o unless it is another).
+template <bool KLO, bool SPLIT>
+__device__ __forceinline__ void pf_issue_values(uint32_t t_o, uint32_t t_ol, uint32_t pa, uint32_t vh, bool acc) {
   constexpr uint32_t id = umma_idesc(128, 128, false, true);
   constexpr uint32_t hi = umma_desc_hi_sw128(1024);
   const uint32_t lo_h = umma_desc_lo(vh, kPfBox), lo_l = lo_h + (2 * kPfBox >> 4);
 #pragma unroll
-  for (int ks = 0; ks < kPfT / 16; ++ks) {
+  for (int ks = 0; ks < 4; ++ks) {
     umma_f16_ts_w(t_o, pa + 8 * ks, lo_h + 128 * ks, hi, id, acc || ks > 0);
-    if (KLO) umma_f16_ts_w(t_o, pa + 8 * ks, lo_l + 128 * ks, hi, id, true);
-    umma_f16_ts_w(t_o, pa + 32 + 8 * ks, lo_h + 128 * ks, hi, id, true);
+    if (KLO) umma_f16_ts_w(t_ol, pa + 8 * ks, lo_l + 128 * ks, hi, id, !SPLIT || acc || ks > 0);
+    umma_f16_ts_w(t_ol, pa + 64 + 8 * ks, lo_h + 128 * ks, hi, id, true);
   }
 }
 
+template <bool MLA>
 __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, const PfPlan p) {
   constexpr int D = 128;
   constexpr uint32_t kLimit = 1u << 20;  // polls of up to 2 us each
+  constexpr uint32_t kSpins = 1u << 26;  // polls of tens of cycles
   extern __shared__ uint8_t pf_raw[];
   uint8_t *sm = pf_raw + ((1024u - (smem_u32(pf_raw) & 1023u)) & 1023u);
-  // barriers: kfull[6] keys of a stage landed, kfree[6] its score product
-  // done, vfull[6] / vfree[6] the same for values; per tile parity: sdone[2]
-  // scores done, epi[2] the workers' epilogue done (16 arrivals), pvdone[2]
-  // value product done; qready the job's query rows staged (16 arrivals),
-  // drain[3] (one per MMA warp).  A barrier per parity completes every other tile, and the next
+  // barriers: kfull[8] keys of a unit landed, kfree[8] its score products
+  // done, vfull[8] / vfree[8] the same for values, rfull[2] / rfree[2] for
+  // the positional keys; per tile parity: sdone[2] scores done, epi[2][2] the
+  // workers' P of either value unit's positions written (16 arrivals),
+  // pvdone[2] value products done;
+  // qready the job's query rows staged (16 arrivals), drain[2] (one per MMA
+  // warp).  A barrier per parity completes every other tile, and the next
   // completion of one always depends on the wait for its previous one, so
   // no wait can fall two phases behind.
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm + p.off_bar);
-  constexpr int S6 = kPfMaxStages;
-  uint64_t *kfull = bar, *kfree = bar + S6, *vfull = bar + 2 * S6, *vfree = bar + 3 * S6;
-  uint64_t *sdone = bar + 4 * S6, *epi = sdone + 2, *pvdone = sdone + 4, *qready = sdone + 6, *drain = sdone + 7;
-  constexpr int kBars = 4 * S6 + 10;
+  constexpr int S8 = kPfMaxStages;
+  uint64_t *kfull = bar, *kfree = bar + S8, *vfull = bar + 2 * S8, *vfree = bar + 3 * S8;
+  uint64_t *rfull = bar + 4 * S8, *rfree = rfull + 2;
+  uint64_t *sdone = rfree + 2, *epi = sdone + 2, *pvdone = epi + 4, *qready = pvdone + 2, *drain = qready + 1;
+  constexpr int kBars = 4 * S8 + 4 + 11;
   static_assert(kBars * 8 + 12 <= kPfBarBytes, "barrier region");
   uint32_t *tbase = reinterpret_cast<uint32_t *>(sm + p.off_bar + kBars * 8);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + p.off_bar + kBars * 8 + 4);
@@ -246,12 +306,11 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
   const int quarter = warp & 3, slice = warp >> 2;
   const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
   const float sg = a.sig_log2;
-  const int vbytes = p.tbytes - p.kbytes;
 
   if (tid == 0) {
     for (int i = 0; i < kBars; ++i) {
       uint64_t *b = &bar[i];
-      mbar_init(b, (b == epi || b == epi + 1 || b == qready) ? kPfWorkers / 32 : 1);
+      mbar_init(b, ((b >= epi && b < epi + 4) || b == qready) ? kPfWorkers / 32 : 1);
     }
     *abort_flag = 0;
     fence_mbar_init();
@@ -270,13 +329,14 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
   tc_fence_after();
   const uint32_t tmem = *tbase;
   // TMEM columns (lane = the job's row in every region): scores of tile k
-  // at 64 (k & 1), fp32; the job's query rows as bf16 pairs (hi 64 columns,
-  // then lo), the A operand of the score products; output pass: O at 128
-  // (fp32, 128 channels) and P of tile k at 256 + 64 (k & 1) (bf16 pairs,
-  // hi 32 columns, then lo), the A operand of the value products.
-  const uint32_t t_o = tmem + 128;
+  // at 128 (k & 1), fp32, and in their place, once they are read, the tile's
+  // P (bf16 pairs, hi 64 columns, then lo), the A operand of the value
+  // products; O at 256 (fp32, 128 channels); at 384 the job's query rows as
+  // bf16 pairs (hi 64 columns, then lo), the A operand of the score products,
+  // or (MLA) the sum of the value products with a lo half.
+  const uint32_t t_o = tmem + 256, t_ol = MLA ? tmem + 384 : t_o;
   const uint32_t t_q = tmem + 384;
-  auto t_p = [&](int k) { return tmem + 256 + 64 * (k & 1); };
+  auto t_s = [&](int k) { return tmem + 128u * (k & 1); };
 
   // Jobs are handed out one at a time from a counter, so CTAs finish
   // together although jobs differ in length.  Order: bands of p.band units
@@ -306,6 +366,10 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
     const int rb = p.n_rb - 1 - step;
     J.b = J.unit / v.Hkv;
     J.j = J.unit - J.b * v.Hkv;
+    if constexpr (MLA) {
+      J.b += a.b0;
+      J.j += a.h0;
+    }
     J.r0 = rb * kPfRows;
     J.nr = min(kPfRows, R - J.r0);
     J.len = v.lens[J.b];
@@ -315,33 +379,46 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
   auto sleepy = [&](uint64_t *b, uint32_t parity) {
     return mbar_wait_sleepy(b, parity, kLimit, abort_flag, 2000);
   };
+  auto spin = [&](uint64_t *b, uint32_t parity) { return mbar_spin_or_abort(b, parity, kSpins, abort_flag); };
 
-  if (warp == kPfWorkers / 32 + 1) {
-    // ======================= copy warp ====================================
-    // lane 0 copies each tile's keys (and values) into the next stage once
-    // the products that read the stage's previous tile are done
-    int kk = 0;
+  if (warp == kPfWorkers / 32 + 1 || warp == kPfWorkers / 32 + 3) {
+    // ======================= copy warps ===================================
+    // lane 0 of one copies each tile's key units (and positional keys), of
+    // the other its value units, once the products that read the unit's
+    // place before are done
+    const bool keys = warp == kPfWorkers / 32 + 1;
+    uint64_t *full = keys ? kfull : vfull, *free_ = keys ? kfree : vfree;
+    const int n = keys ? p.nk : p.nv;
+    uint8_t *ring = sm + (keys ? 0 : p.off_v);
+    int c = 0, rc = 0;  // units (and positional tiles) copied
+    PfRing ru, rr;
     bool ok = true;
     for (int job = next_job(); job < p.n_jobs; job = next_job()) {
       if (ok && lane == 0) {
         const Job J = job_at(job);
-        const uint8_t *src0 = a.tiles + (size_t)J.unit * p.n_t64 * p.tbytes;
-        for (int k = 0; k < J.n_t && ok; ++k, ++kk) {
-          const int s = kk % p.ns, u = kk / p.ns;
-          if (u > 0) ok = sleepy(&kfree[s], (u - 1) & 1);
-          // the stage is written only by bulk copies and read only by the
-          // products (both async proxy, ordered by the commit's release of
-          // kfree): no proxy fence
-          if (ok) {
-            mbar_expect_tx(&kfull[s], p.kbytes);
-            bulk_g2s(sm + s * p.kbytes, src0 + (size_t)k * p.tbytes, p.kbytes, &kfull[s]);
-          }
-          if (ok) {
-            const int sv = kk % p.nv, uv = kk / p.nv;
-            if (uv > 0) ok = sleepy(&vfree[sv], (uv - 1) & 1);
+        const uint8_t *src = a.tiles + (size_t)J.unit * p.n_t * p.tbytes + (keys ? 0 : 2 * p.ub);
+        for (int k = 0; k < J.n_t && ok; ++k) {
+          for (int u = 0; u < 2 && ok; ++u) {
+            const int s = ru.s;
+            ok = sleepy(&free_[s], ru.ph ^ 1);
+            // the unit's place is written only by bulk copies and read only
+            // by the products (both async proxy, ordered by the commit's
+            // release of kfree / vfree): no proxy fence
             if (ok) {
-              mbar_expect_tx(&vfull[sv], vbytes);
-              bulk_g2s(sm + p.off_v + sv * vbytes, src0 + (size_t)k * p.tbytes + p.kbytes, vbytes, &vfull[sv]);
+              mbar_expect_tx(&full[s], p.ub);
+              bulk_g2s(ring + s * p.ub, src + (size_t)k * p.tbytes + u * p.ub, p.ub, &full[s]);
+              ++c;
+              ru.next(n);
+            }
+          }
+          if (MLA && keys && ok) {
+            const int s = rr.s;
+            ok = sleepy(&rfree[s], rr.ph ^ 1);
+            if (ok) {
+              mbar_expect_tx(&rfull[s], p.krb);
+              bulk_g2s(sm + p.off_r + s * p.krb, a.kr + ((size_t)(J.b - a.b0) * p.n_t + k) * p.krb, p.krb, &rfull[s]);
+              ++rc;
+              rr.next(p.nr);
             }
           }
         }
@@ -351,57 +428,22 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
     }
     // the last copies land before the CTA leaves (bounded; at once when
     // they were consumed)
-    if (lane == 0)
-      for (int c = max(0, kk - max(p.ns, p.nv)); c < kk; ++c) {
-        if (c >= kk - p.ns) mbar_wait(&kfull[c % p.ns], (c / p.ns) & 1, 1u << 22);
-        if (c >= kk - p.nv) mbar_wait(&vfull[c % p.nv], (c / p.nv) & 1, 1u << 22);
-      }
+    if (lane == 0) {
+      for (int u = max(0, c - n); u < c; ++u) mbar_wait(&full[u % n], (u / n) & 1, 1u << 22);
+      for (int u = max(0, rc - p.nr); u < rc; ++u) mbar_wait(&rfull[u % p.nr], (u / p.nr) & 1, 1u << 22);
+    }
     __syncwarp();
   } else if (warp >= kPfWorkers / 32) {
     // ======================= MMA warps ====================================
-    // Each warp's lane 0 issues a stream of products (one thread issues at
-    // most one product per ~45 cycles, so several streams keep the tensor
-    // cores busy): warps 16 and 18 the score products of the even and the
-    // odd tiles, warp 19 (output pass) the value products.  A commit covers
-    // the products its own thread issued.
-    const int role = warp == kPfWorkers / 32 ? 0 : warp == kPfWorkers / 32 + 2 ? 1 : 2;
-    auto issue_s = [&](int kk, int s) {  // S = Q K^T of the tile in key stage s
-      tc_fence_after();
-      const uint32_t kh = smem_u32(sm + s * p.kbytes), d0 = tmem + 64u * (kk & 1);
-      if (p.k_lo) {
-        if (p.q_lo) pf_issue_scores<true, true>(d0, t_q, kh);
-        else pf_issue_scores<true, false>(d0, t_q, kh);
-      } else {
-        if (p.q_lo) pf_issue_scores<false, true>(d0, t_q, kh);
-        else pf_issue_scores<false, false>(d0, t_q, kh);
-      }
-      umma_commit(&sdone[kk & 1]);
-      umma_commit(&kfree[s]);
-    };
-    auto issue_pv = [&](int c, int s, bool acc) {  // O += P V of tile c, values in stage s
-      tc_fence_after();
-      const uint32_t vh = smem_u32(sm + p.off_v + s * vbytes);
-      if (p.k_lo) pf_issue_values<true>(t_o, t_p(c), vh, acc);
-      else pf_issue_values<false>(t_o, t_p(c), vh, acc);
-      umma_commit(&pvdone[c & 1]);
-      umma_commit(&vfree[s]);
-    };
-    auto wait_epi = [&](int c) -> bool {  // the workers' epilogue of tile c
-      return c < 0 || sleepy(&epi[c & 1], (c >> 1) & 1);
-    };
-    auto pv = [&](int c, bool acc) -> bool {  // value product of tile c once its P is written
-      const int s = c % p.nv;
-      bool ok = wait_epi(c);
-      if (ok) ok = sleepy(&vfull[s], (c / p.nv) & 1);
-      if (ok) issue_pv(c, s, acc);
-      return ok;
-    };
-    // Barrier phases: a score warp waits for epi(c) (its parity's previous
-    // phase) before S(c + 2), and epi[c & 1] completes for tile c + 2 only
-    // after S(c + 2); the value warp waits for every epi(c) in order before
-    // PV(c), which the workers await before the epilogue of c + 2.  So every
-    // wait is for the phase after the one its warp last saw.
-    int kk = 0, njob = 0, issued = 0;
+    // lane 0 of one issues the score products, of the other the value
+    // products; a commit covers the products its own thread issued
+    const bool scores = warp == kPfWorkers / 32;
+    // Barrier phases: S(c + 2) takes the columns of P(c), so its warp waits
+    // for PV(c) first, and PV(c + 2) needs S(c + 2); the value warp waits for
+    // every epi(c) in order before PV(c), and epi(c + 2) needs S(c + 2).  So
+    // every wait is for the phase after the one its warp last saw.
+    int kk = 0, njob = 0, c = 0;
+    PfRing ru, rr;
     bool ok = true;
     for (int job = next_job(); job < p.n_jobs; job = next_job()) {
       if (ok && lane == 0) {
@@ -410,15 +452,51 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
         ok = sleepy(qready, njob & 1);
         ++njob;
         for (int k = 0; k < J.n_t && ok; ++k, ++kk) {
-          if ((kk & 1) == role) {
-            const int s = kk % p.ns;
-            if (kk >= 2) ok = wait_epi(kk - 2);  // the score buffer of tile kk - 2 is read
-            if (ok) ok = sleepy(&kfull[s], (kk / p.ns) & 1);
-            if (ok) issue_s(kk, s);
-            ++issued;
-          } else if (role == 2) {
-            ok = pv(kk, k > 0);
-            ++issued;
+          if (scores) {
+            if (kk >= 2) ok = spin(&pvdone[kk & 1], ((kk >> 1) - 1) & 1);  // P(kk - 2) is read
+            for (int u = 0; u < 2 && ok; ++u, ++c, ru.next(scores ? p.nk : p.nv)) {
+              const int s = ru.s;
+              ok = spin(&kfull[s], ru.ph);
+              if (!ok) break;
+              tc_fence_after();
+              const uint32_t ku = smem_u32(sm + s * p.ub);
+              if constexpr (MLA) {
+                pf_issue_scores_ss<true>(t_s(kk), smem_u32(sm + p.off_q) + u * 16384, ku, u > 0);
+              } else if (p.k_lo) {
+                if (p.q_lo) pf_issue_scores<true, true>(t_s(kk), t_q + 32 * u, ku, u > 0);
+                else pf_issue_scores<true, false>(t_s(kk), t_q + 32 * u, ku, u > 0);
+              } else {
+                if (p.q_lo) pf_issue_scores<false, true>(t_s(kk), t_q + 32 * u, ku, u > 0);
+                else pf_issue_scores<false, false>(t_s(kk), t_q + 32 * u, ku, u > 0);
+              }
+              umma_commit(&kfree[s]);
+            }
+            if constexpr (MLA) {
+              const int s = rr.s;
+              if (ok) ok = spin(&rfull[s], rr.ph);
+              if (ok) {
+                tc_fence_after();
+                const uint32_t q = smem_u32(sm + p.off_q) + 32768, kr = smem_u32(sm + p.off_r + s * p.krb);
+                if (p.krb > 16384) pf_issue_scores_ss<true>(t_s(kk), q, kr, true);
+                else pf_issue_scores_ss<false>(t_s(kk), q, kr, true);
+                umma_commit(&rfree[s]);
+                rr.next(p.nr);
+              }
+            }
+            if (ok) umma_commit(&sdone[kk & 1]);
+          } else {
+            for (int u = 0; u < 2 && ok; ++u, ++c, ru.next(scores ? p.nk : p.nv)) {
+              const int s = ru.s;
+              ok = spin(&vfull[s], ru.ph);
+              if (ok) ok = spin(&epi[2 * (kk & 1) + u], (kk >> 1) & 1);
+              if (!ok) break;
+              tc_fence_after();
+              const uint32_t vh = smem_u32(sm + p.off_v + s * p.ub), pa = t_s(kk) + 32 * u;
+              if (MLA || p.k_lo) pf_issue_values<true, MLA>(t_o, t_ol, pa, vh, k > 0 || u > 0);
+              else pf_issue_values<false, false>(t_o, t_o, pa, vh, k > 0 || u > 0);
+              umma_commit(&vfree[s]);
+            }
+            if (ok) umma_commit(&pvdone[kk & 1]);
           }
         }
         if (!ok) *abort_flag = 1;
@@ -426,9 +504,10 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
       ok = __shfl_sync(0xffffffffu, ok, 0);
     }
     // every product this warp issued lands before TMEM is released (bounded)
-    if (lane == 0 && issued > 0) {
-      umma_commit(&drain[role]);
-      mbar_wait(&drain[role], 0, 1u << 22);  // drain[0..2]
+    if (lane == 0 && c > 0) {
+      uint64_t *d = &drain[scores ? 0 : 1];
+      umma_commit(d);
+      mbar_wait(d, 0, 1u << 22);
     }
     __syncwarp();
   } else {
@@ -437,9 +516,8 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
     auto wait_pv = [&](int c) -> bool {  // completion of tile c's value product
       return c < 0 || sleepy(&pvdone[c & 1], (c >> 1) & 1);
     };
-    // query rows r0 .. r0 + 127 of the unit (zero past R) into TMEM, this
-    // thread's row and quarter of the channels; output pass: the rows'
-    // log-normalisers (+inf for rows that see no position)
+    // query rows r0 .. r0 + 127 of the unit (zero past R) into TMEM (MLA:
+    // shared memory), this thread's row and quarter of the channels
     auto load_q = [&](const Job &J) {
       const int rl = 32 * quarter + lane;
       float x[32];
@@ -473,15 +551,38 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
       uint32_t hw[16], lw[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) split2<true>(x[2 * i], x[2 * i + 1], hw[i], lw[i]);
-      tmem_st16_nw(t_q + 16 * slice + lane_off, hw);
-      if (p.q_lo) tmem_st16_nw(t_q + 64 + 16 * slice + lane_off, lw);
-      tmem_wait_st();
+      if constexpr (MLA) {
+        // the row's 32 content channels and 16 of its positional ones, K-major
+        // boxes of 64 channels in shared memory
+        uint8_t *q_s = sm + p.off_q;
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc)
+          put_chunk(q_s, rl, 32 * slice + 8 * cc, 16384,
+                    make_uint4(hw[4 * cc], hw[4 * cc + 1], hw[4 * cc + 2], hw[4 * cc + 3]));
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) {
+          uint4 u = make_uint4(0, 0, 0, 0);
+          if (rl < J.nr)
+            u = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(a.q_pe) +
+                                                (((size_t)J.b * a.n_q + J.r0 + rl) * a.Hq + J.j) * 64 + 16 * slice)[cc];
+          put_chunk(q_s, rl, 128 + 16 * slice + 8 * cc, 16384, u);
+        }
+        fence_proxy_async();
+      } else {
+        tmem_st16_nw(t_q + 16 * slice + lane_off, hw);
+        if (p.q_lo) tmem_st16_nw(t_q + 64 + 16 * slice + lane_off, lw);
+        tmem_wait_st();
+      }
       tc_fence_before();  // the rows, stored here, are read by the tensor cores
       workers_sync<kPfWorkers>();
     };
 
     int kk = 0;
-    float *smax = reinterpret_cast<float *>(sm + p.off_red);  // [4 slices][128 rows]
+    // [tile parity][4 slices][128 rows]: the rows' slice maxima
+    float *smax = reinterpret_cast<float *>(sm + p.off_red);
+    // The four warps that share a quarter of the rows meet on a barrier of
+    // their own: a row's maximum and its columns concern no other warp.
+    auto row_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(4 + quarter) : "memory"); };
     for (int job = next_job(); job < p.n_jobs; job = next_job()) {
       if (failed) continue;
       const Job J = job_at(job);
@@ -499,36 +600,39 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
       // threads move it and rescale their channels of O (in TMEM, after the
       // value product of the previous tile) and their sums.  The weights
       // are not normalised: O is divided by the row's sum at the end.
+      // A warp whose wait gave up stays in the tile loop for the barriers.
       float c_ref = -INFINITY, l_run = 0.f;
       for (int k = 0; k < J.n_t; ++k, ++kk) {
-        // scores of this tile, and its P buffer free
-        bool ok = !failed && sleepy(&sdone[kk & 1], (kk >> 1) & 1);
-        if (ok) ok = wait_pv(kk - 2);
-        if (workers_sync_or<kPfWorkers>(!ok)) {
+        // scores of this tile (issued once the buffer's last P was read)
+        if (!failed && !__all_sync(0xffffffffu, spin(&sdone[kk & 1], (kk >> 1) & 1))) {
           failed = true;
           *abort_flag = 1;
-          break;
         }
         tc_fence_after();
-        const int tb = k * kPfT + 16 * slice;  // first position of this thread's slice
-        const int nv = row_live ? min(16, last - tb + 1) : 0;  // live positions (<= 0: none)
-        float y[16];
-        tmem_ld16(tmem + 64u * (kk & 1) + 16 * slice + lane_off, y);
+        // this thread's positions: 16 of either value unit's 64
+        const int tb = k * kPfT + 16 * slice;
+        const int nv0 = row_live ? last - tb + 1 : 0, nv1 = nv0 - 64;  // live ones if < 16 (<= 0: none)
+        float y[32];
+        tmem_ld16x2(t_s(kk) + 16 * slice + lane_off, t_s(kk) + 64 + 16 * slice + lane_off, y);
         float mx = -INFINITY;
-        if (nv >= 16) {  // the whole slice is in the row's range (most tiles)
-          float mm[4];
+        if (row_live && nv1 >= 16) {  // all in the row's range (most tiles)
+          float mm[8];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) mm[i] = fmaxf(fmaxf(y[i], y[4 + i]), fmaxf(y[8 + i], y[12 + i]));
-          mx = fmaxf(fmaxf(mm[0], mm[1]), fmaxf(mm[2], mm[3]));
+          for (int i = 0; i < 8; ++i) mm[i] = fmaxf(fmaxf(y[i], y[8 + i]), fmaxf(y[16 + i], y[24 + i]));
+          mx = fmaxf(fmaxf(fmaxf(mm[0], mm[1]), fmaxf(mm[2], mm[3])), fmaxf(fmaxf(mm[4], mm[5]), fmaxf(mm[6], mm[7])));
         } else {
 #pragma unroll
-          for (int i = 0; i < 16; ++i)
-            if (i < nv) mx = fmaxf(mx, y[i]);
+          for (int i = 0; i < 16; ++i) {
+            if (i < nv0) mx = fmaxf(mx, y[i]);
+            if (i < nv1) mx = fmaxf(mx, y[16 + i]);
+          }
         }
-        smax[slice * kPfRows + rl] = mx;
-        workers_sync<kPfWorkers>();  // the row's four slice maxima
-        const float M = sg * fmaxf(fmaxf(smax[rl], smax[kPfRows + rl]),
-                                   fmaxf(smax[2 * kPfRows + rl], smax[3 * kPfRows + rl]));
+        float *sx = smax + (kk & 1) * 4 * kPfRows + rl;
+        sx[slice * kPfRows] = mx;
+        tc_fence_before();
+        row_sync();  // the row's four slice maxima; its scores are all read
+        tc_fence_after();
+        const float M = sg * fmaxf(fmaxf(sx[0], sx[kPfRows]), fmaxf(sx[2 * kPfRows], sx[3 * kPfRows]));
         const bool move = M > c_ref + 8.f;  // the same decision on the row's four threads
         const bool resc = move && c_ref != -INFINITY;
         if (__any_sync(0xffffffffu, resc)) {
@@ -545,48 +649,47 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
             float z[16];
             uint32_t zw[16];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              tmem_ld16(t_o + 32 * slice + 16 * h + lane_off, z);
+            for (int h = 0; h < (MLA ? 4 : 2); ++h) {
+              const uint32_t at = (h < 2 ? t_o : t_ol) + 32 * slice + 16 * (h & 1) + lane_off;
+              tmem_ld16(at, z);
 #pragma unroll
               for (int i = 0; i < 16; ++i) zw[i] = __float_as_uint(z[i] * f);
-              tmem_st16_nw(t_o + 32 * slice + 16 * h + lane_off, zw);
+              tmem_st16_nw(at, zw);
             }
             l_run *= f;
           }
         }
         if (move) c_ref = M;
-        // P of this row over the slice's 16 positions, hi and lo halves
-        float x0[8], x1[8];
-        if (nv >= 16) {
+        // P of this row over its positions of one value unit, then of the
+        // other, hi and lo halves: 8 columns of bf16 pairs (hi), the same 64
+        // columns on (lo); the unit's value products start as soon as its
+        // positions are written
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int nv = u ? nv1 : nv0;
+          float *yu = y + 16 * u;
+          if (nv >= 16) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) yu[i] = fast_exp2(fmaf(yu[i], sg, -c_ref));
+          } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) yu[i] = i < nv ? fast_exp2(fmaf(yu[i], sg, -c_ref)) : 0.f;
+          }
+          uint32_t hw[8], lw[8];
+          float ls[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            x0[i] = fast_exp2(fmaf(y[i], sg, -c_ref));
-            x1[i] = fast_exp2(fmaf(y[8 + i], sg, -c_ref));
+            split2<true>(yu[2 * i], yu[2 * i + 1], hw[i], lw[i]);
+            ls[i & 3] += yu[2 * i] + yu[2 * i + 1];
           }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            x0[i] = i < nv ? fast_exp2(fmaf(y[i], sg, -c_ref)) : 0.f;
-            x1[i] = 8 + i < nv ? fast_exp2(fmaf(y[8 + i], sg, -c_ref)) : 0.f;
-          }
+          l_run += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+          tmem_st8_nw(t_s(kk) + 32 * u + 8 * slice + lane_off, hw);
+          tmem_st8_nw(t_s(kk) + 64 + 32 * u + 8 * slice + lane_off, lw);
+          tmem_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&epi[2 * (kk & 1) + u]);
         }
-        // positions 16 slice .. 16 slice + 15 of the tile: 8 columns of
-        // bf16 pairs (hi), the same 32 columns on (lo)
-        uint32_t hw[8], lw[8];
-        float ls[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          split2<true>(x0[2 * i], x0[2 * i + 1], hw[i], lw[i]);
-          split2<true>(x1[2 * i], x1[2 * i + 1], hw[4 + i], lw[4 + i]);
-          ls[i] += (x0[2 * i] + x0[2 * i + 1]) + (x1[2 * i] + x1[2 * i + 1]);
-        }
-        l_run += (ls[0] + ls[1]) + (ls[2] + ls[3]);
-        tmem_st8_nw(t_p(kk) + 8 * slice + lane_off, hw);
-        tmem_st8_nw(t_p(kk) + 32 + 8 * slice + lane_off, lw);
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&epi[kk & 1]);
       }
       // a rescale's wait that gave up on the last tile is seen by every worker
       if (workers_sync_or<kPfWorkers>(failed)) {
@@ -594,8 +697,9 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
         *abort_flag = 1;
         continue;
       }
-      // O: lane = the job's row, 32 channels per slice, divided by the sum
-      // of the row's weights (the four slices' sums, same reference)
+      // O (MLA: and the lo products' sum), lane = the job's row, 32 channels
+      // per slice, divided by the sum of the row's weights (the four slices'
+      // sums, same reference)
       float o[32];
       if (J.n_t > 0) {
         const bool ok = wait_pv(kk - 1);
@@ -605,13 +709,16 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
           continue;
         }
         tc_fence_after();
-        float z[16];
-        tmem_ld16(t_o + 32 * slice + lane_off, z);
+        tmem_ld32(t_o + 32 * slice + lane_off, o);
+        if constexpr (MLA) {
+          float z[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) o[i] = z[i];
-        tmem_ld16(t_o + 32 * slice + 16 + lane_off, z);
+          for (int h = 0; h < 2; ++h) {
+            tmem_ld16(t_ol + 32 * slice + 16 * h + lane_off, z);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) o[16 + i] = z[i];
+            for (int i = 0; i < 16; ++i) o[16 * h + i] += z[i];
+          }
+        }
       } else {
 #pragma unroll
         for (int i = 0; i < 32; ++i) o[i] = 0.f;
@@ -642,18 +749,18 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
   pdl_trigger();
 }
 
-// Shared-memory plan.  Attention kernel: the key stages, the value stages,
-// the rows' slice maxima (and at a job's end their sums of weights),
-// barriers; the query rows, S, P and O live in TMEM.  Expand kernel: one
-// tile and its staged records.
+// Shared-memory plan.  Attention kernel: the key units, the value units,
+// MLA's positional keys and query rows, the rows' slice maxima (and at a
+// job's end their sums of weights), barriers; S, P, O and else the query
+// rows live in TMEM.  Expand kernel: half a tile and its staged records.
 PfPlan pf_plan(const PfArgs &a, int sms) {
   PfPlan p;
   const int R = a.n_q * a.G;
   p.n_rb = (R + kPfRows - 1) / kPfRows;
   p.n_jobs = a.v.B * a.v.Hkv * p.n_rb;
-  p.n_t64 = a.v.cap / kPfT;
+  p.n_t = (int)((a.v.cap + kPfT - 1) / kPfT);
   p.q_lo = a.q_f32 ? 1 : 0;
-  p.k_lo = a.v.bits != 16 ? 1 : 0;
+  p.k_lo = a.v.bits != 16 || a.kr_bytes ? 1 : 0;  // formed keys and values have lo halves
   p.fmt = a.v.bits == 16 ? kFmtBf16
           : a.v.scheme == kSchemeSym ? (a.v.bits == 8 ? kFmtS8 : a.v.bits == 4 ? kFmtS4 : kFmtS2)
                                      : (a.v.bits == 8 ? kFmtG8 : kFmtG4);
@@ -665,25 +772,28 @@ PfPlan pf_plan(const PfArgs &a, int sms) {
   const bool sym = p.fmt >= kFmtS8;
   const int bchunks = p.nrec + (sym ? 1 : 0);
   p.b_stride = 16 * (bchunks % 2 ? bchunks : bchunks + 1);
-  p.kbytes = 2 * kPfBox * (p.k_lo ? 2 : 1);
-  p.tbytes = 2 * p.kbytes;
+  p.ub = 2 * kPfBox * (p.k_lo ? 2 : 1);
+  p.tbytes = 4 * p.ub;
+  p.krb = a.kr_bytes;
   // + the (scale, zero) rows of the tile's position groups (per-channel keys)
-  p.smem_x = p.tbytes + kPfT * p.b_stride + (p.kpc ? 2 * 128 * 8 : 0) + 1024;
-  const int vb = p.tbytes - p.kbytes;
-  const int rbytes = 4 * kPfRows * 4;
-  // the most stages that fit.  Value tiles wait for the value product three
-  // tiles back, key tiles only for the score product, so values get the
-  // larger share (int4: 2 key and 5 value stages of 32 KB); keys keep at
-  // least two (a score warp's wait for the stage it skipped relies on ns >= 2).
-  const int avail = 232448 - (rbytes + kPfBarBytes + 1024);
-  const int T = avail / p.kbytes;  // key and value tiles are the same size
-  p.ns = std::min(kPfMaxStages, std::max(2, T / 3));
-  p.nv = std::max(1, std::min(kPfMaxStages, T - p.ns));
+  p.smem_x = 2 * p.ub + 64 * p.b_stride + (p.kpc ? 2 * 128 * 8 : 0) + 1024;
+  const int rbytes = 2 * 4 * kPfRows * 4;
+  const int qbytes = p.krb ? 3 * 16384 : 0;
+  // the most units that fit, values the larger share (a value unit waits for
+  // the epilogue of its tile, key units only for the tile before)
+  int avail = 232448 - (rbytes + kPfBarBytes + 1024) - qbytes;
+  p.nr = p.krb ? (p.krb <= 16384 ? 2 : 1) : 0;
+  avail -= p.nr * p.krb;
+  const int T = avail / p.ub;
+  p.nk = std::min(kPfMaxStages, std::max(2, T / 2));
+  p.nv = std::max(1, std::min(kPfMaxStages, T - p.nk));
   // bands of units whose tiles take up to 32 MB (L2 holds two bands)
-  const long long unit_bytes = (long long)p.n_t64 * p.tbytes;
+  const long long unit_bytes = (long long)p.n_t * p.tbytes;
   p.band = (int)std::max(1LL, std::min<long long>(a.v.B * a.v.Hkv, (32LL << 20) / std::max(1LL, unit_bytes)));
-  p.off_v = p.ns * p.kbytes;
-  p.off_red = p.off_v + p.nv * vb;
+  p.off_v = p.nk * p.ub;
+  p.off_r = p.off_v + p.nv * p.ub;
+  p.off_q = p.off_r + p.nr * p.krb;
+  p.off_red = p.off_q + qbytes;
   p.off_bar = p.off_red + rbytes;
   // + alignment of the base to 1024 bytes; at least half the SM's shared
   // memory, so that one CTA (holding its TMEM columns) runs per SM
@@ -694,33 +804,54 @@ PfPlan pf_plan(const PfArgs &a, int sms) {
 
 }  // namespace
 
-size_t prefill_tile_bytes(int bits) { return (size_t)2 * 2 * kPfBox * (bits != 16 ? 2 : 1); }
+size_t prefill_unit_bytes(int bits, int64_t cap) {
+  return (size_t)((cap + kPfT - 1) / kPfT) * 8 * kPfBox * (bits != 16 ? 2 : 1);
+}
 
 bool prefill_plan_fits(const PfArgs &a) {
   const PfPlan o = pf_plan(a, 1);
-  return o.smem <= 232448 && o.ns >= 2 && o.nv >= 2;
+  return o.smem <= 232448 && o.nk >= 2 && o.nv >= 2;
+}
+
+static cudaError_t pf_sms(int *out) {
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0, n = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    sms = n;
+  }
+  *out = sms;
+  return cudaSuccess;
+}
+
+cudaError_t launch_mla_prefill_formed(const PfArgs &a, cudaStream_t st) {
+  int sms = 0;
+  cudaError_t e = pf_sms(&sms);
+  if (e != cudaSuccess) return e;
+  const PfPlan p = pf_plan(a, sms);
+  e = cudaFuncSetAttribute(prefill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+  if (e == cudaSuccess)
+    e = launch_pdl(prefill_kernel<true>, dim3(p.grid), dim3(kPfThreads), p.smem, st, a, p);
+  return e;
 }
 
 cudaError_t launch_gqa_prefill(const PfArgs &a, cudaStream_t st) {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
+  int sms = 0;
+  cudaError_t e = pf_sms(&sms);
+  if (e != cudaSuccess) return e;
   const PfPlan po = pf_plan(a, sms);
-  cudaError_t e = cudaFuncSetAttribute(prefill_expand_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       po.smem_x);
+  e = cudaFuncSetAttribute(prefill_expand_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, po.smem_x);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, po.smem);
+    e = cudaFuncSetAttribute(prefill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, po.smem);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);  // the job counter
   if (e == cudaSuccess)
-    e = launch_pdl(prefill_expand_kernel, dim3(po.n_t64, a.v.B * a.v.Hkv), dim3(kPfWorkers), po.smem_x, st,
+    e = launch_pdl(prefill_expand_kernel, dim3(2 * po.n_t, a.v.B * a.v.Hkv), dim3(kPfWorkers), po.smem_x, st,
                    a, po);
   if (e == cudaSuccess)
-    e = launch_pdl(prefill_kernel, dim3(po.grid), dim3(kPfThreads), po.smem, st, a, po);
+    e = launch_pdl(prefill_kernel<false>, dim3(po.grid), dim3(kPfThreads), po.smem, st, a, po);
   return e;
 }
 

@@ -56,6 +56,32 @@ __device__ __forceinline__ void umma_f16_ts_w(uint32_t d_tmem, uint32_t a_tmem, 
       "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate ? 1 : 0)
       : "memory");
 }
+// The same three for a whole warp that runs its issue loop uniformly: only
+// the lane with `el` set issues.  Operands then live in uniform registers; a
+// loop under `if (lane == 0)` moves each operand of each product there first.
+__device__ __forceinline__ void umma_f16_ts_el(uint32_t el, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo,
+                                               uint32_t b_hi, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 db;\n setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n mov.b64 db, {%2, %3};\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate ? 1 : 0), "r"(el)
+      : "memory");
+}
+__device__ __forceinline__ void umma_f16_el(uint32_t el, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
+                                            uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n mov.b64 da, {%1, %3};\n"
+      " mov.b64 db, {%2, %3};\n @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate ? 1 : 0), "r"(el)
+      : "memory");
+}
+__device__ __forceinline__ void umma_commit_el(uint32_t el, uint64_t *bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(bar)),
+      "r"(el)
+      : "memory");
+}
 // the words of umma_desc(addr, lbo, sbo, 2) (128-byte swizzle)
 __device__ __forceinline__ uint32_t umma_desc_lo(uint32_t addr, uint32_t lbo) {
   return ((addr >> 4) & 0x3FFF) | (((lbo >> 4) & 0x3FFF) << 16);
@@ -99,6 +125,23 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr)
       : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+// two runs of 16 TMEM columns of this warp's 32 lanes, two loads and one wait
+__device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, float (&v)[32]) {
+  uint32_t r[32];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[16 * h]), "=r"(r[16 * h + 1]), "=r"(r[16 * h + 2]), "=r"(r[16 * h + 3]), "=r"(r[16 * h + 4]),
+          "=r"(r[16 * h + 5]), "=r"(r[16 * h + 6]), "=r"(r[16 * h + 7]), "=r"(r[16 * h + 8]), "=r"(r[16 * h + 9]),
+          "=r"(r[16 * h + 10]), "=r"(r[16 * h + 11]), "=r"(r[16 * h + 12]), "=r"(r[16 * h + 13]),
+          "=r"(r[16 * h + 14]), "=r"(r[16 * h + 15])
+        : "r"(h ? tb : ta)
+        : "memory");
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
@@ -167,6 +210,23 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t *bar, uint32_t parit
         : "memory");
     if (ok) return true;
     if ((i & 63) == 63 && *abort_flag) return false;
+  }
+  return false;
+}
+// The same by polls that never suspend the thread (a suspended waiter takes
+// hundreds of cycles to come back): for the hand-offs of a short chain.
+__device__ __forceinline__ bool mbar_spin_or_abort(uint64_t *bar, uint32_t parity, uint32_t limit,
+                                                   const volatile int *abort_flag) {
+  const uint32_t a = smem_u32(bar);
+  for (uint32_t i = 0; i < limit; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(a), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if ((i & 1023) == 1023 && *abort_flag) return false;
   }
   return false;
 }

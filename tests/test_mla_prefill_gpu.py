@@ -5,6 +5,7 @@ against the oracle's unabsorbed chunk attention on the dequantised cache.
 Ragged lengths, one sequence shorter than the chunk, an inheriting layer;
 bf16 chunks of an even number of rows decode two rows per CTA at d >= 256
 (a pair may hold an empty row beside a one-position row), odd ones one."""
+import ctypes
 import math
 
 import numpy as np
@@ -98,4 +99,78 @@ def test_mla_prefill_row_pairs(width, n_q, heads):
     assert (f32(out[2, :empty]) == 0).all()
     if empty < n_q:
         assert (np.abs(f32(out[2, empty])) > 0).any()  # the one-position row
+    assert c.device_error() == 0
+
+
+def _scratch(c, n_q):
+    out = ctypes.c_size_t()
+    assert c.lib.kvk_prefill_scratch_size(c.handle, 0, n_q, ctypes.byref(out)) == 0
+    return out.value
+
+
+@pytest.mark.parametrize("width,fmt", [(512, None), (256, None), (128, None), (64, None), (512, ("grouped", 8)),
+                                       (256, ("grouped", 4)), (128, ("symmetric", 8)), (64, ("symmetric", 4)),
+                                       (512, ("symmetric", 2))],
+                         ids=lambda x: str(x) if isinstance(x, int) else "bf16" if x is None else f"{x[0][:3]}{x[1]}")
+@pytest.mark.parametrize("n_q,heads", [(256, 16), (387, 5)], ids=["nq256", "nq387-h5"])
+def test_mla_prefill_formed(width, fmt, n_q, heads):
+    """Chunks long enough to attend over keys and values formed per head: two
+    whole row blocks and a remainder, lengths at, one past and one short of
+    the 64- and 128-position blocks, sequences shorter than the chunk and an
+    empty one."""
+    lens = [385, 256, 191, 20, 0, 129]
+    c, wk, wv, c_hat, kr_hat = _setup(width, fmt, lens, 400, seed=width + n_q, H=heads)
+    g = torch.Generator().manual_seed(7)
+    qn = torch.randn((len(lens), n_q, heads, 128), generator=g).to(torch.bfloat16)
+    qp = torch.randn((len(lens), n_q, heads, 64), generator=g).to(torch.bfloat16)
+    sigma = 1.0 / math.sqrt(192)
+    assert _scratch(c, n_q) == _scratch(c, 400)  # the formed tiles' size, which no chunk changes
+    out = c.prefill_mla(0, qn.cuda(), qp.cuda(), wk.cuda(), wv.cuda(), sigma)
+    ref = oatt.mla_prefill_unabsorbed(f32(qn), f32(qp), c_hat, kr_hat, f32(wk), f32(wv), width, lens, sigma)
+    assert_close(f32(out), ref, what=f"formed d={width} {fmt} n_q={n_q} H={heads}")
+    assert (f32(out[3, : n_q - 20]) == 0).all() and (f32(out[4]) == 0).all()
+    assert c.device_error() == 0
+
+
+@pytest.mark.parametrize("cap", [262144, 65536], ids=["head-groups", "sequence-groups"])
+def test_mla_prefill_formed_groups(cap):
+    """Contexts whose formed tiles pass 2 GiB: the heads (262144 positions: 8
+    heads at a time) or the sequences (65536: 2 of 3 at a time) go in groups
+    through the same scratch.  The same call over a small cache is equal."""
+    lens, n_q = [333, 70, 200], 300
+    outs = []
+    for T in (cap, 400):
+        n = lens if T != 262144 and cap != 262144 else lens[:1]
+        c, wk, wv, _, _ = _setup(512, None, n, T, seed=3)
+        g = torch.Generator().manual_seed(8)
+        qn = torch.randn((len(n), n_q, H, 128), generator=g).to(torch.bfloat16)
+        qp = torch.randn((len(n), n_q, H, 64), generator=g).to(torch.bfloat16)
+        outs.append(f32(c.prefill_mla(0, qn.cuda(), qp.cuda(), wk.cuda(), wv.cuda(), 0.07)))
+        assert c.device_error() == 0
+    assert np.array_equal(outs[0], outs[1])
+
+
+def test_mla_prefill_scratch_limits():
+    """The scratch size never shrinks with the chunk; a buffer that holds the
+    absorbed path's rows but not the formed tiles still serves the call."""
+    c, wk, wv, _, _ = _setup(512, None, [300, 80], 8192, seed=9)
+    sizes = [_scratch(c, n) for n in list(range(1, 321)) + [1000, 8192]]
+    assert sizes == sorted(sizes)
+    n_q = 200
+    g = torch.Generator().manual_seed(4)
+    qn = torch.randn((2, n_q, H, 128), generator=g).to(torch.bfloat16).cuda()
+    qp = torch.randn((2, n_q, H, 64), generator=g).to(torch.bfloat16).cuda()
+    wk, wv = wk.cuda(), wv.cuda()
+    full = c.prefill_mla(0, qn, qp, wk, wv, 0.07)
+    rows = 2 * n_q * H
+    small = rows * (2 * 512 + 64) * 2 + 256 + rows * 514 * 4  # absorbed queries and latent partials
+    assert 1024 < small < _scratch(c, n_q) == sizes[-1]
+    out = torch.empty_like(full)
+    buf = torch.empty(small, dtype=torch.uint8, device="cuda")
+    st = torch.cuda.current_stream().cuda_stream
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    args = (c.handle, 0, p(qn), p(qp), p(wk), p(wv), n_q, 0.07, p(out), p(buf))
+    assert c.lib.kvk_prefill_attention_mla(*args, small, ctypes.c_void_p(st)) == 0
+    assert_close(f32(out), f32(full), max_abs=2e-4, rel_l2=1e-4, what="absorbed = formed")
+    assert c.lib.kvk_prefill_attention_mla(*args, 1024, ctypes.c_void_p(st)) != 0
     assert c.device_error() == 0
