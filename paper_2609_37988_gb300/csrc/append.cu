@@ -367,79 +367,6 @@ __global__ void __launch_bounds__(128)
 // layout.h, derived per format below) and stored as whole words, the 128-
 // to 512-byte record in one to four coalesced store instructions.
 
-// 4-bit codes (grouped int4 or symmetric 4-bit): p = K codes | V codes << 16.
-// Lanes 0-15 build K word T = lane (lane column c = T / 4, word w = T % 4
-// holds k-steps 2w, 2w+1: nibble h + 2 jj from lane 4 (2w + jj) + c/2 + 2h
-// element 2 (c%2), nibble 4 + h + 2 jj from its element 2 (c%2) + 1).
-// Lanes 16-31 build logical V word U = lane - 16 (chunk k = U / 4, word
-// wd = U % 4: M-blocks 2k + mm, rows g = 2 wd + gg, g + 8 e: bits
-// 8 (2 gg + mm) + 4 e from lane 4 (2k + mm) + 2e + wd/2, element
-// 2 (wd%2) + gg).
-struct Gather4 {
-  int src[4], sh, dlo[4], dhi[4];
-  __device__ explicit Gather4(int lane) {
-    if (lane < 16) {
-      const int c = lane >> 2, w = lane & 3;
-      sh = 8 * (c & 1);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int jj = q >> 1, h = q & 1;
-        src[q] = 4 * (2 * w + jj) + (c >> 1) + 2 * h;
-        dlo[q] = 4 * (h + 2 * jj);
-        dhi[q] = 4 * (4 + h + 2 * jj);
-      }
-    } else {
-      const int u = lane - 16, k = u >> 2, wd = u & 3;
-      sh = 16 + 8 * (wd & 1);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int mm = q >> 1, e = q & 1;
-        src[q] = 4 * (2 * k + mm) + 2 * e + (wd >> 1);
-        dlo[q] = 8 * mm + 4 * e;
-        dhi[q] = 16 + 8 * mm + 4 * e;
-      }
-    }
-  }
-  __device__ __forceinline__ uint32_t word(uint32_t p) const {
-    uint32_t x = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint32_t b = __shfl_sync(0xffffffffu, p, src[q]) >> sh;
-      x |= ((b & 0xFu) << dlo[q]) | (((b >> 4) & 0xFu) << dhi[q]);
-    }
-    return x;
-  }
-};
-
-// 8-bit codes: every lane builds K word T = lane (chunk T / 4 = 4 (bp / 16)
-// + c, k-step j = 4 (chunk / 4) + T % 4: bytes 0-1 from lane 4j + c/2,
-// bytes 2-3 from lane 4j + c/2 + 2, each lane's elements 2 (c%2), +1) and
-// logical V word U = lane (M-block m = U / 4, word wd = U % 4: bytes 2 gg + e
-// from lane 4m + 2e + wd/2, element 2 (wd%2) + gg).
-struct Gather8 {
-  int ks0, ks1, ksh, vs0, vs1, vsh;
-  __device__ explicit Gather8(int lane) {
-    const int chunk = lane >> 2, c = chunk & 3, j = 4 * (chunk >> 2) + (lane & 3);
-    ks0 = 4 * j + (c >> 1);
-    ks1 = ks0 + 2;
-    ksh = 16 * (c & 1);
-    const int m = lane >> 2, wd = lane & 3;
-    vs0 = 4 * m + (wd >> 1);
-    vs1 = vs0 + 2;
-    vsh = 16 * (wd & 1);
-  }
-  __device__ __forceinline__ uint32_t kword(uint32_t pk) const {
-    const uint32_t a = (__shfl_sync(0xffffffffu, pk, ks0) >> ksh) & 0xFFFFu;
-    const uint32_t b = (__shfl_sync(0xffffffffu, pk, ks1) >> ksh) & 0xFFFFu;
-    return a | (b << 16);
-  }
-  __device__ __forceinline__ uint32_t vword(uint32_t pv) const {
-    const uint32_t a = __shfl_sync(0xffffffffu, pv, vs0) >> vsh;
-    const uint32_t b = __shfl_sync(0xffffffffu, pv, vs1) >> vsh;
-    return __byte_perm(a, b, 0x5140);
-  }
-};
-
 // bf16 values: lane owns K words T = lane, lane + 32 (chunk T / 4, c =
 // chunk % 4, j = 2 (chunk / 4) + (T % 4) / 2, h = T % 2: the bf16 pair of
 // elements 2 (c%2), +1 of lane 4j + c/2 + 2h) and V words W = lane, lane + 32
@@ -479,139 +406,8 @@ struct Gather16 {
   }
 };
 
-// Codes of one lane's four channels in one register (code e at bits BITS e).
-template <int BITS>
-__device__ __forceinline__ uint32_t pack_codes(const uint32_t (&c)[4]) {
-  return c[0] | (c[1] << BITS) | (c[2] << (2 * BITS)) | (c[3] << (3 * BITS));
-}
-
-// KPC: keys with per-channel groups -- the kernel writes the value section
-// and its metadata only (the key codes are written when a group of
-// positions completes, by gqa_append_kgroups) and leaves the lengths to the
-// residual kernel, which runs last.
-template <int BITS, int GS, bool SYM, bool KPC = false>
-__global__ void __launch_bounds__(256)
-    gqa_append_bulk(const GqaView v, const void *kin, const void *vin, int in_f32, int n_new,
-                    const int32_t *n_per_seq, int32_t *err) {
-  pdl_wait();
-  pdl_trigger();
-  static_assert(!KPC || (!SYM && BITS != 16), "per-channel keys: grouped codes");
-  constexpr int D = 128, E = 4;
-  constexpr int SEC = D * BITS / 8;                       // bytes per section
-  constexpr int MBY = ((D / GS) * 8 + 15) & ~15;          // one section's group metadata
-  constexpr int REC = SYM ? 2 * SEC : BITS == 16 ? 2 * SEC : 2 * SEC + (KPC ? 1 : 2) * MBY;
-  constexpr int KM = 2 * SEC, VM = KPC ? 2 * SEC : KM + MBY;
-  constexpr int NC = SEC / 16;                            // chunks per code section
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int wpb = blockDim.x >> 5;
-  const size_t total = (size_t)v.B * n_new * v.Hkv;
-  Gather4 g4(lane);
-  Gather8 g8(lane);
-  Gather16 g16(lane);
-  (void)g4; (void)g8; (void)g16;
-  // two rows per iteration, their loads issued together and their
-  // arithmetic independent (rows past the end compute on row 0's inputs and
-  // store nothing)
-  auto process = [&](const float (&xk)[E], const float (&xv)[E], bool ok, size_t row, int t) {
-    uint8_t *rec = v.rec + row * REC;
-    if constexpr (BITS == 16) {
-      uint32_t k0 = pack2<true>(xk[0], xk[1]), k1 = pack2<true>(xk[2], xk[3]);
-      uint32_t v0 = pack2<true>(xv[0], xv[1]), v1 = pack2<true>(xv[2], xv[3]);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint32_t kw = g16.kword(k0, k1, h), vw = g16.vword(v0, v1, h);
-        if (ok) {
-          reinterpret_cast<uint32_t *>(rec)[lane + 32 * h] = kw;
-          reinterpret_cast<uint32_t *>(rec + SEC)[lane + 32 * h] = vw;
-        }
-      }
-    } else {
-      uint32_t ck[E], cv[E];
-      if constexpr (SYM) {
-        const uint32_t sk = quant_sym_lane<E>(xk, BITS, ck);
-        const uint32_t sv = quant_sym_lane<E>(xv, BITS, cv);
-        if (ok && lane == 0) v.scales[row] = sk | (sv << 16);
-      } else {
-        float ks = 0.f, kz = 0.f, vs, vz;
-        if constexpr (!KPC) quant_lane<E>(xk, GS, (1 << BITS) - 1, ck, ks, kz);
-        else for (int e = 0; e < E; ++e) ck[e] = 0u;
-        quant_lane<E>(xv, GS, (1 << BITS) - 1, cv, vs, vz);
-        if (ok && (lane * E) % GS == 0) {
-          if constexpr (!KPC) reinterpret_cast<float2 *>(rec + KM)[(lane * E) / GS] = make_float2(ks, kz);
-          reinterpret_cast<float2 *>(rec + VM)[(lane * E) / GS] = make_float2(vs, vz);
-        }
-      }
-      const uint32_t pk = pack_codes<BITS>(ck), pv = pack_codes<BITS>(cv);
-      // logical chunk of this lane's word(s) and its physical 16-byte slot:
-      // symmetric records rotate all chunks by sym_rot(t), grouped ones the
-      // V chunks by v_rot(t)
-      if constexpr (BITS == 4) {
-        const uint32_t w = g4.word(pk | (pv << 16));
-        int off;
-        if (lane < 16) {
-          off = SYM ? 16 * (((lane >> 2) + sym_rot(t, REC / 16)) & (REC / 16 - 1)) + 4 * (lane & 3)
-                    : 4 * lane;
-        } else {
-          const int u = lane - 16, k = u >> 2;
-          off = SYM ? 16 * ((NC + k + sym_rot(t, REC / 16)) & (REC / 16 - 1)) + 4 * (u & 3)
-                    : SEC + 16 * ((k + v_rot(t, REC, NC)) & (NC - 1)) + 4 * (u & 3);
-        }
-        if (ok && (!KPC || lane >= 16)) *reinterpret_cast<uint32_t *>(rec + off) = w;
-      } else {
-        const uint32_t kw = g8.kword(pk), vw = g8.vword(pv);
-        const int kc = lane >> 2;
-        const int koff = SYM ? 16 * ((kc + sym_rot(t, REC / 16)) & (REC / 16 - 1)) + 4 * (lane & 3)
-                             : 4 * lane;
-        const int voff = SYM ? 16 * ((NC + kc + sym_rot(t, REC / 16)) & (REC / 16 - 1)) + 4 * (lane & 3)
-                             : SEC + 16 * ((kc + v_rot(t, REC, NC)) & (NC - 1)) + 4 * (lane & 3);
-        if (ok) {
-          if constexpr (!KPC) *reinterpret_cast<uint32_t *>(rec + koff) = kw;
-          *reinterpret_cast<uint32_t *>(rec + voff) = vw;
-        }
-      }
-    }
-  };
-  const size_t step = (size_t)gridDim.x * wpb;
-  // 32-bit index arithmetic (the launcher sends fewer than 2^31 rows)
-  const RowStep rstep((uint32_t)step, (uint32_t)v.Hkv, (uint32_t)n_new);
-  RowIdx ridx = rstep.at((uint32_t)min((size_t)blockIdx.x * wpb + warp, total));
-  for (size_t w0 = (size_t)blockIdx.x * wpb + warp; w0 < total; w0 += 2 * step) {
-    bool ok[2];
-    size_t row[2];
-    int tt[2];
-    float xk[2][E], xv[2][E];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const size_t wid = w0 + u * step;
-      const RowIdx r = ridx;
-      ridx = rstep.next(ridx);  // row wid + step
-      ok[u] = false;
-      row[u] = 0;
-      tt[u] = 0;
-      size_t in_off = 0;
-      if (wid < total) {
-        const int kvh = (int)r.kvh, i = (int)r.i, b = (int)r.b;
-        in_off = wid * D;  // inputs are [B, n_new, H_kv, D], row wid
-        const int nb = seq_count(n_per_seq, b, n_new, err);
-        const int t = v.lens[b] + i;
-        if (i < nb) {
-          if (t >= v.cap) {
-            if (lane == 0) set_err(err, 2);
-          } else {
-            ok[u] = true;
-            row[u] = ((size_t)b * v.Hkv + kvh) * v.cap + t;
-            tt[u] = t;
-          }
-        }
-      }
-      load_row<D>(kin, vin, in_f32, in_off, lane, xk[u], xv[u]);
-    }
-    process(xk[0], xv[0], ok[0], row[0], tt[0]);
-    process(xk[1], xv[1], ok[1], row[1], tt[1]);
-  }
-  // the last CTA advances the lengths (per-channel keys: the residual
-  // kernel does, after this one)
-  if constexpr (KPC) return;
+// The last CTA to finish advances the lengths (completion counter).
+__device__ __forceinline__ void advance_lengths(const GqaView &v, int n_new, const int32_t *n_per_seq) {
   __syncthreads();
   __shared__ int last;
   if (threadIdx.x == 0) {
@@ -626,6 +422,354 @@ __global__ void __launch_bounds__(256)
     }
     if (threadIdx.x == 0) *v.counter = 0;
   }
+}
+
+// 32 consecutive elements of one lane, from 16-byte aligned bf16 or fp32
+__device__ __forceinline__ void load_quarter(const void *p, bool f32, float (&x)[32]) {
+  if (f32) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float4 u = static_cast<const float4 *>(p)[j];
+      x[4 * j] = u.x; x[4 * j + 1] = u.y; x[4 * j + 2] = u.z; x[4 * j + 3] = u.w;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint4 u = static_cast<const uint4 *>(p)[j];
+      const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        x[8 * j + 2 * k] = __uint_as_float(w[k] << 16);
+        x[8 * j + 2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
+      }
+    }
+  }
+}
+
+// Two floats in one 64-bit register pair for the packed binary32 units
+// (each half rounded as the scalar operation is).
+__device__ __forceinline__ uint64_t pair_f32(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpair_f32(uint64_t v, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// 1.5 2^23: adding it to |y| < 2^22 rounds y to the nearest integer, half to
+// even, and leaves that integer in the low bits of the sum's pattern.
+constexpr float kRintBias = 12582912.f;
+constexpr uint32_t kRintBits = 0x4B400000u;
+
+// Codes of one lane's 32 channels (a quarter of a row), given the group's
+// scale and zero (symmetric: zero 0): bits[e] = kRintBits + rint(fl((x - zr) /
+// sc)), clamped to [lo, hi].  The quotients are the correctly rounded ones,
+// by residuals: with y = RN(1/sc), q within an ulp of d/sc and r = d - q sc
+// (exact in one FMA), RN(q + r y) = RN(d/sc) (Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", 1990); the
+// first residual step brings RN(d y) within that ulp, the second rounds.
+// (Deciding near-halves by the division instead cost half the kernel: bf16
+// inputs put exact ties into nearly every warp.)  The theorem wants no
+// underflow and no overflow, so scales outside [2^-96, 2^96] (0 among them)
+// and groups with a value that is not finite take the division.  `over`: the
+// largest quotient may pass hi (a scale rounded down).
+__device__ __forceinline__ void quarter_codes(const float (&x)[32], float sc, float zr, float lo, float hi, bool over,
+                                              uint32_t (&bits)[32]) {
+  const float y = __frcp_rn(sc);
+  const uint64_t nz = pair_f32(-zr, -zr), y2 = pair_f32(y, y), ns = pair_f32(-sc, -sc),
+                 b2 = pair_f32(kRintBias, kRintBias);
+  uint64_t sum = pair_f32(0.f, 0.f);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const uint64_t d = add_f32x2(pair_f32(x[2 * i], x[2 * i + 1]), nz);
+    uint64_t q = mul_f32x2(d, y2);
+    q = fma_f32x2(fma_f32x2(q, ns, d), y2, q);
+    q = fma_f32x2(fma_f32x2(q, ns, d), y2, q);
+    sum = add_f32x2(sum, d);
+    float t0, t1;
+    unpair_f32(add_f32x2(q, b2), t0, t1);
+    bits[2 * i] = __float_as_uint(t0);
+    bits[2 * i + 1] = __float_as_uint(t1);
+  }
+  float s0, s1;
+  unpair_f32(sum, s0, s1);
+  if (!(fabsf(s0 + s1) < INFINITY) || !(sc >= 0x1p-96f && sc <= 0x1p96f) || over) {
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+      const float r = sc == 0.f ? 0.f : fminf(fmaxf(rintf(__fdiv_rn(__fsub_rn(x[e], zr), sc)), lo), hi);
+      bits[e] = __float_as_uint(r + kRintBias);
+    }
+  }
+}
+
+// Word sums of a quarter's codes at their places (layout.h): sum of (bits[e]
+// - kRintBits + off) << shift, the constant part taken off at once.
+template <int BITS, bool KEY>
+__device__ __forceinline__ void quarter_words(const uint32_t (&bits)[32], uint32_t off, uint32_t (&w)[BITS]) {
+  uint32_t c[BITS];
+#pragma unroll
+  for (int i = 0; i < BITS; ++i) w[i] = c[i] = 0u;
+#pragma unroll
+  for (int l = 0; l < 32; ++l) {
+    int wi, sh;
+    if (KEY) {
+      int byte, hi;
+      k_pos(l, BITS, 128, &byte, &hi);
+      wi = BITS == 8 ? 2 * (byte >> 4) + ((byte & 15) >> 2) : byte >> 4;
+      sh = 8 * (byte & 3) + 4 * hi;
+    } else {
+      const int g = l & 7, e = (l >> 3) & 1, hh = l >> 4;
+      const int bl = BITS == 8 ? 16 * hh + 2 * g + e : 2 * g + hh;
+      wi = bl >> 2;
+      sh = 8 * (bl & 3) + (BITS == 4 ? 4 * e : 0);
+    }
+    w[wi] += bits[l] << sh;
+    c[wi] += 1u << sh;
+  }
+#pragma unroll
+  for (int i = 0; i < BITS; ++i) w[i] -= (kRintBits - off) * c[i];
+}
+
+// Bulk appends of 8- and 4-bit codes, head_dim 128: a lane quantises 32
+// channels (a quarter of a row's keys, then of its values), a warp 8 rows per
+// iteration.  A warp per row with 4 channels per lane spent 420 warp
+// instructions per row (3 shuffle rounds per extremum, a division per 8 lanes
+// of a group, 4 shuffles per packed word); here the extrema stay in
+// registers, a group of 32 divides once, the words are summed in place and
+// the arithmetic is packed (81 instructions per row).  bf16 inputs come one
+// iteration ahead through shared memory: a warp copies its next 8 rows in
+// whole 512-byte runs, each lane's 64 bytes to a place of its own, 80 bytes
+// apart (no bank conflicts); with plain loads the kernel waited for memory
+// most of the time.  At the 14B shape (32 x 2048 x 8 rows) int4 g32: 223 us
+// with a warp per row, 89 with plain loads.
+// GS: group (32, 64; 128 for the symmetric scheme's rows); lanes of a group
+// meet by 0, 1 or 2 shuffles.  KPC: keys with per-channel groups -- values
+// only; the key codes are written when a group of positions completes
+// (gqa_append_kgroups) and the lengths advance in the residual kernel.
+constexpr int kQuadStage = 2 * 32 * 80;  // a warp's 8 rows, keys and values, one iteration
+constexpr int kQuadSmem = 8 * 2 * kQuadStage;
+template <int BITS, int GS, bool SYM, bool KPC>
+__global__ void __launch_bounds__(256)
+    gqa_append_quads(const GqaView v, const void *kin, const void *vin, int in_f32, int n_new,
+                     const int32_t *n_per_seq, int32_t *err) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int SEC = 16 * BITS, NC = BITS;               // bytes and 16-byte chunks per section
+  constexpr int MBY = ((128 / GS) * 8 + 15) & ~15;        // one section's group metadata
+  constexpr int REC = SYM ? 2 * SEC : 2 * SEC + (KPC ? 1 : 2) * MBY;
+  constexpr int KM = 2 * SEC, VM = KPC ? KM : KM + MBY;
+  constexpr float LEV = (float)((1 << BITS) - 1), QL = (float)((1 << (BITS - 1)) - 1);
+  extern __shared__ __align__(16) uint8_t quads_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, qc = lane & 3;
+  const uint32_t total = (uint32_t)((size_t)v.B * n_new * v.Hkv);  // the launcher sends fewer than 2^31 rows
+  const uint32_t step = gridDim.x * 64;
+  const RowStep rstep(step, (uint32_t)v.Hkv, (uint32_t)n_new);
+  uint32_t row0 = (blockIdx.x * 8 + warp) * 8;
+  RowIdx ri = rstep.at(min(row0 + (lane >> 2), total));
+  uint8_t *stage = quads_smem + warp * 2 * kQuadStage;
+  // the warp's 8 rows from r0 on into a stage, keys then values (bf16)
+  auto fetch = [&](uint32_t r0, int s) {
+#pragma unroll
+    for (int sec = KPC ? 1 : 0; sec < 2; ++sec)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = 32 * j + lane;  // 16-byte piece of the 8 rows
+        const bool in = r0 + (c >> 4) < total;
+        cp_async16(stage + s * kQuadStage + sec * (kQuadStage / 2) + (c >> 2) * 80 + (c & 3) * 16,
+                   static_cast<const uint8_t *>(sec ? vin : kin) + (in ? (size_t)r0 * 256 + 16 * c : 0), in);
+      }
+    cp_async_commit();
+  };
+  if (!in_f32 && row0 < total) fetch(row0, 0);
+  for (int s = 0; row0 < total; row0 += step, ri = rstep.next(ri), s ^= 1) {
+    const uint32_t row = row0 + (lane >> 2);
+    bool ok = row < total;
+    float xk[32], xv[32];
+    if (in_f32) {
+      const size_t in_off = (size_t)(ok ? row : 0) * 128 + 32 * qc;  // inputs are [B, n_new, H_kv, 128], row `row`
+      if constexpr (!KPC) load_quarter(static_cast<const float *>(kin) + in_off, true, xk);
+      load_quarter(static_cast<const float *>(vin) + in_off, true, xv);
+    } else {
+      __syncwarp();  // the stage's last rows are read
+      if (row0 + step < total) fetch(row0 + step, s ^ 1);
+      else cp_async_commit();
+      cp_async_wait<1>();
+      __syncwarp();
+      const uint8_t *mine = stage + s * kQuadStage + lane * 80;
+      if constexpr (!KPC) load_quarter(mine, false, xk);
+      load_quarter(mine + kQuadStage / 2, false, xv);
+    }
+    int t = 0;
+    size_t slot = 0;
+    if (ok) {
+      const int b = (int)ri.b, nb = seq_count(n_per_seq, b, n_new, err);
+      t = v.lens[b] + (int)ri.i;
+      ok = (int)ri.i < nb;
+      if (ok && t >= v.cap) {
+        if (qc == 0) set_err(err, 2);
+        ok = false;
+      }
+      if (ok) slot = ((size_t)b * v.Hkv + ri.kvh) * v.cap + t;
+    }
+    uint8_t *rec = v.rec + slot * REC;
+    // physical 16-byte place of a record's logical chunk: symmetric records
+    // rotate all chunks by sym_rot(t), grouped ones the V chunks by v_rot(t)
+    auto at = [&](int chunk) -> uint4 * {
+      const int c = SYM          ? (chunk + sym_rot(t, REC / 16)) & (REC / 16 - 1)
+                    : chunk < NC ? chunk
+                                 : NC + ((chunk - NC + v_rot(t, REC, NC)) & (NC - 1));
+      return reinterpret_cast<uint4 *>(rec) + c;
+    };
+    uint32_t ssym = 0;
+#pragma unroll
+    for (int sec = KPC ? 1 : 0; sec < 2; ++sec) {
+      const float(&x)[32] = sec ? xv : xk;
+      float mn = x[0], mx = x[0];
+#pragma unroll
+      for (int e = 1; e < 32; ++e) {
+        mn = fminf(mn, x[e]);
+        mx = fmaxf(mx, x[e]);
+      }
+#pragma unroll
+      for (int o = 1; o < GS / 32; o <<= 1) {
+        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      }
+      uint32_t bits[32], w[BITS];
+      if constexpr (SYM) {
+        const float am = fmaxf(fmaxf(mx, -mn), 0.f);
+        const uint16_t sb = f32_to_bf16_bits(__fdiv_rn(am, QL));
+        const float s = bf16_to_f32(sb);
+        const float top = s == 0.f ? 0.f : __fmul_rn(am, __fdividef(1.f, s));
+        quarter_codes(x, s, 0.f, -QL, QL, !(top <= QL + 0.4f), bits);
+        ssym |= (uint32_t)sb << (16 * sec);
+      } else {
+        const float s = __fdiv_rn(__fsub_rn(mx, mn), LEV);
+        quarter_codes(x, s, mn, 0.f, LEV, false, bits);
+        if (ok && (32 * qc) % GS == 0)
+          reinterpret_cast<float2 *>(rec + (sec ? VM : KM))[32 * qc / GS] = make_float2(s, mn);
+      }
+      constexpr uint32_t off = SYM ? (uint32_t)QL : 0u;
+      if (sec) {
+        // values: the quarter is BITS / 4 whole chunks
+        quarter_words<BITS, false>(bits, off, w);
+#pragma unroll
+        for (int c = 0; c < BITS / 4; ++c)
+          if (ok) *at(NC + BITS / 4 * qc + c) = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+      } else if constexpr (BITS == 4) {
+        // keys: word c belongs to chunk c at place qc; the row's four lanes
+        // transpose (two exchanges), lane qc stores chunk qc
+        quarter_words<BITS, true>(bits, off, w);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {  // pairs (0, 1) and (2, 3) with lane ^ 1
+          const uint32_t give = qc & 1 ? w[2 * h] : w[2 * h + 1];
+          const uint32_t got = __shfl_xor_sync(0xffffffffu, give, 1);
+          if (qc & 1) w[2 * h] = got;
+          else w[2 * h + 1] = got;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {  // pairs (0, 2) and (1, 3) with lane ^ 2
+          const uint32_t give = qc & 2 ? w[h] : w[h + 2];
+          const uint32_t got = __shfl_xor_sync(0xffffffffu, give, 2);
+          if (qc & 2) w[h] = got;
+          else w[h + 2] = got;
+        }
+        if (ok) *at(qc) = make_uint4(w[0], w[1], w[2], w[3]);
+      } else {
+        // keys: words 2c, 2c + 1 are half qc % 2 of chunk 4 (qc / 2) + c; the
+        // even lane of a pair stores chunks c = 0, 1, the odd one c = 2, 3
+        quarter_words<BITS, true>(bits, off, w);
+        uint32_t g[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) g[i] = __shfl_xor_sync(0xffffffffu, qc & 1 ? w[i] : w[4 + i], 1);
+        if (ok) {
+          const int c0 = 4 * (qc >> 1) + (qc & 1 ? 2 : 0);
+          *at(c0) = qc & 1 ? make_uint4(g[0], g[1], w[4], w[5]) : make_uint4(w[0], w[1], g[0], g[1]);
+          *at(c0 + 1) = qc & 1 ? make_uint4(g[2], g[3], w[6], w[7]) : make_uint4(w[2], w[3], g[2], g[3]);
+        }
+      }
+    }
+    if (SYM && ok && qc == 0) v.scales[slot] = ssym;
+  }
+  if constexpr (!KPC) advance_lengths(v, n_new, n_per_seq);
+}
+
+// Bulk appends of bf16 caches, head_dim 128: a warp per row, two rows per
+// iteration, their loads issued together (rows past the end compute on row
+// 0's inputs and store nothing).
+__global__ void __launch_bounds__(256)
+    gqa_append_bulk_bf16(const GqaView v, const void *kin, const void *vin, int in_f32, int n_new,
+                         const int32_t *n_per_seq, int32_t *err) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int D = 128, E = 4, SEC = 2 * D, REC = 2 * SEC;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wpb = blockDim.x >> 5;
+  const size_t total = (size_t)v.B * n_new * v.Hkv;
+  const Gather16 g16(lane);
+  const size_t step = (size_t)gridDim.x * wpb;
+  // 32-bit index arithmetic (the launcher sends fewer than 2^31 rows)
+  const RowStep rstep((uint32_t)step, (uint32_t)v.Hkv, (uint32_t)n_new);
+  RowIdx ridx = rstep.at((uint32_t)min((size_t)blockIdx.x * wpb + warp, total));
+  for (size_t w0 = (size_t)blockIdx.x * wpb + warp; w0 < total; w0 += 2 * step) {
+    bool ok[2];
+    size_t row[2];
+    float xk[2][E], xv[2][E];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const size_t wid = w0 + u * step;
+      const RowIdx r = ridx;
+      ridx = rstep.next(ridx);  // row wid + step
+      ok[u] = false;
+      row[u] = 0;
+      size_t in_off = 0;
+      if (wid < total) {
+        const int kvh = (int)r.kvh, i = (int)r.i, b = (int)r.b;
+        in_off = wid * D;  // inputs are [B, n_new, H_kv, D], row wid
+        const int nb = seq_count(n_per_seq, b, n_new, err);
+        const int t = v.lens[b] + i;
+        if (i < nb) {
+          if (t >= v.cap) {
+            if (lane == 0) set_err(err, 2);
+          } else {
+            ok[u] = true;
+            row[u] = ((size_t)b * v.Hkv + kvh) * v.cap + t;
+          }
+        }
+      }
+      load_row<D>(kin, vin, in_f32, in_off, lane, xk[u], xv[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      uint8_t *rec = v.rec + row[u] * REC;
+      const uint32_t k0 = pack2<true>(xk[u][0], xk[u][1]), k1 = pack2<true>(xk[u][2], xk[u][3]);
+      const uint32_t v0 = pack2<true>(xv[u][0], xv[u][1]), v1 = pack2<true>(xv[u][2], xv[u][3]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t kw = g16.kword(k0, k1, h), vw = g16.vword(v0, v1, h);
+        if (ok[u]) {
+          reinterpret_cast<uint32_t *>(rec)[lane + 32 * h] = kw;
+          reinterpret_cast<uint32_t *>(rec + SEC)[lane + 32 * h] = vw;
+        }
+      }
+    }
+  }
+  advance_lengths(v, n_new, n_per_seq);
 }
 
 // Short appends (a decode step: n_new x H_kv <= 64 rows per sequence,
@@ -969,9 +1113,9 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-// CTAs of `wpc` row warps for `rows` rows: one per wpc rows, up to 2048
-// threads per SM of the current device; the kernels loop over the rest
-unsigned row_blocks(size_t rows, int wpc = 4) {
+// CTAs of `wpc` rows for `rows` rows: one per wpc rows, up to `ctas_per_sm`
+// per SM of the current device; the kernels loop over the rest
+unsigned row_blocks(size_t rows, int wpc = 4, int ctas_per_sm = 16) {
   static int sms = 0;
   if (!sms) {
     int dev = 0;
@@ -979,7 +1123,7 @@ unsigned row_blocks(size_t rows, int wpc = 4) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
       sms = 148;
   }
-  const size_t need = (rows + wpc - 1) / wpc, cap = (size_t)sms * (64 / wpc);
+  const size_t need = (rows + wpc - 1) / wpc, cap = (size_t)sms * ctas_per_sm;
   return (unsigned)(need < cap ? (need > 0 ? need : 1) : cap);
 }
 
@@ -1014,25 +1158,26 @@ cudaError_t launch_gqa_append(const GqaView &v, const void *k, const void *vv, i
                    max_groups);
   }
   if (e == cudaSuccess) {
-    const dim3 bg(row_blocks(rows, 8));
-    if (kpc && (size_t)n_new * v.Hkv > 64 && d128 && rows < (1u << 31) && (v.bits == 8 || v.bits == 4)) {
-      // bulk appends of the values beside per-channel keys (head_dim 128)
-      auto bulk = [&](auto kern) {
-        return launch_pdl(kern, bg, dim3(256), 0, st, v, k, vv, in_f32, n_new, n_per_seq, err);
-      };
-      if (v.bits == 8) e = v.group == 32 ? bulk(gqa_append_bulk<8, 32, false, true>) : bulk(gqa_append_bulk<8, 64, false, true>);
-      else e = v.group == 32 ? bulk(gqa_append_bulk<4, 32, false, true>) : bulk(gqa_append_bulk<4, 64, false, true>);
-    } else if (!kpc && (size_t)n_new * v.Hkv > 64 && d128 && rows < (1u << 31) &&
-        (v.bits == 16 || v.bits == 8 || v.bits == 4)) {
-      // bulk appends of the per-token layouts with head_dim 128
-      const bool sym = v.scheme == kSchemeSym;
-      auto bulk = [&](auto kern) {
-        return launch_pdl(kern, bg, dim3(256), 0, st, v, k, vv, in_f32, n_new, n_per_seq, err);
-      };
-      if (v.bits == 16) e = bulk(gqa_append_bulk<16, 64, false>);
-      else if (sym) e = v.bits == 8 ? bulk(gqa_append_bulk<8, 64, true>) : bulk(gqa_append_bulk<4, 64, true>);
-      else if (v.bits == 8) e = v.group == 32 ? bulk(gqa_append_bulk<8, 32, false>) : bulk(gqa_append_bulk<8, 64, false>);
-      else e = v.group == 32 ? bulk(gqa_append_bulk<4, 32, false>) : bulk(gqa_append_bulk<4, 64, false>);
+    // bulk appends (head_dim 128): a warp per row for bf16, a lane per 32
+    // channels for 8- and 4-bit codes
+    const bool bulk = (size_t)n_new * v.Hkv > 64 && d128 && rows < (1u << 31);
+    const bool sym = v.scheme == kSchemeSym;
+    auto quads = [&](auto kern) {
+      cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kQuadSmem);
+      if (r != cudaSuccess) return r;
+      return launch_pdl(kern, dim3(row_blocks(rows, 64, 2)), dim3(256), kQuadSmem, st, v, k, vv, in_f32, n_new,
+                        n_per_seq, err);
+    };
+    if (bulk && v.bits == 16) {
+      e = launch_pdl(gqa_append_bulk_bf16, dim3(row_blocks(rows, 8, 8)), dim3(256), 0, st, v, k, vv, in_f32, n_new,
+                     n_per_seq, err);
+    } else if (bulk && (v.bits == 8 || v.bits == 4)) {
+      const bool g32 = v.group == 32;
+      if (sym) e = v.bits == 8 ? quads(gqa_append_quads<8, 128, true, false>) : quads(gqa_append_quads<4, 128, true, false>);
+      else if (kpc && v.bits == 8) e = g32 ? quads(gqa_append_quads<8, 32, false, true>) : quads(gqa_append_quads<8, 64, false, true>);
+      else if (kpc) e = g32 ? quads(gqa_append_quads<4, 32, false, true>) : quads(gqa_append_quads<4, 64, false, true>);
+      else if (v.bits == 8) e = g32 ? quads(gqa_append_quads<8, 32, false, false>) : quads(gqa_append_quads<8, 64, false, false>);
+      else e = g32 ? quads(gqa_append_quads<4, 32, false, false>) : quads(gqa_append_quads<4, 64, false, false>);
     } else if (!kpc && (size_t)n_new * v.Hkv <= 64)
       e = launch_pdl(d128 ? gqa_append_seq<128> : gqa_append_seq<64>, dim3(v.B), dim3(256), 0, st,
                      v, k, vv, in_f32, n_new, n_per_seq, err);

@@ -293,3 +293,64 @@ def test_append_rounding_ties(fmt):
     st = oracle_state(k, v, lens, cfg)
     check_codes(c.export(0), st, lens, cfg)
     assert c.device_error() == 0
+
+
+@pytest.mark.parametrize("in_dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
+@pytest.mark.parametrize("fmt", [
+    dict(bits=8, group=32, key_axis="token"), dict(bits=8, group=64, key_axis="token"),
+    dict(bits=4, group=32, key_axis="token"), dict(bits=4, group=64, key_axis="token"),
+    dict(bits=8, group=64, key_axis="channel"), dict(bits=4, group=32, key_axis="channel"),
+    dict(bits=8, scheme="symmetric"), dict(bits=4, scheme="symmetric"), dict(bits=16),
+], ids=lambda f: f"{f.get('scheme', 'grouped')[:3]}{f['bits']}g{f.get('group', 128)}-{f.get('key_axis', 'token')[:1]}")
+def test_bulk_append_equals_short_appends(fmt, in_dtype):
+    """One bulk append stores byte for byte what appends of a few rows (a
+    kernel of their own) store: row counts that leave part of a warp's and of
+    a CTA's rows over, per-sequence counts, and rows of the values where a
+    quotient by residuals could differ from a division: exact ties, constant
+    and zero groups, tiny and huge scales, infinities and NaN."""
+    from paper_2609_37988_gb300.cache import Cache, Layer
+    B, Hkv, D, n = 3, 3, 128, 67
+    g = torch.Generator().manual_seed(fmt["bits"])
+    def rows():
+        x = torch.randn((B, n, Hkv, D), generator=g)
+        x[0, 1] = 0.0
+        x[0, 2] = 3.25
+        x[0, 3] *= 1e-38
+        x[0, 4] *= 1e-42
+        x[0, 5] *= 1e30
+        x[0, 6] = torch.where(torch.rand((Hkv, D), generator=g) < 0.5, -3e38, 3e38)
+        x[0, 7, :, 5] = float("inf")
+        x[0, 8, :, 40] = float("-inf")
+        x[0, 9, :, 77] = float("nan")
+        x[0, 10, 0] = float("nan")
+        x[0, 11] = torch.arange(D) % 31 * 0.5  # quotients on half-integers
+        x[0, 12] = (torch.arange(D) % 16).float()
+        x[0, 13] *= 2.0 ** -95
+        x[0, 14] *= 2.0 ** -100
+        x[0, 15] = -0.0
+        return x.to(in_dtype).cuda()
+    k, v = rows(), rows()
+    count = torch.tensor([n, 41, 66], dtype=torch.int32, device="cuda")
+    caches = []
+    for step in (n, 21):  # 201 rows per sequence at once, 63 at a time
+        c = Cache(n_layers=1, n_q_heads=6, n_kv_heads=Hkv, head_dim=D, max_batch=B, max_ctx=n + 21, layers=[Layer(**fmt)])
+        c.arenas[0].zero_()
+        c.reset()
+        for i in range(0, n, step):
+            part = (count - i).clamp(0, min(step, n - i)).to(torch.int32)
+            c.append(0, k[:, i:i + step].contiguous(), v[:, i:i + step].contiguous(), part)
+        caches.append(c)
+    torch.cuda.synchronize()
+    a, b = caches
+    assert a.lengths(0).tolist() == b.lengths(0).tolist() == count.tolist()
+    x, y = a.export(0), b.export(0)
+    for key in x:
+        if x[key] is None or key == "k_residual":
+            continue
+        for s in range(B):
+            m = int(count[s]) // fmt.get("group", 1) if key in ("k_scale", "k_zero") and fmt.get("key_axis") == "channel" else int(count[s])
+            p, q = x[key][s, :, :m].contiguous(), y[key][s, :, :m].contiguous()
+            if p.is_floating_point():
+                p, q = p.float().view(torch.int32), q.float().view(torch.int32)
+            assert torch.equal(p, q), (key, s)
+    assert a.device_error() == 0 and b.device_error() == 0
