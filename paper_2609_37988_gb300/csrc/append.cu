@@ -360,12 +360,11 @@ __global__ void __launch_bounds__(128)
 }
 
 // ---- bulk appends, head_dim 128, per-token layouts -------------------------
-// One warp per (sequence, new position, KV head) row over a bounded grid,
-// lane L holding channels 4L .. 4L+3.  Each lane packs its codes into one
-// register per section; the record's 32-bit words are then gathered from
-// the lanes that hold their channels by warp shuffles (the channel order of
-// layout.h, derived per format below) and stored as whole words, the 128-
-// to 512-byte record in one to four coalesced store instructions.
+// bf16: one warp per (sequence, new position, KV head) row over a bounded
+// grid, lane L holding channels 4L .. 4L+3; the record's 32-bit words are
+// gathered from the lanes that hold their channels by warp shuffles (the
+// channel order of layout.h, derived below) and stored as whole words.
+// 8- and 4-bit codes: a lane per 32 channels (gqa_append_quads).
 
 // bf16 values: lane owns K words T = lane, lane + 32 (chunk T / 4, c =
 // chunk % 4, j = 2 (chunk / 4) + (T % 4) / 2, h = T % 2: the bf16 pair of
@@ -556,7 +555,8 @@ __device__ __forceinline__ void quarter_words(const uint32_t (&bits)[32], uint32
 // whole 512-byte runs, each lane's 64 bytes to a place of its own, 80 bytes
 // apart (no bank conflicts); with plain loads the kernel waited for memory
 // most of the time.  At the 14B shape (32 x 2048 x 8 rows) int4 g32: 223 us
-// with a warp per row, 89 with plain loads.
+// with a warp per row, 89 with plain loads, 72 now (5.1 TB/s of inputs and
+// records; issue 57 % busy).
 // GS: group (32, 64; 128 for the symmetric scheme's rows); lanes of a group
 // meet by 0, 1 or 2 shuffles.  KPC: keys with per-channel groups -- values
 // only; the key codes are written when a group of positions completes
