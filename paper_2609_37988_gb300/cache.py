@@ -43,21 +43,29 @@ class Layer:
                         QUANT_SYMMETRIC if self.scheme == "symmetric" else QUANT_GROUPED)
 
 
+# Call overhead counts in a decode step: a small layer's kernels take 3-5 us
+# each.  Pointers and streams go to ctypes as plain integers (the argument
+# types are declared), and the current stream is read as a raw handle:
+# torch.cuda.current_stream() builds a Stream object, 2.8 us of the 8 us that
+# a rewind took and of the 15.6 us of a decode.
+_DTYPES = {torch.float32: DTYPE_F32, torch.bfloat16: DTYPE_BF16}
+
+
 def _ptr(t):
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+    return 0 if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return DTYPE_F32
-    if t.dtype == torch.bfloat16:
-        return DTYPE_BF16
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    code = _DTYPES.get(t.dtype)
+    if code is None:
+        raise TypeError(f"unsupported dtype {t.dtype}")
+    return code
 
 
 def _need(t: torch.Tensor, name: str):
@@ -98,6 +106,9 @@ class Cache:
                                             _ptr(self.workspace), ws.value, max_splits,
                                             ctypes.byref(h)))
         self.handle = h
+        # the calls of a step, looked up once
+        self._append, self._rewind = self.lib.kvk_append, self.lib.kvk_rewind
+        self._decode, self._decode_mla = self.lib.kvk_decode_attention, self.lib.kvk_decode_attention_mla
         self.max_splits = max_splits
         self.reset()
 
@@ -156,11 +167,12 @@ class Cache:
         """GQA: k, v ``[B, n, H_kv, D]`` (fp32/bf16).  MLA: k = latent
         ``[B, n, r]`` bf16, v = positional key ``[B, n, d_R]`` bf16."""
         _need(k, "k"); _need(v, "v")
-        n = int(k.shape[1])
         if n_per_seq is not None:
             _need(n_per_seq, "n_per_seq")
-        check(self.lib.kvk_append(self.handle, layer, _ptr(k), _ptr(v), _dtype_code(k), n,
-                                  _ptr(n_per_seq), _stream(stream)))
+        st = self._append(self.handle, layer, k.data_ptr(), v.data_ptr(), _dtype_code(k), k.shape[1],
+                          _ptr(n_per_seq), _stream(stream))
+        if st:
+            check(st)
 
     def set_kept(self, layer: int, idx: torch.Tensor = None, n_kept: torch.Tensor = None,
                  stream=None):
@@ -259,7 +271,9 @@ class Cache:
 
     def rewind(self, n: int, stream=None):
         """Drop the last ``n`` positions of every sequence of every anchor."""
-        check(self.lib.kvk_rewind(self.handle, n, _stream(stream)))
+        st = self._rewind(self.handle, n, _stream(stream))
+        if st:
+            check(st)
 
     # -- reads ---------------------------------------------------------------
     def plan_splits(self, layer: int) -> int:
@@ -272,8 +286,10 @@ class Cache:
         _need(q, "q")
         if out is None:
             out = torch.empty(q.shape, dtype=torch.float32, device=q.device)
-        check(self.lib.kvk_decode_attention(self.handle, layer, _ptr(q), _dtype_code(q),
-                                            float(scale), _ptr(out), n_splits, _stream(stream)))
+        st = self._decode(self.handle, layer, q.data_ptr(), _dtype_code(q), float(scale), out.data_ptr(), n_splits,
+                          _stream(stream))
+        if st:
+            check(st)
         return out
 
     def decode_partial(self, layer: int, q: torch.Tensor, scale: float, n_splits: int,
@@ -289,13 +305,13 @@ class Cache:
 
     def decode_mla(self, layer: int, q_nope, q_pe, w_uk, w_uv, scale: float, out=None,
                    n_splits: int = 0, stream=None) -> torch.Tensor:
-        for t, nm in ((q_nope, "q_nope"), (q_pe, "q_pe"), (w_uk, "w_uk"), (w_uv, "w_uv")):
-            _need(t, nm)
+        _need(q_nope, "q_nope"); _need(q_pe, "q_pe"); _need(w_uk, "w_uk"); _need(w_uv, "w_uv")
         if out is None:
             out = torch.empty(q_nope.shape, dtype=torch.float32, device=q_nope.device)
-        check(self.lib.kvk_decode_attention_mla(self.handle, layer, _ptr(q_nope), _ptr(q_pe),
-                                                _ptr(w_uk), _ptr(w_uv), float(scale), _ptr(out),
-                                                n_splits, _stream(stream)))
+        st = self._decode_mla(self.handle, layer, q_nope.data_ptr(), q_pe.data_ptr(), w_uk.data_ptr(),
+                              w_uv.data_ptr(), float(scale), out.data_ptr(), n_splits, _stream(stream))
+        if st:
+            check(st)
         return out
 
     def export(self, layer: int, stream=None) -> dict:
