@@ -237,7 +237,12 @@ __global__ void __launch_bounds__(32 * kMergeWarps) evict_merge_stats_kernel(con
   const int unit = id / R, r = id % R, b = unit / v.Hkv;
   const int len = v.lens[b];
   if (len <= a.budget) return;
-  const int nt = min((len + kT - 1) / kT, a.n_tiles) * a.stat_sub;
+  int nt = min((len + kT - 1) / kT, a.n_tiles);
+  if (a.items_per_cta) {  // one entry set per CTA that walked tiles of the unit
+    const int i0 = unit * a.n_tiles;
+    nt = (i0 + nt - 1) / a.items_per_cta - i0 / a.items_per_cta + 1;
+  }
+  nt *= a.stat_sub;
   const float2 *st = a.stats + ((size_t)unit * R + r) * a.n_tiles * a.stat_sub;
   float M = -INFINITY;
   for (int i = lane; i < nt; i += 32) M = fmaxf(M, st[i].x);
@@ -297,96 +302,161 @@ __device__ __forceinline__ void load8(const uint32_t *key, int t0, int n, uint32
   }
 }
 
+// ---- thread-block clusters -------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the int at the same shared-memory place of CTA `rank` of the cluster
+__device__ __forceinline__ int cluster_ld(const int *p, uint32_t rank) {
+  uint32_t a;
+  int x;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(x) : "r"(a) : "memory");
+  return x;
+}
+
 // Kept list of one (sequence, kv head): the budget - n_win largest votes by
 // a radix select on their bit patterns (votes are >= 0, so the patterns
 // order as the values), then the chosen positions in increasing order and
-// the window.
-__global__ void __launch_bounds__(1024) evict_select_kernel(const EvictArgs a) {
+// the window.  A cluster of 8 CTAs per unit, each over an eighth of the
+// positions: a unit's votes are read five times, which one CTA per unit did
+// in 110 us for 32 units of 131072 positions with 120 SMs idle.  Per pass
+// the CTAs add each other's histograms through distributed shared memory and
+// decide alike (one cluster barrier per pass: two histograms in turn).
+constexpr int kSelParts = 8;
+__global__ void __cluster_dims__(kSelParts, 1, 1) __launch_bounds__(1024) evict_select_kernel(const EvictArgs a) {
   pdl_wait();
   pdl_trigger();
   const GqaView &v = a.v;
-  const int j = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+  const int j = blockIdx.x / kSelParts, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int part = (int)cluster_rank();
   const int unit = b * v.Hkv + j;
   const int len = v.lens[b];
   int32_t *out = v.kept_idx + (size_t)unit * v.kept_cap;
-  if (len <= a.budget) {  // everything is kept
-    for (int t = tid; t < len; t += 1024) out[t] = t;
-    if (tid == 0) v.kept_n[unit] = len;
+  if (len <= a.budget) {  // everything is kept (the whole cluster leaves)
+    for (int t = part * 1024 + tid; t < len; t += kSelParts * 1024) out[t] = t;
+    if (part == 0 && tid == 0) v.kept_n[unit] = len;
     return;
   }
   const int P = len - a.n_win, k = a.budget - a.n_win;
   const uint32_t *key = reinterpret_cast<const uint32_t *>(a.votes + (size_t)unit * v.cap);
-  __shared__ int hist[256];
+  const int per = ((P + kSelParts - 1) / kSelParts + 7) / 8 * 8;
+  const int p0 = min(P, part * per), p1 = min(P, p0 + per);  // this CTA's positions
+  __shared__ int hist[2][256];
   __shared__ uint32_t s_prefix;
   __shared__ int s_rank;
   __shared__ int wsum[32];
   __shared__ int s_total;
+  __shared__ int s_cnt[2];
   uint32_t prefix = 0, mask = 0;
   int rank = k;  // 1-based rank (from the top) of the wanted key among the matches
   if (k > 0) {
     for (int pass = 0; pass < 4; ++pass) {
       const int shift = 24 - 8 * pass;
-      for (int d = tid; d < 256; d += 1024) hist[d] = 0;
+      int *h = hist[pass & 1];
+      if (tid < 256) h[tid] = 0;
       __syncthreads();
       // votes of similar size share their leading bytes, so most lanes of a
       // warp hit the bin of lane 0: those are counted with one atomic, the
       // others one by one.  Eight consecutive votes per thread per round
       // keep eight loads in flight.
-      for (int c0 = 0; c0 < P; c0 += 8 * 1024) {
+      for (int c0 = p0; c0 < p1; c0 += 8 * 1024) {
         uint32_t kk[8];
-        load8(key, c0 + 8 * tid, P, kk);
+        load8(key, c0 + 8 * tid, p1, kk);
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const bool hit = c0 + 8 * tid + u < P && (kk[u] & mask) == prefix;
+          const bool hit = c0 + 8 * tid + u < p1 && (kk[u] & mask) == prefix;
           const uint32_t bin = hit ? (kk[u] >> shift) & 255 : 256u;
           const uint32_t bin0 = __shfl_sync(0xffffffffu, bin, 0);
           const uint32_t same = __ballot_sync(0xffffffffu, bin == bin0);
           if (bin == bin0) {
-            if ((threadIdx.x & 31) == 0 && bin0 < 256u) atomicAdd(&hist[bin0], __popc(same));
+            if (lane == 0 && bin0 < 256u) atomicAdd(&h[bin0], __popc(same));
           } else if (hit) {
-            atomicAdd(&hist[bin], 1);
+            atomicAdd(&h[bin], 1);
           }
         }
       }
-      __syncthreads();
-      if (tid == 0) {
-        int cum = 0, sel = 0;
-        for (int d = 255; d >= 0; --d) {
-          if (cum + hist[d] >= rank) { sel = d; break; }
-          cum += hist[d];
+      cluster_sync();
+      // bins from the top: the one in which the count reaches the rank
+      int n = 0, inc = 0;
+      if (tid < 256) {
+        for (uint32_t r = 0; r < kSelParts; ++r) n += cluster_ld(&h[255 - tid], r);
+        inc = n;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, inc, off);
+          if (lane >= off) inc += y;
         }
-        s_prefix = prefix | ((uint32_t)sel << shift);
-        s_rank = rank - cum;
+        if (lane == 31) wsum[warp] = inc;
+      }
+      __syncthreads();
+      if (tid < 256) {
+        for (int w = 0; w < warp; ++w) inc += wsum[w];
+        if (inc >= rank && inc - n < rank) {
+          s_prefix = prefix | ((uint32_t)(255 - tid) << shift);
+          s_rank = rank - (inc - n);
+        }
       }
       __syncthreads();
       prefix = s_prefix;
       rank = s_rank;
       mask |= 0xFFu << shift;
-      __syncthreads();
     }
   }
   // positions above the threshold key, and the first `rank` equal to it
   // (one scan of the packed counts: greater in the high half, equal in the
   // low half; a taken position's slot is the greater ones before it plus
-  // the equal ones before it, at most `rank`)
+  // the equal ones before it, at most `rank`); first the counts of the
+  // positions before this CTA's
   const uint32_t theta = prefix;
   int gt_carry = 0, eq_carry = 0;
-  for (int c0 = 0; c0 < P && k > 0; c0 += 8 * 1024) {
+  if (k > 0) {
+    if (tid < 2) s_cnt[tid] = 0;
+    __syncthreads();
+    int ngt = 0, neq = 0;
+    for (int c0 = p0; c0 < p1; c0 += 8 * 1024) {
+      uint32_t kk[8];
+      load8(key, c0 + 8 * tid, p1, kk);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const bool in = c0 + 8 * tid + u < p1;
+        ngt += in && kk[u] > theta;
+        neq += in && kk[u] == theta;
+      }
+    }
+    ngt = __reduce_add_sync(0xffffffffu, ngt);
+    neq = __reduce_add_sync(0xffffffffu, neq);
+    if (lane == 0) {
+      if (ngt) atomicAdd(&s_cnt[0], ngt);
+      if (neq) atomicAdd(&s_cnt[1], neq);
+    }
+    cluster_sync();
+    for (int r = 0; r < part; ++r) {
+      gt_carry += cluster_ld(&s_cnt[0], r);
+      eq_carry += cluster_ld(&s_cnt[1], r);
+    }
+  }
+  for (int c0 = p0; c0 < p1 && k > 0; c0 += 8 * 1024) {
     const int tb = c0 + 8 * tid;  // this thread's eight consecutive positions
     uint32_t kk[8];
-    load8(key, tb, P, kk);
+    load8(key, tb, p1, kk);
     int ngt = 0, neq = 0;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      ngt += tb + u < P && kk[u] > theta;
-      neq += tb + u < P && kk[u] == theta;
+      ngt += tb + u < p1 && kk[u] > theta;
+      neq += tb + u < p1 && kk[u] == theta;
     }
     const int ex = block_scan_1024((ngt << 16) | neq, wsum, &s_total);
     const int tot = s_total;
     int gt_before = gt_carry + (ex >> 16), eq_before = eq_carry + (ex & 0xFFFF);
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const bool gt = tb + u < P && kk[u] > theta, eq = tb + u < P && kk[u] == theta;
+      const bool gt = tb + u < p1 && kk[u] > theta, eq = tb + u < p1 && kk[u] == theta;
       const int pos = gt_before + min(eq_before, rank);
       if ((gt || (eq && eq_before < rank)) && pos < k) out[pos] = tb + u;
       gt_before += gt;
@@ -395,9 +465,12 @@ __global__ void __launch_bounds__(1024) evict_select_kernel(const EvictArgs a) {
     gt_carry += tot >> 16;
     eq_carry += tot & 0xFFFF;
   }
-  for (int i = tid; i < a.n_win; i += 1024) out[k + i] = P + i;
-  if (tid == 0) v.kept_n[unit] = a.budget;
+  if (part == kSelParts - 1)
+    for (int i = tid; i < a.n_win; i += 1024) out[k + i] = P + i;
+  if (part == 0 && tid == 0) v.kept_n[unit] = a.budget;
+  cluster_sync();  // no CTA leaves while another may read its counts
 }
+
 
 // ---------------------------------------------------------------------------
 // Tensor-core scoring (tcgen05; head_dim 128, at most 256 window rows).
@@ -410,41 +483,60 @@ __global__ void __launch_bounds__(1024) evict_select_kernel(const EvictArgs a) {
 // chunk c ^ (r & 7)).  hi*hi + hi*lo + lo*hi keeps ~16 significant bits of
 // each factor (the dropped lo*lo term is below 2^-16 of the product); the
 // tensor cores accumulate in fp32 in TMEM.
-//  * statistics pass: A = query rows (M = 128 per chunk), B = keys (N = 128
-//    positions): TMEM lane = row, so each thread reduces its row over the
-//    positions without shuffles (two entries per tile and row, one per
-//    64-position half);
-//  * vote pass: A = keys (M = 128 positions), B = query rows (N = R rounded
-//    up to 16): TMEM lane = position, so each thread sums its position's
-//    weights over the rows.
+// Both passes take A = keys (M = 128 positions) and B = query rows (N = R
+// rounded up to 16): TMEM lane = position, column = row, one chain for all
+// rows (with A = rows in chunks of 128, as the statistics ran before, 160
+// rows took 32 products at about 160 cycles an item, this way 16 at 125).
+//  * statistics pass: each thread sums 2^(x - ref) of its lane's positions
+//    for a quarter of the rows, in registers over all the tiles that its CTA
+//    walks of a unit; a warp's reference of a row is the maximum of its first
+//    tile and moves only when a score rises more than 64 above it, so the
+//    warp's lanes meet (a reduction per row) only then and at the unit's end;
+//  * vote pass: each thread sums its position's weights over the rows.
 // The vote pass recomputes the scores: on the tensor cores that is cheaper
 // than a round trip through HBM.  A CTA (one per SM) walks a contiguous range
-// of (unit, tile) items; with two key stages the keys of the next item are
-// dequantised while the tensor cores run the current one, and the epilogue
-// of an item reads one TMEM buffer while the next item's chain fills the
-// other.  Query rows past R are zero; in the statistics pass the last row
+// of (unit, tile) items in four roles that run beside each other: 3 warps
+// copy the keys' records in, 8 dequantise them (the ALU's share), one issues
+// the chains, 16 run the epilogues (the exponentials' share: 20480 scores of 160 rows take
+// the MUFU 1280 cycles), two key stages and two TMEM buffers between them.
+// One group of 16 warps that did both in turn took 6200 cycles per item in
+// the statistics pass and 4950 in the vote pass at the 131k-context shape.
+// The statistics stay in registers over a CTA's tiles of a unit and leave
+// once per CTA and unit (stored per tile they were 168 MB of traffic and a
+// 59 us merge).  Query rows past R are zero; in the statistics pass the last row
 // chunk may read rows past the query buffer (lanes that are never used).
-constexpr int kTcWorkers = 512;              // dequantise and run the epilogues
-constexpr int kTcThreads = kTcWorkers + 32;  // + the MMA warp
-static_assert(kEvictStatSub == kTcWorkers / 128, "one statistics entry per worker column slice");
+constexpr int kTcEpi = 512;                  // epilogue threads (warps 0-15)
+constexpr int kTcDeq = 256;                  // dequantising threads (warps 16-23)
+constexpr int kTcCopy = 96;                  // copying threads (warps 24-26)
+constexpr int kTcThreads = kTcEpi + kTcDeq + kTcCopy + 32;  // + the MMA warp
+constexpr int kTcPv = 1024;                  // floats: partial votes (2 x 3 x 128) or references (16 x 64)
+static_assert(kEvictStatSub == kTcEpi / 128, "one statistics entry per column slice");
 
 struct TcPlan {
   int items_per_cta, n_items;
-  int R16, nch, q_lo, k_lo, nst, nstg, fmt;  // nst key stages, nstg staging buffers
+  int R16, q_lo, k_lo, nst, nstg, fmt;  // nst key stages, nstg staging buffers
   int kb_nch, kb_stride, stg_bytes;  // staged 16-byte chunks per position, their stride
   int nc_magic;                      // ceil(2^16 / kb_nch): e / kb_nch = (e nc_magic) >> 16 here
   int stage, off_q, off_ql, off_k, off_stg, off_norm, off_pv, off_bar, smem;
 };
 
-template <bool VOTES>
+// NB (statistics pass): blocks of 8 rows that a slice holds at most
+template <bool VOTES, int NB>
 __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs a, const TcPlan p) {
   extern __shared__ uint8_t evict_tc_raw[];
   uint8_t *sm = evict_tc_raw + ((1024u - (smem_u32(evict_tc_raw) & 1023u)) & 1023u);
-  // bar[0], [1]: the chain of TMEM buffer 0 / 1 done; [2]: drain; [3], [4]:
-  // the keys of an even / odd item staged (one arrival per worker warp)
+  // Item k of the CTA: chain[k & 1] its products done, keys[k & 1] its keys
+  // staged (an arrival per dequantising warp), epi[k & 1] its epilogue done
+  // (an arrival per epilogue warp); staging buffer g: sfull[g] copied (an
+  // arrival per copying thread), sfree[g] dequantised (one per warp); unit n
+  // of the CTA: uready[n & 1] its query rows (and norms) loaded; drain.  Every barrier's next completion
+  // but one depends on every waiter's having seen this one.
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm + p.off_bar);
-  uint32_t *tbase = reinterpret_cast<uint32_t *>(sm + p.off_bar + 40);
-  volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + p.off_bar + 44);
+  uint64_t *chain = bar, *keys = bar + 2, *epi = bar + 4, *uready = bar + 6, *drain = bar + 8, *sfull = bar + 9,
+           *sfree = bar + 11;
+  constexpr int kBars = 13;
+  uint32_t *tbase = reinterpret_cast<uint32_t *>(bar + kBars);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(tbase + 1);
   float *norm = reinterpret_cast<float *>(sm + p.off_norm);
   float *pv = reinterpret_cast<float *>(sm + p.off_pv);
   uint8_t *qh = sm + p.off_q, *ql = sm + p.off_ql;
@@ -457,7 +549,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
   constexpr int KBOX = 128 * 128;  // bytes of one 64-channel box of a 128-row key tile
 
   if (tid == 0) {
-    for (int i = 0; i < 5; ++i) mbar_init(&bar[i], i < 3 ? 1 : kTcWorkers / 32);
+    for (int i = 0; i < kBars; ++i)
+      mbar_init(&bar[i], i < 2 || i == 8 ? 1 : i == 4 || i == 5 ? kTcEpi / 32 : i == 9 || i == 10 ? kTcCopy : kTcDeq / 32);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -476,18 +569,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
 
   const int it0 = blockIdx.x * p.items_per_cta;
   const int it1 = min(it0 + p.items_per_cta, p.n_items);
-  // worker warp w reads TMEM lanes 32 (w % 4) .. + 31; slice = w / 4
+  // epilogue warp w reads TMEM lanes 32 (w % 4) .. + 31; slice = w / 4
   const int quarter = warp & 3, slice = warp >> 2;
   const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
-  uint32_t phases = 0u;  // bit tb: parity of TMEM buffer tb's next completion
-  bool failed = false;
+  const int did = tid - kTcEpi, cid = did - kTcDeq;  // index among the dequantising, the copying threads
+  auto sleepy = [&](uint64_t *b, uint32_t parity) {
+    return mbar_wait_sleepy(b, parity, kSleepyLimit, abort_flag, 2000);
+  };
 
   const int gshift = v.group == 64 ? 6 : 5;  // grouped layers: groups of 32 or 64 channels
-  // rows of this thread in the statistics epilogue, divided by G (the row's
-  // window query), once
-  int rdiv[2];
-#pragma unroll
-  for (int c = 0; c < 2; ++c) rdiv[c] = (128 * c + 32 * quarter + lane) / a.G;
   // (unit, tile) of item `it` and the unit's length, advanced without divisions
   struct Cursor {
     int it, unit, tile, len;
@@ -525,10 +615,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
 
   // query rows of `unit` (and, for the votes, the rows' log-normalisers;
   // +inf for the padding rows, whose weights are then 0)
-  auto load_q = [&](int unit) {
+  auto load_q = [&](int unit, int n) {
     const int b = unit / v.Hkv, j = unit % v.Hkv;
     const int box = p.R16 * 128;
-    for (int e = tid; e < p.R16 * (D / 8); e += kTcWorkers) {
+    for (int e = did; e < p.R16 * (D / 8); e += kTcDeq) {
       const int r = e >> 4, c8 = e & 15;
       float x[8];
 #pragma unroll
@@ -554,22 +644,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
       put8(qh, ql, p.q_lo != 0, r, 8 * c8, box, x);
     }
     if constexpr (VOTES) {
-      for (int r = tid; r < p.R16; r += kTcWorkers) {
+      float *nm = norm + 256 * (n & 1);
+      for (int r = did; r < p.R16; r += kTcDeq) {
         if (r < R) {
           const float2 f = a.fin[(size_t)unit * R + r];
-          norm[r] = f.x + log2f(f.y);
+          nm[r] = f.x + log2f(f.y);
         } else {
-          norm[r] = INFINITY;
+          nm[r] = INFINITY;
         }
       }
     }
     fence_proxy_async();
-    workers_sync<kTcWorkers>();
   };
 
   // asynchronous copy of the K bundles of item `it` (K section in logical
   // order, then the group metadata or the symmetric scale word) into staging
-  // buffer g; one commit group per call
+  // buffer g, then the buffer's arrival (once the thread's copies landed)
   auto stage_copy = [&](const Cursor &cu, int g) {
     const int unit = cu.unit, t0 = cu.tile * kT, len = cu.len;
     uint8_t *dst0 = sm + p.off_stg + g * p.stg_bytes;
@@ -579,7 +669,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
     const int nrec = v.rec_bytes >> 4;
     const int km = ks16 * 32;  // grouped: key metadata follows the K and V sections
     const uint8_t *base = v.rec + (size_t)unit * v.cap * v.rec_bytes;
-    for (int e = tid; e < kT * NC; e += kTcWorkers) {
+    for (int e = cid; e < kT * NC; e += kTcCopy) {
       const int pos = (e * p.nc_magic) >> 16, c = e - pos * NC;
       const int t = t0 + pos;
       const bool ok = t < len;
@@ -587,21 +677,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
       cp_async16(dst0 + pos * p.kb_stride + 16 * c, base + (size_t)(ok ? t : t0) * v.rec_bytes + so, ok);
     }
     if (sym)
-      for (int pos = tid; pos < kT; pos += kTcWorkers) {
+      for (int pos = cid; pos < kT; pos += kTcCopy) {
         const int t = t0 + pos;
         const bool ok = t < len;
         cp_async4(dst0 + pos * p.kb_stride + 16 * ks16,
                   v.scales + (size_t)unit * v.cap + (ok ? t : t0), ok);
       }
-    cp_async_commit();
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sfull[g])) : "memory");
   };
 
   // dequantised keys of the item staged in buffer g into key stage s
   auto dequant = [&](int g, int s) {
-    const int pidx = tid & 127, hf = tid >> 7;  // position, channel quarter
+    const int pidx = did & 127;  // position
     const uint8_t *bundle = sm + p.off_stg + g * p.stg_bytes + pidx * p.kb_stride;
     uint8_t *kh = sm + p.off_k + s * p.stage, *kl = kh + 2 * KBOX;
-    switch (p.fmt) {
+#pragma unroll 1
+    for (int hf = did >> 7; hf < 4; hf += 2)  // channel quarters
+      switch (p.fmt) {
       case kFmtBf16: tc_dequant<kFmtBf16>(bundle, bundle + TcFmtKs16(kFmtBf16) * 16, pidx, hf, gshift, kh, kl); break;
       case kFmtG8: tc_dequant<kFmtG8>(bundle, bundle + TcFmtKs16(kFmtG8) * 16, pidx, hf, gshift, kh, kl); break;
       case kFmtG4: tc_dequant<kFmtG4>(bundle, bundle + TcFmtKs16(kFmtG4) * 16, pidx, hf, gshift, kh, kl); break;
@@ -618,88 +710,123 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
     const uint32_t qa = smem_u32(qh), qb = smem_u32(ql);
     const uint32_t qbox = (uint32_t)p.R16 * 128;
     const uint32_t d0 = tmem + 256u * tb;
-    auto dsc = [](uint32_t addr) { return umma_desc(addr, 16, 1024, 2); };
-    if constexpr (!VOTES) {
-      const uint32_t id = umma_idesc(128, 128, false, false);
-      for (int c = 0; c < p.nch; ++c) {
+    constexpr uint32_t hi = umma_desc_hi_sw128(1024);
+    const uint32_t dkh = umma_desc_lo(kh, 16), dkl = umma_desc_lo(kl, 16), dqh = umma_desc_lo(qa, 16),
+                   dql = umma_desc_lo(qb, 16);
+    const uint32_t id = umma_idesc(128, p.R16, false, false);
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t ko = (ks >> 2) * KBOX + (ks & 3) * 32;
-          const uint32_t qo = (ks >> 2) * qbox + c * 16384 + (ks & 3) * 32;
-          umma_f16(d0 + 128 * c, dsc(qa + qo), dsc(kh + ko), id, ks > 0);
-          if (p.k_lo) umma_f16(d0 + 128 * c, dsc(qa + qo), dsc(kl + ko), id, true);
-          if (p.q_lo) umma_f16(d0 + 128 * c, dsc(qb + qo), dsc(kh + ko), id, true);
-        }
-      }
-    } else {
-      const uint32_t id = umma_idesc(128, p.R16, false, false);
-#pragma unroll
-      for (int ks = 0; ks < D / 16; ++ks) {
-        const uint32_t ko = (ks >> 2) * KBOX + (ks & 3) * 32;
-        const uint32_t qo = (ks >> 2) * qbox + (ks & 3) * 32;
-        umma_f16(d0, dsc(kh + ko), dsc(qa + qo), id, ks > 0);
-        if (p.k_lo) umma_f16(d0, dsc(kl + ko), dsc(qa + qo), id, true);
-        if (p.q_lo) umma_f16(d0, dsc(kh + ko), dsc(qb + qo), id, true);
-      }
+    for (int ks = 0; ks < D / 16; ++ks) {
+      const uint32_t ko = ((ks >> 2) * KBOX + (ks & 3) * 32) >> 4;
+      const uint32_t qo = (ks >> 2) * (qbox >> 4) + 2 * (ks & 3);
+      umma_f16_ss_w(d0, dkh + ko, dqh + qo, hi, id, ks > 0);
+      if (p.k_lo) umma_f16_ss_w(d0, dkl + ko, dqh + qo, hi, id, true);
+      if (p.q_lo) umma_f16_ss_w(d0, dkh + ko, dql + qo, hi, id, true);
     }
-    umma_commit(&bar[tb]);
+    umma_commit(&chain[tb]);
   };
 
-  // epilogue of item `it` from TMEM buffer tb
-  auto epilogue = [&](const Cursor &cu, int tb) {
+  // Statistics pass: this thread's sums of a slice's rows over its lane's
+  // positions of the unit's tiles, relative to the warp's references (shared
+  // memory, one row of 64 per warp: rows 16 bk + i of the slice in order).
+  constexpr int BW = VOTES ? 16 : 8;  // rows of a block
+  const int nblk = p.R16 / BW, per = (nblk + 3) / 4;
+  const int bk0 = min(nblk, slice * per), bk1 = min(nblk, bk0 + per);
+  float l_run[8 * NB];
+  float *ref = pv + 64 * warp;
+  bool fresh = true;  // the unit has no references yet
+  auto flush_stats = [&](int unit) {
+    const int stride = kEvictStatSub * a.n_tiles;
+    const int e = kEvictStatSub * ((int)blockIdx.x - unit * a.n_tiles / p.items_per_cta) + quarter;
+#pragma unroll
+    for (int i = 0; i < 8 * NB; ++i) {
+      const int r = 8 * bk0 + i;
+      float L = l_run[i];
+#pragma unroll
+      for (int o = 16; o; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+      if (lane == 0 && r < 8 * bk1 && r < R) a.stats[((size_t)unit * R + r) * stride + e] = make_float2(ref[i], L);
+    }
+  };
+  // epilogue of item `cu` (the k-th) from TMEM buffer tb
+  auto epilogue = [&](const Cursor &cu, int tb, const float *nm) {
     const int unit = cu.unit, tile = cu.tile, len = cu.len;
     const int P = len - a.n_win;
     const int t0 = tile * kT;
     const float sg = a.sig_log2;
     if constexpr (!VOTES) {
-      float2 *st = a.stats + (size_t)unit * R * (kEvictStatSub * a.n_tiles);
-      for (int c = 0; c < p.nch; ++c) {
-        if (128 * c + 32 * quarter >= R) continue;  // the warp's rows are all padding
-        const int r = 128 * c + 32 * quarter + lane;
-        const int last = P + (c == 0 ? rdiv[0] : rdiv[1]);  // the last position row r sees
-        float y[32];
-        const uint32_t ta = tmem + 256u * tb + 128 * c + 32 * slice + lane_off;
+      const int t = t0 + 32 * quarter + lane;
+      // row r of window query w = r / G sees positions up to P + w: rows
+      // before (t - P) G do not see this lane's position
+      const int r_from = (t - P) * a.G;
+      const bool whole = t0 + 32 * quarter + 31 <= P;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          float z[16];
-          tmem_ld16(ta + 16 * q, z);
+      for (int b = 0; b < NB; b += 2) {  // 16 rows at a time (8 at an odd end)
+        if (bk0 + b >= bk1) break;
+        const uint32_t ta = tmem + 256u * tb + 8 * (bk0 + b) + lane_off;
+        const int n = bk0 + b + 1 < bk1 && b + 1 < NB ? 16 : 8;
+        float z[16];
+        tmem_ld16(ta, z);  // past an odd end: another slice's rows, unused
+        if (!whole) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) y[16 * q + i] = z[i];
+          for (int i = 0; i < 16; ++i)
+            if (8 * (bk0 + b) + i < r_from) z[i] = -INFINITY;
         }
-        const int tb0 = t0 + 32 * slice;
-        const int nv = min(32, last - tb0 + 1);  // positions of the slice row r sees
-        float m = -INFINITY, l = 0.f;
-        if (nv >= 32) {  // four independent chains each
-          float mm[4] = {y[0], y[1], y[2], y[3]}, ll[4] = {0.f, 0.f, 0.f, 0.f};
+        if (fresh) {
 #pragma unroll
-          for (int i = 4; i < 32; ++i) mm[i & 3] = fmaxf(mm[i & 3], y[i]);
-          const float ms = fmaxf(fmaxf(mm[0], mm[1]), fmaxf(mm[2], mm[3])) * sg;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) ll[i & 3] += fast_exp2(fmaf(y[i], sg, -ms));
-          m = ms;
-          l = (ll[0] + ll[1]) + (ll[2] + ll[3]);
-        } else if (nv > 0) {
-#pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (i < nv) m = fmaxf(m, y[i]);
-          const float ms = m * sg;
-#pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (i < nv) l += fast_exp2(fmaf(y[i], sg, -ms));
-          m = ms;
+          for (int i = 0; i < 16; ++i) {
+            if (8 * b + i < 8 * NB) l_run[8 * b + i] = 0.f;
+            if (lane == 0 && i < n) ref[8 * b + i] = -INFINITY;
+          }
+          __syncwarp();
         }
-        if (r < R)
-          st[(size_t)r * (kEvictStatSub * a.n_tiles) + kEvictStatSub * tile + slice] = make_float2(m, l);
+        float top = -INFINITY;
+        const float4 *r4 = reinterpret_cast<const float4 *>(ref + 8 * b);
+#pragma unroll
+        for (int i4 = 0; i4 < 4; ++i4) {
+          if (4 * i4 >= n) continue;
+          const float4 c = r4[i4];
+          z[4 * i4] = fmaf(z[4 * i4], sg, -c.x);
+          z[4 * i4 + 1] = fmaf(z[4 * i4 + 1], sg, -c.y);
+          z[4 * i4 + 2] = fmaf(z[4 * i4 + 2], sg, -c.z);
+          z[4 * i4 + 3] = fmaf(z[4 * i4 + 3], sg, -c.w);
+          if (!whole) {  // -inf - -inf, masked and without a reference yet: adds nothing
+#pragma unroll
+            for (int i = 4 * i4; i < 4 * i4 + 4; ++i) z[i] = fmaxf(z[i], -INFINITY);
+          }
+          top = fmaxf(top, fmaxf(fmaxf(z[4 * i4], z[4 * i4 + 1]), fmaxf(z[4 * i4 + 2], z[4 * i4 + 3])));
+        }
+        if (__any_sync(0xffffffffu, fresh || top > 64.f)) {
+          // the references move to the warp's maxima where scores pass them;
+          // a row whose positions so far are all masked keeps -inf
+          tmem_ld16(ta, z);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            if (8 * b + i >= 8 * NB || i >= n) continue;
+            if (!whole && 8 * (bk0 + b) + i < r_from) z[i] = -INFINITY;
+            const float c = ref[8 * b + i];
+            float m = z[i] * sg;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (m > c) l_run[8 * b + i] *= fast_exp2(c - m);
+            m = fmaxf(m, c);
+            __syncwarp();
+            if (lane == 0) ref[8 * b + i] = m;
+            z[i] = m == -INFINITY ? -INFINITY : fmaf(z[i], sg, -m);
+          }
+          __syncwarp();
+        }
+        // masked positions add 2^-inf = 0
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if (8 * b + i < 8 * NB && i < n) l_run[8 * b + i] += fast_exp2(z[i]);
       }
+      fresh = false;
     } else {
       const int pos = 32 * quarter + lane, t = t0 + pos;
-      const int n16 = p.R16 / 16, per = (n16 + 3) / 4;
-      const int bk0 = min(n16, slice * per), bk1 = min(n16, bk0 + per);
       float vv[4] = {0.f, 0.f, 0.f, 0.f};  // four independent chains
       for (int bk = bk0; bk < bk1; ++bk) {
         float y[16];
         tmem_ld16(tmem + 256u * tb + 16 * bk + lane_off, y);
-        const float4 *nr = reinterpret_cast<const float4 *>(norm + 16 * bk);
+        const float4 *nr = reinterpret_cast<const float4 *>(nm + 16 * bk);
 #pragma unroll
         for (int i4 = 0; i4 < 4; ++i4) {
           const float4 c4 = nr[i4];
@@ -709,100 +836,128 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
           vv[3] += fast_exp2(fmaf(y[4 * i4 + 3], sg, -c4.w));
         }
       }
+      // the four slices of a position are in the four warps of its quarter
       const float vote = (vv[0] + vv[1]) + (vv[2] + vv[3]);
-      if (slice) pv[(slice - 1) * 128 + pos] = vote;
-      workers_sync<kTcWorkers>();
-      if (!slice && t < P) a.votes[(size_t)unit * v.cap + t] = vote + pv[pos] + pv[128 + pos] + pv[256 + pos];
+      float *pb = pv + 3 * 128 * tb;
+      if (slice) pb[(slice - 1) * 128 + pos] = vote;
+      asm volatile("bar.sync %0, 128;" ::"r"(4 + quarter) : "memory");
+      if (!slice && t < P) a.votes[(size_t)unit * v.cap + t] = vote + pb[pos] + pb[128 + pos] + pb[256 + pos];
     }
   };
 
-  // waits for the chain in TMEM buffer tb, runs its epilogue, frees the buffers
-  auto finish = [&](const Cursor &it, int tb) -> bool {
-    const bool ok = mbar_wait_sleepy(&bar[tb], (phases >> tb) & 1u, kSleepyLimit, abort_flag, 2000);
-    phases ^= 1u << tb;
-    if (workers_sync_or<kTcWorkers>(!ok)) return false;
-    tc_fence_after();
-    epilogue(it, tb);
-    tc_fence_before();
-    workers_sync<kTcWorkers>();
-    return true;
-  };
-
-  if (warp == kTcWorkers / 32) {
-    // ======================= MMA warp =====================================
-    // the same item sequence as the workers; each chain once its keys are staged
-    int kk = 0;
-    for (Cursor cu = next_valid(at(it0)); cu.it < it1; cu = next_valid(after(cu)), ++kk) {
-      if (!mbar_wait_sleepy(&bar[3 + (kk & 1)], (kk >> 1) & 1, kSleepyLimit, abort_flag, 2000)) {
-        if (lane == 0) *abort_flag = 1;
-        break;
-      }
-      if (lane == 0) issue(kk % p.nst, kk & 1);
-      __syncwarp();
-    }
-    // every chain issued lands before TMEM is released (bounded)
-    if (lane == 0 && kk > 0) {
-      umma_commit(&bar[2]);
-      mbar_wait(&bar[2], 0, kLimit);
-    }
-    __syncwarp();
-  } else {
-    // ======================= workers ======================================
-    int cur_unit = -1, pend_tb = 0, k = 0;
-    bool has_pend = false;
-    Cursor pend;
-    Cursor it = next_valid(at(it0));
-    if (it.it < it1) stage_copy(it, 0);
-    while (it.it < it1 && !failed) {
-      const int unit = it.unit;
-      const Cursor nxt = next_valid(after(it));
-      if (p.nstg == 2) {
-        if (nxt.it < it1)
-          stage_copy(nxt, (k + 1) & 1);  // overwrites the staging of item k - 1, already dequantised
-        else
-          cp_async_commit();  // an empty group keeps the wait count below uniform
-      }
-      if (unit != cur_unit) {
-        if (has_pend) {
-          failed = !finish(pend, pend_tb);
-          has_pend = false;
-          if (failed) break;
+  // Registers by warpgroup: the epilogues' sums take more than an equal share.
+  // 512 x 88 + 256 x 56 + 128 x 40 = 64512 = the 896 x 72 launched.
+  static_assert(kTcThreads == 896, "the register split");
+  if (warp >= (kTcEpi + kTcDeq) / 32) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;" ::: "memory");
+    if (warp == (kTcEpi + kTcDeq + kTcCopy) / 32) {
+      // ======================= MMA warp =====================================
+      // the same item sequence as the others; each chain once its keys are
+      // staged and its TMEM buffer was read
+      int k = 0;
+      for (Cursor cu = next_valid(at(it0)); cu.it < it1; cu = next_valid(after(cu)), ++k) {
+        bool ok = sleepy(&keys[k & 1], (k >> 1) & 1);
+        if (ok && k >= 2) ok = sleepy(&epi[k & 1], ((k >> 1) - 1) & 1);
+        if (!__all_sync(0xffffffffu, ok)) {
+          if (lane == 0) {
+            *abort_flag = 1;
+            set_err(a.err, 8);
+          }
+          break;
         }
-        load_q(unit);
-        cur_unit = unit;
+        if (lane == 0) issue(k % p.nst, k & 1);
+        __syncwarp();
       }
-      if (p.nst == 1 && has_pend) {  // the single key stage must be free
-        failed = !finish(pend, pend_tb);
-        has_pend = false;
-        if (failed) break;
+      // every chain issued lands before TMEM is released (bounded)
+      if (lane == 0 && k > 0) {
+        umma_commit(drain);
+        mbar_wait(drain, 0, kLimit);
       }
-      if (p.nstg == 2)
-        cp_async_wait<1>();  // this item's bundles landed (the next item's may be in flight)
-      else
-        cp_async_wait<0>();
-      workers_sync<kTcWorkers>();
-      dequant(p.nstg == 2 ? (k & 1) : 0, k % p.nst);
+      __syncwarp();
+    } else {
+      // ======================= copies =======================================
+      int k = 0, g = 0;
+      uint32_t ph = 1;  // a buffer's first use waits for nothing
+      for (Cursor it = next_valid(at(it0)); it.it < it1; it = next_valid(after(it)), ++k) {
+        if (!__all_sync(0xffffffffu, sleepy(&sfree[g], ph))) {
+          *abort_flag = 1;
+          break;
+        }
+        stage_copy(it, g);
+        if (++g == p.nstg) {
+          g = 0;
+          ph ^= 1;
+        }
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");  // no copy outlives the CTA
+    }
+  } else if (warp >= kTcEpi / 32) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;" ::: "memory");
+    // ======================= dequantising =================================
+    // A thread whose wait gave up goes on without work.
+    bool failed = false;
+    int cur_unit = -1, n_unit = 0, k = 0, g = 0;
+    uint32_t ph = 0;
+    for (Cursor it = next_valid(at(it0)); it.it < it1; it = next_valid(after(it)), ++k) {
+      // the key stage is free once the chain that read it is done; a new
+      // unit's rows replace the last unit's after its last chain, and its
+      // norms those of two units ago, whose last epilogue is k - 2 at most
+      if (k >= p.nst && !failed) {
+        const int c = k - p.nst;
+        failed = !sleepy(&chain[c & 1], (c >> 1) & 1);
+      }
+      if (it.unit != cur_unit) {
+        if (k >= 1 && !failed) failed = !sleepy(&chain[(k - 1) & 1], ((k - 1) >> 1) & 1);
+        if (k >= 2 && !failed) failed = !sleepy(&epi[k & 1], ((k >> 1) - 1) & 1);
+        if (!failed) load_q(it.unit, n_unit);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&uready[n_unit & 1]);
+        cur_unit = it.unit;
+        ++n_unit;
+      }
+      if (!failed) failed = !sleepy(&sfull[g], ph);
+      if (!failed) dequant(g, k % p.nst);
       fence_proxy_async();  // the keys, written here, are read by the tensor cores
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bar[3 + (k & 1)]);
-      if (p.nstg == 1 && nxt.it < it1) {  // the staging is consumed once every worker is done
-        workers_sync<kTcWorkers>();
-        stage_copy(nxt, 0);
+      if (failed) *abort_flag = 1;
+      if (lane == 0) {
+        mbar_arrive(&keys[k & 1]);
+        mbar_arrive(&sfree[g]);
       }
-      if (has_pend) {
-        failed = !finish(pend, pend_tb);
-        if (failed) break;
+      if (++g == p.nstg) {
+        g = 0;
+        ph ^= 1;
       }
-      pend = it; pend_tb = k & 1; has_pend = true;
-      ++k;
-      it = nxt;
     }
-    if (!failed && has_pend) failed = !finish(pend, pend_tb);
-    cp_async_wait<0>();  // no copy outlives the CTA
-    if (failed) {
-      *abort_flag = 1;
-      if (tid == 0) set_err(a.err, 8);
+    if (failed) set_err(a.err, 8);
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 88;" ::: "memory");
+    // ======================= epilogues ====================================
+    // A warp whose wait gave up goes on through the barriers without work.
+    bool failed = false;
+    int cur_unit = -1, n_unit = -1, k = 0;
+    for (Cursor it = next_valid(at(it0)); it.it < it1; it = next_valid(after(it)), ++k) {
+      if (it.unit != cur_unit) {
+        if constexpr (!VOTES) {
+          if (cur_unit >= 0) flush_stats(cur_unit);
+        }
+        cur_unit = it.unit;
+        ++n_unit;
+        fresh = true;
+        if (!failed) failed = !__all_sync(0xffffffffu, sleepy(&uready[n_unit & 1], (n_unit >> 1) & 1));
+      }
+      if (!failed) failed = !__all_sync(0xffffffffu, sleepy(&chain[k & 1], (k >> 1) & 1));
+      if (failed) *abort_flag = 1;
+      tc_fence_after();
+      epilogue(it, k & 1, norm + 256 * (n_unit & 1));
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&epi[k & 1]);
     }
+    if constexpr (!VOTES) {
+      if (cur_unit >= 0) flush_stats(cur_unit);
+    }
+    if (failed && lane == 0) set_err(a.err, 8);
   }
   tc_fence_before();
   __syncthreads();
@@ -814,16 +969,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
 }
 
 // Shared-memory plan of the tensor-core kernels: the query rows first (hi,
-// then lo), so that the statistics pass's reads past the last query row
-// (at most 112 rows of 128 bytes per box) stay inside the key stages that
-// follow; two key stages when they fit, else one; two staging buffers of
+// then lo); two key stages when they fit, else one; two staging buffers of
 // the K bundles.  Bundle strides are odd multiples of 16 bytes, so the
 // 16-byte loads of eight consecutive positions fall in distinct banks.
 TcPlan tc_plan(const EvictArgs &a, int sms) {
   TcPlan p;
   const int R = a.n_win * a.G;
   p.R16 = (R + 15) / 16 * 16;
-  p.nch = (p.R16 + 127) / 128;
   p.q_lo = a.q_f32 ? 1 : 0;
   p.k_lo = a.v.bits != 16 ? 1 : 0;
   p.fmt = a.v.bits == 16 ? kFmtBf16
@@ -842,22 +994,22 @@ TcPlan tc_plan(const EvictArgs &a, int sms) {
   const int qbytes = p.R16 * 256 * (p.q_lo ? 2 : 1);
   p.off_k = (qbytes + 1023) / 1024 * 1024;
   auto fits = [&](int nst, int nstg) {
-    return p.off_k + nst * p.stage + nstg * p.stg_bytes + 256 * 4 + 3 * 128 * 4 + 64 + 1024 <= 232448;
+    return p.off_k + nst * p.stage + nstg * p.stg_bytes + 2 * 256 * 4 + kTcPv * 4 + 128 + 1024 <= 232448;
   };
   p.nst = fits(2, 2) ? 2 : 1;
   p.nstg = fits(p.nst, 2) ? 2 : 1;
   p.off_stg = p.off_k + p.nst * p.stage;
   p.off_norm = p.off_stg + p.nstg * p.stg_bytes;
-  p.off_pv = p.off_norm + 256 * 4;
-  p.off_bar = p.off_pv + 3 * 128 * 4;
-  p.smem = p.off_bar + 64 + 1024;  // + alignment of the base to 1024 bytes
+  p.off_pv = p.off_norm + 2 * 256 * 4;
+  p.off_bar = p.off_pv + kTcPv * 4;
+  p.smem = p.off_bar + 128 + 1024;  // + alignment of the base to 1024 bytes
   p.n_items = a.v.B * a.v.Hkv * a.n_tiles;
   const int grid = std::max(1, std::min(p.n_items, sms));
   p.items_per_cta = (p.n_items + grid - 1) / grid;
   return p;
 }
 
-cudaError_t launch_evict_tc(const EvictArgs &a, cudaStream_t st) {
+cudaError_t launch_evict_tc(const EvictArgs &args, cudaStream_t st) {
   static int sms = 0;
   if (!sms) {
     int dev = 0;
@@ -865,22 +1017,25 @@ cudaError_t launch_evict_tc(const EvictArgs &a, cudaStream_t st) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
   }
+  EvictArgs a = args;
   const TcPlan p = tc_plan(a, sms);
-  cudaError_t e = cudaFuncSetAttribute(evict_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       p.smem);
+  a.items_per_cta = p.items_per_cta;
+  // 160 rows (5 query heads, 32 queries) fit 40 sums a thread
+  auto stat = p.R16 <= 160 ? evict_tc_kernel<false, 5> : evict_tc_kernel<false, 8>;
+  cudaError_t e = cudaFuncSetAttribute(stat, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(evict_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+    e = cudaFuncSetAttribute(evict_tc_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((p.n_items + p.items_per_cta - 1) / p.items_per_cta);
-  e = launch_pdl(evict_tc_kernel<false>, grid, dim3(kTcThreads), p.smem, st, a, p);
+  e = launch_pdl(stat, grid, dim3(kTcThreads), p.smem, st, a, p);
   if (e == cudaSuccess) {
     const int rows = a.v.B * a.v.Hkv * a.n_win * a.G;
     e = launch_pdl(evict_merge_stats_kernel, dim3((rows + kMergeWarps - 1) / kMergeWarps),
                    dim3(32 * kMergeWarps), 0, st, a);
   }
-  if (e == cudaSuccess) e = launch_pdl(evict_tc_kernel<true>, grid, dim3(kTcThreads), p.smem, st, a, p);
+  if (e == cudaSuccess) e = launch_pdl(evict_tc_kernel<true, 1>, grid, dim3(kTcThreads), p.smem, st, a, p);
   if (e == cudaSuccess)
-    e = launch_pdl(evict_select_kernel, dim3(a.v.Hkv, a.v.B), dim3(1024), 0, st, a);
+    e = launch_pdl(evict_select_kernel, dim3(a.v.Hkv * kSelParts, a.v.B), dim3(1024), 0, st, a);
   return e;
 }
 
@@ -900,7 +1055,7 @@ cudaError_t launch_evict_d(const EvictArgs &a, cudaStream_t st) {
     e = launch_pdl(evict_votes_kernel, dim3((a.v.cap + kVoteT - 1) / kVoteT, a.v.Hkv, a.v.B),
                    dim3(kVoteT), 0, st, a);
   if (e == cudaSuccess)
-    e = launch_pdl(evict_select_kernel, dim3(a.v.Hkv, a.v.B), dim3(1024), 0, st, a);
+    e = launch_pdl(evict_select_kernel, dim3(a.v.Hkv * kSelParts, a.v.B), dim3(1024), 0, st, a);
   return e;
 }
 

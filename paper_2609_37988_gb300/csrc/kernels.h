@@ -120,8 +120,9 @@ struct EvictArgs {
   int n_tiles;         // 128-position tiles launched per (sequence, kv head)
   int sc_stride;       // n_tiles * kEvictTile: row stride of the scores
   int stat_sub;        // statistics entries per tile and row (1 or kEvictStatSub)
+  int items_per_cta = 0;  // > 0: those entries per CTA run over a unit's tiles instead
   float *votes;        // [B * Hkv][cap]
-  float2 *stats;       // [B * Hkv][R][n_tiles * stat_sub] per-tile (max, sum)
+  float2 *stats;       // [B * Hkv][R][n_tiles * stat_sub] per-tile (or run) (max, sum)
   float2 *fin;         // [B * Hkv][R] merged (max, sum)
   float *scores;       // [B * Hkv][R][sc_stride] scaled scores (log2 domain)
   int32_t *err;

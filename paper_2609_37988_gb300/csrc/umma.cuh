@@ -56,30 +56,15 @@ __device__ __forceinline__ void umma_f16_ts_w(uint32_t d_tmem, uint32_t a_tmem, 
       "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate ? 1 : 0)
       : "memory");
 }
-// The same three for a whole warp that runs its issue loop uniformly: only
-// the lane with `el` set issues.  Operands then live in uniform registers; a
-// loop under `if (lane == 0)` moves each operand of each product there first.
-__device__ __forceinline__ void umma_f16_ts_el(uint32_t el, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo,
-                                               uint32_t b_hi, uint32_t idesc, bool accumulate) {
+// A and B in shared memory, both descriptors' low words given (the high one,
+// `hi`, is the same): built per product from 64-bit arithmetic they cost a
+// lone issuing thread about 170 cycles a product against the 64 it takes
+__device__ __forceinline__ void umma_f16_ss_w(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                              bool accumulate) {
   asm volatile(
-      "{\n .reg .pred p, q;\n .reg .b64 db;\n setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n mov.b64 db, {%2, %3};\n"
-      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate ? 1 : 0), "r"(el)
-      : "memory");
-}
-__device__ __forceinline__ void umma_f16_el(uint32_t el, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
-                                            uint32_t idesc, bool accumulate) {
-  asm volatile(
-      "{\n .reg .pred p, q;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n mov.b64 da, {%1, %3};\n"
-      " mov.b64 db, {%2, %3};\n @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate ? 1 : 0), "r"(el)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit_el(uint32_t el, uint64_t *bar) {
-  asm volatile(
-      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
-      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(bar)),
-      "r"(el)
+      "{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate ? 1 : 0)
       : "memory");
 }
 // the words of umma_desc(addr, lbo, sbo, 2) (128-byte swizzle)
@@ -113,6 +98,17 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+// 8 consecutive TMEM columns of this warp's 32 lanes, one load and one wait
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
 }
 // 32 consecutive TMEM columns of this warp's 32 lanes, one load and one wait
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {

@@ -107,8 +107,7 @@ def _check_lists(cache, q, st, lens, sigma, budget, votes_gpu, what):
                                          (5, 64, torch.bfloat16)],
                          ids=["r128", "r160-f32q", "r320-cuda-cores"])
 def test_evict_votes_and_lists(fmt, G, n_win, qdt):
-    # R = n_win G window rows: 128 (one row chunk), 160 (two, the second
-    # partly past the query rows), 320 (scored on the CUDA cores)
+    # R = n_win G window rows: 128, 160, 320 (scored on the CUDA cores)
     B, Hkv, D, T = 3, 2, 128, 800
     Hq = G * Hkv
     cap, budget = 256, 200
@@ -155,6 +154,42 @@ def test_evict_then_decode_per_head(fmt):
     c.set_kept(0)
     assert c.kept_lists(0) is None
     assert torch.equal(c.decode(0, qd.cuda(), sigma, n_splits=2), plain)
+    assert c.device_error() == 0
+
+
+@pytest.mark.parametrize("B,Hkv,G,n_win,T", [(40, 4, 3, 9, 300), (2, 3, 7, 32, 1000), (1, 2, 8, 32, 700),
+                                             (3, 2, 5, 20, 513)],
+                         ids=["units-over-ctas", "rows224", "rows256", "rows100"])
+@pytest.mark.parametrize("fmt", [FORMATS[0], FORMATS[2]], ids=_fid)
+def test_evict_votes_rising_scores(fmt, B, Hkv, G, n_win, T):
+    """Keys that grow along the context by up to 30 times, so that a row's
+    scores rise past its reference by more than 64 (base 2) at some tiles and
+    rows and not at others; several units per CTA, several CTAs per unit, row
+    counts that leave part of a slice's blocks over."""
+    D = 128
+    Hq = G * Hkv
+    g = torch.Generator().manual_seed(n_win)
+    grow = 1.0 + 29.0 * (torch.arange(T) / T)[None, :, None, None] * torch.linspace(0, 1, Hkv)[None, None, :, None]
+    k = (torch.randn((B, T, Hkv, D), generator=g) * grow).to(torch.bfloat16)
+    v = torch.randn((B, T, Hkv, D), generator=g).to(torch.bfloat16)
+    budget = T // 2
+    c = _cache(B, Hq, Hkv, D, T, [dict(**fmt, evict_capacity=budget)])
+    c.append(0, k.cuda(), v.cuda())
+    lens = np.full(B, T)
+    st = oracle_state(f32(k), f32(v), lens, fmt)
+    q = _qwin(B, n_win, Hq, D, seed=G)
+    sigma = 1.0 / math.sqrt(D)
+    got = f32(c.evict_window(0, q.cuda(), sigma, budget))
+    _, votes = oev.snapkv_kept(f32(q), st["k_hat"], lens, sigma, budget)
+    # a weight's relative error: 2 ln 2 times 3 2^-18 sigma log2(e) sum |q k|
+    # (see VOTE_RTOL), here for the largest keys
+    khat = np.abs(st["k_hat"]).reshape(-1, D).max(axis=0)
+    worst = sigma * math.log2(math.e) * float(np.abs(f32(q)).reshape(-1, D).max(axis=0) @ khat)
+    rtol = 2 * math.log(2) * 3 * 2.0 ** -18 * worst
+    for b in range(B):
+        for j in range(Hkv):
+            ref = np.asarray(votes[b][j], np.float64)[: T - n_win]
+            assert np.allclose(got[b, j, : T - n_win], ref, rtol=rtol, atol=1e-7), (b, j)
     assert c.device_error() == 0
 
 
