@@ -323,29 +323,32 @@ __device__ __forceinline__ int cluster_ld(const int *p, uint32_t rank) {
 // Kept list of one (sequence, kv head): the budget - n_win largest votes by
 // a radix select on their bit patterns (votes are >= 0, so the patterns
 // order as the values), then the chosen positions in increasing order and
-// the window.  A cluster of 8 CTAs per unit, each over an eighth of the
-// positions: a unit's votes are read five times, which one CTA per unit did
-// in 110 us for 32 units of 131072 positions with 120 SMs idle.  Per pass
-// the CTAs add each other's histograms through distributed shared memory and
-// decide alike (one cluster barrier per pass: two histograms in turn).
-constexpr int kSelParts = 8;
-__global__ void __cluster_dims__(kSelParts, 1, 1) __launch_bounds__(1024) evict_select_kernel(const EvictArgs a) {
+// the window.  PARTS = 8: a cluster of 8 CTAs per unit, each over an eighth
+// of the positions: a unit's votes are read five times, which one CTA per
+// unit did in 110 us for 32 units of 131072 positions with 120 SMs idle (64
+// us so).  Per pass the CTAs add each other's histograms through distributed
+// shared memory and decide alike (one cluster barrier per pass: two
+// histograms in turn).  Up to 16384 positions one CTA (PARTS = 1) is faster:
+// the barriers cost more than its few rounds (8153 positions: 27 us, 43).
+constexpr int kSelParts = 8, kSelOneCta = 16384;
+template <int PARTS>
+__global__ void __cluster_dims__(PARTS, 1, 1) __launch_bounds__(1024) evict_select_kernel(const EvictArgs a) {
   pdl_wait();
   pdl_trigger();
   const GqaView &v = a.v;
-  const int j = blockIdx.x / kSelParts, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int part = (int)cluster_rank();
+  const int j = blockIdx.x / PARTS, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int part = PARTS > 1 ? (int)cluster_rank() : 0;
   const int unit = b * v.Hkv + j;
   const int len = v.lens[b];
   int32_t *out = v.kept_idx + (size_t)unit * v.kept_cap;
   if (len <= a.budget) {  // everything is kept (the whole cluster leaves)
-    for (int t = part * 1024 + tid; t < len; t += kSelParts * 1024) out[t] = t;
+    for (int t = part * 1024 + tid; t < len; t += PARTS * 1024) out[t] = t;
     if (part == 0 && tid == 0) v.kept_n[unit] = len;
     return;
   }
   const int P = len - a.n_win, k = a.budget - a.n_win;
   const uint32_t *key = reinterpret_cast<const uint32_t *>(a.votes + (size_t)unit * v.cap);
-  const int per = ((P + kSelParts - 1) / kSelParts + 7) / 8 * 8;
+  const int per = ((P + PARTS - 1) / PARTS + 7) / 8 * 8;
   const int p0 = min(P, part * per), p1 = min(P, p0 + per);  // this CTA's positions
   __shared__ int hist[2][256];
   __shared__ uint32_t s_prefix;
@@ -381,11 +384,17 @@ __global__ void __cluster_dims__(kSelParts, 1, 1) __launch_bounds__(1024) evict_
           }
         }
       }
-      cluster_sync();
+      if (PARTS > 1) cluster_sync();
+      else __syncthreads();
       // bins from the top: the one in which the count reaches the rank
       int n = 0, inc = 0;
       if (tid < 256) {
-        for (uint32_t r = 0; r < kSelParts; ++r) n += cluster_ld(&h[255 - tid], r);
+        if (PARTS > 1) {
+#pragma unroll
+          for (uint32_t r = 0; r < PARTS; ++r) n += cluster_ld(&h[255 - tid], r);
+        } else {
+          n = h[255 - tid];
+        }
         inc = n;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -415,7 +424,7 @@ __global__ void __cluster_dims__(kSelParts, 1, 1) __launch_bounds__(1024) evict_
   // positions before this CTA's
   const uint32_t theta = prefix;
   int gt_carry = 0, eq_carry = 0;
-  if (k > 0) {
+  if (PARTS > 1 && k > 0) {
     if (tid < 2) s_cnt[tid] = 0;
     __syncthreads();
     int ngt = 0, neq = 0;
@@ -465,12 +474,17 @@ __global__ void __cluster_dims__(kSelParts, 1, 1) __launch_bounds__(1024) evict_
     gt_carry += tot >> 16;
     eq_carry += tot & 0xFFFF;
   }
-  if (part == kSelParts - 1)
+  if (part == PARTS - 1)
     for (int i = tid; i < a.n_win; i += 1024) out[k + i] = P + i;
   if (part == 0 && tid == 0) v.kept_n[unit] = a.budget;
-  cluster_sync();  // no CTA leaves while another may read its counts
+  if (PARTS > 1) cluster_sync();  // no CTA leaves while another may read its counts
 }
 
+
+cudaError_t launch_evict_select(const EvictArgs &a, cudaStream_t st) {
+  if (a.v.cap <= kSelOneCta) return launch_pdl(evict_select_kernel<1>, dim3(a.v.Hkv, a.v.B), dim3(1024), 0, st, a);
+  return launch_pdl(evict_select_kernel<kSelParts>, dim3(a.v.Hkv * kSelParts, a.v.B), dim3(1024), 0, st, a);
+}
 
 // ---------------------------------------------------------------------------
 // Tensor-core scoring (tcgen05; head_dim 128, at most 256 window rows).
@@ -797,22 +811,43 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
         if (__any_sync(0xffffffffu, fresh || top > 64.f)) {
           // the references move to the warp's maxima where scores pass them;
           // a row whose positions so far are all masked keeps -inf
-          tmem_ld16(ta, z);
+          auto scores = [&]() {
+            tmem_ld16(ta, z);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            if (8 * b + i >= 8 * NB || i >= n) continue;
-            if (!whole && 8 * (bk0 + b) + i < r_from) z[i] = -INFINITY;
-            const float c = ref[8 * b + i];
-            float m = z[i] * sg;
+            for (int i = 0; i < 16; ++i)
+              if (!whole && 8 * (bk0 + b) + i < r_from) z[i] = -INFINITY;
+          };
+          scores();
 #pragma unroll
-            for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (m > c) l_run[8 * b + i] *= fast_exp2(c - m);
-            m = fmaxf(m, c);
+          for (int o = 16; o; o >>= 1)  // 16 reductions side by side
+#pragma unroll
+            for (int i = 0; i < 16; ++i) z[i] = fmaxf(z[i], __shfl_xor_sync(0xffffffffu, z[i], o));
+          __syncwarp();
+#pragma unroll
+          for (int i4 = 0; i4 < 4; ++i4) {
+            if (4 * i4 >= n) continue;
+            const float4 c4 = r4[i4];
+            const float c[4] = {c4.x, c4.y, c4.z, c4.w};
+            float m[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              m[u] = fmaxf(z[4 * i4 + u] * sg, c[u]);
+              if (8 * b + 4 * i4 + u < 8 * NB && m[u] > c[u]) l_run[8 * b + 4 * i4 + u] *= fast_exp2(c[u] - m[u]);
+            }
             __syncwarp();
-            if (lane == 0) ref[8 * b + i] = m;
-            z[i] = m == -INFINITY ? -INFINITY : fmaf(z[i], sg, -m);
+            if (lane == 0) reinterpret_cast<float4 *>(ref + 8 * b)[i4] = make_float4(m[0], m[1], m[2], m[3]);
           }
           __syncwarp();
+          scores();
+#pragma unroll
+          for (int i4 = 0; i4 < 4; ++i4) {
+            if (4 * i4 >= n) continue;
+            const float4 c = r4[i4];
+            z[4 * i4] = fmaxf(fmaf(z[4 * i4], sg, -c.x), -INFINITY);
+            z[4 * i4 + 1] = fmaxf(fmaf(z[4 * i4 + 1], sg, -c.y), -INFINITY);
+            z[4 * i4 + 2] = fmaxf(fmaf(z[4 * i4 + 2], sg, -c.z), -INFINITY);
+            z[4 * i4 + 3] = fmaxf(fmaf(z[4 * i4 + 3], sg, -c.w), -INFINITY);
+          }
         }
         // masked positions add 2^-inf = 0
 #pragma unroll
@@ -1035,7 +1070,7 @@ cudaError_t launch_evict_tc(const EvictArgs &args, cudaStream_t st) {
   }
   if (e == cudaSuccess) e = launch_pdl(evict_tc_kernel<true, 1>, grid, dim3(kTcThreads), p.smem, st, a, p);
   if (e == cudaSuccess)
-    e = launch_pdl(evict_select_kernel, dim3(a.v.Hkv * kSelParts, a.v.B), dim3(1024), 0, st, a);
+    e = launch_evict_select(a, st);
   return e;
 }
 
@@ -1055,7 +1090,7 @@ cudaError_t launch_evict_d(const EvictArgs &a, cudaStream_t st) {
     e = launch_pdl(evict_votes_kernel, dim3((a.v.cap + kVoteT - 1) / kVoteT, a.v.Hkv, a.v.B),
                    dim3(kVoteT), 0, st, a);
   if (e == cudaSuccess)
-    e = launch_pdl(evict_select_kernel, dim3(a.v.Hkv * kSelParts, a.v.B), dim3(1024), 0, st, a);
+    e = launch_evict_select(a, st);
   return e;
 }
 
