@@ -199,7 +199,10 @@ kvk_status kvk_rewind(kvk_cache *cache, int32_t n, kvk_stream stream);
  * for `layer` with n_splits = 0 (host only; depends on the host-side bound
  * on the anchor's lengths, the SM count and the decode schedule).  Under the
  * run schedule (kvk_set_decode_schedule) it is the number of partial slots
- * per (sequence, KV head) that kvk_decode_partial with n_splits = 0 writes. */
+ * per (sequence, KV head) that kvk_decode_partial with n_splits = 0 writes.
+ * kvk_decode_attention over several sequences whose units all fit one wave
+ * of CTAs may split each sequence by its own length instead (the same count
+ * where the lengths are equal). */
 kvk_status kvk_decode_plan_splits(kvk_cache *cache, int32_t layer, int32_t *n_splits);
 
 /* Install the kept-position list of anchor `layer` (eviction, Sec. 3.4):
@@ -453,7 +456,10 @@ kvk_status kvk_set_wait_limit(kvk_cache *cache, uint32_t polls);
  *  KVK_SCHEDULE_AUTO (default): the runs where the split grid would give
  *      each CTA at most 13 tiles and leave its last wave of CTAs less than
  *      90 % full (and every run CTA gets at least four tiles), else the
- *      splits.
+ *      splits; kvk_decode_attention takes splits in proportion to each
+ *      sequence's length instead where they make one wave (2 to 62
+ *      sequences, contiguous reads; instead of the runs where whole splits
+ *      fill at least 85 % of it).
  * run_ctas: the number of run CTAs (clamped to [units, tiles], units = B *
  * H_kv, tiles of 64 or 128 positions per unit); 0 = the fewest whole waves
  * of resident CTAs that are at least the units.  run_setup: planned tiles

@@ -1167,6 +1167,65 @@ __device__ __forceinline__ bool gqa_run_segment(const GqaDecodeArgs &a, int k, G
   return true;
 }
 
+// Balanced splits: unit (b, kvh), items [i0, i1) (i1 = -1: to the end) and
+// partial slot of CTA blockIdx.x of a one-dimensional grid of n CTAs.  With
+// t_b kernel tiles of sequence b (from its length on the device), R is the
+// smallest number of tiles per CTA for which sum_b Hkv ceil(t_b / R) <= n and
+// no unit takes more than bal_cap slots: the least possible longest CTA of
+// one wave with a unit's tiles in equal splits.  The split grid cuts every
+// sequence by the longest one's length, so a short sequence's last splits
+// find nothing to do: ragged batches (lengths from half to all of 8192,
+// 16 x 4 units of int4 with per-channel keys) left a quarter of the CTAs
+// empty.  Every warp finds the same answer (lane: sequences lane, lane + 32).
+struct GqaBalSeg {
+  int b, kvh, i0, i1, slot;
+};
+template <int TILE>
+__device__ __forceinline__ bool gqa_balanced_split(const GqaDecodeArgs &a, GqaBalSeg &sg) {
+  const GqaView &v = a.v;
+  const int lane = threadIdx.x & 31, n = gridDim.x, x = blockIdx.x;
+  int t[2], k[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int b = lane + 32 * h;
+    t[h] = b < v.B ? max(1, (v.lens[b] + TILE - 1) / TILE) : 0;
+  }
+  const int sum = __reduce_add_sync(0xffffffffu, t[0] + t[1]) * v.Hkv;
+  const int top = __reduce_max_sync(0xffffffffu, max(t[0], t[1]));
+  int r = max((sum + n - 1) / n, (top + a.bal_cap - 1) / a.bal_cap);
+  for (;; ++r) {  // ends: at r = top every unit takes one CTA
+#pragma unroll
+    for (int h = 0; h < 2; ++h) k[h] = (t[h] + r - 1) / r;
+    if (r >= top || __reduce_add_sync(0xffffffffu, k[0] + k[1]) * v.Hkv <= n) break;
+  }
+  // CTAs in order of (sequence, kv head, slot): this one's sequence
+  int base = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int inc = k[h];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    const int lo = v.Hkv * (base + inc - k[h]), hi = v.Hkv * (base + inc);
+    const uint32_t m = __ballot_sync(0xffffffffu, x >= lo && x < hi);
+    if (m) {
+      const int l = __ffs(m) - 1;
+      const int kb = __shfl_sync(0xffffffffu, k[h], l), rel = x - __shfl_sync(0xffffffffu, lo, l);
+      sg.b = l + 32 * h;
+      sg.kvh = rel / kb;
+      sg.slot = rel - sg.kvh * kb;
+      sg.i0 = sg.slot * r * TILE;
+      sg.i1 = sg.slot == kb - 1 ? -1 : sg.i0 + r * TILE;
+      if (rel == 0 && threadIdx.x == 0) a.bal_counts[sg.b] = kb;
+      return true;
+    }
+    base += __shfl_sync(0xffffffffu, inc, 31);
+  }
+  return false;  // more CTAs than splits
+}
+
 // RUN = false: grid (split, kv head, sequence); CTA (x, y, z) decodes items
 // [x ips, (x + 1) ips) of unit (z, y) into partial slot x (ips =
 // a.items_per_split; the last split runs to the end, so a launch recorded
@@ -1206,6 +1265,14 @@ __global__ void __launch_bounds__(128, GqaCfg<BITS, D, KAX, GS>::MIN_CTAS)
     __syncthreads();
   }
   if constexpr (!RUN) {
+    if constexpr (!GATHER) {
+      if (a.bal_ctas > 0) {
+        GqaBalSeg sg;
+        if (gqa_balanced_split<C::TILE>(a, sg))
+          gqa_decode_unit<BITS, D, KAX, GS, GATHER>(a, &rows, sg.b, sg.kvh, sg.i0, sg.i1, sg.slot, 0);
+        return;
+      }
+    }
     const int split = blockIdx.x;
     const int i0 = split * a.items_per_split;
     const int i1 = split == a.n_splits - 1 ? -1 : i0 + a.items_per_split;
@@ -1261,6 +1328,7 @@ cudaError_t launch_gqa_decode_g(const GqaDecodeArgs &a, cudaStream_t st) {
   }
   if constexpr (RUN) return launch_pdl(k, dim3(a.run_ctas), dim3(128), C::SMEM, st, rows, a);
   dim3 grid(a.n_splits, a.v.Hkv, a.v.B);
+  if (a.bal_ctas > 0) grid = dim3(a.bal_ctas);
   return launch_pdl(k, grid, dim3(128), C::SMEM, st, rows, a);
 }
 

@@ -402,6 +402,32 @@ bool plan_runs(kvk_cache *c, int a, RunPlan *p) {
   return true;
 }
 
+// Balanced splits of an automatic decode of anchor a (kernel side in
+// decode_gqa.cuh, gqa_balanced_split), given what plan_runs and auto_splits
+// (`splits`) chose: the number of CTAs, 0 if the decode keeps their schedule.
+// Taken where one wave of resident CTAs holds the units at two or more splits
+// each and the other plan is one wave too; over sequences of equal length the
+// splits are then those of the split grid.  Instead of the runs only if whole
+// splits fill 85 % of the wave (the runs fill all of it, but only if the
+// lengths are equal).  *cap: partial slots per unit, twice the even share (a
+// sequence twice as long as the average takes it), in the merge's steps.
+int plan_balanced(kvk_cache *c, int a, bool runs, int splits, int *cap) {
+  if (c->schedule != KVK_SCHEDULE_AUTO || c->kept_on[a]) return 0;
+  if (c->desc.max_batch < 2 || c->desc.max_batch > kBalanceMaxBatch) return 0;
+  const kvk_layer_cfg &L = c->cfg[a];
+  const int units = c->desc.max_batch * c->desc.n_kv_heads, slots = c->sm_count * c->ctas[a];
+  const int share = slots / units;
+  if (share < 2 || splits < 2) return 0;
+  if (runs ? share * units < 0.85 * slots : splits * units > slots) return 0;
+  const int per = gqa_decode_tile(L.bits, c->desc.head_dim, L.bits == 16 ? 0 : L.key_axis, layer_group(&c->desc, &L),
+                                  layer_scheme(&L)) / kTile;
+  const int ktiles = (layer_tiles(c, a) + per - 1) / per;
+  if (ktiles < 2) return 0;
+  *cap = std::min(c->max_splits, share <= 4 ? 8 : share <= 12 ? 16 : 2 * share);
+  if (*cap < std::min(share, ktiles)) return 0;
+  return (int)std::min<long long>(slots, (long long)units * ktiles);
+}
+
 // The shortest chunk of layer `a` that attends over formed keys and values;
 // shorter ones run the absorbed decode per row.  Both costs in ns per cached
 // position, measured (4 x 4096, 1 x 8192 and 8 x 1024 positions, 8-128
@@ -977,13 +1003,20 @@ static kvk_status gqa_decode_common(kvk_cache *c, int32_t layer, const void *q, 
   args.gather = c->kept_on[a];
   const int tiles = layer_tiles(c, a);
   RunPlan rp;
-  const bool runs = n_splits == 0 && plan_runs(c, a, &rp);
+  const bool automatic = n_splits == 0;
+  bool runs = automatic && plan_runs(c, a, &rp);
   if (runs) n_splits = rp.slots;
   if (n_splits == 0) n_splits = auto_splits(c, a);
+  int bal_cap = 0;
+  const int bal = automatic && merge && !partial ? plan_balanced(c, a, runs, std::min(n_splits, tiles), &bal_cap) : 0;
+  if (bal) {
+    runs = false;
+    n_splits = bal_cap;  // slots
+  }
   // a partial-only call keeps the caller's split count (extra splits are
   // empty and write m = -inf, l = 0); a full call never uses more splits
   // than tiles.
-  if (merge && !runs) n_splits = std::min(n_splits, tiles);
+  if (merge && !runs && !bal) n_splits = std::min(n_splits, tiles);
   args.q = q;
   args.q_f32 = q_dtype == KVK_DTYPE_F32;
   args.Hq = c->desc.n_q_heads;
@@ -1008,7 +1041,12 @@ static kvk_status gqa_decode_common(kvk_cache *c, int32_t layer, const void *q, 
     args.run_setup = rp.setup;
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (merge && n_splits == 1 && !runs) {
+  if (bal) {
+    args.bal_ctas = bal;
+    args.bal_cap = bal_cap;
+    args.bal_counts = c->err() + 1;  // the workspace's first block, after the error word
+  }
+  if (merge && n_splits == 1 && !runs && !bal) {
     args.out = out;  // one split: the kernel normalises and writes the output
     args.partial = nullptr;
   } else {
@@ -1017,9 +1055,9 @@ static kvk_status gqa_decode_common(kvk_cache *c, int32_t layer, const void *q, 
   }
   cudaError_t e = launch_gqa_decode(args, st);
   if (e != cudaSuccess) return cuda_fail(e, "decode launch");
-  if (merge && (n_splits > 1 || runs)) {
+  if (merge && (n_splits > 1 || runs || bal)) {
     e = launch_splitk_merge(args.partial, n_splits, c->desc.max_batch * c->desc.n_q_heads,
-                            c->desc.head_dim, out, st);
+                            c->desc.head_dim, out, st, args.bal_counts, c->desc.n_q_heads);
     if (e != cudaSuccess) return cuda_fail(e, "merge launch");
   }
   return KVK_OK;

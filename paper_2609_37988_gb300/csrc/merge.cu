@@ -23,7 +23,7 @@ namespace {
 template <int SB>
 __global__ void __launch_bounds__(128)
     splitk_merge_kernel(const float *P, int S, int n_rows, int dim,
-                        float *__restrict__ out) {
+                        float *__restrict__ out, const int32_t *counts, int rows_per) {
   pdl_wait();
   pdl_trigger();
   const int width = dim >= 128 ? 128 : dim;  // threads per row
@@ -34,6 +34,9 @@ __global__ void __launch_bounds__(128)
   const size_t RS = (size_t)dim + 2;
   const size_t SS = (size_t)n_rows * RS;  // split stride
   const float *pr = P + (size_t)row * RS;
+  // with per-sequence counts every slot up to S is loaded beside the count
+  // (the slots exist) and those past it are dropped
+  const int n = counts ? counts[row / rows_per] : S;
   float m[SB], l[SB];
 #pragma unroll
   for (int s = 0; s < SB; ++s) {
@@ -44,6 +47,12 @@ __global__ void __launch_bounds__(128)
     float x[SB];
 #pragma unroll
     for (int s = 0; s < SB; ++s) x[s] = s < S ? pr[s * SS + ch] : 0.f;
+#pragma unroll
+    for (int s = 0; s < SB; ++s)
+      if (s >= n) {
+        m[s] = -INFINITY;
+        x[s] = l[s] = 0.f;
+      }
     float M = -INFINITY;
 #pragma unroll
     for (int s = 0; s < SB; ++s) M = fmaxf(M, m[s]);
@@ -70,7 +79,8 @@ __global__ void __launch_bounds__(128)
 // around it (one sequence of 32769 int8 positions) went 40.3 -> 33.4 us.
 constexpr int kWideWarps = 8, kWideRound = 8;
 __global__ void __launch_bounds__(32 * kWideWarps)
-    splitk_merge_wide(const float *P, int S, int n_rows, int dim, float *__restrict__ out) {
+    splitk_merge_wide(const float *P, int S, int n_rows, int dim, float *__restrict__ out,
+                      const int32_t *counts, int rows_per) {
   pdl_wait();
   pdl_trigger();
   __shared__ float s_m[kWideWarps], s_l[kWideWarps], s_a[kWideWarps][128];
@@ -98,16 +108,31 @@ __global__ void __launch_bounds__(32 * kWideWarps)
     l[i] = s < S ? pr[s * SS + dim + 1] : 0.f;
   }
   load_acc(0);
+  // per-sequence counts: the slots past the row's own are dropped (every
+  // slot up to S exists)
+  const int n = counts ? counts[row / rows_per] : S;
+  auto drop = [&]() {
+#pragma unroll
+    for (int i = 0; i < kWideRound; ++i)
+      if (warp + kWideWarps * i >= n) {
+        m[i] = -INFINITY;
+        l[i] = x[i][0] = x[i][1] = x[i][2] = x[i][3] = 0.f;
+      }
+  };
+  drop();
   float M = -INFINITY;
 #pragma unroll
   for (int i = 0; i < kWideRound; ++i) M = fmaxf(M, m[i]);
-  for (int s = warp + kWideWarps * kWideRound; s < S; s += kWideWarps) M = fmaxf(M, pr[s * SS + dim]);
+  for (int s = warp + kWideWarps * kWideRound; s < n; s += kWideWarps) M = fmaxf(M, pr[s * SS + dim]);
   if (lane == 0) s_m[warp] = M;
   __syncthreads();
 #pragma unroll
   for (int w = 0; w < kWideWarps; ++w) M = fmaxf(M, s_m[w]);
   for (int ch0 = 0; ch0 < dim; ch0 += 128) {
-    if (ch0 > 0) load_acc(ch0);
+    if (ch0 > 0) {
+      load_acc(ch0);
+      drop();
+    }
     float L = 0.f, A[4] = {0.f, 0.f, 0.f, 0.f};
     if (M != -INFINITY) {
 #pragma unroll
@@ -117,7 +142,7 @@ __global__ void __launch_bounds__(32 * kWideWarps)
 #pragma unroll
         for (int j = 0; j < 4; ++j) A[j] = fmaf(w, x[i][j], A[j]);
       }
-      for (int s = warp + kWideWarps * kWideRound; s < S; s += kWideWarps) {
+      for (int s = warp + kWideWarps * kWideRound; s < n; s += kWideWarps) {
         const float ms = pr[s * SS + dim];
         const float w = ms == -INFINITY ? 0.f : exp2f(ms - M);
         L = fmaf(w, pr[s * SS + dim + 1], L);
@@ -162,17 +187,20 @@ cudaError_t launch_rewind(const RewindArgs &a, cudaStream_t st) {
 }
 
 cudaError_t launch_splitk_merge(const float *partials, int n_splits, int n_rows, int dim,
-                                float *out, cudaStream_t st) {
+                                float *out, cudaStream_t st, const int32_t *counts, int rows_per) {
   if (n_splits < 1 || n_rows < 0 || dim < 1) return cudaErrorInvalidValue;
   if (n_rows == 0) return cudaSuccess;
   const int rpc = dim >= 128 ? 1 : 128 / dim;
   const int grid = (n_rows + rpc - 1) / rpc;
   if (n_splits <= 8)
-    return launch_pdl(splitk_merge_kernel<8>, grid, dim3(128), 0, st, partials, n_splits, n_rows, dim, out);
+    return launch_pdl(splitk_merge_kernel<8>, grid, dim3(128), 0, st, partials, n_splits, n_rows, dim, out, counts,
+                      rows_per);
   else if (n_splits <= 16)
-    return launch_pdl(splitk_merge_kernel<16>, grid, dim3(128), 0, st, partials, n_splits, n_rows, dim, out);
+    return launch_pdl(splitk_merge_kernel<16>, grid, dim3(128), 0, st, partials, n_splits, n_rows, dim, out, counts,
+                      rows_per);
   else
-    return launch_pdl(splitk_merge_wide, n_rows, dim3(32 * kWideWarps), 0, st, partials, n_splits, n_rows, dim, out);
+    return launch_pdl(splitk_merge_wide, n_rows, dim3(32 * kWideWarps), 0, st, partials, n_splits, n_rows, dim, out, counts,
+                      rows_per);
 }
 
 }  // namespace kvk

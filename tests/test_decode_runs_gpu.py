@@ -209,3 +209,63 @@ def test_schedule_argument_checks():
         c.set_decode_schedule(3)
     with pytest.raises(KVKError, match="INVALID_ARG"):
         c.set_decode_schedule(RUNS, -1)
+
+
+BAL_FORMATS = FORMATS[:1] + FORMATS[4:7] + [dict(bits=16, group=64, key_axis="token"),
+                                            dict(bits=8, group=64, key_axis="channel"),
+                                            dict(bits=4, group=32, key_axis="channel")]
+
+
+@pytest.mark.parametrize("fmt", BAL_FORMATS, ids=lambda f: _fid(f) + f["key_axis"][0])
+@pytest.mark.parametrize("lens", [[3000, 0, 1, 777, 129], [130, 64, 65, 3000], [2999] * 3,
+                                  [(37 * i) % 700 for i in range(41)]],
+                         ids=["one-long", "long-last", "equal", "41-sequences"])
+def test_balanced_splits_match_the_oracle(fmt, lens):
+    """Automatic decodes of a few units split each sequence by its own length
+    (a sequence's splits in proportion, one wave): every position read once,
+    empty and one-position sequences, sequences in both halves of the lanes,
+    a long sequence that reaches the slot limit."""
+    B, Hkv, G, D = len(lens), 2, 5, 128
+    c = _cache(B, G * Hkv, Hkv, D, 3008, fmt, max_splits=16)
+    K, V = _fill(c, B, Hkv, D, lens, seed=fmt["bits"] + len(lens))
+    st = oracle_state(K, V, np.array(lens), fmt)
+    sigma = 1.0 / math.sqrt(D)
+    q = torch.randn((B, G * Hkv, D), generator=torch.Generator().manual_seed(2)).to(torch.bfloat16)
+    ref = gqa_expected(q, st, np.array(lens), sigma)
+    out = c.decode(0, q.cuda(), sigma)
+    assert_close(f32(out), ref, what=f"balanced {_fid(fmt)}")
+    assert (f32(out)[np.array(lens) == 0] == 0).all()
+    c.set_decode_schedule(SPLITS)
+    assert_close(f32(c.decode(0, q.cuda(), sigma)), f32(out), max_abs=1e-4, rel_l2=1e-4, what="balanced = splits")
+    assert c.device_error() == 0
+
+
+def test_recorded_balanced_launch_covers_longer_sequences():
+    """Recorded at one length bound, replayed after one sequence grew past
+    it: the splits follow the lengths on the device."""
+    fmt = dict(bits=4, group=32, key_axis="token")
+    B, Hkv, G, D = 3, 2, 4, 128
+    c = _cache(B, G * Hkv, Hkv, D, 4096, fmt)
+    g = torch.Generator().manual_seed(3)
+    k = torch.randn((B, 4000, Hkv, D), generator=g).to(torch.bfloat16)
+    v = torch.randn((B, 4000, Hkv, D), generator=g).to(torch.bfloat16)
+    c.append(0, k[:, :300].contiguous().cuda(), v[:, :300].contiguous().cuda())
+    q = torch.randn((B, G * Hkv, D), generator=g).to(torch.bfloat16).cuda()
+    out = torch.empty((B, G * Hkv, D), device="cuda")
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        c.decode(0, q, 0.1, out=out, stream=s)  # warm (kernel attributes set outside capture)
+        s.synchronize()
+        gr = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(gr, stream=s):
+            c.decode(0, q, 0.1, out=out, stream=s)
+    torch.cuda.synchronize()
+    more = torch.tensor([3700, 0, 411], dtype=torch.int32, device="cuda")
+    c.append(0, k[:, 300:].contiguous().cuda(), v[:, 300:].contiguous().cuda(), more)
+    torch.cuda.synchronize()
+    gr.replay()
+    torch.cuda.synchronize()
+    lens = np.array([4000, 300, 711])
+    st = oracle_state(f32(k), f32(v), lens, fmt)
+    assert_close(f32(out), gqa_expected(q.cpu(), st, lens, 0.1), what="replayed")
+    assert c.device_error() == 0
