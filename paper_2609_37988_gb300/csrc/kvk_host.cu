@@ -429,16 +429,17 @@ int plan_balanced(kvk_cache *c, int a, bool runs, int splits, int *cap) {
 }
 
 // The shortest chunk of layer `a` that attends over formed keys and values;
-// shorter ones run the absorbed decode per row.  Both costs in ns per cached
-// position, measured (4 x 4096, 1 x 8192 and 8 x 1024 positions, 8-128
-// queries, every width; e.g. bf16 d = 512, 4 x 4096, absorbed / formed us: 48
-// queries 162 / 163, 64 170 / 162, 96 309 / 163; d = 64: 128 92 / 134, 1 x
-// 8192 d = 512: 8 266 / 203):
-//  absorbed: a wave of resident CTAs (one row each, or two at d >= 256 over
-//            bf16 latents) takes `full` (`half` if at most half of it is
-//            there), plus about 10 us;
-//  formed:   a wave of jobs (128 rows of one head) 14.8, the forming itself
-//            `form` per sequence, plus about 15 us.
+// shorter ones run the absorbed decode per row.  Both costs in ns, fitted to
+// measured calls (1 x 1500, 4 x 300, 4 x 4096, 8 x 1024, 16 x 600 positions,
+// 16-250 queries, every width; e.g. bf16 d = 512, 4 x 4096, absorbed / formed
+// us: 48 queries 162 / 163, 96 308 / 163; d = 64: 128 92 / 134, 250 170 / 137;
+// 8-bit d = 512, 8 x 1024: 16 55 / 92, 48 150 / 92):
+//  absorbed: per position, a wave of resident CTAs (one row each, or two at
+//            d >= 256 over bf16 latents) takes kFull (kHalf if at most half
+//            of it is there); absorption and merge kRow per row; 10 us;
+//  formed:   per position, a wave of jobs (128 rows of one head) takes 14.8
+//            and the forming kForm per sequence (quantised 0.6 more); 30 us
+//            (quantised 33, grouped 41 with the weights' column sums).
 // The answer is one more than the longest chunk (of up to 1024 queries) that
 // the absorbed path serves faster; at least 16 (a handful of queries is not
 // worth the formed tiles' memory), never where one head's tiles pass 2 GiB.
@@ -446,22 +447,25 @@ int mla_formed_from(const kvk_cache *c, int a) {
   const kvk_layer_cfg &L = c->cfg[a];
   const int w = L.width == 512 ? 0 : L.width == 256 ? 1 : L.width == 128 ? 2 : 3;
   static const double kHalf[4] = {36.0, 14.5, 10.0, 8.5}, kFull[4] = {41.0, 18.5, 15.6, 12.0};
-  static const double kQuant[4] = {37.0, 18.5, 10.5, 10.0};
-  static const double kForm[4] = {5.1, 3.9, 3.5, 3.3}, kFormQ[4] = {3.5, 2.5, 1.8, 1.5};
+  static const double kQuant[4] = {37.0, 18.5, 10.5, 10.0}, kRow[4] = {75.0, 40.0, 22.0, 14.0};
+  static const double kForm[4] = {4.4, 3.2, 2.9, 2.7};
+  const bool quant = L.bits != 16;
   if (c->lay[a].cap > (1 << 21)) return INT32_MAX;
   const double B = c->desc.max_batch, H = c->desc.n_q_heads, T = c->desc.max_ctx, sms = c->sm_count;
   for (int n = std::min(1024, c->desc.max_ctx); n >= 1; --n) {
     const double rows = B * n;
-    double absorbed;
-    if (L.bits != 16) {
-      absorbed = kQuant[w] * std::ceil(rows / sms);
+    double wave;
+    if (quant) {
+      wave = kQuant[w] * std::ceil(rows / sms);
     } else {
       const double slots = w >= 2 || n % 2 == 0 ? 2.0 * sms : sms;
-      absorbed = rows <= slots / 2 ? kHalf[w] : kFull[w] * std::ceil(rows / slots);
+      wave = rows <= slots / 2 ? kHalf[w] : kFull[w] * std::ceil(rows / slots);
     }
+    const double absorbed = wave * T + kRow[w] * rows + 10e3;
     const double jobs = B * H * ((n + 127) / 128);
-    const double formed = 14.8 * std::ceil(jobs / sms) + B * (kForm[w] + (L.bits != 16 ? kFormQ[w] : 0.0));
-    if (absorbed * T + 10e3 < formed * T + 15e3) return std::max(16, n + 1);
+    const double formed = (14.8 * std::ceil(jobs / sms) + B * (kForm[w] + (quant ? 0.6 : 0.0))) * T +
+                          (!quant ? 30e3 : layer_scheme(&L) == kSchemeSym ? 33e3 : 41e3);
+    if (absorbed < formed) return std::max(16, n + 1);
   }
   return 16;
 }

@@ -70,19 +70,15 @@ __device__ __forceinline__ void st_sector(void *p, uint4 a, uint4 b) {
                : "memory");
 }
 
-// Codes 8 j .. 8 j + 7 of a quantised record (layout.h), as small integers.
+// Codes of chunk j (8 codes, layout.h) of 16 bytes of a quantised record.
 template <int BITS>
-__device__ __forceinline__ void fm_codes(const uint8_t *rec, int j, int (&u)[8]) {
+__device__ __forceinline__ void fm_codes(const uint4 &q, int j, int (&u)[8]) {
+  const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
   if constexpr (BITS == 8) {
-    const uint2 w = reinterpret_cast<const uint2 *>(rec)[j];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      u[k] = (w.x >> (8 * k)) & 255u;
-      u[4 + k] = (w.y >> (8 * k)) & 255u;
-    }
+    for (int k = 0; k < 8; ++k) u[k] = (w4[2 * j + (k >> 2)] >> (8 * (k & 3))) & 255u;
   } else {
-    const uint32_t w = BITS == 4 ? reinterpret_cast<const uint32_t *>(rec)[j]
-                                 : (uint32_t)reinterpret_cast<const uint16_t *>(rec)[j];
+    const uint32_t w = BITS == 4 ? w4[j] : w4[j >> 1] >> (16 * (j & 1));
 #pragma unroll
     for (int k = 0; k < 8; ++k) u[k] = (w >> mla_q_bit(k, BITS)) & ((1u << BITS) - 1u);
   }
@@ -294,22 +290,46 @@ __global__ void __launch_bounds__(kFmThreads, 1)
         } else {
           const bool sym = v.scheme == kSchemeSym;
           const int C0 = sym ? (1 << (BITS - 1)) - 1 : 1 << (BITS - 1);
-          for (int e = tid; e < kFmRows * (per + 8); e += kFmEpi) {
-            const int r = e / (per + 8), c = e - r * (per + 8);
-            const bool ok = t0 + r < len;
-            int u[8];
-            uint32_t w[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
-            if (ok) fm_codes<BITS>(rec + (size_t)r * v.rec_bytes, c, u);
-            if (c < per) {
-              if (ok) {
+          // the record as 16-byte pieces of CH chunks (records, and the
+          // latent's share of one, are whole pieces; a power of two of them)
+          constexpr int CH = 16 / BITS, U = 4;
+          const int sh = 31 - __clz(W * BITS / 128), pieces = kFmRows << sh;
+          for (int e0 = tid; e0 < pieces; e0 += U * kFmEpi) {
+            uint4 q[U];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) w[k] = pack_bf16((float)(u[2 * k] - C0), (float)(u[2 * k + 1] - C0));
+            for (int i = 0; i < U; ++i) {  // U loads in flight
+              const int e = e0 + i * kFmEpi, r = e >> sh, c = e & ((1 << sh) - 1);
+              q[i] = e < pieces && t0 + r < len
+                         ? *reinterpret_cast<const uint4 *>(rec + (size_t)r * v.rec_bytes + 16 * c)
+                         : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+              const int e = e0 + i * kFmEpi, r = e >> sh, c16 = e & ((1 << sh) - 1);
+              if (e >= pieces) break;
+              const bool ok = t0 + r < len;
+#pragma unroll
+              for (int j = 0; j < CH; ++j) {
+                int u[8];
+                fm_codes<BITS>(q[i], j, u);
+                uint32_t w[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) w[k] = ok ? pack_bf16((float)(u[2 * k] - C0), (float)(u[2 * k + 1] - C0)) : 0u;
+                const int c = CH * c16 + j;
+                *reinterpret_cast<uint4 *>(sm + (c >> 3) * kFmABox + r * 128 + (((c & 7) ^ (r & 7)) << 4)) =
+                    make_uint4(w[0], w[1], w[2], w[3]);
               }
-              *reinterpret_cast<uint4 *>(sm + (c >> 3) * kFmABox + r * 128 + (((c & 7) ^ (r & 7)) << 4)) =
-                  make_uint4(w[0], w[1], w[2], w[3]);
-            } else if (cur.h == 0) {
+            }
+          }
+          if (cur.h == 0) {  // the block's positional keys, once per group of heads
+            constexpr int RP = BITS / 2;  // 16-byte pieces of k^R (64 codes)
+            for (int e = tid; e < kFmRows * RP; e += kFmEpi) {
+              const int r = e / RP, c16 = e - r * RP;
+              const bool ok = t0 + r < len;
+              uint4 q = make_uint4(0, 0, 0, 0);
+              float s = 0.f, z = 0.f;
               if (ok) {
-                float s, z;
+                q = *reinterpret_cast<const uint4 *>(rec + (size_t)r * v.rec_bytes + W * BITS / 8 + 16 * c16);
                 if (sym) {
                   s = __uint_as_float(reinterpret_cast<const uint32_t *>(v.meta)[(size_t)b * v.cap + t0 + r] & 0xFFFF0000u);
                   z = -(float)C0 * s;
@@ -318,13 +338,20 @@ __global__ void __launch_bounds__(kFmThreads, 1)
                   s = m.z;
                   z = m.w;
                 }
+              }
+#pragma unroll
+              for (int j = 0; j < CH; ++j) {
+                int u[8];
+                fm_codes<BITS>(q, j, u);
+                uint32_t w[4], lo[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
                   split2<true>(fmaf((float)u[2 * k], s, z), fmaf((float)u[2 * k + 1], s, z), w[k], lo[k]);
+                uint8_t *dst = a.kr + ((size_t)cur.b * a.n_t + cur.t) * a.kr_bytes + r * 128 +
+                               (((CH * c16 + j) ^ (r & 7)) << 4);
+                *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4 *>(dst + 16384) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
               }
-              uint8_t *dst = a.kr + ((size_t)cur.b * a.n_t + cur.t) * a.kr_bytes + r * 128 + (((c - per) ^ (r & 7)) << 4);
-              *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-              *reinterpret_cast<uint4 *>(dst + 16384) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             }
           }
           if (tid < kFmRows) {
