@@ -810,36 +810,38 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) v.lens[b] = min((long long)len + nb, (long long)v.cap);
 }
 
-// Per-channel key groups completed by this append: one warp per (sequence,
-// KV head, group of GS positions).  The group's keys (residual rows for
-// positions already stored, the appended rows for new ones, rounded to
-// bf16 as the residual holds them) are staged in natural channel order in
-// shared memory; lane L quantises the channel pairs {c, c + 8} of pairs L
-// (and L + 32 when D = 128; c = 16 (p / 8) + p % 8: the two channels of one
-// 4-bit byte)
-// over the group's positions: scale = fl((max - min) / levels) correctly
-// rounded, codes rint((x - min) / scale) through the fast reciprocal with
-// the rounding check of rint_quot_fast (the correctly rounded division
-// where it cannot decide), the codes packed into the positions' key
-// sections in shared memory and stored as whole 16-byte chunks.
-constexpr int kKgWarps = 4;
-// dynamic shared memory of gqa_append_kgroups: per warp the staged keys
-// (GS rows of D + 8 bf16) and the key sections (GS rows of D bits / 8 bytes)
-__host__ __device__ constexpr int kg_warp_bytes(int D, int GS, int bits) {
+// Per-channel key groups completed by this append: one CTA of 128 threads per
+// (sequence, KV head, group of GS positions).  The group's keys (residual
+// rows for positions already stored, the appended rows for new ones, rounded
+// to bf16 as the residual holds them) are staged in natural channel order in
+// shared memory; the channel pairs {c, c + 8} (c = 16 (p / 8) + p % 8: the two
+// channels of one 4-bit byte) are shared by 128 / (D / 2) threads that take
+// a part of the positions each and meet over their extrema: scale = fl((max
+// - min) / levels) correctly rounded, codes rint((x - min) / scale) by
+// residual steps (quarter_codes; the division for scales out of their
+// range), packed into the
+// positions' key sections in shared memory and stored as whole 16-byte
+// chunks.  Bound by the latency of that chain: a warp per group, with two
+// passes over all positions, took 48 us for a single group per (sequence, KV
+// head) and held 8 warps per SM by its shared memory.
+constexpr int kKgThreads = 128;
+// dynamic shared memory of gqa_append_kgroups: the staged keys (GS rows of
+// D + 8 bf16) and the key sections (GS rows of D bits / 8 bytes)
+__host__ __device__ constexpr int kg_bytes(int D, int GS, int bits) {
   return ((GS * (D + 8) * 2 + GS * D * bits / 8) + 15) & ~15;
 }
 template <int D>
-__global__ void __launch_bounds__(32 * kKgWarps)
+__global__ void __launch_bounds__(kKgThreads)
     gqa_append_kgroups(const GqaView v, const void *kin, int in_f32, int n_new,
-                       const int32_t *n_per_seq, int32_t *err, int max_groups) {
+                       const int32_t *n_per_seq, int max_groups) {
   pdl_wait();
   pdl_trigger();
   constexpr int PAD = D + 8;                      // bf16 per staged row (conflict-free columns)
+  constexpr int PAIRS = D / 2, PARTS = kKgThreads / PAIRS;
   extern __shared__ __align__(16) uint8_t kg_smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const size_t wid = (size_t)blockIdx.x * kKgWarps + warp;
-  const size_t total = (size_t)v.B * v.Hkv * max_groups;
-  if (wid >= total) return;
+  __shared__ float s_mn[kKgThreads][2], s_mx[kKgThreads][2];
+  const int tid = threadIdx.x;
+  const size_t wid = blockIdx.x;
   const int gidx = (int)(wid % max_groups);
   const int kvh = (int)((wid / max_groups) % v.Hkv);
   const int b = (int)(wid / ((size_t)max_groups * v.Hkv));
@@ -847,106 +849,110 @@ __global__ void __launch_bounds__(32 * kKgWarps)
   const int nb = seq_count(n_per_seq, b, n_new, nullptr);
   const int len0 = v.lens[b];
   const int G = len0 / GS + gidx;  // candidate group
-  if ((G + 1) * GS > len0 + nb || (G + 1) * GS > v.cap) return;  // not completed now (warp-uniform)
+  if ((G + 1) * GS > len0 + nb || (G + 1) * GS > v.cap) return;  // not completed now (CTA-uniform)
   const size_t slab = (size_t)b * v.Hkv + kvh;
   const RecLayout L = rec_layout(v.bits, D, GS, 1);
   const int sec = D * v.bits / 8;
   const uint8_t *res = v.resid + slab * (size_t)GS * D * 2;
-  uint8_t *wbase = kg_smem + warp * kg_warp_bytes(D, GS, v.bits);
-  uint16_t *xs = reinterpret_cast<uint16_t *>(wbase);
-  uint8_t *ks = wbase + GS * PAD * 2;
+  uint16_t *xs = reinterpret_cast<uint16_t *>(kg_smem);
+  uint8_t *ks = kg_smem + GS * PAD * 2;
   // ---- the group's keys, natural channel order ----
   constexpr int CPR = D / 8;  // 8-channel pieces per row
-  for (int q = lane; q < GS * CPR; q += 32) {
+#pragma unroll 4
+  for (int q = tid; q < GS * CPR; q += kKgThreads) {
     const int r = q / CPR, c8 = 8 * (q - r * CPR);
     const int p = G * GS + r;
-    uint16_t h[8];
+    uint4 o;
     if (p < len0) {
-      // residual row r: bf16 in the key fragment order
+      // residual row r: bf16 in the key fragment order (channels 2 i, 2 i + 1
+      // of a piece are neighbours)
+      uint32_t w[4];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
+      for (int e = 0; e < 4; ++e) {
         int kb, khi;
-        k_pos(c8 + e, 16, D, &kb, &khi);
-        h[e] = *reinterpret_cast<const uint16_t *>(res + (size_t)r * D * 2 + kb);
+        k_pos(c8 + 2 * e, 16, D, &kb, &khi);
+        w[e] = *reinterpret_cast<const uint32_t *>(res + (size_t)r * D * 2 + kb);
       }
+      o = make_uint4(w[0], w[1], w[2], w[3]);
     } else {
       const size_t ii = (((size_t)b * n_new + (p - len0)) * v.Hkv + kvh) * D + c8;
       if (in_f32) {
         const float4 *src = reinterpret_cast<const float4 *>(static_cast<const float *>(kin) + ii);
         const float4 u0 = src[0], u1 = src[1];
-        const float f[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-#pragma unroll
-        for (int e = 0; e < 8; ++e) h[e] = f32_to_bf16_bits(f[e]);
+        o = make_uint4(pack_bf16(u0.x, u0.y), pack_bf16(u0.z, u0.w), pack_bf16(u1.x, u1.y), pack_bf16(u1.z, u1.w));
       } else {
-        const uint4 u = *reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(kin) + ii);
-        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) { h[2 * e] = (uint16_t)(w[e] & 0xffffu); h[2 * e + 1] = (uint16_t)(w[e] >> 16); }
+        o = *reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(kin) + ii);
       }
     }
-    uint4 o;
-    o.x = h[0] | ((uint32_t)h[1] << 16); o.y = h[2] | ((uint32_t)h[3] << 16);
-    o.z = h[4] | ((uint32_t)h[5] << 16); o.w = h[6] | ((uint32_t)h[7] << 16);
     *reinterpret_cast<uint4 *>(xs + r * PAD + c8) = o;
   }
-  for (int q = lane; q < GS * sec / 16; q += 32) reinterpret_cast<uint4 *>(ks)[q] = make_uint4(0, 0, 0, 0);
-  __syncwarp();
+  __syncthreads();
   // ---- per channel: scale, zero, codes ----
   const float lev = (float)((1 << v.bits) - 1);
-#pragma unroll
-  for (int pp = 0; pp < D / 64; ++pp) {  // D / 2 channel pairs, 32 per pass
-    const int pr = lane + 32 * pp;
-    const int ch0 = (pr >> 3) * 16 + (pr & 7);
-    float sc[2], zr[2], rs[2];
+  const int pr = tid % PAIRS, part = tid / PAIRS;
+  const int ch0 = (pr >> 3) * 16 + (pr & 7);
+  const int r0 = part * GS / PARTS, r1 = (part + 1) * GS / PARTS;
+  float mn[2] = {INFINITY, INFINITY}, mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll 4
+  for (int r = r0; r < r1; ++r)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int ch = ch0 + 8 * h;
-      float mn = INFINITY, mx = -INFINITY;
-      for (int r = 0; r < GS; ++r) {
-        const float x = bf16_to_f32(xs[r * PAD + ch]);
-        mn = fminf(mn, x);
-        mx = fmaxf(mx, x);
-      }
-      sc[h] = __fdiv_rn(__fsub_rn(mx, mn), lev);
-      zr[h] = mn;
-      rs[h] = sc[h] == 0.f ? 0.f : __fdividef(1.f, sc[h]);
-      v.gmeta[(slab * (v.cap / GS) + G) * D + ch] = make_float2(sc[h], mn);
+      const float x = bf16_to_f32(xs[r * PAD + ch0 + 8 * h]);
+      mn[h] = fminf(mn[h], x);
+      mx[h] = fmaxf(mx[h], x);
     }
-    int kb0, kh0, kb1, kh1;
-    k_pos(ch0, v.bits, D, &kb0, &kh0);
-    k_pos(ch0 + 8, v.bits, D, &kb1, &kh1);
-    for (int r = 0; r < GS; ++r) {
-      uint32_t c[2];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (sc[h] == 0.f) {
-          c[h] = 0u;
-        } else {
-          const float d = __fsub_rn(bf16_to_f32(xs[r * PAD + ch0 + 8 * h]), zr[h]);
-          bool near;
-          float q = rint_quot_fast(d, rs[h], near);
-          if (near) q = rintf(__fdiv_rn(d, sc[h]));
-          c[h] = (uint32_t)fminf(fmaxf(q, 0.f), lev);
-        }
-      }
-      if (v.bits == 8) {
-        ks[r * sec + kb0] = (uint8_t)c[0];
-        ks[r * sec + kb1] = (uint8_t)c[1];
-      } else {
-        // channels ch0 and ch0 + 8 share one byte (low and high nibble)
-        ks[r * sec + kb0] = (uint8_t)(c[0] | (c[1] << 4));
-      }
+  for (int h = 0; h < 2; ++h) {
+    s_mn[tid][h] = mn[h];
+    s_mx[tid][h] = mx[h];
+  }
+  __syncthreads();
+  float sc[2], zr[2], rs[2];
+  bool wide[2];  // a scale out of the residual steps' range (quarter_codes)
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int o = 0; o < PARTS; ++o) {
+      mn[h] = fminf(mn[h], s_mn[o * PAIRS + pr][h]);
+      mx[h] = fmaxf(mx[h], s_mx[o * PAIRS + pr][h]);
+    }
+    sc[h] = __fdiv_rn(__fsub_rn(mx[h], mn[h]), lev);
+    zr[h] = mn[h];
+    rs[h] = __frcp_rn(sc[h]);
+    wide[h] = !(sc[h] >= 0x1p-96f && sc[h] <= 0x1p96f);
+    if (part == 0) v.gmeta[(slab * (v.cap / GS) + G) * D + ch0 + 8 * h] = make_float2(sc[h], mn[h]);
+  }
+  int kb0, kh0, kb1, kh1;
+  k_pos(ch0, v.bits, D, &kb0, &kh0);
+  k_pos(ch0 + 8, v.bits, D, &kb1, &kh1);
+#pragma unroll 2
+  for (int r = r0; r < r1; ++r) {
+    uint32_t c[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float d = __fsub_rn(bf16_to_f32(xs[r * PAD + ch0 + 8 * h]), zr[h]);
+      float q = __fmul_rn(d, rs[h]);
+      q = fmaf(fmaf(q, -sc[h], d), rs[h], q);
+      q = fmaf(fmaf(q, -sc[h], d), rs[h], q);
+      if (wide[h]) q = sc[h] == 0.f ? 0.f : __fdiv_rn(d, sc[h]);
+      c[h] = (uint32_t)fminf(fmaxf(rintf(q), 0.f), lev);
+    }
+    if (v.bits == 8) {
+      ks[r * sec + kb0] = (uint8_t)c[0];
+      ks[r * sec + kb1] = (uint8_t)c[1];
+    } else {
+      // channels ch0 and ch0 + 8 share one byte (low and high nibble)
+      ks[r * sec + kb0] = (uint8_t)(c[0] | (c[1] << 4));
     }
   }
-  __syncwarp();
+  __syncthreads();
   // ---- the group's key sections, whole 16-byte chunks ----
   const int cps = sec / 16;
-  for (int q = lane; q < GS * cps; q += 32) {
+  for (int q = tid; q < GS * cps; q += kKgThreads) {
     const int r = q / cps, u = q - r * cps;
     uint8_t *rec = v.rec + (slab * v.cap + (size_t)G * GS + r) * L.rec + L.k_off;
     reinterpret_cast<uint4 *>(rec)[u] = reinterpret_cast<const uint4 *>(ks + r * sec)[u];
   }
-  (void)err;
 }
 
 // Positions of the group left open after this append go to the residual
@@ -1154,22 +1160,11 @@ cudaError_t launch_gqa_append(const GqaView &v, const void *k, const void *vv, i
   if (kpc) {
     // groups first (they read residual rows the open group may overwrite)
     const int max_groups = (n_new + v.group - 1) / v.group + 1;
-    const size_t warps = (size_t)v.B * v.Hkv * max_groups;
-    const dim3 grid((unsigned)((warps + kKgWarps - 1) / kKgWarps));
+    const dim3 grid((unsigned)((size_t)v.B * v.Hkv * max_groups));
     auto kern = d128 ? gqa_append_kgroups<128> : gqa_append_kgroups<64>;
-    const int smem = kKgWarps * kg_warp_bytes(v.D, v.group, v.bits);
-    static bool attr_set = false;
-    if (!attr_set) {
-      // the largest need: head_dim 128, groups of 64, 8-bit codes
-      const int most = kKgWarps * kg_warp_bytes(128, 64, 8);
-      e = cudaFuncSetAttribute(gqa_append_kgroups<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gqa_append_kgroups<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-      if (e != cudaSuccess) return e;
-      attr_set = true;
-    }
-    e = launch_pdl(kern, grid, dim3(32 * kKgWarps), (size_t)smem, st, v, k, in_f32, n_new, n_per_seq, err,
-                   max_groups);
+    // at most 25.6 KB (head_dim 128, groups of 64, 8-bit codes)
+    e = launch_pdl(kern, grid, dim3(kKgThreads), (size_t)kg_bytes(v.D, v.group, v.bits), st, v, k, in_f32, n_new,
+                   n_per_seq, max_groups);
   }
   if (e == cudaSuccess) {
     // bulk appends (head_dim 128): a warp per row for bf16, a lane per 32
