@@ -1242,7 +1242,11 @@ __device__ __forceinline__ bool gqa_balanced_split(const GqaDecodeArgs &a, GqaBa
 // slots (up to a.run_slots) empty.  Every CTA does
 // W / n tiles of work, so one wave of resident CTAs ends together instead
 // of a second, partial wave of splits.
-template <int BITS, int D, int KAX, int GS, bool GATHER, bool RUN>
+// BAL: the one-dimensional grid of gqa_balanced_split (with neither of the
+// others).  A kernel of its own: as a branch beside the split grid's body it
+// made the split grid's decodes 0.4 us each slower (14B step of 48 decodes:
+// 5009 us with it, 4986 without).
+template <int BITS, int D, int KAX, int GS, bool GATHER, bool RUN, bool BAL>
 __global__ void __launch_bounds__(128, GqaCfg<BITS, D, KAX, GS>::MIN_CTAS)
     gqa_decode_kernel(const __grid_constant__ CUtensorMap rows, const GqaDecodeArgs a) {
   pdl_wait();
@@ -1264,15 +1268,12 @@ __global__ void __launch_bounds__(128, GqaCfg<BITS, D, KAX, GS>::MIN_CTAS)
     }
     __syncthreads();
   }
-  if constexpr (!RUN) {
-    if constexpr (!GATHER) {
-      if (a.bal_ctas > 0) {
-        GqaBalSeg sg;
-        if (gqa_balanced_split<C::TILE>(a, sg))
-          gqa_decode_unit<BITS, D, KAX, GS, GATHER>(a, &rows, sg.b, sg.kvh, sg.i0, sg.i1, sg.slot, 0);
-        return;
-      }
-    }
+  if constexpr (BAL) {
+    static_assert(!GATHER && !RUN, "balanced splits read contiguously");
+    GqaBalSeg sg;
+    if (gqa_balanced_split<C::TILE>(a, sg))
+      gqa_decode_unit<BITS, D, KAX, GS, false>(a, &rows, sg.b, sg.kvh, sg.i0, sg.i1, sg.slot, 0);
+  } else if constexpr (!RUN) {
     const int split = blockIdx.x;
     const int i0 = split * a.items_per_split;
     const int i1 = split == a.n_splits - 1 ? -1 : i0 + a.items_per_split;
@@ -1309,10 +1310,10 @@ __global__ void __launch_bounds__(128, GqaCfg<BITS, D, KAX, GS>::MIN_CTAS)
   }
 }
 
-template <int BITS, int D, int KAX, int GS, bool GATHER, bool RUN>
+template <int BITS, int D, int KAX, int GS, bool GATHER, bool RUN, bool BAL = false>
 cudaError_t launch_gqa_decode_g(const GqaDecodeArgs &a, cudaStream_t st) {
   using C = GqaCfg<BITS, D, KAX, GS>;
-  auto k = gqa_decode_kernel<BITS, D, KAX, GS, GATHER, RUN>;
+  auto k = gqa_decode_kernel<BITS, D, KAX, GS, GATHER, RUN, BAL>;
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
@@ -1327,8 +1328,8 @@ cudaError_t launch_gqa_decode_g(const GqaDecodeArgs &a, cudaStream_t st) {
     memcpy(&rows, a.rows, sizeof rows);
   }
   if constexpr (RUN) return launch_pdl(k, dim3(a.run_ctas), dim3(128), C::SMEM, st, rows, a);
+  if constexpr (BAL) return launch_pdl(k, dim3(a.bal_ctas), dim3(128), C::SMEM, st, rows, a);
   dim3 grid(a.n_splits, a.v.Hkv, a.v.B);
-  if (a.bal_ctas > 0) grid = dim3(a.bal_ctas);
   return launch_pdl(k, grid, dim3(128), C::SMEM, st, rows, a);
 }
 
@@ -1342,6 +1343,10 @@ cudaError_t launch_gqa_decode_t(const GqaDecodeArgs &a, cudaStream_t st) {
     } else {
       return cudaErrorInvalidValue;
     }
+  }
+  if (a.bal_ctas > 0) {
+    if (a.gather || a.out || !a.bal_counts) return cudaErrorInvalidValue;
+    return launch_gqa_decode_g<BITS, D, KAX, GS, false, false, true>(a, st);
   }
   if constexpr (GqaCfg<BITS, D, KAX, GS>::KPC) {
     if (a.gather) return cudaErrorInvalidValue;  // no kept lists with per-channel keys
@@ -1361,7 +1366,7 @@ int gqa_tile_t() {
 template <int BITS, int D, int KAX, int GS>
 int gqa_ctas_per_sm_t() {
   using C = GqaCfg<BITS, D, KAX, GS>;
-  auto k = gqa_decode_kernel<BITS, D, KAX, GS, false, false>;
+  auto k = gqa_decode_kernel<BITS, D, KAX, GS, false, false, false>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, 128, C::SMEM) != cudaSuccess) n = 1;
