@@ -210,6 +210,41 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t &hi, uint32_t 
   lo = pack2<BF16>(x - h.x, y - h.y);
 }
 
+// Two floats in one 64-bit register pair for the packed binary32 units
+// (each half rounded as the scalar operation is).
+__device__ __forceinline__ uint64_t pair_f32(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpair_f32(uint64_t v, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// split2 of a packed pair, bf16: the same halves with one packed subtraction
+__device__ __forceinline__ void split2_bf16(uint64_t x2, uint32_t &hi, uint32_t &lo) {
+  float x, y, dx, dy;
+  unpair_f32(x2, x, y);
+  hi = pack2<true>(x, y);
+  const float2 h = unpack2<true>(hi);
+  unpair_f32(fma_f32x2(pair_f32(h.x, h.y), pair_f32(-1.f, -1.f), x2), dx, dy);
+  lo = pack2<true>(dx, dy);
+}
+
 __device__ __forceinline__ float bf16_to_f32(uint16_t b) {
   return __uint_as_float(static_cast<uint32_t>(b) << 16);
 }

@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -503,28 +504,64 @@ cudaError_t launch_evict_select(const EvictArgs &a, cudaStream_t st) {
 // rows took 32 products at about 160 cycles an item, this way 16 at 125).
 //  * statistics pass: each thread sums 2^(x - ref) of its lane's positions
 //    for a quarter of the rows, in registers over all the tiles that its CTA
-//    walks of a unit; a warp's reference of a row is the maximum of its first
-//    tile and moves only when a score rises more than 64 above it, so the
-//    warp's lanes meet (a reduction per row) only then and at the unit's end;
+//    walks of a unit; a warp's reference of a row is its first lane's first
+//    score and moves (to the warp's maximum) only when a score rises more
+//    than 64 above it, so the warp's lanes meet only then and, 31 shuffles
+//    for 32 rows, at the unit's end.  Tiles that every row sees in full, past
+//    the unit's first, run a copy of the code without masks;
 //  * vote pass: each thread sums its position's weights over the rows.
 // The vote pass recomputes the scores: on the tensor cores that is cheaper
 // than a round trip through HBM.  A CTA (one per SM) walks a contiguous range
 // of (unit, tile) items in four roles that run beside each other: 3 warps
 // copy the keys' records in, 8 dequantise them (the ALU's share), one issues
-// the chains, 16 run the epilogues (the exponentials' share: 20480 scores of 160 rows take
-// the MUFU 1280 cycles), two key stages and two TMEM buffers between them.
-// One group of 16 warps that did both in turn took 6200 cycles per item in
-// the statistics pass and 4950 in the vote pass at the 131k-context shape.
+// the chains, 16 run the epilogues (the exponentials' share), two key stages
+// and two TMEM buffers between them.
+//
+// What bounds it: issue slots (69-71 % busy), about evenly over the roles.
+// At the 131k-context shape (32 units of int4 records, 160 rows) an item takes
+// 3950 cycles in the statistics pass (452 us) and 3250 in the vote pass (384
+// us), of which a dequantising warp works 3250 and 2750, the chain's issue
+// 3450 and 2750 (16 products at 125-160 cycles beside the others' shared-
+// memory traffic, 80 alone) and an epilogue warp 3250 and 1950.  One group of
+// 16 warps that dequantised and ran the epilogues in turn took 6200 and 4950
+// cycles (704 and 560 us).  Of what the roles' own code cost, the cursor over
+// the items was a tenth (28 warps each checked the unit's limits per item;
+// now once per unit), the masks in the statistics epilogue 400 cycles, and
+// per unit the shuffles of a butterfly per row and the query rows' loads one
+// at a time 25 us.  Packed binary32 arithmetic in the epilogues gained
+// nothing (945 and 944 us a call).
 // The statistics stay in registers over a CTA's tiles of a unit and leave
 // once per CTA and unit (stored per tile they were 168 MB of traffic and a
-// 59 us merge).  Query rows past R are zero; in the statistics pass the last row
-// chunk may read rows past the query buffer (lanes that are never used).
+// 59 us merge).  Query rows past R are zero.
 constexpr int kTcEpi = 512;                  // epilogue threads (warps 0-15)
 constexpr int kTcDeq = 256;                  // dequantising threads (warps 16-23)
 constexpr int kTcCopy = 96;                  // copying threads (warps 24-26)
 constexpr int kTcThreads = kTcEpi + kTcDeq + kTcCopy + 32;  // + the MMA warp
 constexpr int kTcPv = 1024;                  // floats: partial votes (2 x 3 x 128) or references (16 x 64)
 static_assert(kEvictStatSub == kTcEpi / 128, "one statistics entry per column slice");
+
+// Sums over the warp of N values a lane (8 or 32): x[0] of lane L becomes the
+// sum of value L (N = 32) or L / 4 (N = 8).  Each step halves the values that
+// a lane carries, 31 or 9 shuffles where a butterfly per value takes 5 N (16
+// warps' 64 sums each took 19500 cycles so).
+template <int N>
+__device__ __forceinline__ void lanes_sum(float (&x)[N]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    const int h = N * o / 32;  // values kept by a step that halves them
+    if (h) {
+#pragma unroll
+      for (int i = 0; i < h; ++i) {
+        const bool up = lane & o;
+        const float send = up ? x[i] : x[i + h];
+        x[i] = (up ? x[i + h] : x[i]) + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    } else {
+      x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+    }
+  }
+}
 
 struct TcPlan {
   int items_per_cta, n_items;
@@ -592,39 +629,40 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
   };
 
   const int gshift = v.group == 64 ? 6 : 5;  // grouped layers: groups of 32 or 64 channels
-  // (unit, tile) of item `it` and the unit's length, advanced without divisions
+  // (unit, tile) of item `it`, the unit's length and the item after its last
+  // valid tile (none: at most `it`), advanced without divisions; within a
+  // unit a step is two additions and a compare
   struct Cursor {
-    int it, unit, tile, len;
+    int it, unit, tile, len, end;
   };
   const int units = v.B * v.Hkv;
-  auto at = [&](int it) {
-    Cursor c;
-    c.it = it;
-    c.unit = it / a.n_tiles;
-    c.tile = it - c.unit * a.n_tiles;
+  auto unit_end = [&](Cursor &c) {  // c at tile c.tile of c.unit
     c.len = c.unit < units ? v.lens[c.unit / v.Hkv] : 0;
-    return c;
+    const int n = c.len > a.budget ? ((VOTES ? c.len - a.n_win : c.len) + kT - 1) / kT : 0;  // valid tiles
+    c.end = min(it1, c.it + n - c.tile);
   };
-  auto next_valid = [&](Cursor c) {  // c or the first valid item after it (c.it == it1: none)
-    while (c.it < it1) {
-      if (c.len > a.budget && c.tile * kT < (VOTES ? c.len - a.n_win : c.len)) break;
-      // an invalid item has no valid successor in its unit: on to the next unit
+  auto next_unit = [&](Cursor c) {  // the first valid item at or after c (c.it == it1: none)
+    while (c.it < it1 && c.it >= c.end) {
       c.it += a.n_tiles - c.tile;
       c.tile = 0;
       ++c.unit;
-      c.len = c.unit < units ? v.lens[c.unit / v.Hkv] : 0;
+      unit_end(c);
     }
     c.it = min(c.it, it1);
     return c;
   };
-  auto after = [&](Cursor c) {  // the item after c
+  auto first = [&]() {
+    Cursor c;
+    c.it = it0;
+    c.unit = it0 / a.n_tiles;
+    c.tile = it0 - c.unit * a.n_tiles;
+    unit_end(c);
+    return next_unit(c);
+  };
+  auto step = [&](Cursor c) {
     ++c.it;
-    if (++c.tile == a.n_tiles) {
-      c.tile = 0;
-      ++c.unit;
-      c.len = c.unit < units ? v.lens[c.unit / v.Hkv] : 0;
-    }
-    return c;
+    ++c.tile;
+    return c.it < c.end ? c : next_unit(c);
   };
 
   // query rows of `unit` (and, for the votes, the rows' log-normalisers;
@@ -632,33 +670,36 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
   auto load_q = [&](int unit, int n) {
     const int b = unit / v.Hkv, j = unit % v.Hkv;
     const int box = p.R16 * 128;
-    for (int e = did; e < p.R16 * (D / 8); e += kTcDeq) {
-      const int r = e >> 4, c8 = e & 15;
-      float x[8];
+    // thread: chunk c8 of rows did / 16 + 16 i; row r is query w = r / G of
+    // head r % G, carried from row to row
+    const int c8 = did & 15, dw = (kTcDeq / 16) / a.G, dg = kTcDeq / 16 - dw * a.G;
+    int r = did >> 4, w = r / a.G, g = r - w * a.G;
+    for (; r < p.R16; r += kTcDeq / 16) {
+      const size_t qi = (((size_t)b * a.n_win + (r < R ? w : 0)) * a.Hq + j * a.G + g) * D + 8 * c8;
+      if (a.q_f32) {
+        float x[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = 0.f;
-      if (r < R) {
-        const int w = r / a.G, h = j * a.G + r % a.G;
-        const size_t qi = (((size_t)b * a.n_win + w) * a.Hq + h) * D + 8 * c8;
-        if (a.q_f32) {
+        for (int i = 0; i < 8; ++i) x[i] = 0.f;
+        if (r < R) {
           const float4 u0 = *reinterpret_cast<const float4 *>(static_cast<const float *>(a.q) + qi);
           const float4 u1 = *reinterpret_cast<const float4 *>(static_cast<const float *>(a.q) + qi + 4);
           x[0] = u0.x; x[1] = u0.y; x[2] = u0.z; x[3] = u0.w;
           x[4] = u1.x; x[5] = u1.y; x[6] = u1.z; x[7] = u1.w;
-        } else {
-          const uint4 u = *reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(a.q) + qi);
-          const uint32_t ww[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            x[2 * i] = __uint_as_float(ww[i] << 16);
-            x[2 * i + 1] = __uint_as_float(ww[i] & 0xFFFF0000u);
-          }
         }
+        put8(qh, ql, true, r, 8 * c8, box, x);
+      } else {
+        cp_async16(qh + (c8 >> 3) * box + r * 128 + (((c8 & 7) ^ (r & 7)) << 4), static_cast<const uint16_t *>(a.q) + qi,
+                   r < R);
       }
-      put8(qh, ql, p.q_lo != 0, r, 8 * c8, box, x);
+      w += dw;
+      g += dg;
+      if (g >= a.G) {
+        g -= a.G;
+        ++w;
+      }
     }
     if constexpr (VOTES) {
-      float *nm = norm + 256 * (n & 1);
+      float *nm = norm + p.R16 * (n & 1);
       for (int r = did; r < p.R16; r += kTcDeq) {
         if (r < R) {
           const float2 f = a.fin[(size_t)unit * R + r];
@@ -668,6 +709,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
         }
       }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     fence_proxy_async();
   };
 
@@ -741,7 +783,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
 
   // Statistics pass: this thread's sums of a slice's rows over its lane's
   // positions of the unit's tiles, relative to the warp's references (shared
-  // memory, one row of 64 per warp: rows 16 bk + i of the slice in order).
+  // memory, 64 per warp: the slice's rows in order).
   constexpr int BW = VOTES ? 16 : 8;  // rows of a block
   const int nblk = p.R16 / BW, per = (nblk + 3) / 4;
   const int bk0 = min(nblk, slice * per), bk1 = min(nblk, bk0 + per);
@@ -751,13 +793,25 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
   auto flush_stats = [&](int unit) {
     const int stride = kEvictStatSub * a.n_tiles;
     const int e = kEvictStatSub * ((int)blockIdx.x - unit * a.n_tiles / p.items_per_cta) + quarter;
-#pragma unroll
-    for (int i = 0; i < 8 * NB; ++i) {
+    auto put = [&](int i, float L) {  // the slice's row i
       const int r = 8 * bk0 + i;
-      float L = l_run[i];
+      if (r < 8 * bk1 && r < R) a.stats[((size_t)unit * R + r) * stride + e] = make_float2(ref[i], L);
+    };
 #pragma unroll
-      for (int o = 16; o; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-      if (lane == 0 && r < 8 * bk1 && r < R) a.stats[((size_t)unit * R + r) * stride + e] = make_float2(ref[i], L);
+    for (int b = 0; b + 4 <= NB; b += 4) {  // 32 rows at a time
+      float x[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) x[i] = l_run[8 * b + i];
+      lanes_sum(x);
+      put(8 * b + lane, x[0]);
+    }
+#pragma unroll
+    for (int b = NB / 4 * 4; b < NB; ++b) {  // 8
+      float x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = l_run[8 * b + i];
+      lanes_sum(x);
+      if ((lane & 3) == 0) put(8 * b + (lane >> 2), x[0]);
     }
   };
   // epilogue of item `cu` (the k-th) from TMEM buffer tb
@@ -772,6 +826,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
       // before (t - P) G do not see this lane's position
       const int r_from = (t - P) * a.G;
       const bool whole = t0 + 32 * quarter + 31 <= P;
+      // tiles that every row sees in full, past the unit's first: no masks
+      auto tiles = [&](auto hot_t) {
+        constexpr bool hot = decltype(hot_t)::value;
 #pragma unroll
       for (int b = 0; b < NB; b += 2) {  // 16 rows at a time (8 at an odd end)
         if (bk0 + b >= bk1) break;
@@ -779,17 +836,21 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
         const int n = bk0 + b + 1 < bk1 && b + 1 < NB ? 16 : 8;
         float z[16];
         tmem_ld16(ta, z);  // past an odd end: another slice's rows, unused
-        if (!whole) {
+        if (!hot && !whole) {
 #pragma unroll
           for (int i = 0; i < 16; ++i)
             if (8 * (bk0 + b) + i < r_from) z[i] = -INFINITY;
         }
-        if (fresh) {
+        if (!hot && fresh) {
+          // lane 0's scores (its position is visible where any lane's is)
+          if (lane == 0) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            if (8 * b + i < 8 * NB) l_run[8 * b + i] = 0.f;
-            if (lane == 0 && i < n) ref[8 * b + i] = -INFINITY;
+            for (int i = 0; i < 16; ++i)
+              if (i < n) ref[8 * b + i] = z[i] * sg;
           }
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (8 * b + i < 8 * NB) l_run[8 * b + i] = 0.f;
           __syncwarp();
         }
         float top = -INFINITY;
@@ -802,20 +863,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
           z[4 * i4 + 1] = fmaf(z[4 * i4 + 1], sg, -c.y);
           z[4 * i4 + 2] = fmaf(z[4 * i4 + 2], sg, -c.z);
           z[4 * i4 + 3] = fmaf(z[4 * i4 + 3], sg, -c.w);
-          if (!whole) {  // -inf - -inf, masked and without a reference yet: adds nothing
+          if (!hot && !whole) {  // -inf - -inf, masked and without a reference yet: adds nothing
 #pragma unroll
             for (int i = 4 * i4; i < 4 * i4 + 4; ++i) z[i] = fmaxf(z[i], -INFINITY);
           }
           top = fmaxf(top, fmaxf(fmaxf(z[4 * i4], z[4 * i4 + 1]), fmaxf(z[4 * i4 + 2], z[4 * i4 + 3])));
         }
-        if (__any_sync(0xffffffffu, fresh || top > 64.f)) {
+        if (__builtin_expect(__any_sync(0xffffffffu, top > 64.f), 0)) {
           // the references move to the warp's maxima where scores pass them;
           // a row whose positions so far are all masked keeps -inf
           auto scores = [&]() {
             tmem_ld16(ta, z);
 #pragma unroll
             for (int i = 0; i < 16; ++i)
-              if (!whole && 8 * (bk0 + b) + i < r_from) z[i] = -INFINITY;
+              if (!hot && !whole && 8 * (bk0 + b) + i < r_from) z[i] = -INFINITY;
           };
           scores();
 #pragma unroll
@@ -854,6 +915,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
         for (int i = 0; i < 16; ++i)
           if (8 * b + i < 8 * NB && i < n) l_run[8 * b + i] += fast_exp2(z[i]);
       }
+      };
+      if (whole && !fresh)
+        tiles(std::true_type{});
+      else
+        tiles(std::false_type{});
       fresh = false;
     } else {
       const int pos = 32 * quarter + lane, t = t0 + pos;
@@ -890,7 +956,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
       // the same item sequence as the others; each chain once its keys are
       // staged and its TMEM buffer was read
       int k = 0;
-      for (Cursor cu = next_valid(at(it0)); cu.it < it1; cu = next_valid(after(cu)), ++k) {
+      for (Cursor cu = first(); cu.it < it1; cu = step(cu), ++k) {
         bool ok = sleepy(&keys[k & 1], (k >> 1) & 1);
         if (ok && k >= 2) ok = sleepy(&epi[k & 1], ((k >> 1) - 1) & 1);
         if (!__all_sync(0xffffffffu, ok)) {
@@ -913,7 +979,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
       // ======================= copies =======================================
       int k = 0, g = 0;
       uint32_t ph = 1;  // a buffer's first use waits for nothing
-      for (Cursor it = next_valid(at(it0)); it.it < it1; it = next_valid(after(it)), ++k) {
+      for (Cursor it = first(); it.it < it1; it = step(it), ++k) {
         if (!__all_sync(0xffffffffu, sleepy(&sfree[g], ph))) {
           *abort_flag = 1;
           break;
@@ -933,7 +999,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
     bool failed = false;
     int cur_unit = -1, n_unit = 0, k = 0, g = 0;
     uint32_t ph = 0;
-    for (Cursor it = next_valid(at(it0)); it.it < it1; it = next_valid(after(it)), ++k) {
+    for (Cursor it = first(); it.it < it1; it = step(it), ++k) {
       // the key stage is free once the chain that read it is done; a new
       // unit's rows replace the last unit's after its last chain, and its
       // norms those of two units ago, whose last epilogue is k - 2 at most
@@ -971,7 +1037,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
     // A warp whose wait gave up goes on through the barriers without work.
     bool failed = false;
     int cur_unit = -1, n_unit = -1, k = 0;
-    for (Cursor it = next_valid(at(it0)); it.it < it1; it = next_valid(after(it)), ++k) {
+    for (Cursor it = first(); it.it < it1; it = step(it), ++k) {
       if (it.unit != cur_unit) {
         if constexpr (!VOTES) {
           if (cur_unit >= 0) flush_stats(cur_unit);
@@ -984,7 +1050,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
       if (!failed) failed = !__all_sync(0xffffffffu, sleepy(&chain[k & 1], (k >> 1) & 1));
       if (failed) *abort_flag = 1;
       tc_fence_after();
-      epilogue(it, k & 1, norm + 256 * (n_unit & 1));
+      epilogue(it, k & 1, norm + p.R16 * (n_unit & 1));
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&epi[k & 1]);
@@ -1029,13 +1095,13 @@ TcPlan tc_plan(const EvictArgs &a, int sms) {
   const int qbytes = p.R16 * 256 * (p.q_lo ? 2 : 1);
   p.off_k = (qbytes + 1023) / 1024 * 1024;
   auto fits = [&](int nst, int nstg) {
-    return p.off_k + nst * p.stage + nstg * p.stg_bytes + 2 * 256 * 4 + kTcPv * 4 + 128 + 1024 <= 232448;
+    return p.off_k + nst * p.stage + nstg * p.stg_bytes + 2 * p.R16 * 4 + kTcPv * 4 + 128 + 1024 <= 232448;
   };
   p.nst = fits(2, 2) ? 2 : 1;
   p.nstg = fits(p.nst, 2) ? 2 : 1;
   p.off_stg = p.off_k + p.nst * p.stage;
   p.off_norm = p.off_stg + p.nstg * p.stg_bytes;
-  p.off_pv = p.off_norm + 2 * 256 * 4;
+  p.off_pv = p.off_norm + 2 * p.R16 * 4;
   p.off_bar = p.off_pv + kTcPv * 4;
   p.smem = p.off_bar + 128 + 1024;  // + alignment of the base to 1024 bytes
   p.n_items = a.v.B * a.v.Hkv * a.n_tiles;

@@ -33,7 +33,10 @@
 // in TMEM took 77-90 cycles (a clock64 trace of the 64-position version: 16
 // of them 1450 cycles, 12 value products 800 alone) against 64 for N = 128,
 // and the two products of a tile then cost 2560 cycles per 128 positions
-// (16 + 24 at 64), under which the epilogue (about 1500) hides.
+// (16 + 24 at 64).  Measured: about 3500 cycles per 128 positions, the chain
+// of a tile's scores, epilogue (about 1500) and values with two tiles in
+// flight; the 64-position version took 2.33 ms where this one takes 2.12
+// (14B int4 layer, 4 x 8192 positions, the last 2048 the chunk).
 //
 // MLA chunks run the same attention kernel over keys and values formed per
 // head (mla_form.cu): units are heads (G = 1), and the score products go on

@@ -57,8 +57,8 @@ __device__ __forceinline__ void umma_f16_ts_w(uint32_t d_tmem, uint32_t a_tmem, 
       : "memory");
 }
 // A and B in shared memory, both descriptors' low words given (the high one,
-// `hi`, is the same): built per product from 64-bit arithmetic they cost a
-// lone issuing thread about 170 cycles a product against the 64 it takes
+// `hi`, is the same).  Both operands come from shared memory: M = 128, N = 128
+// took 130-160 cycles beside other shared-memory traffic (64 with A in TMEM)
 __device__ __forceinline__ void umma_f16_ss_w(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
                                               bool accumulate) {
   asm volatile(

@@ -158,8 +158,8 @@ def test_evict_then_decode_per_head(fmt):
 
 
 @pytest.mark.parametrize("B,Hkv,G,n_win,T", [(40, 4, 3, 9, 300), (2, 3, 7, 32, 1000), (1, 2, 8, 32, 700),
-                                             (3, 2, 5, 20, 513)],
-                         ids=["units-over-ctas", "rows224", "rows256", "rows100"])
+                                             (3, 2, 5, 20, 513), (24, 4, 8, 32, 700)],
+                         ids=["units-over-ctas", "rows224", "rows256", "rows100", "rows256-tiles-per-cta"])
 @pytest.mark.parametrize("fmt", [FORMATS[0], FORMATS[2]], ids=_fid)
 def test_evict_votes_rising_scores(fmt, B, Hkv, G, n_win, T):
     """Keys that grow along the context by up to 30 times, so that a row's
