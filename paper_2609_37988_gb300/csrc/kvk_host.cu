@@ -175,6 +175,7 @@ struct kvk_cache {
   std::vector<uint8_t *> arena;
   std::vector<ArenaLayout> lay;
   std::vector<long long> len_hi;  // host upper bound on every sequence's length
+  std::vector<uint8_t> ragged;    // sequences may differ in length (an append with per-sequence counts)
   std::vector<int> kept_on;
   uint8_t *ws;
   size_t ws_bytes;
@@ -405,14 +406,17 @@ bool plan_runs(kvk_cache *c, int a, RunPlan *p) {
 // Balanced splits of an automatic decode of anchor a (kernel side in
 // decode_gqa.cuh, gqa_balanced_split), given what plan_runs and auto_splits
 // (`splits`) chose: the number of CTAs, 0 if the decode keeps their schedule.
-// Taken where one wave of resident CTAs holds the units at two or more splits
-// each and the other plan is one wave too; over sequences of equal length the
-// splits are then those of the split grid.  Instead of the runs only if whole
+// Taken once an append has named per-sequence counts (sequences of equal
+// length have nothing to balance, and finding its split on the device costs a
+// CTA about 1 us: the 7B step, 16 equal sequences, took 1.115 ms with it and 1.078
+// without), where one wave
+// of resident CTAs holds the units at two or more splits each and the other
+// plan is one wave too.  Instead of the runs only if whole
 // splits fill 85 % of the wave (the runs fill all of it, but only if the
 // lengths are equal).  *cap: partial slots per unit, twice the even share (a
 // sequence twice as long as the average takes it), in the merge's steps.
 int plan_balanced(kvk_cache *c, int a, bool runs, int splits, int *cap) {
-  if (c->schedule != KVK_SCHEDULE_AUTO || c->kept_on[a]) return 0;
+  if (c->schedule != KVK_SCHEDULE_AUTO || c->kept_on[a] || !c->ragged[a]) return 0;
   if (c->desc.max_batch < 2 || c->desc.max_batch > kBalanceMaxBatch) return 0;
   const kvk_layer_cfg &L = c->cfg[a];
   const int units = c->desc.max_batch * c->desc.n_kv_heads, slots = c->sm_count * c->ctas[a];
@@ -541,6 +545,7 @@ kvk_status kvk_cache_create(const kvk_model_desc *desc, const kvk_layer_cfg *cfg
   c->arena.assign(desc->n_layers, nullptr);
   c->lay.resize(desc->n_layers);
   c->len_hi.assign(desc->n_layers, 0);
+  c->ragged.assign(desc->n_layers, 0);
   c->kept_on.assign(desc->n_layers, 0);
   c->ctas.assign(desc->n_layers, 0);
   c->formed_from.assign(desc->n_layers, 0);
@@ -630,6 +635,7 @@ kvk_status kvk_cache_reset(kvk_cache *c, kvk_stream stream) {
     cudaError_t e = cudaMemsetAsync(c->arena[l], 0, (size_t)A.kept_idx, st);
     if (e != cudaSuccess) return cuda_fail(e, "resetting lengths");
     c->len_hi[l] = 0;
+    c->ragged[l] = 0;
     c->kept_on[l] = 0;
   }
   cudaError_t e = cudaMemsetAsync(c->err(), 0, 4, st);
@@ -681,6 +687,7 @@ kvk_status kvk_append(kvk_cache *c, int32_t layer, const void *k, const void *v,
   }
   if (e != cudaSuccess) return cuda_fail(e, "append launch");
   c->len_hi[layer] += n_new;
+  if (n_new_per_seq) c->ragged[layer] = 1;
   return KVK_OK;
 }
 

@@ -249,7 +249,8 @@ def test_recorded_balanced_launch_covers_longer_sequences():
     g = torch.Generator().manual_seed(3)
     k = torch.randn((B, 4000, Hkv, D), generator=g).to(torch.bfloat16)
     v = torch.randn((B, 4000, Hkv, D), generator=g).to(torch.bfloat16)
-    c.append(0, k[:, :300].contiguous().cuda(), v[:, :300].contiguous().cuda())
+    c.append(0, k[:, :300].contiguous().cuda(), v[:, :300].contiguous().cuda(),
+             torch.full((B,), 300, dtype=torch.int32, device="cuda"))
     q = torch.randn((B, G * Hkv, D), generator=g).to(torch.bfloat16).cuda()
     out = torch.empty((B, G * Hkv, D), device="cuda")
     s = torch.cuda.Stream()
