@@ -408,8 +408,8 @@ bool plan_runs(kvk_cache *c, int a, RunPlan *p) {
 // (`splits`) chose: the number of CTAs, 0 if the decode keeps their schedule.
 // Taken once an append has named per-sequence counts (sequences of equal
 // length have nothing to balance, and finding its split on the device costs a
-// CTA about 1 us: the 7B step, 16 equal sequences, took 1.115 ms with it and 1.078
-// without), where one wave
+// CTA about 1 us: the 7B step, 16 equal sequences, took 1.115 ms with it and
+// 1.078 without), where one wave
 // of resident CTAs holds the units at two or more splits each and the other
 // plan is one wave too.  Instead of the runs only if whole
 // splits fill 85 % of the wave (the runs fill all of it, but only if the

@@ -20,7 +20,7 @@ namespace {
 // maxima, sums and this element's accumulators) is issued before any is
 // used, so the merge costs one memory round trip.  Rows per CTA: 128 / dim
 // (dim <= 128), else one row with a channel loop.
-template <int SB>
+template <int SB, bool COUNTS>
 __global__ void __launch_bounds__(128)
     splitk_merge_kernel(const float *P, int S, int n_rows, int dim,
                         float *__restrict__ out, const int32_t *counts, int rows_per) {
@@ -36,7 +36,8 @@ __global__ void __launch_bounds__(128)
   const float *pr = P + (size_t)row * RS;
   // with per-sequence counts every slot up to S is loaded beside the count
   // (the slots exist) and those past it are dropped
-  const int n = counts ? counts[row / rows_per] : S;
+  int n = S;
+  if constexpr (COUNTS) n = counts[row / rows_per];
   float m[SB], l[SB];
 #pragma unroll
   for (int s = 0; s < SB; ++s) {
@@ -47,12 +48,14 @@ __global__ void __launch_bounds__(128)
     float x[SB];
 #pragma unroll
     for (int s = 0; s < SB; ++s) x[s] = s < S ? pr[s * SS + ch] : 0.f;
+    if constexpr (COUNTS) {
 #pragma unroll
-    for (int s = 0; s < SB; ++s)
-      if (s >= n) {
-        m[s] = -INFINITY;
-        x[s] = l[s] = 0.f;
-      }
+      for (int s = 0; s < SB; ++s)
+        if (s >= n) {
+          m[s] = -INFINITY;
+          x[s] = l[s] = 0.f;
+        }
+    }
     float M = -INFINITY;
 #pragma unroll
     for (int s = 0; s < SB; ++s) M = fmaxf(M, m[s]);
@@ -193,10 +196,10 @@ cudaError_t launch_splitk_merge(const float *partials, int n_splits, int n_rows,
   const int rpc = dim >= 128 ? 1 : 128 / dim;
   const int grid = (n_rows + rpc - 1) / rpc;
   if (n_splits <= 8)
-    return launch_pdl(splitk_merge_kernel<8>, grid, dim3(128), 0, st, partials, n_splits, n_rows, dim, out, counts,
+    return launch_pdl(counts ? splitk_merge_kernel<8, true> : splitk_merge_kernel<8, false>, grid, dim3(128), 0, st, partials, n_splits, n_rows, dim, out, counts,
                       rows_per);
   else if (n_splits <= 16)
-    return launch_pdl(splitk_merge_kernel<16>, grid, dim3(128), 0, st, partials, n_splits, n_rows, dim, out, counts,
+    return launch_pdl(counts ? splitk_merge_kernel<16, true> : splitk_merge_kernel<16, false>, grid, dim3(128), 0, st, partials, n_splits, n_rows, dim, out, counts,
                       rows_per);
   else
     return launch_pdl(splitk_merge_wide, n_rows, dim3(32 * kWideWarps), 0, st, partials, n_splits, n_rows, dim, out, counts,
