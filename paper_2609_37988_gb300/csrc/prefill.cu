@@ -36,7 +36,11 @@
 // (16 + 24 at 64).  Measured: about 3500 cycles per 128 positions, the chain
 // of a tile's scores, epilogue (about 1500) and values with two tiles in
 // flight; the 64-position version took 2.33 ms where this one takes 2.12
-// (14B int4 layer, 4 x 8192 positions, the last 2048 the chunk).
+// (14B int4 layer, 4 x 8192 positions, the last 2048 the chunk).  The chain's
+// share of the epilogue: packed binary32 arithmetic (2025 -> 1995 us, repeated
+// calls) and 104 registers for the workers (-> 1946 us); the first unit's
+// weights computed before the row's barrier instead, with the reference as it
+// stands, was slower (1985 us).
 //
 // MLA chunks run the same attention kernel over keys and values formed per
 // head (mla_form.cu): units are heads (G = 1), and the score products go on
@@ -384,136 +388,144 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
   };
   auto spin = [&](uint64_t *b, uint32_t parity) { return mbar_spin_or_abort(b, parity, kSpins, abort_flag); };
 
-  if (warp == kPfWorkers / 32 + 1 || warp == kPfWorkers / 32 + 3) {
-    // ======================= copy warps ===================================
-    // lane 0 of one copies each tile's key units (and positional keys), of
-    // the other its value units, once the products that read the unit's
-    // place before are done
-    const bool keys = warp == kPfWorkers / 32 + 1;
-    uint64_t *full = keys ? kfull : vfull, *free_ = keys ? kfree : vfree;
-    const int n = keys ? p.nk : p.nv;
-    uint8_t *ring = sm + (keys ? 0 : p.off_v);
-    int c = 0, rc = 0;  // units (and positional tiles) copied
-    PfRing ru, rr;
-    bool ok = true;
-    for (int job = next_job(); job < p.n_jobs; job = next_job()) {
-      if (ok && lane == 0) {
-        const Job J = job_at(job);
-        const uint8_t *src = a.tiles + (size_t)J.unit * p.n_t * p.tbytes + (keys ? 0 : 2 * p.ub);
-        for (int k = 0; k < J.n_t && ok; ++k) {
-          for (int u = 0; u < 2 && ok; ++u) {
-            const int s = ru.s;
-            ok = sleepy(&free_[s], ru.ph ^ 1);
-            // the unit's place is written only by bulk copies and read only
-            // by the products (both async proxy, ordered by the commit's
-            // release of kfree / vfree): no proxy fence
-            if (ok) {
-              mbar_expect_tx(&full[s], p.ub);
-              bulk_g2s(ring + s * p.ub, src + (size_t)k * p.tbytes + u * p.ub, p.ub, &full[s]);
-              ++c;
-              ru.next(n);
-            }
-          }
-          if (MLA && keys && ok) {
-            const int s = rr.s;
-            ok = sleepy(&rfree[s], rr.ph ^ 1);
-            if (ok) {
-              mbar_expect_tx(&rfull[s], p.krb);
-              bulk_g2s(sm + p.off_r + s * p.krb, a.kr + ((size_t)(J.b - a.b0) * p.n_t + k) * p.krb, p.krb, &rfull[s]);
-              ++rc;
-              rr.next(p.nr);
-            }
-          }
-        }
-        if (!ok) *abort_flag = 1;
-      }
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-    }
-    // the last copies land before the CTA leaves (bounded; at once when
-    // they were consumed)
-    if (lane == 0) {
-      for (int u = max(0, c - n); u < c; ++u) mbar_wait(&full[u % n], (u / n) & 1, 1u << 22);
-      for (int u = max(0, rc - p.nr); u < rc; ++u) mbar_wait(&rfull[u % p.nr], (u / p.nr) & 1, 1u << 22);
-    }
-    __syncwarp();
-  } else if (warp >= kPfWorkers / 32) {
-    // ======================= MMA warps ====================================
-    // lane 0 of one issues the score products, of the other the value
-    // products; a commit covers the products its own thread issued
-    const bool scores = warp == kPfWorkers / 32;
-    // Barrier phases: S(c + 2) takes the columns of P(c), so its warp waits
-    // for PV(c) first, and PV(c + 2) needs S(c + 2); the value warp waits for
-    // every epi(c) in order before PV(c), and epi(c + 2) needs S(c + 2).  So
-    // every wait is for the phase after the one its warp last saw.
-    int kk = 0, njob = 0, c = 0;
-    PfRing ru, rr;
-    bool ok = true;
-    for (int job = next_job(); job < p.n_jobs; job = next_job()) {
-      if (ok && lane == 0) {
-        const Job J = job_at(job);
-        // this job's query rows are staged (and the last job's O was read)
-        ok = sleepy(qready, njob & 1);
-        ++njob;
-        for (int k = 0; k < J.n_t && ok; ++k, ++kk) {
-          if (scores) {
-            if (kk >= 2) ok = spin(&pvdone[kk & 1], ((kk >> 1) - 1) & 1);  // P(kk - 2) is read
-            for (int u = 0; u < 2 && ok; ++u, ++c, ru.next(scores ? p.nk : p.nv)) {
+  // Registers by warpgroup, 512 x 104 + 128 x 64 = the 640 x 96 launched: the
+  // workers hold 32 scores, their weights and both halves without spills
+  // (each set inside its branch: ahead of the branches the workers spilled).
+  static_assert(kPfThreads == 640, "the register split");
+  if (warp >= kPfWorkers / 32) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;" ::: "memory");
+    if (warp == kPfWorkers / 32 + 1 || warp == kPfWorkers / 32 + 3) {
+      // ======================= copy warps ===================================
+      // lane 0 of one copies each tile's key units (and positional keys), of
+      // the other its value units, once the products that read the unit's
+      // place before are done
+      const bool keys = warp == kPfWorkers / 32 + 1;
+      uint64_t *full = keys ? kfull : vfull, *free_ = keys ? kfree : vfree;
+      const int n = keys ? p.nk : p.nv;
+      uint8_t *ring = sm + (keys ? 0 : p.off_v);
+      int c = 0, rc = 0;  // units (and positional tiles) copied
+      PfRing ru, rr;
+      bool ok = true;
+      for (int job = next_job(); job < p.n_jobs; job = next_job()) {
+        if (ok && lane == 0) {
+          const Job J = job_at(job);
+          const uint8_t *src = a.tiles + (size_t)J.unit * p.n_t * p.tbytes + (keys ? 0 : 2 * p.ub);
+          for (int k = 0; k < J.n_t && ok; ++k) {
+            for (int u = 0; u < 2 && ok; ++u) {
               const int s = ru.s;
-              ok = spin(&kfull[s], ru.ph);
-              if (!ok) break;
-              tc_fence_after();
-              const uint32_t ku = smem_u32(sm + s * p.ub);
-              if constexpr (MLA) {
-                pf_issue_scores_ss<true>(t_s(kk), smem_u32(sm + p.off_q) + u * 16384, ku, u > 0);
-              } else if (p.k_lo) {
-                if (p.q_lo) pf_issue_scores<true, true>(t_s(kk), t_q + 32 * u, ku, u > 0);
-                else pf_issue_scores<true, false>(t_s(kk), t_q + 32 * u, ku, u > 0);
-              } else {
-                if (p.q_lo) pf_issue_scores<false, true>(t_s(kk), t_q + 32 * u, ku, u > 0);
-                else pf_issue_scores<false, false>(t_s(kk), t_q + 32 * u, ku, u > 0);
-              }
-              umma_commit(&kfree[s]);
-            }
-            if constexpr (MLA) {
-              const int s = rr.s;
-              if (ok) ok = spin(&rfull[s], rr.ph);
+              ok = sleepy(&free_[s], ru.ph ^ 1);
+              // the unit's place is written only by bulk copies and read only
+              // by the products (both async proxy, ordered by the commit's
+              // release of kfree / vfree): no proxy fence
               if (ok) {
-                tc_fence_after();
-                const uint32_t q = smem_u32(sm + p.off_q) + 32768, kr = smem_u32(sm + p.off_r + s * p.krb);
-                if (p.krb > 16384) pf_issue_scores_ss<true>(t_s(kk), q, kr, true);
-                else pf_issue_scores_ss<false>(t_s(kk), q, kr, true);
-                umma_commit(&rfree[s]);
+                mbar_expect_tx(&full[s], p.ub);
+                bulk_g2s(ring + s * p.ub, src + (size_t)k * p.tbytes + u * p.ub, p.ub, &full[s]);
+                ++c;
+                ru.next(n);
+              }
+            }
+            if (MLA && keys && ok) {
+              const int s = rr.s;
+              ok = sleepy(&rfree[s], rr.ph ^ 1);
+              if (ok) {
+                mbar_expect_tx(&rfull[s], p.krb);
+                bulk_g2s(sm + p.off_r + s * p.krb, a.kr + ((size_t)(J.b - a.b0) * p.n_t + k) * p.krb, p.krb, &rfull[s]);
+                ++rc;
                 rr.next(p.nr);
               }
             }
-            if (ok) umma_commit(&sdone[kk & 1]);
-          } else {
-            for (int u = 0; u < 2 && ok; ++u, ++c, ru.next(scores ? p.nk : p.nv)) {
-              const int s = ru.s;
-              ok = spin(&vfull[s], ru.ph);
-              if (ok) ok = spin(&epi[2 * (kk & 1) + u], (kk >> 1) & 1);
-              if (!ok) break;
-              tc_fence_after();
-              const uint32_t vh = smem_u32(sm + p.off_v + s * p.ub), pa = t_s(kk) + 32 * u;
-              if (MLA || p.k_lo) pf_issue_values<true, MLA>(t_o, t_ol, pa, vh, k > 0 || u > 0);
-              else pf_issue_values<false, false>(t_o, t_o, pa, vh, k > 0 || u > 0);
-              umma_commit(&vfree[s]);
-            }
-            if (ok) umma_commit(&pvdone[kk & 1]);
           }
+          if (!ok) *abort_flag = 1;
         }
-        if (!ok) *abort_flag = 1;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
       }
-      ok = __shfl_sync(0xffffffffu, ok, 0);
+      // the last copies land before the CTA leaves (bounded; at once when
+      // they were consumed)
+      if (lane == 0) {
+        for (int u = max(0, c - n); u < c; ++u) mbar_wait(&full[u % n], (u / n) & 1, 1u << 22);
+        for (int u = max(0, rc - p.nr); u < rc; ++u) mbar_wait(&rfull[u % p.nr], (u / p.nr) & 1, 1u << 22);
+      }
+      __syncwarp();
+    } else {
+      // ======================= MMA warps ====================================
+      // lane 0 of one issues the score products, of the other the value
+      // products; a commit covers the products its own thread issued
+      const bool scores = warp == kPfWorkers / 32;
+      // Barrier phases: S(c + 2) takes the columns of P(c), so its warp waits
+      // for PV(c) first, and PV(c + 2) needs S(c + 2); the value warp waits for
+      // every epi(c) in order before PV(c), and epi(c + 2) needs S(c + 2).  So
+      // every wait is for the phase after the one its warp last saw.
+      int kk = 0, njob = 0, c = 0;
+      PfRing ru, rr;
+      bool ok = true;
+      for (int job = next_job(); job < p.n_jobs; job = next_job()) {
+        if (ok && lane == 0) {
+          const Job J = job_at(job);
+          // this job's query rows are staged (and the last job's O was read)
+          ok = sleepy(qready, njob & 1);
+          ++njob;
+          for (int k = 0; k < J.n_t && ok; ++k, ++kk) {
+            if (scores) {
+              if (kk >= 2) ok = spin(&pvdone[kk & 1], ((kk >> 1) - 1) & 1);  // P(kk - 2) is read
+              for (int u = 0; u < 2 && ok; ++u, ++c, ru.next(scores ? p.nk : p.nv)) {
+                const int s = ru.s;
+                ok = spin(&kfull[s], ru.ph);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t ku = smem_u32(sm + s * p.ub);
+                if constexpr (MLA) {
+                  pf_issue_scores_ss<true>(t_s(kk), smem_u32(sm + p.off_q) + u * 16384, ku, u > 0);
+                } else if (p.k_lo) {
+                  if (p.q_lo) pf_issue_scores<true, true>(t_s(kk), t_q + 32 * u, ku, u > 0);
+                  else pf_issue_scores<true, false>(t_s(kk), t_q + 32 * u, ku, u > 0);
+                } else {
+                  if (p.q_lo) pf_issue_scores<false, true>(t_s(kk), t_q + 32 * u, ku, u > 0);
+                  else pf_issue_scores<false, false>(t_s(kk), t_q + 32 * u, ku, u > 0);
+                }
+                umma_commit(&kfree[s]);
+              }
+              if constexpr (MLA) {
+                const int s = rr.s;
+                if (ok) ok = spin(&rfull[s], rr.ph);
+                if (ok) {
+                  tc_fence_after();
+                  const uint32_t q = smem_u32(sm + p.off_q) + 32768, kr = smem_u32(sm + p.off_r + s * p.krb);
+                  if (p.krb > 16384) pf_issue_scores_ss<true>(t_s(kk), q, kr, true);
+                  else pf_issue_scores_ss<false>(t_s(kk), q, kr, true);
+                  umma_commit(&rfree[s]);
+                  rr.next(p.nr);
+                }
+              }
+              if (ok) umma_commit(&sdone[kk & 1]);
+            } else {
+              for (int u = 0; u < 2 && ok; ++u, ++c, ru.next(scores ? p.nk : p.nv)) {
+                const int s = ru.s;
+                ok = spin(&vfull[s], ru.ph);
+                if (ok) ok = spin(&epi[2 * (kk & 1) + u], (kk >> 1) & 1);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t vh = smem_u32(sm + p.off_v + s * p.ub), pa = t_s(kk) + 32 * u;
+                if (MLA || p.k_lo) pf_issue_values<true, MLA>(t_o, t_ol, pa, vh, k > 0 || u > 0);
+                else pf_issue_values<false, false>(t_o, t_o, pa, vh, k > 0 || u > 0);
+                umma_commit(&vfree[s]);
+              }
+              if (ok) umma_commit(&pvdone[kk & 1]);
+            }
+          }
+          if (!ok) *abort_flag = 1;
+        }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+      }
+      // every product this warp issued lands before TMEM is released (bounded)
+      if (lane == 0 && c > 0) {
+        uint64_t *d = &drain[scores ? 0 : 1];
+        umma_commit(d);
+        mbar_wait(d, 0, 1u << 22);
+      }
+      __syncwarp();
     }
-    // every product this warp issued lands before TMEM is released (bounded)
-    if (lane == 0 && c > 0) {
-      uint64_t *d = &drain[scores ? 0 : 1];
-      umma_commit(d);
-      mbar_wait(d, 0, 1u << 22);
-    }
-    __syncwarp();
   } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 104;" ::: "memory");
     // ======================= workers ======================================
     bool failed = false;
     auto wait_pv = [&](int c) -> bool {  // completion of tile c's value product
@@ -605,6 +617,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
       // are not normalised: O is divided by the row's sum at the end.
       // A warp whose wait gave up stays in the tile loop for the barriers.
       float c_ref = -INFINITY, l_run = 0.f;
+      const uint64_t sg2 = pair_f32(sg, sg);
       for (int k = 0; k < J.n_t; ++k, ++kk) {
         // scores of this tile (issued once the buffer's last P was read)
         if (!failed && !__all_sync(0xffffffffu, spin(&sdone[kk & 1], (kk >> 1) & 1))) {
@@ -671,21 +684,30 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
         for (int u = 0; u < 2; ++u) {
           const int nv = u ? nv1 : nv0;
           float *yu = y + 16 * u;
+          uint64_t y2[8];
           if (nv >= 16) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) yu[i] = fast_exp2(fmaf(yu[i], sg, -c_ref));
+            for (int i = 0; i < 8; ++i) {
+              float e0, e1;
+              unpair_f32(fma_f32x2(pair_f32(yu[2 * i], yu[2 * i + 1]), sg2, pair_f32(-c_ref, -c_ref)), e0, e1);
+              y2[i] = pair_f32(fast_exp2(e0), fast_exp2(e1));
+            }
           } else {
 #pragma unroll
             for (int i = 0; i < 16; ++i) yu[i] = i < nv ? fast_exp2(fmaf(yu[i], sg, -c_ref)) : 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) y2[i] = pair_f32(yu[2 * i], yu[2 * i + 1]);
           }
           uint32_t hw[8], lw[8];
-          float ls[4] = {0.f, 0.f, 0.f, 0.f};
+          uint64_t ls[2] = {0, 0};
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            split2<true>(yu[2 * i], yu[2 * i + 1], hw[i], lw[i]);
-            ls[i & 3] += yu[2 * i] + yu[2 * i + 1];
+            split2_bf16(y2[i], hw[i], lw[i]);
+            ls[i & 1] = add_f32x2(ls[i & 1], y2[i]);
           }
-          l_run += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+          float l0, l1;
+          unpair_f32(add_f32x2(ls[0], ls[1]), l0, l1);
+          l_run += l0 + l1;
           tmem_st8_nw(t_s(kk) + 32 * u + 8 * slice + lane_off, hw);
           tmem_st8_nw(t_s(kk) + 64 + 32 * u + 8 * slice + lane_off, lw);
           tmem_wait_st();
