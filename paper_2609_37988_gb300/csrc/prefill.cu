@@ -33,9 +33,9 @@
 // in TMEM took 77-90 cycles (a clock64 trace of the 64-position version: 16
 // of them 1450 cycles, 12 value products 800 alone) against 64 for N = 128,
 // and the two products of a tile then cost 2560 cycles per 128 positions
-// (16 + 24 at 64).  Measured: about 3500 cycles per 128 positions, the chain
+// (16 + 24 at 64).  Measured: about 3400 cycles per 128 positions, the chain
 // of a tile's scores, epilogue (about 1500) and values with two tiles in
-// flight; the 64-position version took 2.33 ms where this one takes 2.12
+// flight; the 64-position version took 2.33 ms, this one then 2.12
 // (14B int4 layer, 4 x 8192 positions, the last 2048 the chunk).  The chain's
 // share of the epilogue: packed binary32 arithmetic (2025 -> 1995 us, repeated
 // calls) and 104 registers for the workers (-> 1946 us); the first unit's
