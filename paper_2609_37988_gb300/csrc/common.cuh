@@ -6,6 +6,10 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
+
+#include "regsplit.h"
+
 namespace kvk {
 
 // ---- programmatic dependent launch ----------------------------------------
@@ -37,6 +41,20 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Whether kernel K was compiled to the register count that its setmaxnreg
+// split needs (regsplit.h); asked of the runtime until it says so once.
+template <auto K>
+inline cudaError_t check_reg_split(const RegSplit &split) {
+  static std::atomic<bool> known{false};
+  if (known.load(std::memory_order_relaxed)) return cudaSuccess;
+  cudaFuncAttributes fa;
+  const cudaError_t e = cudaFuncGetAttributes(&fa, reinterpret_cast<const void *>(K));
+  if (e != cudaSuccess) return e;
+  if (!split.fits(fa.numRegs)) return cudaErrorLaunchOutOfResources;
+  known.store(true, std::memory_order_relaxed);
+  return cudaSuccess;
 }
 
 __device__ __forceinline__ void set_err(int32_t *err, int code) {

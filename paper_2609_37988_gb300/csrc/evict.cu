@@ -948,9 +948,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
 
   // Registers by warpgroup: the epilogues' sums take more than an equal share.
   // 512 x 88 + 256 x 56 + 128 x 40 = 64512 = the 896 x 72 launched.
-  static_assert(kTcThreads == 896, "the register split");
+  static_assert(kEvictRegs.threads[0] == kTcEpi && kEvictRegs.threads[1] == kTcDeq &&
+                    kEvictRegs.all_threads() == kTcThreads && kEvictRegs.fits(72),
+                "the register split");
   if (warp >= (kTcEpi + kTcDeq) / 32) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;" ::: "memory");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kEvictRegs.regs[2]) : "memory");
     if (warp == (kTcEpi + kTcDeq + kTcCopy) / 32) {
       // ======================= MMA warp =====================================
       // the same item sequence as the others; each chain once its keys are
@@ -993,7 +995,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
       asm volatile("cp.async.wait_all;" ::: "memory");  // no copy outlives the CTA
     }
   } else if (warp >= kTcEpi / 32) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;" ::: "memory");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kEvictRegs.regs[1]) : "memory");
     // ======================= dequantising =================================
     // A thread whose wait gave up goes on without work.
     bool failed = false;
@@ -1032,7 +1034,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
     }
     if (failed) set_err(a.err, 8);
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 88;" ::: "memory");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEvictRegs.regs[0]) : "memory");
     // ======================= epilogues ====================================
     // A warp whose wait gave up goes on through the barriers without work.
     bool failed = false;
@@ -1122,8 +1124,13 @@ cudaError_t launch_evict_tc(const EvictArgs &args, cudaStream_t st) {
   const TcPlan p = tc_plan(a, sms);
   a.items_per_cta = p.items_per_cta;
   // 160 rows (5 query heads, 32 queries) fit 40 sums a thread
-  auto stat = p.R16 <= 160 ? evict_tc_kernel<false, 5> : evict_tc_kernel<false, 8>;
-  cudaError_t e = cudaFuncSetAttribute(stat, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+  const bool few = p.R16 <= 160;
+  auto stat = few ? evict_tc_kernel<false, 5> : evict_tc_kernel<false, 8>;
+  cudaError_t e = few ? check_reg_split<&evict_tc_kernel<false, 5>>(kEvictRegs)
+                      : check_reg_split<&evict_tc_kernel<false, 8>>(kEvictRegs);
+  if (e == cudaSuccess) e = check_reg_split<&evict_tc_kernel<true, 1>>(kEvictRegs);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(stat, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(evict_tc_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
   if (e != cudaSuccess) return e;

@@ -253,8 +253,10 @@ __global__ void __launch_bounds__(kMlaQThreads, 1)
   // in all): expansion 80 + 80, products 96, softmax 256, in all
   // (80 + 80 + 96 + 256) x 128 = 65536; each warpgroup's role begins with its
   // own (the softmax increase waits for the decreases).
+  static_assert(kMlaQRegs.all_threads() == kMlaQThreads && kMlaQRegs.threads[2] == kExpThreads && kMlaQRegs.fits(128),
+                "the register split");
   if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 80;\n" ::: "memory");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kMlaQRegs.regs[2]) : "memory");
     // ======================= expansion warps ==============================
     // tile t -> operand stage t % NST (free once the values of tile t - NST
     // were computed); rows past the split's end are zero, with zero scales
@@ -364,7 +366,7 @@ __global__ void __launch_bounds__(kMlaQThreads, 1)
     __syncwarp();
     pdl_trigger();
   } else if (warp >= 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 96;\n" ::: "memory");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kMlaQRegs.regs[1]) : "memory");
     if (warp == 5) {
       // no role: the tiles come from global memory (see the expansion warps)
       pdl_trigger();
@@ -446,7 +448,7 @@ __global__ void __launch_bounds__(kMlaQThreads, 1)
       pdl_trigger();
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 256;\n" ::: "memory");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kMlaQRegs.regs[0]) : "memory");
     // ======================= softmax warps ================================
     const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
     // this lane's tile position: M = 128 puts row r in lane r; M = 64 puts
@@ -674,7 +676,9 @@ cudaError_t launch_mla_q_t(const MlaDecodeArgs &a, cudaStream_t st) {
   constexpr int MU_SMEM = (64 * (W + 8)) * 2 + (2 * 64 * 16 + 16) * 4;
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    cudaError_t e = check_reg_split<&mla_decode_q_kernel<W, BITS, SYM>>(kMlaQRegs);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(mla_merge_upv_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                MU_SMEM);

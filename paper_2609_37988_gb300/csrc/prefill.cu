@@ -391,9 +391,10 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
   // Registers by warpgroup, 512 x 104 + 128 x 64 = the 640 x 96 launched: the
   // workers hold 32 scores, their weights and both halves without spills
   // (each set inside its branch: ahead of the branches the workers spilled).
-  static_assert(kPfThreads == 640, "the register split");
+  static_assert(kPfRegs.threads[0] == kPfWorkers && kPfRegs.all_threads() == kPfThreads && kPfRegs.fits(96),
+                "the register split");
   if (warp >= kPfWorkers / 32) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;" ::: "memory");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPfRegs.regs[1]) : "memory");
     if (warp == kPfWorkers / 32 + 1 || warp == kPfWorkers / 32 + 3) {
       // ======================= copy warps ===================================
       // lane 0 of one copies each tile's key units (and positional keys), of
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
       __syncwarp();
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 104;" ::: "memory");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPfRegs.regs[0]) : "memory");
     // ======================= workers ======================================
     bool failed = false;
     auto wait_pv = [&](int c) -> bool {  // completion of tile c's value product
@@ -856,7 +857,9 @@ cudaError_t launch_mla_prefill_formed(const PfArgs &a, cudaStream_t st) {
   cudaError_t e = pf_sms(&sms);
   if (e != cudaSuccess) return e;
   const PfPlan p = pf_plan(a, sms);
-  e = cudaFuncSetAttribute(prefill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+  e = check_reg_split<&prefill_kernel<true>>(kPfRegs);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(prefill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
   if (e == cudaSuccess)
     e = launch_pdl(prefill_kernel<true>, dim3(p.grid), dim3(kPfThreads), p.smem, st, a, p);
   return e;
@@ -867,7 +870,9 @@ cudaError_t launch_gqa_prefill(const PfArgs &a, cudaStream_t st) {
   cudaError_t e = pf_sms(&sms);
   if (e != cudaSuccess) return e;
   const PfPlan po = pf_plan(a, sms);
-  e = cudaFuncSetAttribute(prefill_expand_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, po.smem_x);
+  e = check_reg_split<&prefill_kernel<false>>(kPfRegs);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(prefill_expand_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, po.smem_x);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(prefill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, po.smem);
   if (e != cudaSuccess) return e;
