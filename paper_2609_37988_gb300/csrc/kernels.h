@@ -146,7 +146,10 @@ struct PfArgs {
   int Hq, G, n_q;
   float sig_log2;      // softmax scale * log2(e)
   float *out;          // [B, n_q, Hq, D]
-  int *counter;        // the job counter, zeroed by the launch
+  int *counter;        // the job counter, zero when the attention kernel starts
+  int *bad;            // [units] records of kPfBadStride ints, zero when the tiles are written:
+                       // cap - t of the first position t whose value is not finite, per
+                       // channel, then of any channel (0: none)
   uint8_t *tiles;      // [B * Hkv] units of prefill_unit_bytes(bits, cap): expanded tiles
   int32_t *err;
   // MLA chunks over formed keys and values (units = heads: v.B sequences from
@@ -157,8 +160,11 @@ struct PfArgs {
   int kr_bytes = 0;             // 0: GQA
   int b0 = 0, h0 = 0;
 };
+constexpr int kPfBadStride = 132;  // 128 channels, the unit's word, 16-byte multiple
+// zeroes counter and bad (bad 1024 bytes behind the counter)
 cudaError_t launch_gqa_prefill(const PfArgs &a, cudaStream_t st);
-// the attention over tiles that launch_mla_form wrote (prefill.cu)
+// the attention over tiles that launch_mla_form wrote (prefill.cu); the caller
+// zeroed counter and bad before the forming
 cudaError_t launch_mla_prefill_formed(const PfArgs &a, cudaStream_t st);
 bool prefill_plan_fits(const PfArgs &a);
 // expanded tiles of one unit (a KV head of a sequence of capacity cap)
@@ -205,6 +211,7 @@ struct MlaFormArgs {
   uint8_t *tiles;      // [nb][nh][n_t] tiles of 128 KB (layout: prefill.cu)
   uint8_t *kr;         // [nb][n_t] tiles of kr_bytes (16 KB hi; quantised latents + 16 KB lo)
   int kr_bytes;
+  int *bad;            // [nb * nh] records (PfArgs::bad)
   int32_t *err;
 };
 cudaError_t launch_mla_wsum(const void *w_uk, const void *w_uv, int H, int r, int W, float *wsum, cudaStream_t st);

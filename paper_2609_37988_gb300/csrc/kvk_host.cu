@@ -856,18 +856,21 @@ kvk_status check_prefill(const kvk_cache *c, int32_t layer, int32_t n_q) {
     return fail(KVK_ERR_INVALID_ARG, "n_q %d outside [1, max_ctx]", n_q);
   return KVK_OK;
 }
-// Pre-fill scratch: the job counter, then the expanded tiles (every
-// 64-position tile of every unit, dequantised once).
+// Pre-fill scratch: the job counter, the units' records of non-finite values,
+// then the expanded tiles (every 128-position tile of every unit, dequantised
+// once).
 struct PrefillScratch {
-  size_t counters, tiles, total;
+  size_t counters, bad, tiles, total;
 };
+size_t prefill_bad_bytes(size_t units) { return (size_t)align256((int64_t)units * kPfBadStride * 4); }
 PrefillScratch prefill_scratch(const kvk_cache *c, int32_t layer, int32_t n_q) {
   (void)n_q;
   PrefillScratch p;
   const int a = c->src[layer];
-  p.counters = 0;
-  p.tiles = 1024;
   const size_t units = (size_t)c->desc.max_batch * c->desc.n_kv_heads;
+  p.counters = 0;
+  p.bad = 1024;
+  p.tiles = p.bad + prefill_bad_bytes(units);
   p.total = p.tiles + units * prefill_unit_bytes(c->cfg[a].bits, c->lay[a].cap);
   return p;
 }
@@ -890,11 +893,11 @@ MlaPrefillScratch mla_prefill_scratch(const kvk_cache *c, int32_t layer, int32_t
   return p;
 }
 // MLA chunks over formed keys and values (mla_form.cu): the job counter, the
-// weights' column sums, then the positional keys' tiles and the formed tiles
+// units' records of non-finite values, the weights' column sums, then the positional keys' tiles and the formed tiles
 // of one group of nb sequences x nh heads (at most 2 GiB of tiles, or one
 // head of one sequence; the groups run one after another in the same space).
 struct MlaFormedScratch {
-  size_t wsum, kr, tiles, total;
+  size_t bad, wsum, kr, tiles, total;
   int nb, nh, kr_bytes;
 };
 MlaFormedScratch mla_formed_scratch(const kvk_cache *c, int32_t layer) {
@@ -906,7 +909,8 @@ MlaFormedScratch mla_formed_scratch(const kvk_cache *c, int32_t layer) {
   p.nh = (int)std::min(H, fit);
   p.nb = (int)std::max(1LL, std::min(B, fit / p.nh));
   p.kr_bytes = c->cfg[a].bits == 16 ? 16384 : 32768;
-  p.wsum = 1024;
+  p.bad = 1024;
+  p.wsum = p.bad + prefill_bad_bytes((size_t)p.nb * p.nh);
   p.kr = p.wsum + (size_t)align256(H * 256 * 4);
   p.tiles = p.kr + (size_t)p.nb * n_t * p.kr_bytes;
   p.total = p.tiles + (size_t)p.nb * p.nh * unit;
@@ -965,6 +969,7 @@ kvk_status kvk_prefill_attention(kvk_cache *c, int32_t layer, const void *q, int
   a.n_q = n_q;
   a.sig_log2 = softmax_scale * 1.4426950408889634f;
   a.counter = reinterpret_cast<int *>(static_cast<uint8_t *>(scratch) + ps.counters);
+  a.bad = reinterpret_cast<int *>(static_cast<uint8_t *>(scratch) + ps.bad);
   a.tiles = static_cast<uint8_t *>(scratch) + ps.tiles;
   a.out = out;
   a.err = c->err();
@@ -1231,6 +1236,7 @@ kvk_status kvk_prefill_attention_mla(kvk_cache *c, int32_t layer, const void *q_
     f.tiles = sc + fs.tiles;
     f.kr = sc + fs.kr;
     f.kr_bytes = fs.kr_bytes;
+    f.bad = reinterpret_cast<int *>(sc + fs.bad);
     f.err = c->err();
     PfArgs p;
     p.v = GqaView{};
@@ -1246,6 +1252,7 @@ kvk_status kvk_prefill_attention_mla(kvk_cache *c, int32_t layer, const void *q_
     p.sig_log2 = softmax_scale * 1.4426950408889634f;
     p.out = out;
     p.counter = reinterpret_cast<int *>(sc);
+    p.bad = f.bad;
     p.tiles = f.tiles;
     p.err = c->err();
     p.q_pe = q_pe;
@@ -1259,7 +1266,7 @@ kvk_status kvk_prefill_attention_mla(kvk_cache *c, int32_t layer, const void *q_
         f.h0 = p.h0 = h0;
         f.nb = p.v.B = std::min(fs.nb, mv.B - b0);
         f.nh = p.v.Hkv = std::min(fs.nh, H - h0);
-        e = cudaMemsetAsync(p.counter, 0, sizeof(int), st);
+        e = cudaMemsetAsync(sc, 0, fs.wsum, st);  // the counter and the group's records
         if (e == cudaSuccess) e = launch_mla_form(f, w_uk, w_uv, H, r, c->sm_count, st);
         if (e == cudaSuccess) e = launch_mla_prefill_formed(p, st);
       }

@@ -19,10 +19,12 @@
 // and the epilogue applies each position's scale, and its offset times the
 // weights' column sums (mla_wsum_kernel): one product either way.
 // Results leave as bf16 hi + lo halves in the tile layout prefill.cu copies
-// (128 positions: key units by 64 channels, value units by 64 positions), 32 bytes (16 channels) per
-// thread and store: the swizzle keeps such a pair of 16-byte chunks in one
-// aligned sector.  The positional keys are copied beside (hi, and lo for
-// quantised latents) once per block.
+// (128 positions: key units by 64 channels, value units by 64 positions), 32
+// bytes (16 channels) per thread and store: the swizzle keeps such a pair of
+// 16-byte chunks in one aligned sector.  Values that are not finite (of a
+// latent that is not) enter as zeros and are recorded (PfArgs::bad).  The
+// positional keys are copied beside (hi, and lo for quantised latents) once
+// per block.
 //
 // Bound by the weights' L2 traffic (64 bytes per cycle and SM at d = 512) and
 // the 64 KB per tile and head it writes.
@@ -393,6 +395,21 @@ __global__ void __launch_bounds__(kFmThreads, 1)
           if constexpr (BITS != 16) {
 #pragma unroll
             for (int k = 0; k < 32; ++k) x[k] = ws ? fmaf(x[k], sc, zc * ws[c0 + k]) : x[k] * sc;
+          }
+          if (half) {
+            uint32_t top = 0;
+#pragma unroll
+            for (int k = 0; k < 32; ++k) top = max(top, __float_as_uint(x[k]) & 0x7FFFFFFFu);
+            if (top >= 0x7F800000u) {
+              int *bad = a.bad + ((size_t)cur.b * a.nh + cur.h) * kPfBadStride;
+#pragma unroll
+              for (int k = 0; k < 32; ++k)
+                if ((__float_as_uint(x[k]) & 0x7FFFFFFFu) >= 0x7F800000u) {
+                  x[k] = 0.f;
+                  atomicMax(bad + c0 + k, (int)v.cap - (t0 + row));
+                }
+              atomicMax(bad + 128, (int)v.cap - (t0 + row));
+            }
           }
           {
 #pragma unroll

@@ -29,6 +29,12 @@
 // are handed out from a counter in bands of units whose tiles stay in L2,
 // the longest row blocks first.
 //
+// A position that a row does not see has weight 0 in its products, and 0
+// times an infinite or NaN value is NaN: such values enter the tiles as 0,
+// and each unit records, per channel, the first position that has one
+// (PfArgs::bad).  A row that sees it gets NaN in that channel, the others
+// do not depend on it.
+//
 // Why tiles of 128 positions: a score product of N = 64 with its A operand
 // in TMEM took 77-90 cycles (a clock64 trace of the 64-position version: 16
 // of them 1450 cycles, 12 value products 800 alone) against 64 for N = 128,
@@ -109,6 +115,29 @@ struct PfRing {
 __device__ __forceinline__ int pf_tiles(int len, int n_q, int G, int r_last) {
   const int p_max = len - n_q + r_last / G;
   return p_max >= 0 ? p_max / kPfT + 1 : 0;
+}
+
+// The non-finite halves of 8 bf16 values (channels ch.. of position t) set to
+// zero and recorded in `bad` (null: already recorded with their hi parts).
+__device__ __noinline__ uint4 pf_scrub(uint4 u, int *bad, int ch, int cap_t) {
+  uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if ((w[i] >> (16 * h) & 0x7F80u) == 0x7F80u) {
+        w[i] &= h ? 0xFFFFu : 0xFFFF0000u;
+        if (bad) {
+          atomicMax(bad + ch + 2 * i + h, cap_t);
+          atomicMax(bad + 128, cap_t);
+        }
+      }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ bool pf_finite(uint4 u) {
+  // an exponent of all ones carries out of its half's top bit
+  auto ok = [](uint32_t w) { return (((w & 0x7F807F80u) + 0x00800080u) & 0x80008000u) == 0; };
+  return ok(u.x) && ok(u.y) && ok(u.z) && ok(u.w);
 }
 
 // Expand: the keys and values of 64 positions (half a tile) of one unit,
@@ -234,7 +263,14 @@ __global__ void __launch_bounds__(kPfWorkers) prefill_expand_kernel(const PfArgs
     reinterpret_cast<uint4 *>(dst + b * p.ub + h * 2 * kPfBox + hf * kPfBox)[i - x * B16] = src[i];
   }
   uint4 *dv = reinterpret_cast<uint4 *>(dst + (2 + hf) * p.ub);
-  for (int i = tid; i < p.ub / 16; i += kPfWorkers) dv[i] = src[kbytes / 16 + i];
+  for (int i = tid; i < p.ub / 16; i += kPfWorkers) {
+    uint4 u = src[kbytes / 16 + i];
+    if (!pf_finite(u)) {
+      const int x = i / B16, row = i >> 3 & 63, ch = 64 * (x & 1) + 8 * ((i & 7) ^ (row & 7));
+      u = pf_scrub(u, x < 2 ? a.bad + (size_t)unit * kPfBadStride : nullptr, ch, (int)v.cap - (t0 + row));
+    }
+    dv[i] = u;
+  }
   pdl_trigger();
 }
 
@@ -727,6 +763,8 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
       // per slice, divided by the sum of the row's weights (the four slices'
       // sums, same reference)
       float o[32];
+      const int *bad = a.bad + (size_t)J.unit * kPfBadStride;
+      const bool sees_bad = (int)v.cap - last <= __ldg(bad + 128);  // a position that is not finite in some channel
       if (J.n_t > 0) {
         const bool ok = wait_pv(kk - 1);
         if (workers_sync_or<kPfWorkers>(!ok)) {
@@ -753,6 +791,17 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
       workers_sync<kPfWorkers>();
       const float L = (smax[rl] + smax[kPfRows + rl]) + (smax[2 * kPfRows + rl] + smax[3 * kPfRows + rl]);
       const float inv = L > 0.f ? 1.f / L : 0.f;
+      if (sees_bad) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int4 x = reinterpret_cast<const int4 *>(bad + 32 * slice)[c];
+          const int at = (int)v.cap - last;
+          if (at <= x.x) o[4 * c] = NAN;
+          if (at <= x.y) o[4 * c + 1] = NAN;
+          if (at <= x.z) o[4 * c + 2] = NAN;
+          if (at <= x.w) o[4 * c + 3] = NAN;
+        }
+      }
       if (row_live) {
         const int r = J.r0 + rl;
         const int qi = r / a.G, h = J.j * a.G + (r - qi * a.G);
@@ -876,7 +925,8 @@ cudaError_t launch_gqa_prefill(const PfArgs &a, cudaStream_t st) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(prefill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, po.smem);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);  // the job counter
+  // the job counter and the records of non-finite values behind it
+  e = cudaMemsetAsync(a.counter, 0, 1024 + (size_t)a.v.B * a.v.Hkv * kPfBadStride * 4, st);
   if (e == cudaSuccess)
     e = launch_pdl(prefill_expand_kernel, dim3(2 * po.n_t, a.v.B * a.v.Hkv), dim3(kPfWorkers), po.smem_x, st,
                    a, po);

@@ -174,3 +174,33 @@ def test_mla_prefill_scratch_limits():
     assert_close(f32(out), f32(full), max_abs=2e-4, rel_l2=1e-4, what="absorbed = formed")
     assert c.lib.kvk_prefill_attention_mla(*args, 1024, ctypes.c_void_p(st)) != 0
     assert c.device_error() == 0
+
+
+@pytest.mark.parametrize("width,fmt", [(512, None), (64, None), (128, ("symmetric", 8))],
+                         ids=["bf16-d512", "bf16-d64", "sym8-d128"])
+def test_mla_prefill_non_finite_latents_stay_with_their_readers(width, fmt):
+    """A latent with an infinite coordinate spoils the rows that see its
+    position and no others, formed keys and values or not."""
+    from paper_2609_37988_gb300.cache import Cache, Layer
+    T, n_q, at = 700, 600, 555
+    layer = dict(bits=16, width=width) if fmt is None else dict(bits=fmt[1], scheme=fmt[0], width=width)
+    g = torch.Generator().manual_seed(9)
+    cl = torch.randn((2, T, 512), generator=g).to(torch.bfloat16)
+    kr = torch.randn((2, T, 64), generator=g).to(torch.bfloat16)
+    wk, wv = ((torch.randn((H, 128, 512), generator=g) / math.sqrt(512)).to(torch.bfloat16).cuda() for _ in range(2))
+    qn = torch.randn((2, n_q, H, 128), generator=g).to(torch.bfloat16).cuda()
+    qp = torch.randn((2, n_q, H, 64), generator=g).to(torch.bfloat16).cuda()
+    dirty = cl.clone()
+    dirty[1, at, 7] = math.inf
+    outs = []
+    for x in (cl, dirty):
+        c = Cache(kind="mla", n_layers=1, n_q_heads=H, head_dim=128, latent_dim=512, rope_dim=64, max_batch=2,
+                  max_ctx=T, layers=[Layer(**layer)])
+        c.append(0, x.cuda(), kr.cuda())
+        outs.append(f32(c.prefill_mla(0, qn, qp, wk, wv, 0.07)).copy())
+        assert c.device_error() == 0
+    clean, out = outs
+    first = at - (T - n_q)
+    assert np.array_equal(out[0], clean[0])
+    assert np.array_equal(out[1, :first], clean[1, :first])
+    assert np.isnan(out[1, first:]).all()

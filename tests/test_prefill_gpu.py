@@ -111,6 +111,36 @@ def test_prefill_row_maxima_rise(fmt):
     assert c.device_error() == 0
 
 
+@pytest.mark.parametrize("fmt,hit", [(FORMATS[0], 1), (FORMATS[2], 32), (FORMATS[6], 128)],
+                         ids=["bf16", "int4", "sym4"])
+def test_prefill_non_finite_values_stay_with_their_readers(fmt, hit):
+    """An infinite (bf16: also a NaN) value reaches the rows that see its
+    position, in the channels that its stored group spoils, and no others:
+    rows before it, of the same job and tile, are those of a clean cache."""
+    Hkv, G, T, n_q = 2, 5, 300, 150
+    g = torch.Generator().manual_seed(12)
+    K = torch.randn((1, T, Hkv, 128), generator=g).to(torch.bfloat16)
+    V = torch.randn((1, T, Hkv, 128), generator=g).to(torch.bfloat16)
+    q = _queries(1, n_q, G * Hkv, seed=5, dtype=torch.bfloat16).cuda()
+    spots = [(200, 0, 3, math.inf), (263, 1, 70, math.nan if hit == 1 else -math.inf)]
+    dirty = V.clone()
+    for t, h, ch, x in spots:
+        dirty[0, t, h, ch] = x
+    outs = []
+    for v in (V, dirty):
+        c = _cache(1, G * Hkv, Hkv, T, [fmt])
+        c.append(0, K.cuda(), v.cuda())
+        outs.append(f32(c.prefill(0, q, 0.08)).copy())
+        assert c.device_error() == 0
+    clean, out = outs
+    spoilt = np.zeros(clean.shape, bool)
+    for t, h, ch, _ in spots:
+        c0 = ch // hit * hit
+        spoilt[0, t - (T - n_q):, h * G:(h + 1) * G, c0:c0 + hit] = True
+    assert np.isnan(out[spoilt]).all()
+    assert np.array_equal(out[~spoilt], clean[~spoilt])
+
+
 def test_prefill_one_query_is_decode_and_inheritor_reads_anchor():
     B, Hkv, G, T = 2, 4, 5, 600
     fmt = dict(bits=4, group=32, key_axis="token")
