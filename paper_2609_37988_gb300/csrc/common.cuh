@@ -193,6 +193,37 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
+// 32 bytes (a sector) at a 32-byte aligned global address
+__device__ __forceinline__ void st_sector(void *p, uint4 a, uint4 b) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
+               "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+               : "memory");
+}
+// 8 floats at a 16-byte aligned global address, one access where `sector`
+// (the same for the warp) says that it is 32-byte aligned
+__device__ __forceinline__ void st8(float *p, const float *x, bool sector) {
+  if (sector) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]),
+                 "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7])
+                 : "memory");
+  } else {
+    reinterpret_cast<float4 *>(p)[0] = make_float4(x[0], x[1], x[2], x[3]);
+    reinterpret_cast<float4 *>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
+  }
+}
+__device__ __forceinline__ void ld8(const float *p, float (&x)[8], bool sector) {
+  if (sector) {
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
+                 : "l"(p)
+                 : "memory");
+  } else {
+    const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
+    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+    x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+  }
+}
+
 // ---- packing -------------------------------------------------------------
 __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
   __half2 h = __floats2half2_rn(lo, hi);
@@ -261,6 +292,15 @@ __device__ __forceinline__ void split2_bf16(uint64_t x2, uint32_t &hi, uint32_t 
   const float2 h = unpack2<true>(hi);
   unpair_f32(fma_f32x2(pair_f32(h.x, h.y), pair_f32(-1.f, -1.f), x2), dx, dy);
   lo = pack2<true>(dx, dy);
+}
+// the same in f16 halves (22 bits of values within f16's normal range)
+__device__ __forceinline__ void split2_f16(uint64_t x2, uint32_t &hi, uint32_t &lo) {
+  float x, y, dx, dy;
+  unpair_f32(x2, x, y);
+  hi = pack2<false>(x, y);
+  const float2 h = unpack2<false>(hi);
+  unpair_f32(fma_f32x2(pair_f32(h.x, h.y), pair_f32(-1.f, -1.f), x2), dx, dy);
+  lo = pack2<false>(dx, dy);
 }
 
 __device__ __forceinline__ float bf16_to_f32(uint16_t b) {

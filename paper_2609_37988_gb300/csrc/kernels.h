@@ -158,6 +158,8 @@ struct PfArgs {
   const void *q_pe = nullptr;   // bf16 [B, n_q, Hq, 64]
   const uint8_t *kr = nullptr;  // [v.B][tiles of 128 positions] of kr_bytes: hi box, lo box if quantised
   int kr_bytes = 0;             // 0: GQA
+  int flush = 0;                // tiles summed in TMEM before O leaves it (a power of two)
+  const uint32_t *vexp = nullptr;  // [units][tiles]: exponents of the formed values (MlaFormArgs)
   int b0 = 0, h0 = 0;
 };
 constexpr int kPfBadStride = 132;  // 128 channels, the unit's word, 16-byte multiple
@@ -211,6 +213,8 @@ struct MlaFormArgs {
   uint8_t *tiles;      // [nb][nh][n_t] tiles of 128 KB (layout: prefill.cu)
   uint8_t *kr;         // [nb][n_t] tiles of kr_bytes (16 KB hi; quantised latents + 16 KB lo)
   int kr_bytes;
+  uint32_t *vexp;      // [nb][nh][n_t]: byte j the exponent e (signed) of positions 32 j .. + 31 of the
+                       // tile, whose values are stored divided by 2^e
   int *bad;            // [nb * nh] records (PfArgs::bad)
   int32_t *err;
 };

@@ -893,11 +893,12 @@ MlaPrefillScratch mla_prefill_scratch(const kvk_cache *c, int32_t layer, int32_t
   return p;
 }
 // MLA chunks over formed keys and values (mla_form.cu): the job counter, the
-// units' records of non-finite values, the weights' column sums, then the positional keys' tiles and the formed tiles
-// of one group of nb sequences x nh heads (at most 2 GiB of tiles, or one
-// head of one sequence; the groups run one after another in the same space).
+// units' records of non-finite values, the weights' column sums, the formed
+// values' exponents, then the positional keys' tiles and the formed tiles of
+// one group of nb sequences x nh heads (at most 2 GiB of tiles, or one head of
+// one sequence; the groups run one after another in the same space).
 struct MlaFormedScratch {
-  size_t bad, wsum, kr, tiles, total;
+  size_t bad, wsum, vexp, kr, tiles, total;
   int nb, nh, kr_bytes;
 };
 MlaFormedScratch mla_formed_scratch(const kvk_cache *c, int32_t layer) {
@@ -911,7 +912,8 @@ MlaFormedScratch mla_formed_scratch(const kvk_cache *c, int32_t layer) {
   p.kr_bytes = c->cfg[a].bits == 16 ? 16384 : 32768;
   p.bad = 1024;
   p.wsum = p.bad + prefill_bad_bytes((size_t)p.nb * p.nh);
-  p.kr = p.wsum + (size_t)align256(H * 256 * 4);
+  p.vexp = p.wsum + (size_t)align256(H * 256 * 4);
+  p.kr = p.vexp + (size_t)align256((int64_t)p.nb * p.nh * n_t * 4);
   p.tiles = p.kr + (size_t)p.nb * n_t * p.kr_bytes;
   p.total = p.tiles + (size_t)p.nb * p.nh * unit;
   return p;
@@ -1236,6 +1238,7 @@ kvk_status kvk_prefill_attention_mla(kvk_cache *c, int32_t layer, const void *q_
     f.tiles = sc + fs.tiles;
     f.kr = sc + fs.kr;
     f.kr_bytes = fs.kr_bytes;
+    f.vexp = reinterpret_cast<uint32_t *>(sc + fs.vexp);
     f.bad = reinterpret_cast<int *>(sc + fs.bad);
     f.err = c->err();
     PfArgs p;
@@ -1256,6 +1259,8 @@ kvk_status kvk_prefill_attention_mla(kvk_cache *c, int32_t layer, const void *q_
     p.tiles = f.tiles;
     p.err = c->err();
     p.q_pe = q_pe;
+    p.flush = mv.bits == 4 ? 16 : 32;
+    p.vexp = f.vexp;
     p.kr = f.kr;
     p.kr_bytes = fs.kr_bytes;
     cudaError_t e = cudaSuccess;

@@ -18,13 +18,17 @@
 // Quantised latents enter as centred codes, exact in bf16 (|code| <= 255),
 // and the epilogue applies each position's scale, and its offset times the
 // weights' column sums (mla_wsum_kernel): one product either way.
-// Results leave as bf16 hi + lo halves in the tile layout prefill.cu copies
-// (128 positions: key units by 64 channels, value units by 64 positions), 32
-// bytes (16 channels) per thread and store: the swizzle keeps such a pair of
-// 16-byte chunks in one aligned sector.  Values that are not finite (of a
-// latent that is not) enter as zeros and are recorded (PfArgs::bad).  The
-// positional keys are copied beside (hi, and lo for quantised latents) once
-// per block.
+// Results leave as hi + lo halves in the tile layout prefill.cu copies (128
+// positions: key units by 64 channels, value units by 64 positions), 32 bytes
+// (16 channels) per thread and store: the swizzle keeps such a pair of
+// 16-byte chunks in one aligned sector.  Keys split into bf16 (their rounding
+// reaches the output through the scores: 2e-7 of it), values into f16 with a
+// power-of-two scale per 32 positions: bf16 halves of the values, and of the
+// weights that multiply them, each cost 2.4e-6 of the output and the dropped
+// lo x lo products 2.8e-6, in all 4.4e-6 where the absorbed form has 2.7e-6
+// (4-bit latents, 700 positions).  Values that are not finite (of a latent
+// that is not) enter as zeros and are recorded (PfArgs::bad).  The positional
+// keys are copied beside (hi, and lo for quantised latents) once per block.
 //
 // Bound by the weights' L2 traffic (64 bytes per cycle and SM at d = 512) and
 // the 64 KB per tile and head it writes.
@@ -47,6 +51,10 @@ constexpr int kFmABox = kFmRows * 128;       // 64 coordinates of a block (16 KB
 constexpr int kFmWStage = 256 * 128;         // 64 coordinates of a head's 256 weight rows (32 KB)
 constexpr int kFmMaxStages = 6;
 constexpr int kFmTile = 131072;              // one expanded tile of 128 positions
+// smallest biased exponent of 32 positions' largest value: their exponent e
+// stays in [-90, 113], so that 2^-e is a normal number, weights relative to
+// the values' scale keep their range, and e fits a byte
+constexpr int kFmMinExp = 51;
 constexpr int kFmTail = kFmRows * 8 + 256;   // row scales and offsets, barriers, shared words
 
 __host__ __device__ constexpr int fm_stages(int W) {
@@ -65,11 +73,11 @@ __device__ __forceinline__ void fm_tma_load(void *dst, const CUtensorMap *tmap, 
       "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
 }
-// 32 bytes to a 32-byte aligned global address, one sector
-__device__ __forceinline__ void st_sector(void *p, uint4 a, uint4 b) {
-  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
-               "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
-               : "memory");
+// the larger, NaN if either is
+__device__ __forceinline__ float fmax_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
 }
 
 // Codes of chunk j (8 codes, layout.h) of 16 bytes of a quantised record.
@@ -388,43 +396,111 @@ __global__ void __launch_bounds__(kFmThreads, 1)
         uint8_t *tile = a.tiles + (((size_t)cur.b * a.nh + cur.h) * a.n_t + cur.t) * kFmTile;
         uint8_t *dst = half ? tile + 65536 + (row >> 6) * 32768 + (row & 63) * 128 : tile + row * 128;
         const int box = half ? 8192 : 32768;
+        // this row's channels c0 .. c0 + 31 as the products left them, and
+        // with the row's scale and offset (times m) applied
+        auto load = [&](int c0, float (&x)[32]) { tmem_ld32(tmem + 256 * (i & 1) + 128 * half + c0 + lane_off, x); };
+        auto apply = [&](int c0, float (&x)[32], float m) {
+          if (ws) {
+            const float s = sc * m, z = zc * m;
 #pragma unroll
-        for (int c0 = 0; c0 < 128; c0 += 32) {
-          float x[32];
-          tmem_ld32(tmem + 256 * (i & 1) + 128 * half + c0 + lane_off, x);
-          if constexpr (BITS != 16) {
+            for (int k4 = 0; k4 < 8; ++k4) {
+              const float4 w = *reinterpret_cast<const float4 *>(ws + c0 + 4 * k4);
+              x[4 * k4] = fmaf(x[4 * k4], s, z * w.x);
+              x[4 * k4 + 1] = fmaf(x[4 * k4 + 1], s, z * w.y);
+              x[4 * k4 + 2] = fmaf(x[4 * k4 + 2], s, z * w.z);
+              x[4 * k4 + 3] = fmaf(x[4 * k4 + 3], s, z * w.w);
+            }
+          } else {
+            const float s = sc * m;
 #pragma unroll
-            for (int k = 0; k < 32; ++k) x[k] = ws ? fmaf(x[k], sc, zc * ws[c0 + k]) : x[k] * sc;
+            for (int k = 0; k < 32; ++k) x[k] *= s;
           }
-          if (half) {
-            uint32_t top = 0;
+        };
+        auto store = [&](int c0, const uint32_t (&hw)[16], const uint32_t (&lw)[16]) {
 #pragma unroll
-            for (int k = 0; k < 32; ++k) top = max(top, __float_as_uint(x[k]) & 0x7FFFFFFFu);
-            if (top >= 0x7F800000u) {
+          for (int p = 0; p < 2; ++p) {
+            const int j = c0 / 16 + p;  // pair of 8-channel chunks
+            const uint32_t *h = hw + 8 * p, *l = lw + 8 * p;
+            const uint4 h0 = make_uint4(h[0], h[1], h[2], h[3]), h1 = make_uint4(h[4], h[5], h[6], h[7]);
+            const uint4 l0 = make_uint4(l[0], l[1], l[2], l[3]), l1 = make_uint4(l[4], l[5], l[6], l[7]);
+            uint8_t *q = dst + (j >> 2) * box + (((2 * (j & 3)) ^ (row & 6)) << 4);
+            const bool odd = row & 1;
+            st_sector(q, odd ? h1 : h0, odd ? h0 : h1);
+            st_sector(q + 16384, odd ? l1 : l0, odd ? l0 : l1);
+          }
+        };
+        if (!half) {
+#pragma unroll
+          for (int c0 = 0; c0 < 128; c0 += 32) {
+            float x[32];
+            uint32_t hw[16], lw[16];
+            load(c0, x);
+            if constexpr (BITS != 16) apply(c0, x, 1.f);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) split2<true>(x[2 * k], x[2 * k + 1], hw[k], lw[k]);
+            store(c0, hw, lw);
+          }
+        } else {
+          // the largest value of the warp's 32 positions (grouped codes: a
+          // bound on it) gives their exponent, it becomes 2^14 .. 2^15 at
+          // most; NaN and infinities stick to the maximum
+          float top = 0.f;
+#pragma unroll 1
+          for (int c0 = 0; c0 < 128; c0 += 32) {
+            float x[32];
+            load(c0, x);
+#pragma unroll
+            for (int k = 0; k < 32; ++k) top = fmax_nan(top, fabsf(x[k]));
+          }
+          if constexpr (BITS != 16) {
+            top *= fabsf(sc);
+            if (ws) {
+              const float4 w = *reinterpret_cast<const float4 *>(ws + 4 * lane);
+              const float wm = fmax_nan(fmax_nan(fabsf(w.x), fabsf(w.y)), fmax_nan(fabsf(w.z), fabsf(w.w)));
+              top = fmaf(fabsf(zc), __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(wm))), top);
+            }
+          }
+          const bool odd_row = !(top < INFINITY);  // a value (or the bound) is not finite
+          if (__any_sync(0xffffffffu, odd_row)) {
+            if (odd_row) top = 0.f;
+#pragma unroll 1
+            for (int c0 = 0; c0 < 128; c0 += 32) {
+              float x[32];
+              load(c0, x);
+              if (!odd_row) continue;
+              apply(c0, x, 1.f);
               int *bad = a.bad + ((size_t)cur.b * a.nh + cur.h) * kPfBadStride;
+              const int at = (int)v.cap - (t0 + row);
+#pragma unroll
+              for (int k = 0; k < 32; ++k) {
+                if (fabsf(x[k]) < INFINITY) {
+                  top = fmaxf(top, fabsf(x[k]));
+                } else {
+                  atomicMax(bad + c0 + k, at);
+                  atomicMax(bad + 128, at);
+                }
+              }
+            }
+          }
+          const uint32_t tb = __reduce_max_sync(0xffffffffu, __float_as_uint(top)) >> 23;
+          const int e = max((int)tb, kFmMinExp) - 141;
+          const float down = __uint_as_float((uint32_t)(127 - e) << 23);  // 2^-e
+          if (lane == 0)
+            reinterpret_cast<int8_t *>(a.vexp)[4 * (((size_t)cur.b * a.nh + cur.h) * a.n_t + cur.t) + quarter] = (int8_t)e;
+#pragma unroll
+          for (int c0 = 0; c0 < 128; c0 += 32) {
+            float x[32];
+            uint32_t hw[16], lw[16];
+            load(c0, x);
+            apply(c0, x, down);
+            if (odd_row) {
 #pragma unroll
               for (int k = 0; k < 32; ++k)
-                if ((__float_as_uint(x[k]) & 0x7FFFFFFFu) >= 0x7F800000u) {
-                  x[k] = 0.f;
-                  atomicMax(bad + c0 + k, (int)v.cap - (t0 + row));
-                }
-              atomicMax(bad + 128, (int)v.cap - (t0 + row));
+                if (!(fabsf(x[k]) < INFINITY)) x[k] = 0.f;
             }
-          }
-          {
 #pragma unroll
-            for (int p = 0; p < 2; ++p) {
-              uint32_t hw[8], lw[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k) split2<true>(x[16 * p + 2 * k], x[16 * p + 2 * k + 1], hw[k], lw[k]);
-              const int j = c0 / 16 + p;  // pair of 8-channel chunks
-              const uint4 h0 = make_uint4(hw[0], hw[1], hw[2], hw[3]), h1 = make_uint4(hw[4], hw[5], hw[6], hw[7]);
-              const uint4 l0 = make_uint4(lw[0], lw[1], lw[2], lw[3]), l1 = make_uint4(lw[4], lw[5], lw[6], lw[7]);
-              uint8_t *q = dst + (j >> 2) * box + (((2 * (j & 3)) ^ (row & 6)) << 4);
-              const bool odd = row & 1;
-              st_sector(q, odd ? h1 : h0, odd ? h0 : h1);
-              st_sector(q + 16384, odd ? l1 : l0, odd ? l0 : l1);
-            }
+            for (int k = 0; k < 16; ++k) split2<false>(x[2 * k], x[2 * k + 1], hw[k], lw[k]);
+            store(c0, hw, lw);
           }
         }
         tc_fence_before();

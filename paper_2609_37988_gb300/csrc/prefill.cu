@@ -57,7 +57,10 @@
 // zero, so each one costs its accumulator about 2^-25 of its value in one
 // direction, and three per k-step into one accumulator left 1.3e-5 of the
 // result over 3584 positions where the absorbed path has 5.6e-6 (the lo
-// products' own sum is 2^-8 of the result).
+// products' own sum is 2^-11 of the result).  One per k-step still costs
+// 1e-6 of the result per 1000 positions, so O is added to the row's partial
+// result in the output, in binary32, after every 16 tiles over 4-bit latents
+// and 32 over others, whose absorbed forms have 2.8e-6 and 3.5e-6 or more.
 #include <math.h>
 
 #include <algorithm>
@@ -91,6 +94,7 @@ struct PfPlan {
   int b_stride;       // expand: staged record stride (odd multiple of 16 bytes)
   int ub, tbytes;     // a unit; the whole tile (two key and two value units)
   int krb;            // positional keys of a tile (MLA; else 0)
+  int flush;          // tiles that an MLA job sums in TMEM before O is added to its output
   int nk, nv, nr;     // key and value units and positional tiles in shared memory
   int band;           // units per band of the job order
   int off_v, off_r, off_q, off_red, off_bar, smem, smem_x;  // key units at offset 0
@@ -303,16 +307,18 @@ __device__ __forceinline__ void pf_issue_scores_ss(uint32_t d0, uint32_t q, uint
 // O += P V of one value unit (64 positions): P (bf16 pairs, hi then lo 64
 // columns on) from TMEM at pa, the values (hi, then lo 2 boxes on) MN-major
 // in shared memory at vh (64-channel boxes kPfBox apart), 16 positions per
-// k-step; the products with a lo half into t_ol (t_o unless it is another).
+// k-step; the products with a lo half into t_ol (t_o unless it is another:
+// SPLIT, whose halves are f16, and which starts anew unless acc_l).
 template <bool KLO, bool SPLIT>
-__device__ __forceinline__ void pf_issue_values(uint32_t t_o, uint32_t t_ol, uint32_t pa, uint32_t vh, bool acc) {
-  constexpr uint32_t id = umma_idesc(128, 128, false, true);
+__device__ __forceinline__ void pf_issue_values(uint32_t t_o, uint32_t t_ol, uint32_t pa, uint32_t vh, bool acc,
+                                                bool acc_l) {
+  constexpr uint32_t id = SPLIT ? umma_idesc_f16(128, 128, false, true) : umma_idesc(128, 128, false, true);
   constexpr uint32_t hi = umma_desc_hi_sw128(1024);
   const uint32_t lo_h = umma_desc_lo(vh, kPfBox), lo_l = lo_h + (2 * kPfBox >> 4);
 #pragma unroll
   for (int ks = 0; ks < 4; ++ks) {
     umma_f16_ts_w(t_o, pa + 8 * ks, lo_h + 128 * ks, hi, id, acc || ks > 0);
-    if (KLO) umma_f16_ts_w(t_ol, pa + 8 * ks, lo_l + 128 * ks, hi, id, !SPLIT || acc || ks > 0);
+    if (KLO) umma_f16_ts_w(t_ol, pa + 8 * ks, lo_l + 128 * ks, hi, id, !SPLIT || acc_l || ks > 0);
     umma_f16_ts_w(t_ol, pa + 64 + 8 * ks, lo_h + 128 * ks, hi, id, true);
   }
 }
@@ -542,8 +548,10 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t vh = smem_u32(sm + p.off_v + s * p.ub), pa = t_s(kk) + 32 * u;
-                if (MLA || p.k_lo) pf_issue_values<true, MLA>(t_o, t_ol, pa, vh, k > 0 || u > 0);
-                else pf_issue_values<false, false>(t_o, t_o, pa, vh, k > 0 || u > 0);
+                const bool acc = k > 0 || u > 0;
+                if constexpr (MLA) pf_issue_values<true, true>(t_o, t_ol, pa, vh, (k & (p.flush - 1)) > 0 || u > 0, acc);
+                else if (p.k_lo) pf_issue_values<true, false>(t_o, t_o, pa, vh, acc, true);
+                else pf_issue_values<false, false>(t_o, t_o, pa, vh, acc, true);
                 umma_commit(&vfree[s]);
               }
               if (ok) umma_commit(&pvdone[kk & 1]);
@@ -632,6 +640,13 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
     int kk = 0;
     // [tile parity][4 slices][128 rows]: the rows' slice maxima
     float *smax = reinterpret_cast<float *>(sm + p.off_red);
+    float *ref_out = smax + 2 * 4 * kPfRows;  // (MLA) each thread's reference at its last flush
+    const bool sector = (reinterpret_cast<uintptr_t>(a.out) & 31) == 0;  // rows start on 32 bytes
+    // this thread's 32 channels of row rl of a job in the output
+    auto out_row = [&](const Job &J, int rl) {
+      const int r = J.r0 + rl, qi = r / a.G, h = J.j * a.G + (r - qi * a.G);
+      return a.out + (((size_t)J.b * a.n_q + qi) * a.Hq + h) * D + 32 * slice;
+    };
     // The four warps that share a quarter of the rows meet on a barrier of
     // their own: a row's maximum and its columns concern no other warp.
     auto row_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(4 + quarter) : "memory"); };
@@ -653,8 +668,16 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
       // value product of the previous tile) and their sums.  The weights
       // are not normalised: O is divided by the row's sum at the end.
       // A warp whose wait gave up stays in the tile loop for the barriers.
+      // Formed values (MLA) are stored divided by 2^e, e by 32 positions, and
+      // weights and values are split into f16: the reference is that of x +
+      // e and moves at a rise of 4, and the weights are 2^(x + e - m + 11) (at
+      // most 2^15; f16 halves keep 22 bits of those above 2^-3, and 2^-36 of
+      // 2^11 of the others), whose sum takes 2^-e.
+      constexpr float kRise = MLA ? 4.f : 8.f;
       float c_ref = -INFINITY, l_run = 0.f;
       const uint64_t sg2 = pair_f32(sg, sg);
+      const uint32_t *vexp = MLA ? a.vexp + (size_t)J.unit * p.n_t : nullptr;
+      uint32_t ve = MLA && J.n_t > 0 ? __ldg(vexp) : 0;
       for (int k = 0; k < J.n_t; ++k, ++kk) {
         // scores of this tile (issued once the buffer's last P was read)
         if (!failed && !__all_sync(0xffffffffu, spin(&sdone[kk & 1], (kk >> 1) & 1))) {
@@ -668,7 +691,30 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
         float y[32];
         tmem_ld16x2(t_s(kk) + 16 * slice + lane_off, t_s(kk) + 64 + 16 * slice + lane_off, y);
         float mx = -INFINITY;
-        if (row_live && nv1 >= 16) {  // all in the row's range (most tiles)
+        int ev[2] = {0, 0};  // exponents of this thread's positions of either value unit
+        if constexpr (MLA) {
+          ev[0] = (int8_t)(ve >> (8 * (slice >> 1)));
+          ev[1] = (int8_t)(ve >> (8 * (slice >> 1) + 16));
+          if (k + 1 < J.n_t) ve = __ldg(vexp + k + 1);
+          float mu[2] = {-INFINITY, -INFINITY};
+          if (row_live && nv1 >= 16) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              float mm[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                mm[i] = fmaxf(fmaxf(y[16 * u + i], y[16 * u + 4 + i]), fmaxf(y[16 * u + 8 + i], y[16 * u + 12 + i]));
+              mu[u] = fmaxf(fmaxf(mm[0], mm[1]), fmaxf(mm[2], mm[3]));
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              if (i < nv0) mu[0] = fmaxf(mu[0], y[i]);
+              if (i < nv1) mu[1] = fmaxf(mu[1], y[16 + i]);
+            }
+          }
+          mx = fmaxf(fmaf(mu[0], sg, (float)ev[0]), fmaf(mu[1], sg, (float)ev[1]));
+        } else if (row_live && nv1 >= 16) {  // all in the row's range (most tiles)
           float mm[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) mm[i] = fmaxf(fmaxf(y[i], y[8 + i]), fmaxf(y[16 + i], y[24 + i]));
@@ -685,31 +731,57 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
         tc_fence_before();
         row_sync();  // the row's four slice maxima; its scores are all read
         tc_fence_after();
-        const float M = sg * fmaxf(fmaxf(sx[0], sx[kPfRows]), fmaxf(sx[2 * kPfRows], sx[3 * kPfRows]));
-        const bool move = M > c_ref + 8.f;  // the same decision on the row's four threads
+        const float M = (MLA ? 1.f : sg) * fmaxf(fmaxf(sx[0], sx[kPfRows]), fmaxf(sx[2 * kPfRows], sx[3 * kPfRows]));
+        const bool move = M > c_ref + kRise;  // the same decision on the row's four threads
         const bool resc = move && c_ref != -INFINITY;
-        if (__any_sync(0xffffffffu, resc)) {
+        const bool any_resc = __any_sync(0xffffffffu, resc);
+        const bool flush = MLA && k > 0 && (k & (p.flush - 1)) == 0;
+        if (any_resc || flush) {
           // O holds this job's earlier tiles: rescale this thread's 32
           // channels once the previous tile's value product is done.  Lanes
           // are rows and the TMEM accesses are warp-wide (.sync.aligned), so
           // the whole warp takes part, rows that do not move with factor 1.
+          // A flush adds O to the row's partial result in the output (with
+          // the reference it has there kept in shared memory); the next
+          // value product starts O anew.
           if (!__all_sync(0xffffffffu, wait_pv(kk - 1))) {
             failed = true;
             *abort_flag = 1;
           } else {
             tc_fence_after();
             const float f = resc ? fast_exp2(c_ref - M) : 1.f;
+            const float c_new = move ? M : c_ref, c_old = flush ? ref_out[tid] : 0.f;
+            const float f_old = flush && k > p.flush && c_old != -INFINITY ? fast_exp2(c_old - c_new) : 0.f;
             float z[16];
             uint32_t zw[16];
 #pragma unroll
             for (int h = 0; h < (MLA ? 4 : 2); ++h) {
+              if (h >= 2 && !any_resc) continue;
               const uint32_t at = (h < 2 ? t_o : t_ol) + 32 * slice + 16 * (h & 1) + lane_off;
               tmem_ld16(at, z);
+              if (MLA && h < 2 && flush) {
+                if (row_live) {
+                  float *dst = out_row(J, rl) + 16 * h;
 #pragma unroll
-              for (int i = 0; i < 16; ++i) zw[i] = __float_as_uint(z[i] * f);
-              tmem_st16_nw(at, zw);
+                  for (int i = 0; i < 16; ++i) z[i] *= f;
+                  if (k > p.flush) {
+                    float x[2][8];
+                    ld8(dst, x[0], sector);
+                    ld8(dst + 8, x[1], sector);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) z[i] = fmaf(x[i >> 3][i & 7], f_old, z[i]);
+                  }
+                  st8(dst, z, sector);
+                  st8(dst + 8, z + 8, sector);
+                }
+              } else {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) zw[i] = __float_as_uint(z[i] * f);
+                tmem_st16_nw(at, zw);
+              }
             }
             l_run *= f;
+            if (flush) ref_out[tid] = c_new;
           }
         }
         if (move) c_ref = M;
@@ -722,16 +794,17 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
           const int nv = u ? nv1 : nv0;
           float *yu = y + 16 * u;
           uint64_t y2[8];
+          const float off = MLA ? (float)(ev[u] + 11) - c_ref : -c_ref;
           if (nv >= 16) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
               float e0, e1;
-              unpair_f32(fma_f32x2(pair_f32(yu[2 * i], yu[2 * i + 1]), sg2, pair_f32(-c_ref, -c_ref)), e0, e1);
+              unpair_f32(fma_f32x2(pair_f32(yu[2 * i], yu[2 * i + 1]), sg2, pair_f32(off, off)), e0, e1);
               y2[i] = pair_f32(fast_exp2(e0), fast_exp2(e1));
             }
           } else {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) yu[i] = i < nv ? fast_exp2(fmaf(yu[i], sg, -c_ref)) : 0.f;
+            for (int i = 0; i < 16; ++i) yu[i] = i < nv ? fast_exp2(fmaf(yu[i], sg, off)) : 0.f;
 #pragma unroll
             for (int i = 0; i < 8; ++i) y2[i] = pair_f32(yu[2 * i], yu[2 * i + 1]);
           }
@@ -739,12 +812,14 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
           uint64_t ls[2] = {0, 0};
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            split2_bf16(y2[i], hw[i], lw[i]);
+            if constexpr (MLA) split2_f16(y2[i], hw[i], lw[i]);
+            else split2_bf16(y2[i], hw[i], lw[i]);
             ls[i & 1] = add_f32x2(ls[i & 1], y2[i]);
           }
           float l0, l1;
           unpair_f32(add_f32x2(ls[0], ls[1]), l0, l1);
-          l_run += l0 + l1;
+          if constexpr (MLA) l_run = fmaf(l0 + l1, __uint_as_float((uint32_t)(127 - ev[u]) << 23), l_run);
+          else l_run += l0 + l1;
           tmem_st8_nw(t_s(kk) + 32 * u + 8 * slice + lane_off, hw);
           tmem_st8_nw(t_s(kk) + 64 + 32 * u + 8 * slice + lane_off, lw);
           tmem_wait_st();
@@ -782,6 +857,17 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
 #pragma unroll
             for (int i = 0; i < 16; ++i) o[16 * h + i] += z[i];
           }
+          if (J.n_t > p.flush && row_live) {
+            const float c_old = ref_out[tid], f_old = c_old != -INFINITY ? fast_exp2(c_old - c_ref) : 0.f;
+            const float *part = out_row(J, rl);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              float x[8];
+              ld8(part + 8 * c, x, sector);
+#pragma unroll
+              for (int i = 0; i < 8; ++i) o[8 * c + i] = fmaf(x[i], f_old, o[8 * c + i]);
+            }
+          }
         }
       } else {
 #pragma unroll
@@ -803,9 +889,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
         }
       }
       if (row_live) {
-        const int r = J.r0 + rl;
-        const int qi = r / a.G, h = J.j * a.G + (r - qi * a.G);
-        float4 *dst = reinterpret_cast<float4 *>(a.out + (((size_t)J.b * a.n_q + qi) * a.Hq + h) * D + 32 * slice);
+        float4 *dst = reinterpret_cast<float4 *>(out_row(J, rl));
 #pragma unroll
         for (int c = 0; c < 8; ++c)
           dst[c] = make_float4(o[4 * c] * inv, o[4 * c + 1] * inv, o[4 * c + 2] * inv, o[4 * c + 3] * inv);
@@ -850,9 +934,10 @@ PfPlan pf_plan(const PfArgs &a, int sms) {
   p.ub = 2 * kPfBox * (p.k_lo ? 2 : 1);
   p.tbytes = 4 * p.ub;
   p.krb = a.kr_bytes;
+  p.flush = a.flush;
   // + the (scale, zero) rows of the tile's position groups (per-channel keys)
   p.smem_x = 2 * p.ub + 64 * p.b_stride + (p.kpc ? 2 * 128 * 8 : 0) + 1024;
-  const int rbytes = 2 * 4 * kPfRows * 4;
+  const int rbytes = 2 * 4 * kPfRows * 4 + (a.kr_bytes ? kPfWorkers * 4 : 0);
   const int qbytes = p.krb ? 3 * 16384 : 0;
   // the most units that fit, values the larger share (a value unit waits for
   // the epilogue of its tile, key units only for the tile before)

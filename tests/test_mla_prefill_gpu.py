@@ -204,3 +204,78 @@ def test_mla_prefill_non_finite_latents_stay_with_their_readers(width, fmt):
     assert np.array_equal(out[0], clean[0])
     assert np.array_equal(out[1, :first], clean[1, :first])
     assert np.isnan(out[1, first:]).all()
+
+
+@pytest.mark.parametrize("fmt", [None, ("symmetric", 4)], ids=["bf16", "sym4"])
+@pytest.mark.parametrize("steep", [0.02, 1.0], ids=["flat", "steep"])
+def test_mla_prefill_formed_scales_and_flushes(fmt, steep):
+    """Formed values stored relative to a power of two per 32 positions
+    (zero, tiny and large latents side by side, the first ones zero) and
+    partial results that leave the accumulator every 16 (4-bit) or 32 tiles:
+    8450 positions, four flushes and more or two, a whole last round.  An
+    output that starts on 16 bytes but not on 32.  Bound: the accumulator
+    drops up to 2^-24 of itself per 16 positions of a round, 32 x 8 x 2^-24 =
+    1.5e-5 at most, 2e-5 with the other roundings (2^-20)."""
+    T, n_q, heads = 8450, 200, 4
+    from paper_2609_37988_gb300.cache import Cache, Layer
+    layer = dict(bits=16, width=512) if fmt is None else dict(bits=fmt[1], scheme=fmt[0], width=512)
+    g = torch.Generator().manual_seed(21)
+    e = torch.randint(-20, 3, (T // 32 + 1,), generator=g)
+    e[:3] = -200  # zeros
+    e[70:73] = -200
+    scale = torch.exp2(e.double()).float().repeat_interleave(32)[:T]
+    cl = (torch.randn((1, T, 512), generator=g) * torch.arange(512).add(1.0).rsqrt() * scale[None, :, None])
+    cl = cl.to(torch.bfloat16)
+    kr = torch.randn((1, T, 64), generator=g).to(torch.bfloat16)
+    wk = (torch.randn((heads, 128, 512), generator=g) / math.sqrt(512)).mul(steep).to(torch.bfloat16)
+    wv = (torch.randn((heads, 128, 512), generator=g) / math.sqrt(512)).to(torch.bfloat16)
+    qn = torch.randn((1, n_q, heads, 128), generator=g).to(torch.bfloat16)
+    qp = torch.randn((1, n_q, heads, 64), generator=g).to(torch.bfloat16)
+    c = Cache(kind="mla", n_layers=1, n_q_heads=heads, head_dim=128, latent_dim=512, rope_dim=64, max_batch=1,
+              max_ctx=T, layers=[Layer(**layer)])
+    c.append(0, cl.cuda(), kr.cuda())
+    sigma = 1.0 / math.sqrt(192)
+    args = (qn.cuda(), qp.cuda(), wk.cuda(), wv.cuda(), sigma)
+    rows = n_q * heads * (2 * 512 + 64) * 2 + n_q * heads * 514 * 4
+    assert _scratch(c, n_q) > 4 * rows  # over formed keys and values
+    out = c.prefill_mla(0, *args)
+    if fmt is None:
+        c_hat, kr_hat = f32(cl), f32(kr)
+    else:
+        st = ocache.mla_anchor_state(f32(cl), f32(kr), [T], 512, fmt[1], fmt[0])
+        c_hat, kr_hat = st["c_hat"], st["kr_hat"]
+    ref = oatt.mla_prefill_unabsorbed(f32(qn), f32(qp), c_hat, kr_hat, f32(wk), f32(wv), 512, [T], sigma)
+    err = np.linalg.norm(f32(out).astype(np.float64) - ref) / np.linalg.norm(ref)
+    assert err < 2e-5, err
+    buf = torch.empty(out.numel() + 8, device="cuda")
+    for off in (0, 4):
+        view = buf[off:off + out.numel()].view(out.shape)
+        assert view.data_ptr() % 32 == 4 * off
+        assert torch.equal(c.prefill_mla(0, *args, out=view), out)
+    assert c.device_error() == 0
+
+
+@pytest.mark.parametrize("fmt", [None, ("grouped", 4), ("symmetric", 4)], ids=["bf16", "int4", "sym4"])
+def test_mla_prefill_formed_is_no_less_exact(fmt):
+    """The same chunk over formed keys and values and (in a buffer too small
+    for them) by absorbed rows, against 64 bits."""
+    n_q, T = 512, 700
+    c, wk, wv, c_hat, kr_hat = _setup(128, fmt, [T, T], T, seed=17)
+    g = torch.Generator().manual_seed(6)
+    qn = torch.randn((2, n_q, H, 128), generator=g).to(torch.bfloat16)
+    qp = torch.randn((2, n_q, H, 64), generator=g).to(torch.bfloat16)
+    sigma = 1.0 / math.sqrt(192)
+    dev = [t.cuda() for t in (qn, qp, wk, wv)]
+    ref = oatt.mla_prefill_unabsorbed(f32(qn), f32(qp), c_hat, kr_hat, f32(wk), f32(wv), 128, [T, T], sigma)
+    small = 2 * n_q * H * ((2 * 128 + 64) * 2 + 130 * 4)
+    assert small < _scratch(c, n_q)
+    rows = torch.empty((2, n_q, H, 128), device="cuda")
+    buf = torch.empty(small, dtype=torch.uint8, device="cuda")
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    assert c.lib.kvk_prefill_attention_mla(c.handle, 0, *map(p, dev), n_q, sigma, p(rows), p(buf), small,
+                                           ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    formed = c.prefill_mla(0, *dev, sigma)
+    assert not torch.equal(formed, rows)
+    err = [np.linalg.norm(f32(x).astype(np.float64) - ref) / np.linalg.norm(ref) for x in (formed, rows)]
+    assert err[0] <= err[1], err
+    assert c.device_error() == 0
