@@ -269,6 +269,10 @@ kvk_status kvk_evict_window(kvk_cache *cache, int32_t layer, const void *q_win, 
  * scale not finite and positive, scratch too small). */
 kvk_status kvk_prefill_scratch_size(const kvk_cache *cache, int32_t layer, int32_t n_q,
                                     size_t *scratch_bytes);
+/* The smallest buffer that always serves the chunk (MLA: its absorbed rows,
+ * at times slower; GQA: kvk_prefill_scratch_size). */
+kvk_status kvk_prefill_scratch_least(const kvk_cache *cache, int32_t layer, int32_t n_q,
+                                     size_t *scratch_bytes);
 kvk_status kvk_prefill_attention(kvk_cache *cache, int32_t layer, const void *q, int32_t q_dtype,
                                  int32_t n_q, float softmax_scale, float *out, void *scratch,
                                  size_t scratch_bytes, kvk_stream stream);
@@ -284,18 +288,21 @@ kvk_status kvk_prefill_attention(kvk_cache *cache, int32_t layer, const void *q,
  * CTA per row, or per pair of consecutive rows of a sequence for bf16 latents
  * of width >= 256 when n_q is even).  Longer ones form each head's keys
  * W_UK[h][:, :d] c and values W_UV[h][:, :d] c once and attend over them (the
- * same algebra); where the line lies depends on the cache's batch, width and
- * precision.  Queries before position 0 give zeros.
+ * same algebra, and no less exact); the call takes the one that it expects to
+ * be faster for the chunk, the host's bound on the lengths and the anchor's
+ * width and precision.  Queries before position 0 give zeros.
  *  q_nope:  device bf16 [B, n_q, H, head_dim]; q_pe: bf16 [B, n_q, H, rope]
  *           (post-RoPE);
  *  w_uk, w_uv: device bf16 [H, head_dim, latent] as for decode;
  *  out:     device float32 [B, n_q, H, head_dim];
- *  scratch: device, 256-byte aligned, at least kvk_prefill_scratch_size
- *           bytes (which answers for MLA layers too, and never less for a
- *           larger n_q): the rows' absorbed queries and latent partials, or
- *           the formed keys and values (1 KB per position and head, heads and
- *           sequences in groups of at most 2 GiB) and a job counter.  A
- *           buffer that holds only the former serves every chunk by rows;
+ *  scratch: device, 256-byte aligned, at least kvk_prefill_scratch_least
+ *           bytes: the rows' absorbed queries and latent partials.
+ *           kvk_prefill_scratch_size answers for the faster path at the
+ *           lengths of its own call, never less for a larger n_q: where that
+ *           is the formed one, it holds the formed keys and values (1 KB per
+ *           position of the capacity and head; heads and sequences go in
+ *           groups within 256 MiB, or 128 times the rows' memory up to 2 GiB).
+ *           A buffer that holds only one of the two serves by it;
  * all 16-byte aligned.  Errors: INVALID_ARG (not an MLA cache, n_q outside
  * [1, max_ctx], null or misaligned pointers, scale not finite and positive,
  * scratch too small). */

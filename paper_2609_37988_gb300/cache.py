@@ -243,11 +243,17 @@ class Cache:
             out = torch.empty(q_nope.shape, dtype=torch.float32, device=q_nope.device)
         nbytes = ctypes.c_size_t()
         check(self.lib.kvk_prefill_scratch_size(self.handle, layer, n_q, ctypes.byref(nbytes)))
-        scratch = torch.empty(nbytes.value, dtype=torch.uint8, device=self.device)
+        try:
+            scratch = torch.empty(nbytes.value, dtype=torch.uint8, device=self.device)
+        except torch.cuda.OutOfMemoryError:  # the chunk's rows take less
+            check(self.lib.kvk_prefill_scratch_least(self.handle, layer, n_q, ctypes.byref(nbytes)))
+            scratch = torch.empty(nbytes.value, dtype=torch.uint8, device=self.device)
         check(self.lib.kvk_prefill_attention_mla(self.handle, layer, _ptr(q_nope), _ptr(q_pe), _ptr(w_uk),
                                                  _ptr(w_uv), n_q, float(scale), _ptr(out), _ptr(scratch),
                                                  nbytes.value, _stream(stream)))
-        self._prefill_scratch = scratch  # kept alive until the stream is done with it
+        # On the current stream the allocator reuses the buffer in stream
+        # order; another stream's is kept until the next call.
+        self._prefill_scratch = None if stream is None else scratch
         return out
 
     def kept_lists(self, layer: int, stream=None):

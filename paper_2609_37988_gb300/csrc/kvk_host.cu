@@ -184,7 +184,6 @@ struct kvk_cache {
   int sm_count;
   int device;
   std::vector<int> ctas;  // per layer, decode CTAs per SM (0 = not queried)
-  std::vector<int> formed_from;  // per MLA anchor, the shortest chunk over formed keys (mla_formed_from)
   uint32_t wait_limit = KVK_WAIT_LIMIT_DEFAULT;  // decode tile-loop waits (kvk_set_wait_limit)
   int schedule = KVK_SCHEDULE_AUTO;              // decode partition (kvk_set_decode_schedule)
   int run_ctas = 0;                              // CTAs of a run-schedule decode (0: whole waves)
@@ -432,47 +431,6 @@ int plan_balanced(kvk_cache *c, int a, bool runs, int splits, int *cap) {
   return (int)std::min<long long>(slots, (long long)units * ktiles);
 }
 
-// The shortest chunk of layer `a` that attends over formed keys and values;
-// shorter ones run the absorbed decode per row.  Both costs in ns, fitted to
-// measured calls (1 x 1500, 4 x 300, 4 x 4096, 8 x 1024, 16 x 600 positions,
-// 16-250 queries, every width; e.g. bf16 d = 512, 4 x 4096, absorbed / formed
-// us: 48 queries 162 / 163, 96 308 / 163; d = 64: 128 92 / 134, 250 170 / 137;
-// 8-bit d = 512, 8 x 1024: 16 55 / 92, 48 150 / 92):
-//  absorbed: per position, a wave of resident CTAs (one row each, or two at
-//            d >= 256 over bf16 latents) takes kFull (kHalf if at most half
-//            of it is there); absorption and merge kRow per row; 10 us;
-//  formed:   per position, a wave of jobs (128 rows of one head) takes 14.8
-//            and the forming kForm per sequence (quantised 0.6 more); 30 us
-//            (quantised 33, grouped 41 with the weights' column sums).
-// The answer is one more than the longest chunk (of up to 1024 queries) that
-// the absorbed path serves faster; at least 16 (a handful of queries is not
-// worth the formed tiles' memory), never where one head's tiles pass 2 GiB.
-int mla_formed_from(const kvk_cache *c, int a) {
-  const kvk_layer_cfg &L = c->cfg[a];
-  const int w = L.width == 512 ? 0 : L.width == 256 ? 1 : L.width == 128 ? 2 : 3;
-  static const double kHalf[4] = {36.0, 14.5, 10.0, 8.5}, kFull[4] = {41.0, 18.5, 15.6, 12.0};
-  static const double kQuant[4] = {37.0, 18.5, 10.5, 10.0}, kRow[4] = {75.0, 40.0, 22.0, 14.0};
-  static const double kForm[4] = {4.4, 3.2, 2.9, 2.7};
-  const bool quant = L.bits != 16;
-  if (c->lay[a].cap > (1 << 21)) return INT32_MAX;
-  const double B = c->desc.max_batch, H = c->desc.n_q_heads, T = c->desc.max_ctx, sms = c->sm_count;
-  for (int n = std::min(1024, c->desc.max_ctx); n >= 1; --n) {
-    const double rows = B * n;
-    double wave;
-    if (quant) {
-      wave = kQuant[w] * std::ceil(rows / sms);
-    } else {
-      const double slots = w >= 2 || n % 2 == 0 ? 2.0 * sms : sms;
-      wave = rows <= slots / 2 ? kHalf[w] : kFull[w] * std::ceil(rows / slots);
-    }
-    const double absorbed = wave * T + kRow[w] * rows + 10e3;
-    const double jobs = B * H * ((n + 127) / 128);
-    const double formed = (14.8 * std::ceil(jobs / sms) + B * (kForm[w] + (quant ? 0.6 : 0.0))) * T +
-                          (!quant ? 30e3 : layer_scheme(&L) == kSchemeSym ? 33e3 : 41e3);
-    if (absorbed < formed) return std::max(16, n + 1);
-  }
-  return 16;
-}
 }  // namespace
 
 extern "C" {
@@ -548,7 +506,6 @@ kvk_status kvk_cache_create(const kvk_model_desc *desc, const kvk_layer_cfg *cfg
   c->ragged.assign(desc->n_layers, 0);
   c->kept_on.assign(desc->n_layers, 0);
   c->ctas.assign(desc->n_layers, 0);
-  c->formed_from.assign(desc->n_layers, 0);
   int last = 0;
   for (int l = 0; l < desc->n_layers; ++l) {
     if (!cfg[l].inherit) {
@@ -573,7 +530,6 @@ kvk_status kvk_cache_create(const kvk_model_desc *desc, const kvk_layer_cfg *cfg
   for (int l = 0; l < desc->n_layers; ++l) {
     if (cfg[l].inherit) continue;
     if (desc->kind == KVK_KIND_MLA) {
-      c->formed_from[l] = mla_formed_from(c, l);
       if (cfg[l].bits != 16) continue;  // quantised tiles use bulk copies
       e = mla_make_tmap(c->tmap[l].bytes, c->mla_view(l));
     } else {
@@ -895,17 +851,23 @@ MlaPrefillScratch mla_prefill_scratch(const kvk_cache *c, int32_t layer, int32_t
 // MLA chunks over formed keys and values (mla_form.cu): the job counter, the
 // units' records of non-finite values, the weights' column sums, the formed
 // values' exponents, then the positional keys' tiles and the formed tiles of
-// one group of nb sequences x nh heads (at most 2 GiB of tiles, or one head of
-// one sequence; the groups run one after another in the same space).
+// one group of nb sequences x nh heads; the groups run one after another in
+// the same space.  A group takes as many units as 128 times the memory that
+// the chunk's absorbed rows take holds (that, between 256 MiB and 2 GiB; at
+// least one head of one sequence): tiles are laid out by the capacity, since
+// lengths live on the device and may pass the host's bound in a recorded
+// launch, and a short chunk over a large cache is not worth gigabytes.
 struct MlaFormedScratch {
   size_t bad, wsum, vexp, kr, tiles, total;
   int nb, nh, kr_bytes;
 };
-MlaFormedScratch mla_formed_scratch(const kvk_cache *c, int32_t layer) {
+MlaFormedScratch mla_formed_scratch(const kvk_cache *c, int32_t layer, int32_t n_q) {
   const int a = c->src[layer];
   const long long B = c->desc.max_batch, H = c->desc.n_q_heads, n_t = (c->lay[a].cap + 127) / 128;
   const long long unit = n_t * 131072;
-  const long long fit = std::max(1LL, (2LL << 30) / unit);
+  const long long rows = (long long)mla_prefill_scratch(c, layer, n_q).total;
+  const long long space = std::min(2LL << 30, std::max(256LL << 20, 128 * rows));
+  const long long fit = std::max(1LL, space / unit);
   MlaFormedScratch p;
   p.nh = (int)std::min(H, fit);
   p.nb = (int)std::max(1LL, std::min(B, fit / p.nh));
@@ -917,6 +879,56 @@ MlaFormedScratch mla_formed_scratch(const kvk_cache *c, int32_t layer) {
   p.tiles = p.kr + (size_t)p.nb * n_t * p.kr_bytes;
   p.total = p.tiles + (size_t)p.nb * p.nh * unit;
   return p;
+}
+// One head's tiles stay within 2 GiB.
+bool mla_may_form(const kvk_cache *c, int32_t layer) { return c->lay[c->src[layer]].cap <= (1 << 21); }
+
+// Whether n_q queries attend faster over formed keys and values than by the
+// absorbed decode per row, at the host's bound T on the lengths (the capacity
+// where nothing was appended through this handle).  Costs in ns, fitted to
+// calls replayed from graphs (1-8 sequences of 128-16384 positions, 16-1024
+// queries, 16 and 5 heads, every width, three formats; the pick lost 0.2 % to
+// the better path on average, and up to 1.08 times where it left the rows):
+//  rows:   per position, a wave of resident CTAs (one row each, two at d >=
+//          256 over bf16 latents and even n_q, of which half a wave runs at
+//          kHalf) takes kFull or kQuant, over the rows' mean length where
+//          there are several waves; absorption and merge kRow per row and 16
+//          heads, kEach per row.  One row per CTA at d >= 256: kOdd.
+//  formed: per group, the attention 16.5 (quantised 17.9) per position of the
+//          longest job, or of all jobs over the SMs, and the forming kForm
+//          per position of a wave of (128 positions, head) items; further
+//          groups 8 us each.
+// Formed only where it is 5 % faster; never for fewer than 16 queries (a
+// handful is not worth the tiles' memory).
+bool mla_formed_faster(const kvk_cache *c, int32_t layer, int32_t n_q) {
+  if (n_q < 16 || !mla_may_form(c, layer)) return false;
+  const int a = c->src[layer];
+  const kvk_layer_cfg &L = c->cfg[a];
+  const bool quant = L.bits != 16, sym = quant && layer_scheme(&L) == kSchemeSym;
+  const int w = L.width == 512 ? 0 : L.width == 256 ? 1 : L.width == 128 ? 2 : 3, f = !quant ? 0 : sym ? 2 : 1;
+  static const double kFix[2][4] = {{14.6e3, 10.1e3, 8.2e3, 7.1e3}, {9.1e3, 8.0e3, 7.4e3, 6.9e3}};
+  static const double kFull[4] = {29.2, 11.7, 10.6, 8.1}, kHalf[4] = {27.2, 11.8, 8.4, 7.0}, kOdd[2] = {19.2, 10.2};
+  static const double kQuant[2][4] = {{30.8, 14.7, 8.1, 7.6}, {28.6, 13.7, 8.3, 7.4}};
+  static const double kRow[2][4] = {{84.0, 41.0, 23.0, 17.0}, {82.0, 40.0, 21.0, 16.0}};
+  static const double kEach[2][4] = {{35.0, 28.0, 19.0, 17.0}, {38.0, 31.0, 32.0, 27.0}};
+  static const double kFixF[3][4] = {{17.3e3, 16.0e3, 15.0e3, 14.7e3}, {19.8e3, 17.9e3, 16.9e3, 16.6e3},
+                                     {17.8e3, 16.1e3, 15.3e3, 15.2e3}};
+  static const double kForm[3][4] = {{52.0, 42.0, 38.0, 36.0}, {64.0, 53.0, 49.0, 47.0}, {54.0, 45.0, 41.0, 38.0}};
+  const double B = c->desc.max_batch, H = c->desc.n_q_heads, sms = c->sm_count;
+  const double T = c->len_hi[a] > 0 ? (double)c->len_hi[a] : (double)c->desc.max_ctx;
+  const double mean = std::max(T - n_q / 2.0, T / 2.0);
+  const double rows = B * n_q;
+  const bool pairs = w < 2 && !quant && n_q % 2 == 0, one = quant || (w < 2 && !pairs);
+  const double waves = std::ceil(rows / (one ? sms : 2 * sms));
+  const double span = waves <= 1.0 ? T : std::max(T, waves * mean);
+  const double rate = quant ? kQuant[sym][w] : one ? kOdd[w] : rows <= sms ? kHalf[w] : kFull[w];
+  const double by_rows = kFix[quant][w] + rate * span + (kRow[quant][w] * H / 16.0 + kEach[quant][w]) * rows;
+  const MlaFormedScratch fs = mla_formed_scratch(c, layer, n_q);
+  const double groups = std::ceil(B / fs.nb) * std::ceil(H / fs.nh), units = (double)fs.nb * fs.nh;
+  const double att = std::max(T, units * ((n_q + 127) / 128) * mean / sms);
+  const double form = std::ceil(units * std::ceil(T / 128.0) / sms) * 128.0;
+  const double formed = kFixF[f][w] + groups * ((quant ? 17.9 : 16.5) * att + kForm[f][w] * form) + (groups - 1) * 8e3;
+  return formed < 0.95 * by_rows;
 }
 kvk_status check_prefill_mla(const kvk_cache *c, int32_t layer, int32_t n_q) {
   kvk_status s = check_layer_index(c, layer);
@@ -934,16 +946,31 @@ kvk_status kvk_prefill_scratch_size(const kvk_cache *c, int32_t layer, int32_t n
     if (s) return s;
     if (!bytes) return fail(KVK_ERR_INVALID_ARG, "null output");
     // never less for more queries: a buffer sized for the longest chunk
-    // serves every shorter one
-    const int from = c->formed_from[c->src[layer]];
+    // serves every shorter one.  On a grid of chunk lengths: `first` formed,
+    // and all formed from `from` on.
+    static const int grid[] = {16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, INT32_MAX};
+    int first = INT32_MAX, from = mla_may_form(c, layer) ? grid[0] : INT32_MAX;
+    for (int i = 0; from < INT32_MAX && i < 13; ++i) {
+      if (!mla_formed_faster(c, layer, grid[i])) from = grid[i + 1];
+      else first = std::min(first, grid[i]);
+    }
     *bytes = mla_prefill_scratch(c, layer, std::min(n_q, from)).total;
-    if (n_q >= from) *bytes = std::max(*bytes, mla_formed_scratch(c, layer).total);
+    if (n_q >= std::min(first, from)) *bytes = std::max(*bytes, mla_formed_scratch(c, layer, n_q).total);
     return KVK_OK;
   }
   kvk_status s = check_prefill(c, layer, n_q);
   if (s) return s;
   if (!bytes) return fail(KVK_ERR_INVALID_ARG, "null output");
   *bytes = prefill_scratch(c, layer, n_q).total;
+  return KVK_OK;
+}
+
+kvk_status kvk_prefill_scratch_least(const kvk_cache *c, int32_t layer, int32_t n_q, size_t *bytes) {
+  if (!c || c->desc.kind != KVK_KIND_MLA) return kvk_prefill_scratch_size(c, layer, n_q, bytes);
+  kvk_status s = check_prefill_mla(c, layer, n_q);
+  if (s) return s;
+  if (!bytes) return fail(KVK_ERR_INVALID_ARG, "null output");
+  *bytes = mla_prefill_scratch(c, layer, n_q).total;
   return KVK_OK;
 }
 
@@ -1217,13 +1244,13 @@ kvk_status kvk_prefill_attention_mla(kvk_cache *c, int32_t layer, const void *q_
   if (!std::isfinite(softmax_scale) || !(softmax_scale > 0.f))
     return fail(KVK_ERR_INVALID_ARG, "softmax scale must be finite and positive");
   const MlaPrefillScratch ps = mla_prefill_scratch(c, layer, n_q);
-  const MlaFormedScratch fs = mla_formed_scratch(c, layer);
-  const bool formed = n_q >= c->formed_from[c->src[layer]] && scratch_bytes >= fs.total;
-  if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 255u) || (!formed && scratch_bytes < ps.total)) {
-    size_t need = 0;
-    kvk_prefill_scratch_size(c, layer, n_q, &need);
-    return fail(KVK_ERR_INVALID_ARG, "scratch null, not 256-byte aligned or smaller than %zu bytes", need);
-  }
+  const MlaFormedScratch fs = mla_formed_scratch(c, layer, n_q);
+  const bool fits_rows = scratch_bytes >= ps.total;
+  // a buffer that holds only the formed tiles serves by them
+  const bool formed = mla_may_form(c, layer) && scratch_bytes >= fs.total &&
+                      (!fits_rows || mla_formed_faster(c, layer, n_q));
+  if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 255u) || (!formed && !fits_rows))
+    return fail(KVK_ERR_INVALID_ARG, "scratch null, not 256-byte aligned or smaller than %zu bytes", ps.total);
   const int a = c->src[layer];
   if (formed) {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

@@ -279,3 +279,79 @@ def test_mla_prefill_formed_is_no_less_exact(fmt):
     err = [np.linalg.norm(f32(x).astype(np.float64) - ref) / np.linalg.norm(ref) for x in (formed, rows)]
     assert err[0] <= err[1], err
     assert c.device_error() == 0
+
+
+def _rows_bytes(B, n_q, width, H=H):
+    return -(-B * n_q * H * (2 * width + 64) * 2 // 256) * 256 + B * n_q * H * (width + 2) * 4
+
+
+@pytest.mark.parametrize("width,fmt", [(512, ("grouped", 8)), (128, ("symmetric", 4)), (512, None)],
+                         ids=["g8-d512", "sym4-d128", "bf16-d512"])
+def test_mla_prefill_chooses_by_the_lengths(width, fmt):
+    """A short context in a large cache goes by rows, in the rows' memory, and
+    no buffer is kept; the same cache grown takes the formed path where it is
+    faster.  Every buffer that the size call named at one length serves at
+    the others."""
+    from paper_2609_37988_gb300.cache import Cache, Layer
+    layer = dict(bits=16, width=width) if fmt is None else dict(bits=fmt[1], scheme=fmt[0], width=width)
+    cap, n_q, first, grown = 32768, 64, 128, 8192
+    c = Cache(kind="mla", n_layers=1, n_q_heads=H, head_dim=128, latent_dim=512, rope_dim=64, max_batch=1,
+              max_ctx=cap, layers=[Layer(**layer)])
+    g = torch.Generator().manual_seed(2)
+    wk, wv = ((torch.randn((H, 128, 512), generator=g) / math.sqrt(512)).to(torch.bfloat16).cuda() for _ in range(2))
+    qn = torch.randn((1, 512, H, 128), generator=g).to(torch.bfloat16).cuda()
+    qp = torch.randn((1, 512, H, 64), generator=g).to(torch.bfloat16).cuda()
+    c.append(0, torch.randn((1, first, 512), generator=g).to(torch.bfloat16).cuda(),
+             torch.randn((1, first, 64), generator=g).to(torch.bfloat16).cuda())
+    least = ctypes.c_size_t()
+    assert c.lib.kvk_prefill_scratch_least(c.handle, 0, n_q, ctypes.byref(least)) == 0
+    assert least.value == _rows_bytes(1, n_q, width) == _scratch(c, n_q)
+    sizes = {_scratch(c, n) for n in (n_q, 512)}
+    short = c.prefill_mla(0, qn[:, :n_q].contiguous(), qp[:, :n_q].contiguous(), wk, wv, 0.07)
+    assert c._prefill_scratch is None
+    c.append(0, torch.randn((1, grown - first, 512), generator=g).to(torch.bfloat16).cuda(),
+             torch.randn((1, grown - first, 64), generator=g).to(torch.bfloat16).cuda())
+    sizes |= {_scratch(c, n) for n in (n_q, 512)}
+    assert max(sizes) >= 256 << 20
+    ref = c.prefill_mla(0, qn, qp, wk, wv, 0.07)
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    for nbytes in sizes:
+        buf = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        out = torch.full_like(ref, math.nan)
+        st = c.lib.kvk_prefill_attention_mla(c.handle, 0, p(qn), p(qp), p(wk), p(wv), 512, 0.07, p(out), p(buf),
+                                             nbytes, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert st == (0 if nbytes >= min(_rows_bytes(1, 512, width), _scratch(c, 512)) else 1)
+        if st == 0:
+            assert_close(f32(out), f32(ref), max_abs=2e-4, rel_l2=1e-4, what=f"{nbytes} bytes")
+    c.rewind(grown - first)
+    again = c.prefill_mla(0, qn[:, :n_q].contiguous(), qp[:, :n_q].contiguous(), wk, wv, 0.07)
+    assert torch.equal(again, short)
+    assert c.device_error() == 0
+
+
+def test_mla_prefill_falls_back_to_the_rows_memory(monkeypatch):
+    """Where the device has no room for the formed tiles, the call runs by
+    rows in the memory that they take."""
+    c, wk, wv, _, _ = _setup(512, None, [900, 800], 8192, seed=9)
+    n_q = 256
+    g = torch.Generator().manual_seed(4)
+    qn = torch.randn((2, n_q, H, 128), generator=g).to(torch.bfloat16).cuda()
+    qp = torch.randn((2, n_q, H, 64), generator=g).to(torch.bfloat16).cuda()
+    wk, wv = wk.cuda(), wv.cuda()
+    formed = c.prefill_mla(0, qn, qp, wk, wv, 0.07)
+    room, empty, asked = _rows_bytes(2, n_q, 512), torch.empty, []
+
+    def scarce(*size, **kw):
+        if kw.get("dtype") is torch.uint8:
+            asked.append(size[0])
+            if size[0] > room:
+                raise torch.cuda.OutOfMemoryError("no room")
+        return empty(*size, **kw)
+
+    monkeypatch.setattr(torch, "empty", scarce)
+    rows = c.prefill_mla(0, qn, qp, wk, wv, 0.07)
+    monkeypatch.undo()
+    assert asked == [_scratch(c, n_q), room]
+    assert not torch.equal(rows, formed)
+    assert_close(f32(rows), f32(formed), max_abs=2e-4, rel_l2=1e-4, what="rows = formed")
+    assert c.device_error() == 0
