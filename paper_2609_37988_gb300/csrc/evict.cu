@@ -326,12 +326,12 @@ __device__ __forceinline__ int cluster_ld(const int *p, uint32_t rank) {
 // order as the values), then the chosen positions in increasing order and
 // the window.  PARTS = 8: a cluster of 8 CTAs per unit, each over an eighth
 // of the positions: a unit's votes are read five times, which one CTA per
-// unit did in 110 us for 32 units of 131072 positions with 120 SMs idle (64
-// us so).  Per pass the CTAs add each other's histograms through distributed
+// unit did in 99 us for 32 units of 131072 positions with 120 SMs idle (65 us
+// so).  Per pass the CTAs add each other's histograms through distributed
 // shared memory and decide alike (one cluster barrier per pass: two
-// histograms in turn).  Up to 16384 positions one CTA (PARTS = 1) is faster:
-// the barriers cost more than its few rounds (8153 positions: 27 us, 43).
-constexpr int kSelParts = 8, kSelOneCta = 16384;
+// histograms in turn).  The barriers cost more than a few rounds of one CTA:
+// select_one_cta.
+constexpr int kSelParts = 8;
 template <int PARTS>
 __global__ void __cluster_dims__(PARTS, 1, 1) __launch_bounds__(1024) evict_select_kernel(const EvictArgs a) {
   pdl_wait();
@@ -482,8 +482,30 @@ __global__ void __cluster_dims__(PARTS, 1, 1) __launch_bounds__(1024) evict_sele
 }
 
 
+// Whether one CTA per unit selects faster than a cluster of 8, by the host's
+// bound on the lengths (a longer sequence in a recorded launch only takes
+// longer).  Measured (us, one CTA / cluster): 8 units of 4096 positions 10.0 /
+// 14.7, 16384 15.9 / 15.1, 65536 50 / 16; 32 units of 4096 10.3 / 41.9, 32768
+// 27.2 / 42.7, 65536 51 / 45, 131072 101 / 65; 64 units of 65536 51 / 75: 5.6
+// us per round of 8192 positions and CTA, and 14 per wave of clusters.
+bool select_one_cta(const EvictArgs &a, int sms) {
+  auto rounds = [](int64_t n) { return (double)((n + 8191) / 8192); };
+  const double waves = (double)((a.v.B * a.v.Hkv * kSelParts + sms - 1) / sms);
+  const double one = 4.4 + 5.6 * rounds(a.len_hi);
+  const double cluster = (waves > 1.0 ? 14.0 : 1.0) + waves * (4.0 + 10.0 * rounds(a.len_hi / kSelParts));
+  return one <= cluster;
+}
+
 cudaError_t launch_evict_select(const EvictArgs &a, cudaStream_t st) {
-  if (a.v.cap <= kSelOneCta) return launch_pdl(evict_select_kernel<1>, dim3(a.v.Hkv, a.v.B), dim3(1024), 0, st, a);
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0, n = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    sms = n;
+  }
+  if (select_one_cta(a, sms)) return launch_pdl(evict_select_kernel<1>, dim3(a.v.Hkv, a.v.B), dim3(1024), 0, st, a);
   return launch_pdl(evict_select_kernel<kSelParts>, dim3(a.v.Hkv * kSelParts, a.v.B), dim3(1024), 0, st, a);
 }
 

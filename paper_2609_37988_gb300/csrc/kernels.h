@@ -127,6 +127,7 @@ struct EvictArgs {
   int Hq, G, n_win, budget;
   float sig_log2;      // softmax scale * log2(e)
   int n_tiles;         // 128-position tiles launched per (sequence, kv head)
+  int64_t len_hi;      // host-side bound on the lengths (a recorded launch may meet longer ones)
   int sc_stride;       // n_tiles * kEvictTile: row stride of the scores
   int stat_sub;        // statistics entries per tile and row (1 or kEvictStatSub)
   int items_per_cta = 0;  // > 0: those entries per CTA run over a unit's tiles instead

@@ -787,6 +787,7 @@ kvk_status kvk_evict_window(kvk_cache *c, int32_t layer, const void *q_win, int3
   a.budget = budget;
   a.sig_log2 = softmax_scale * 1.4426950408889634f;
   a.n_tiles = es.n_tiles;
+  a.len_hi = c->len_hi[layer] > 0 ? c->len_hi[layer] : c->lay[layer].cap;
   a.sc_stride = es.n_tiles * kEvictTile;
   a.stat_sub = evict_uses_tc(c->desc.head_dim, n_win * a.G) ? kEvictStatSub : 1;
   a.votes = static_cast<float *>(scratch);

@@ -210,6 +210,40 @@ def test_evict_equal_votes_keep_smaller_positions():
     np.testing.assert_array_equal(idx[1, 0, :100], np.r_[np.arange(92), np.arange(122, 130)])
 
 
+@pytest.mark.parametrize("cap,lens", [(20000, [20000, 13001, 130, 0]), (40000, [700, 9000, 41, 8193])],
+                         ids=["cluster", "one-cta-in-a-large-cache"])
+def test_evict_ties_across_the_selecting_ctas(cap, lens):
+    """Keys of three values, so that the cut falls among thousands of equal
+    votes spread over all CTAs of a unit's cluster (lengths past 8192) or over
+    the rounds of the one that selects in shorter contexts of the same large
+    cache: the smaller positions stay, whatever CTA counted them; sequences
+    that keep everything or have no positions beside them."""
+    B, Hkv, G, D, n_win, budget = len(lens), 2, 2, 64, 8, 4000
+    c = _cache(B, G * Hkv, Hkv, D, cap, [dict(bits=8, group=64, key_axis="token", evict_capacity=budget)])
+    g = torch.Generator().manual_seed(7)
+    kind = torch.randint(0, 40, (B, max(lens), Hkv), generator=g).clamp(max=2)  # 0: high, 1: middle, 2: low
+    kind = torch.where(kind == 2, torch.randint(1, 3, kind.shape, generator=g), kind)
+    k = (0.5 - 0.25 * kind.float())[..., None].expand(-1, -1, -1, D).to(torch.bfloat16).contiguous()
+    v = torch.randn((B, max(lens), Hkv, D), generator=g).to(torch.bfloat16)
+    c.append(0, k.cuda(), v.cuda(), n_per_seq=torch.tensor(lens, dtype=torch.int32, device="cuda"))
+    q = torch.full((B, n_win, G * Hkv, D), 0.5, dtype=torch.bfloat16, device="cuda")
+    c.evict_window(0, q, 0.125, budget)
+    idx, n, _ = c.kept_lists(0)
+    idx, n = idx.cpu().numpy(), n.cpu().numpy()
+    for b, L in enumerate(lens):
+        for j in range(Hkv):
+            if L <= budget:
+                want = np.arange(L)
+            else:
+                P, room = L - n_win, budget - n_win
+                cls = kind[b, :P, j].numpy()
+                order = np.lexsort((np.arange(P), cls))[:room]  # by value, then by position
+                want = np.r_[np.sort(order), np.arange(P, L)]
+            assert n[b, j] == len(want)
+            np.testing.assert_array_equal(idx[b, j, :len(want)], want)
+    assert c.device_error() == 0
+
+
 def test_evict_window_only_and_planted_key():
     # budget == n_win keeps only the window; with one more slot the planted
     # key every window query attends to is the one kept
