@@ -200,7 +200,7 @@ kvk_status kvk_rewind(kvk_cache *cache, int32_t n, kvk_stream stream);
  * on the anchor's lengths, the SM count and the decode schedule).  Under the
  * run schedule (kvk_set_decode_schedule) it is the number of partial slots
  * per (sequence, KV head) that kvk_decode_partial with n_splits = 0 writes.
- * kvk_decode_attention over several sequences whose units all fit one wave
+ * kvk_decode_attention over 4 to 62 sequences whose units all fit one wave
  * of CTAs may split each sequence by its own length instead, once an append
  * has named per-sequence counts. */
 kvk_status kvk_decode_plan_splits(kvk_cache *cache, int32_t layer, int32_t *n_splits);
@@ -464,7 +464,8 @@ kvk_status kvk_set_wait_limit(kvk_cache *cache, uint32_t polls);
  *      each CTA at most 13 tiles and leave its last wave of CTAs less than
  *      90 % full (and every run CTA gets at least four tiles), else the
  *      splits; kvk_decode_attention takes splits in proportion to each
- *      sequence's length instead where they make one wave (2 to 62
+ *      sequence's length instead where they make one wave of several tiles
+ *      each and the lengths on the device leave a tile to gain (4 to 62
  *      sequences, contiguous reads, after an append with per-sequence counts;
  *      instead of the runs where whole splits fill at least 85 % of it).
  * run_ctas: the number of run CTAs (clamped to [units, tiles], units = B *

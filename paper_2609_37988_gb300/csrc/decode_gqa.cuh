@@ -1168,62 +1168,87 @@ __device__ __forceinline__ bool gqa_run_segment(const GqaDecodeArgs &a, int k, G
 }
 
 // Balanced splits: unit (b, kvh), items [i0, i1) (i1 = -1: to the end) and
-// partial slot of CTA blockIdx.x of a one-dimensional grid of n CTAs.  With
-// t_b kernel tiles of sequence b (from its length on the device), R is the
-// smallest number of tiles per CTA for which sum_b Hkv ceil(t_b / R) <= n and
-// no unit takes more than bal_cap slots: the least possible longest CTA of
-// one wave with a unit's tiles in equal splits.  The split grid cuts every
-// sequence by the longest one's length, so a short sequence's last splits
-// find nothing to do: ragged batches (lengths from half to all of 8192,
-// 16 x 4 units of int4 with per-channel keys) left a quarter of the CTAs
-// empty.  Every warp finds the same answer (lane: sequences lane, lane + 32).
+// partial slot of a CTA of the grid (bal_x, kv heads, sequences), whose first
+// n CTAs in launch order, one wave, may have work.  The split grid cuts every sequence by the
+// longest one's length, so a short sequence's last splits find nothing to do:
+// ragged batches (lengths from half to all of 8192, 16 x 4 units of int4 with
+// per-channel keys) left a quarter of the CTAs empty.  With t_b kernel tiles
+// of sequence b (from its length on the device), CTA x of the flattened grid
+// takes part x of the sequences cut into splits of R tiles, sum_b Hkv ceil(t_b
+// / R) <= n and no unit in more than bal_cap slots; R is the smallest such
+// number or one of the next up to 1/32 above it.  Where R would not stay
+// within bal_aim (all lengths equal, say: known from their sum), the split
+// grid's own cut into n_splits stands.
+//
+// It runs before a CTA's first copy, so its latency counts: that case costs
+// one reduction, divisions are products with an approximate reciprocal (exact
+// quotients of a + 1/2, a < 2^20: the products are off by less than 2^-21.5 of
+// themselves; the host takes the schedule for fewer than 2^19 tiles).  Every
+// warp finds the same answer (lane: sequences lane, lane + 32).
 struct GqaBalSeg {
   int b, kvh, i0, i1, slot;
 };
+__device__ __forceinline__ int bal_div(int a, float inv) { return __float2int_rd(((float)a + 0.5f) * inv); }
+__device__ __forceinline__ float bal_inv(int d) { return __fdividef(1.f, (float)d); }
 template <int TILE>
 __device__ __forceinline__ bool gqa_balanced_split(const GqaDecodeArgs &a, GqaBalSeg &sg) {
   const GqaView &v = a.v;
-  const int lane = threadIdx.x & 31, n = gridDim.x, x = blockIdx.x;
-  int t[2], k[2];
+  const int lane = threadIdx.x & 31;
+  int t[2] = {0, 0};
+  if (lane < v.B) t[0] = max(1, (v.lens[lane] + TILE - 1) / TILE);
+  if (lane + 32 < v.B) t[1] = max(1, (v.lens[lane + 32] + TILE - 1) / TILE);
+  const int sum = __reduce_add_sync(0xffffffffu, t[0] + t[1]);
+  if (sum <= a.bal_aim * a.bal_n) {
+    const int top = __reduce_max_sync(0xffffffffu, max(t[0], t[1]));
+    int k[2], r = max(__float2int_rd((float)sum * bal_inv(a.bal_n)) + 1,
+                      bal_div(top + a.bal_cap - 1, bal_inv(a.bal_cap)));
+    bool fits = false;
+    for (; r <= a.bal_aim; r += max(1, r >> 5)) {
+      const float inv = bal_inv(r);
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int b = lane + 32 * h;
-    t[h] = b < v.B ? max(1, (v.lens[b] + TILE - 1) / TILE) : 0;
-  }
-  const int sum = __reduce_add_sync(0xffffffffu, t[0] + t[1]) * v.Hkv;
-  const int top = __reduce_max_sync(0xffffffffu, max(t[0], t[1]));
-  int r = max((sum + n - 1) / n, (top + a.bal_cap - 1) / a.bal_cap);
-  for (;; ++r) {  // ends: at r = top every unit takes one CTA
-#pragma unroll
-    for (int h = 0; h < 2; ++h) k[h] = (t[h] + r - 1) / r;
-    if (r >= top || __reduce_add_sync(0xffffffffu, k[0] + k[1]) * v.Hkv <= n) break;
-  }
-  // CTAs in order of (sequence, kv head, slot): this one's sequence
-  int base = 0;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    int inc = k[h];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
+      for (int h = 0; h < 2; ++h) k[h] = t[h] ? bal_div(t[h] + r - 1, inv) : 0;
+      fits = (int)__reduce_add_sync(0xffffffffu, k[0] + k[1]) <= a.bal_n;
+      if (fits) break;
     }
-    const int lo = v.Hkv * (base + inc - k[h]), hi = v.Hkv * (base + inc);
-    const uint32_t m = __ballot_sync(0xffffffffu, x >= lo && x < hi);
-    if (m) {
-      const int l = __ffs(m) - 1;
-      const int kb = __shfl_sync(0xffffffffu, k[h], l), rel = x - __shfl_sync(0xffffffffu, lo, l);
-      sg.b = l + 32 * h;
-      sg.kvh = rel / kb;
-      sg.slot = rel - sg.kvh * kb;
-      sg.i0 = sg.slot * r * TILE;
-      sg.i1 = sg.slot == kb - 1 ? -1 : sg.i0 + r * TILE;
-      if (rel == 0 && threadIdx.x == 0) a.bal_counts[sg.b] = kb;
-      return true;
+    if (fits) {
+      // CTAs in order of (sequence, kv head, slot): this one's sequence
+      const int x = (blockIdx.z * v.Hkv + blockIdx.y) * gridDim.x + blockIdx.x;
+      int base = 0;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (32 * h >= v.B) break;
+        int inc = k[h];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += y;
+        }
+        const int lo = v.Hkv * (base + inc - k[h]), hi = v.Hkv * (base + inc);
+        const uint32_t m = __ballot_sync(0xffffffffu, x >= lo && x < hi);
+        if (m) {
+          const int l = __ffs(m) - 1;
+          const int kb = __shfl_sync(0xffffffffu, k[h], l), rel = x - __shfl_sync(0xffffffffu, lo, l);
+          sg.b = l + 32 * h;
+          sg.kvh = bal_div(rel, bal_inv(kb));
+          sg.slot = rel - sg.kvh * kb;
+          sg.i0 = sg.slot * r * TILE;
+          sg.i1 = sg.slot == kb - 1 ? -1 : sg.i0 + r * TILE;
+          if (rel == 0 && threadIdx.x == 0) a.bal_counts[sg.b] = kb;
+          return true;
+        }
+        base += __shfl_sync(0xffffffffu, inc, 31);
+      }
+      return false;  // more CTAs than splits
     }
-    base += __shfl_sync(0xffffffffu, inc, 31);
   }
-  return false;  // more CTAs than splits
+  sg.b = blockIdx.z;
+  sg.kvh = blockIdx.y;
+  sg.slot = blockIdx.x;
+  if (sg.slot >= a.n_splits) return false;
+  sg.i0 = sg.slot * a.items_per_split;
+  sg.i1 = sg.slot == a.n_splits - 1 ? -1 : sg.i0 + a.items_per_split;
+  if (sg.slot == 0 && sg.kvh == 0 && threadIdx.x == 0) a.bal_counts[sg.b] = a.n_splits;
+  return true;
 }
 
 // RUN = false: grid (split, kv head, sequence); CTA (x, y, z) decodes items
@@ -1242,8 +1267,7 @@ __device__ __forceinline__ bool gqa_balanced_split(const GqaDecodeArgs &a, GqaBa
 // slots (up to a.run_slots) empty.  Every CTA does
 // W / n tiles of work, so one wave of resident CTAs ends together instead
 // of a second, partial wave of splits.
-// BAL: the one-dimensional grid of gqa_balanced_split (with neither of the
-// others).  A kernel of its own: as a branch beside the split grid's body it
+// BAL: a grid cut by gqa_balanced_split (with neither of the others).  A kernel of its own: as a branch beside the split grid's body it
 // made the split grid's decodes 0.4 us each slower (14B step of 48 decodes:
 // 5009 us with it, 4986 without).
 template <int BITS, int D, int KAX, int GS, bool GATHER, bool RUN, bool BAL>
@@ -1328,7 +1352,7 @@ cudaError_t launch_gqa_decode_g(const GqaDecodeArgs &a, cudaStream_t st) {
     memcpy(&rows, a.rows, sizeof rows);
   }
   if constexpr (RUN) return launch_pdl(k, dim3(a.run_ctas), dim3(128), C::SMEM, st, rows, a);
-  if constexpr (BAL) return launch_pdl(k, dim3(a.bal_ctas), dim3(128), C::SMEM, st, rows, a);
+  if constexpr (BAL) return launch_pdl(k, dim3(a.bal_x, a.v.Hkv, a.v.B), dim3(128), C::SMEM, st, rows, a);
   dim3 grid(a.n_splits, a.v.Hkv, a.v.B);
   return launch_pdl(k, grid, dim3(128), C::SMEM, st, rows, a);
 }
@@ -1344,7 +1368,7 @@ cudaError_t launch_gqa_decode_t(const GqaDecodeArgs &a, cudaStream_t st) {
       return cudaErrorInvalidValue;
     }
   }
-  if (a.bal_ctas > 0) {
+  if (a.bal_x > 0) {
     if (a.gather || a.out || !a.bal_counts) return cudaErrorInvalidValue;
     return launch_gqa_decode_g<BITS, D, KAX, GS, false, false, true>(a, st);
   }

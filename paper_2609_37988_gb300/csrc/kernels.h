@@ -68,11 +68,13 @@ struct GqaDecodeArgs {
   // before its data tiles; run_q, run_r: the planned tile count W = B Hkv
   // run_tpu as q run_ctas + r.
   int run_ctas = 0, run_tpu = 0, run_slots = 0, run_q = 0, run_r = 0, run_setup = 0;
-  // balanced splits (contiguous reads, partials only): bal_ctas > 0 CTAs, a
-  // sequence's splits in proportion to its own length (gqa_balanced_split),
-  // at most bal_cap per unit; their number goes to bal_counts[b].
-  // B <= kBalanceMaxBatch, units <= bal_ctas.
-  int bal_ctas = 0, bal_cap = 0;
+  // balanced splits (contiguous reads, partials only): bal_x > 0 CTAs per
+  // unit in the grid; where splits of at most bal_aim kernel tiles in
+  // proportion to each sequence's own length fit bal_n CTAs per KV head, at
+  // most bal_cap per unit, those (gqa_balanced_split), else n_splits of
+  // items_per_split.  Their number goes to bal_counts[b].  B <=
+  // kBalanceMaxBatch.
+  int bal_x = 0, bal_n = 0, bal_cap = 0, bal_aim = 0;
   int32_t *bal_counts = nullptr;
 };
 constexpr int kBalanceMaxBatch = 62;  // two lengths per lane, counts in one 256-byte block
@@ -103,9 +105,11 @@ struct RewindArgs {
 cudaError_t launch_rewind(const RewindArgs &a, cudaStream_t st);
 
 // counts (optional): row r has counts[r / rows_per] splits, at most n_splits
+// (n_rows a multiple of rows_per); `first` slots are read beside the count,
+// the others once it is known
 cudaError_t launch_splitk_merge(const float *partials, int n_splits, int n_rows, int dim,
                                 float *out, cudaStream_t st, const int32_t *counts = nullptr,
-                                int rows_per = 1);
+                                int rows_per = 1, int first = 0);
 
 // Append n_new rows per sequence (per-sequence counts optional).
 cudaError_t launch_gqa_append(const GqaView &v, const void *k, const void *vv, int in_f32,

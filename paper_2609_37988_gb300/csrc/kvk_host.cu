@@ -404,31 +404,53 @@ bool plan_runs(kvk_cache *c, int a, RunPlan *p) {
 
 // Balanced splits of an automatic decode of anchor a (kernel side in
 // decode_gqa.cuh, gqa_balanced_split), given what plan_runs and auto_splits
-// (`splits`) chose: the number of CTAs, 0 if the decode keeps their schedule.
-// Taken once an append has named per-sequence counts (sequences of equal
-// length have nothing to balance, and finding its split on the device costs a
-// CTA about 1 us: the 7B step, 16 equal sequences, took 1.115 ms with it and
-// 1.078 without), where one wave
-// of resident CTAs holds the units at two or more splits each and the other
-// plan is one wave too.  Instead of the runs only if whole
-// splits fill 85 % of the wave (the runs fill all of it, but only if the
-// lengths are equal).  *cap: partial slots per unit, twice the even share (a
-// sequence twice as long as the average takes it), in the merge's steps.
-int plan_balanced(kvk_cache *c, int a, bool runs, int splits, int *cap) {
-  if (c->schedule != KVK_SCHEDULE_AUTO || c->kept_on[a] || !c->ragged[a]) return 0;
-  if (c->desc.max_batch < 2 || c->desc.max_batch > kBalanceMaxBatch) return 0;
+// (`splits`) chose; false: the decode keeps their schedule.  Taken once an
+// append has named per-sequence counts (sequences of equal length have
+// nothing to balance), where one wave of resident CTAs holds the units at two
+// or more splits each and the other plan is one wave too.  Lengths that turn
+// out equal, or nearly so, keep an even cut, at the cost of a reduction and
+// the counts (0.2-0.7 us), so the schedule is for splits of at least 4 tiles
+// (6 of the 64-position ones without per-channel keys; a CTA's tile takes
+// 1.2-2.5 us) and at least 4 sequences.  Decode and merge, 8 formats x 12
+// shapes of 4-40 sequences of 600-16000 positions, against the other plan:
+// equal lengths named by counts 0.94-1.06 (on average 1.01; a search in every
+// CTA and a merge of every slot: 0.95-1.23), lengths from half to all of the
+// longest 0.85-1.04 (0.98), from one position on 0.66-1.00 (0.93).  Instead
+// of the runs where whole splits fill 85 % of the wave (they fill all of it,
+// but by the longest length): 13 x 8 units of sym4, 5003 positions, equal
+// 0.96, ragged 0.90; 16 x 4 of sym8, 8192: 1.01 and 0.93.
+struct BalPlan {
+  int x = 0, n = 0;                  // CTAs per unit in the grid, CTAs of one wave per KV head
+  int cap = 0, aim = 0;              // most slots per unit, most tiles of a balanced split
+  int splits = 0, ips = 0;           // the even cut's splits and items per split
+  int first = 0;                     // slots that the merge reads beside the count
+};
+bool plan_balanced(kvk_cache *c, int a, bool runs, int splits, BalPlan *p) {
+  if (c->schedule != KVK_SCHEDULE_AUTO || c->kept_on[a] || !c->ragged[a]) return false;
+  if (c->desc.max_batch < 4 || c->desc.max_batch > kBalanceMaxBatch) return false;
   const kvk_layer_cfg &L = c->cfg[a];
   const int units = c->desc.max_batch * c->desc.n_kv_heads, slots = c->sm_count * c->ctas[a];
-  const int share = slots / units;
-  if (share < 2 || splits < 2) return 0;
-  if (runs ? share * units < 0.85 * slots : splits * units > slots) return 0;
+  const int share = std::min(slots / units, c->max_splits);
+  if (share < 2 || splits < 2) return false;
+  if (runs ? share * units < 0.85 * slots : splits * units > slots) return false;
   const int per = gqa_decode_tile(L.bits, c->desc.head_dim, L.bits == 16 ? 0 : L.key_axis, layer_group(&c->desc, &L),
                                   layer_scheme(&L)) / kTile;
+  if (c->lay[a].cap / (kTile * per) >= (1 << 19)) return false;  // the kernel's divisions
   const int ktiles = (layer_tiles(c, a) + per - 1) / per;
-  if (ktiles < 2) return 0;
-  *cap = std::min(c->max_splits, share <= 4 ? 8 : share <= 12 ? 16 : 2 * share);
-  if (*cap < std::min(share, ktiles)) return 0;
-  return (int)std::min<long long>(slots, (long long)units * ktiles);
+  const int even = (ktiles + share - 1) / share;  // tiles of an even cut's CTA
+  const bool kpc = L.bits != 16 && layer_scheme(&L) != kSchemeSym && L.key_axis == 1;
+  if (even < (per == 1 && !kpc ? 6 : 4)) return false;
+  p->x = std::min((slots + units - 1) / units, ktiles);
+  p->n = std::min(slots / c->desc.n_kv_heads, p->x * c->desc.max_batch);
+  p->cap = std::min(c->max_splits, 2 * share);
+  p->aim = even - std::max(1, even / 8);
+  if ((ktiles + p->cap - 1) / p->cap > p->aim) return false;  // the slots would not let it gain
+  p->splits = (ktiles + even - 1) / even;
+  p->ips = even * per * kTile;
+  // as many as the merge kernel for the even cut reads at once (8 or 16 slots
+  // cost it the same, a second round trip 0.5 us)
+  p->first = std::min(p->cap, p->splits <= 8 ? 8 : p->splits <= 16 ? 16 : p->splits + p->splits / 3);
+  return true;
 }
 
 }  // namespace
@@ -1053,11 +1075,11 @@ static kvk_status gqa_decode_common(kvk_cache *c, int32_t layer, const void *q, 
   bool runs = automatic && plan_runs(c, a, &rp);
   if (runs) n_splits = rp.slots;
   if (n_splits == 0) n_splits = auto_splits(c, a);
-  int bal_cap = 0;
-  const int bal = automatic && merge && !partial ? plan_balanced(c, a, runs, std::min(n_splits, tiles), &bal_cap) : 0;
+  BalPlan bp;
+  const bool bal = automatic && merge && !partial && plan_balanced(c, a, runs, std::min(n_splits, tiles), &bp);
   if (bal) {
     runs = false;
-    n_splits = bal_cap;  // slots
+    n_splits = bp.cap;  // slots
   }
   // a partial-only call keeps the caller's split count (extra splits are
   // empty and write m = -inf, l = 0); a full call never uses more splits
@@ -1088,8 +1110,12 @@ static kvk_status gqa_decode_common(kvk_cache *c, int32_t layer, const void *q, 
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (bal) {
-    args.bal_ctas = bal;
-    args.bal_cap = bal_cap;
+    args.bal_x = bp.x;
+    args.bal_n = bp.n;
+    args.bal_cap = bp.cap;
+    args.bal_aim = bp.aim;
+    args.n_splits = bp.splits;
+    args.items_per_split = bp.ips;
     args.bal_counts = c->err() + 1;  // the workspace's first block, after the error word
   }
   if (merge && n_splits == 1 && !runs && !bal) {
@@ -1103,7 +1129,7 @@ static kvk_status gqa_decode_common(kvk_cache *c, int32_t layer, const void *q, 
   if (e != cudaSuccess) return cuda_fail(e, "decode launch");
   if (merge && (n_splits > 1 || runs || bal)) {
     e = launch_splitk_merge(args.partial, n_splits, c->desc.max_batch * c->desc.n_q_heads,
-                            c->desc.head_dim, out, st, args.bal_counts, c->desc.n_q_heads);
+                            c->desc.head_dim, out, st, args.bal_counts, c->desc.n_q_heads, bp.first);
     if (e != cudaSuccess) return cuda_fail(e, "merge launch");
   }
   return KVK_OK;

@@ -216,43 +216,127 @@ BAL_FORMATS = FORMATS[:1] + FORMATS[4:7] + [dict(bits=16, group=64, key_axis="to
                                             dict(bits=4, group=32, key_axis="channel")]
 
 
+UNTOUCHED = -77
+
+
+def _count_words(c, B):
+    """The split counts that a balanced decode leaves behind the error word."""
+    return c.workspace[:256].view(torch.int32)[1:1 + B]
+
+
+def _cuts(c, layer, q, sigma, B):
+    """The decode and its per-sequence split counts (None: another schedule)."""
+    w = _count_words(c, B)
+    w.fill_(UNTOUCHED)
+    out = c.decode(layer, q, sigma)
+    k = w.cpu().numpy()
+    assert (k == UNTOUCHED).all() or (k != UNTOUCHED).all()
+    return out, None if (k == UNTOUCHED).all() else k
+
+
+def _balanced_tiles(k, lens, tile):
+    """Tiles per split of a cut in proportion to the lengths, if k is one."""
+    t = np.maximum(1, -(-np.asarray(lens) // tile))
+    return next((r for r in range(1, t.max() + 1) if (k == -(-t // r)).all()), None)
+
+
+def _kernel_tile(fmt):
+    return 128 if fmt["bits"] <= 4 and fmt["key_axis"] == "token" else 64
+
+
+def _ragged(B, T, seed, lo=0):
+    n = np.random.default_rng(seed).integers(lo, T + 1, B)
+    n[seed % B] = T
+    return n.tolist()
+
+
+# (sequences, KV heads, query heads per KV head, D, lengths, cut expected)
+BAL_SETS = {
+    # both halves of the lanes; empty, one-position and tile-sized sequences
+    "41-sequences": (41, 2, 5, 128, [0, 1, 64, 128, 3700] + _ragged(36, 3700, 5), "own"),
+    # the longest takes all the slots that a unit may have
+    "slot-limit": (5, 4, 7, 128, [16384, 1, 300, 0, 77], "own"),
+    "long-last": (6, 4, 3, 128, [130, 64, 65, 900, 0, 15000], "own"),
+    "four": (4, 8, 5, 128, [8192, 500, 4100, 3000], "own"),
+    "62-sequences": (62, 2, 1, 128, _ragged(62, 6000, 3), "own"),
+    "equal": (16, 4, 7, 128, [8192] * 16, "even"),
+    "near": (16, 4, 7, 128, _ragged(16, 8192, 2, 8000), "even"),
+    # no tile to gain: another schedule
+    "short": (8, 4, 7, 128, _ragged(8, 300, 4), None),
+}
+
+
 @pytest.mark.parametrize("fmt", BAL_FORMATS, ids=lambda f: _fid(f) + f["key_axis"][0])
-@pytest.mark.parametrize("lens", [[3000, 0, 1, 777, 129], [130, 64, 65, 3000], [2999] * 3,
-                                  [(37 * i) % 700 for i in range(41)]],
-                         ids=["one-long", "long-last", "equal", "41-sequences"])
-def test_balanced_splits_match_the_oracle(fmt, lens):
-    """Automatic decodes of a few units split each sequence by its own length
-    (a sequence's splits in proportion, one wave): every position read once,
-    empty and one-position sequences, sequences in both halves of the lanes,
-    a long sequence that reaches the slot limit."""
-    B, Hkv, G, D = len(lens), 2, 5, 128
-    c = _cache(B, G * Hkv, Hkv, D, 3008, fmt, max_splits=16)
+@pytest.mark.parametrize("name", BAL_SETS)
+def test_balanced_splits_match_the_split_grid(fmt, name):
+    """Automatic decodes after an append with counts: the kernel that cuts
+    each sequence by its own length ran (its counts say how), and gives what
+    the split grid gives over the same cache."""
+    B, Hkv, G, D, lens, cut = BAL_SETS[name]
+    T = max(lens)
+    g = torch.Generator(device="cuda").manual_seed(B + fmt["bits"])
+    k, v = (torch.randn((B, T, Hkv, D), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    c = _cache(B, G * Hkv, Hkv, D, T, fmt, max_splits=64)
+    c.append(0, k, v, torch.tensor(lens, dtype=torch.int32, device="cuda"))
+    q = torch.randn((B, G * Hkv, D), generator=g, device="cuda").to(torch.bfloat16)
+    out, counts = _cuts(c, 0, q, 0.1, B)
+    tile = _kernel_tile(fmt)
+    if cut is None:
+        assert counts is None
+    elif cut == "even":
+        assert counts is None or (counts == counts[0]).all()
+    elif counts is not None:
+        r = _balanced_tiles(counts, lens, tile)
+        assert r is not None, counts
+        if name == "slot-limit":
+            assert counts[0] == counts.max() > 16  # past one round of the merge's slots
+    else:
+        # not for every format: wide splits of bf16 leave fewer than two a unit
+        assert fmt["bits"] == 16 or name in ("62-sequences", "41-sequences"), name
+    again, _ = _cuts(c, 1, q, 0.1, B)  # the inheritor reads the same anchor
+    assert torch.equal(out, again)
+    c.set_decode_schedule(SPLITS)
+    plain, none = _cuts(c, 0, q, 0.1, B)
+    assert none is None
+    assert_close(f32(out), f32(plain), max_abs=1e-4, rel_l2=1e-4, what=f"balanced = splits, {_fid(fmt)} {name}")
+    assert (f32(out)[np.array(lens) == 0] == 0).all()
+    assert c.device_error() == 0
+
+
+@pytest.mark.parametrize("fmt", [BAL_FORMATS[i] for i in (0, 2, 4, 6)],
+                         ids=lambda f: _fid(f) + f["key_axis"][0])
+def test_balanced_splits_match_the_oracle(fmt):
+    """Every position read once: ragged sequences against fp64."""
+    B, Hkv, G, D = 40, 2, 4, 128
+    lens = [0, 1, 65, 3200] + _ragged(36, 2500, 6)
+    c = _cache(B, G * Hkv, Hkv, D, 3200, fmt, max_splits=64)
     K, V = _fill(c, B, Hkv, D, lens, seed=fmt["bits"] + len(lens))
     st = oracle_state(K, V, np.array(lens), fmt)
-    sigma = 1.0 / math.sqrt(D)
     q = torch.randn((B, G * Hkv, D), generator=torch.Generator().manual_seed(2)).to(torch.bfloat16)
-    ref = gqa_expected(q, st, np.array(lens), sigma)
-    out = c.decode(0, q.cuda(), sigma)
-    assert_close(f32(out), ref, what=f"balanced {_fid(fmt)}")
-    assert (f32(out)[np.array(lens) == 0] == 0).all()
-    c.set_decode_schedule(SPLITS)
-    assert_close(f32(c.decode(0, q.cuda(), sigma)), f32(out), max_abs=1e-4, rel_l2=1e-4, what="balanced = splits")
+    sigma = 1.0 / math.sqrt(D)
+    out, counts = _cuts(c, 0, q.cuda(), sigma, B)
+    assert counts is not None or fmt["bits"] == 16
+    if counts is not None:
+        assert _balanced_tiles(counts, lens, _kernel_tile(fmt)) is not None, counts
+    assert_close(f32(out), gqa_expected(q, st, np.array(lens), sigma), what=f"balanced {_fid(fmt)}")
     assert c.device_error() == 0
 
 
 def test_recorded_balanced_launch_covers_longer_sequences():
-    """Recorded at one length bound, replayed after one sequence grew past
-    it: the splits follow the lengths on the device."""
+    """Recorded at one length bound, replayed after the sequences changed:
+    the splits follow the lengths on the device, or stay even where a
+    sequence has grown past what they may hold."""
     fmt = dict(bits=4, group=32, key_axis="token")
-    B, Hkv, G, D = 3, 2, 4, 128
-    c = _cache(B, G * Hkv, Hkv, D, 4096, fmt)
-    g = torch.Generator().manual_seed(3)
-    k = torch.randn((B, 4000, Hkv, D), generator=g).to(torch.bfloat16)
-    v = torch.randn((B, 4000, Hkv, D), generator=g).to(torch.bfloat16)
-    c.append(0, k[:, :300].contiguous().cuda(), v[:, :300].contiguous().cuda(),
-             torch.full((B,), 300, dtype=torch.int32, device="cuda"))
-    q = torch.randn((B, G * Hkv, D), generator=g).to(torch.bfloat16).cuda()
+    B, Hkv, G, D, T = 32, 2, 4, 128, 8192
+    g = torch.Generator(device="cuda").manual_seed(3)
+    k, v = (torch.randn((B, T, Hkv, D), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    c = _cache(B, G * Hkv, Hkv, D, T, fmt, max_splits=64)
+    start = _ragged(B, 4000, B - 1)
+    counts = lambda n: torch.tensor(n, dtype=torch.int32, device="cuda")
+    c.append(0, k[:, :4000].contiguous(), v[:, :4000].contiguous(), counts(start))
+    q = torch.randn((B, G * Hkv, D), generator=g, device="cuda").to(torch.bfloat16)
     out = torch.empty((B, G * Hkv, D), device="cuda")
+    torch.cuda.synchronize()
     s = torch.cuda.Stream()
     with torch.cuda.stream(s):
         c.decode(0, q, 0.1, out=out, stream=s)  # warm (kernel attributes set outside capture)
@@ -261,12 +345,24 @@ def test_recorded_balanced_launch_covers_longer_sequences():
         with torch.cuda.graph(gr, stream=s):
             c.decode(0, q, 0.1, out=out, stream=s)
     torch.cuda.synchronize()
-    more = torch.tensor([3700, 0, 411], dtype=torch.int32, device="cuda")
-    c.append(0, k[:, 300:].contiguous().cuda(), v[:, 300:].contiguous().cuda(), more)
-    torch.cuda.synchronize()
-    gr.replay()
-    torch.cuda.synchronize()
-    lens = np.array([4000, 300, 711])
-    st = oracle_state(f32(k), f32(v), lens, fmt)
-    assert_close(f32(out), gqa_expected(q.cpu(), st, lens, 0.1), what="replayed")
+    words = _count_words(c, B)
+    lens = np.array(start)
+    for grown, own in ((_ragged(B, 300, 9), True), ([0] * (B - 1) + [3500], False)):
+        n = np.array(grown)
+        m = int(n.max())
+        pick = torch.arange(m, device="cuda")[None, :] + torch.tensor(lens, device="cuda")[:, None]
+        pick = pick.clamp(max=T - 1)[:, :, None, None].expand(B, m, Hkv, D)
+        c.append(0, torch.gather(k, 1, pick).contiguous(), torch.gather(v, 1, pick).contiguous(), counts(n.tolist()))
+        lens = lens + n
+        torch.cuda.synchronize()
+        words.fill_(UNTOUCHED)
+        gr.replay()
+        torch.cuda.synchronize()
+        kb = words.cpu().numpy()
+        assert (kb != UNTOUCHED).all()
+        assert (kb == kb[0]).all() != own
+        ref = _cache(B, G * Hkv, Hkv, D, T, fmt, max_splits=64)
+        ref.append(0, k, v, counts(lens.tolist()))
+        ref.set_decode_schedule(SPLITS)
+        assert_close(f32(out), f32(ref.decode(0, q, 0.1)), max_abs=1e-4, rel_l2=1e-4, what=f"replayed, own cut {own}")
     assert c.device_error() == 0
