@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import quant as oq
 from _parity import (assert_close, check_codes, f32, gqa_expected, oracle_state)
 
 pytestmark = pytest.mark.gpu
@@ -304,7 +305,8 @@ def test_append_rounding_ties(fmt):
 ], ids=lambda f: f"{f.get('scheme', 'grouped')[:3]}{f['bits']}g{f.get('group', 128)}-{f.get('key_axis', 'token')[:1]}")
 def test_bulk_append_equals_short_appends(fmt, in_dtype):
     """One bulk append stores byte for byte what appends of a few rows (a
-    kernel of their own) store: row counts that leave part of a warp's and of
+    kernel of their own; per-channel key groups, which have one kernel, are
+    checked against the oracle below) store: row counts that leave part of a warp's and of
     a CTA's rows over, per-sequence counts, and rows of the values where a
     quotient by residuals could differ from a division: exact ties, constant
     and zero groups, tiny and huge scales, infinities and NaN."""
@@ -345,12 +347,88 @@ def test_bulk_append_equals_short_appends(fmt, in_dtype):
     assert a.lengths(0).tolist() == b.lengths(0).tolist() == count.tolist()
     x, y = a.export(0), b.export(0)
     for key in x:
-        if x[key] is None or key == "k_residual":
+        if x[key] is None:
             continue
         for s in range(B):
+            if key == "k_residual":  # the open group's rows
+                g = fmt["group"]
+                at = torch.arange(int(count[s]) // g * g, int(count[s]), device="cuda") % g
+                assert torch.equal(x[key][s][:, at].view(torch.int16), y[key][s][:, at].view(torch.int16)), (key, s)
+                continue
             m = int(count[s]) // fmt.get("group", 1) if key in ("k_scale", "k_zero") and fmt.get("key_axis") == "channel" else int(count[s])
             p, q = x[key][s, :, :m].contiguous(), y[key][s, :, :m].contiguous()
             if p.is_floating_point():
                 p, q = p.float().view(torch.int32), q.float().view(torch.int32)
             assert torch.equal(p, q), (key, s)
     assert a.device_error() == 0 and b.device_error() == 0
+
+
+@pytest.mark.parametrize("D", [128, 64])
+@pytest.mark.parametrize("in_dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
+@pytest.mark.parametrize("bits,group", [(8, 64), (4, 32), (8, 32), (4, 64)])
+def test_per_channel_key_groups_special_columns(bits, group, in_dtype, D):
+    """The quantiser of per-channel key groups against the oracle, column by
+    column: quotients exactly on half-integers and one bf16 step off, scales
+    on both sides of 2^-96 and 2^96 (where quotients by residuals end), down
+    to subnormals, constant and zero columns, infinities and NaN (the extrema
+    skip a NaN, a quotient that is one gives code 0); appended at once, so
+    that new rows alone make up groups, and a few at a time, so that the
+    residual rows do."""
+    Hkv, n = 2, 3 * group + 5
+    rng = np.random.default_rng(bits + group)
+    levels = (1 << bits) - 1
+    k = np.zeros((1, n, Hkv, D), np.float32)
+    exps = [0, -5, 7, -95, -96, -97, -100, -120, -126, 90, 95, 96, 97, 110]
+    for h in range(Hkv):
+        for c in range(D):
+            for g0 in range(0, n, group):
+                m = min(group, n - g0)
+                col = (rng.integers(0, min(levels, 127), m) + 0.5).astype(np.float32)  # 8 bits: exact in bf16
+                col[0] = 0.0
+                if m > 1:
+                    col[1] = levels
+                step = torch.from_numpy(col).to(torch.bfloat16).view(torch.int16).numpy().copy()
+                step[2:] += rng.integers(-1, 2, max(0, m - 2)).astype(np.int16) * (c % 3 == 1)
+                col = torch.from_numpy(step).view(torch.bfloat16).float().numpy()
+                col = col * np.float32(2.0 ** exps[(c + h) % len(exps)])
+                if c % 5 == 2:
+                    col = -col
+                k[0, g0:g0 + m, h, c] = col
+    k[0, :, 0, 3] = 3.25
+    k[0, :, 0, 4] = 0.0
+    k[0, :, 0, 5] = -0.0
+    k[0, 7, 0, 6] = np.inf
+    k[0, 8, 0, 7] = -np.inf
+    k[0, 9, 1, 8], k[0, 10, 1, 8] = np.inf, -np.inf
+    k[0, 11, 1, 9] = np.nan
+    k[0, :, 1, 10] = np.nan
+    k[0, :, 1, 11] = np.where(np.arange(n) % 2, 3e38, -3e38)
+    k = torch.from_numpy(k).to(torch.bfloat16)  # what the cache rounds keys to
+    v = torch.randn((1, n, Hkv, D), generator=torch.Generator().manual_seed(1))
+    kf = k.float().numpy()
+    nq = n // group * group
+    x = kf[0, :nq].reshape(3, group, Hkv, D)
+    with np.errstate(all="ignore"):
+        mn, mx = np.fmin.reduce(x, axis=1, initial=np.inf), np.fmax.reduce(x, axis=1, initial=-np.inf)
+        scale = ((mx - mn).astype(np.float32) / np.float32(levels)).astype(np.float32)
+        ratio = ((x - mn[:, None]).astype(np.float32) / np.where(scale == 0, np.float32(1), scale)[:, None]).astype(np.float32)
+        code = np.fmin(np.fmax(np.rint(ratio), 0), levels)
+        code = np.where((scale == 0)[:, None], 0, code).astype(np.uint8)
+    plain = np.isfinite(kf[0]).all(axis=0)  # and the oracle, where it has a value
+    plain[1, 11] = False  # its range overflows
+    oc, os_, oz, _ = oq.quantise_per_channel(np.where(plain, kf[0], 0.0).transpose(1, 0, 2), bits, group)
+    keep = np.broadcast_to(plain[:, None, :], oc.shape)
+    assert (oc[keep] == code.reshape(nq, Hkv, D).transpose(1, 0, 2)[keep]).all()
+    for step in (n, 7):
+        c = _cache(1, 2 * Hkv, Hkv, D, n, [dict(bits=bits, group=group, key_axis="channel")])
+        for i in range(0, n, step):
+            c.append(0, k[:, i:i + step].to(in_dtype).contiguous().cuda(), v[:, i:i + step].to(in_dtype).contiguous().cuda())
+        e = c.export(0)
+        np.testing.assert_array_equal(e["k_codes"][0, :, :nq].cpu().numpy(), code.reshape(nq, Hkv, D).transpose(1, 0, 2))
+        for name, want in (("k_scale", scale), ("k_zero", mn)):
+            np.testing.assert_array_equal(e[name][0, :, :3].cpu().numpy(), want.transpose(1, 0, 2), err_msg=name)
+        at = torch.arange(nq, n) % group
+        res, want = e["k_residual"][0][:, at.cuda()].cpu(), k[0, nq:].transpose(0, 1).contiguous()
+        bits16 = lambda t: torch.where(t.isnan(), 0x7FC0, t.view(torch.int16))  # one NaN is as good as another
+        assert torch.equal(bits16(res), bits16(want))
+        assert c.device_error() == 0
