@@ -181,15 +181,27 @@ def test_evict_votes_rising_scores(fmt, B, Hkv, G, n_win, T):
     sigma = 1.0 / math.sqrt(D)
     got = f32(c.evict_window(0, q.cuda(), sigma, budget))
     _, votes = oev.snapkv_kept(f32(q), st["k_hat"], lens, sigma, budget)
-    # a weight's relative error: 2 ln 2 times 3 2^-18 sigma log2(e) sum |q k|
-    # (see VOTE_RTOL), here for the largest keys
-    khat = np.abs(st["k_hat"]).reshape(-1, D).max(axis=0)
-    worst = sigma * math.log2(math.e) * float(np.abs(f32(q)).reshape(-1, D).max(axis=0) @ khat)
-    rtol = 2 * math.log(2) * 3 * 2.0 ** -18 * worst
+    # A weight's relative error is ln 2 times that of its score and of its
+    # row's normaliser: 3 2^-18 sigma log2(e) sum_d |q_d k_d| each (see
+    # VOTE_RTOL), for this position, and at most the row's largest over the
+    # positions that carry weight (within 2^-24 of the row's maximum).
+    unit = 3 * 2.0 ** -18 * sigma  # ln 2 log2(e) = 1
     for b in range(B):
         for j in range(Hkv):
-            ref = np.asarray(votes[b][j], np.float64)[: T - n_win]
-            assert np.allclose(got[b, j, : T - n_win], ref, rtol=rtol, atol=1e-7), (b, j)
+            P = T - n_win
+            kk = np.asarray(st["k_hat"][b, j], np.float64)
+            rows = f32(q)[b, :, j * G:(j + 1) * G].reshape(-1, D).astype(np.float64)
+            s_abs = np.abs(rows) @ np.abs(kk).T                      # [rows, T]
+            x = sigma * (rows @ kk.T)
+            x[np.arange(T)[None, :] > (P + np.repeat(np.arange(n_win), G))[:, None]] = -np.inf
+            live = x > x.max(axis=1, keepdims=True) - 24 * math.log(2)
+            norm = np.where(live, s_abs, 0.0).max(axis=1, keepdims=True)
+            w = np.exp(x - x.max(axis=1, keepdims=True))
+            w /= w.sum(axis=1, keepdims=True)
+            bound = (w * np.expm1(unit * (s_abs + norm)))[:, :P].sum(axis=0)
+            ref = np.asarray(votes[b][j], np.float64)[:P]
+            err = np.abs(got[b, j, :P] - ref)
+            assert (err <= bound + 1e-6 * ref + 1e-7).all(), (b, j, (err / (bound + 1e-6 * ref + 1e-7)).max())
     assert c.device_error() == 0
 
 
