@@ -521,7 +521,7 @@ __device__ __forceinline__ void quarter_words(const uint32_t (&bits)[32], uint32
 // instructions per row (3 shuffle rounds per extremum, a division per 8 lanes
 // of a group, 4 shuffles per packed word); here the extrema stay in
 // registers, a group of 32 divides once, the words are summed in place and
-// the arithmetic is packed (81 instructions per row).  bf16 inputs come one
+// the arithmetic is packed (90 instructions per row).  bf16 inputs come one
 // iteration ahead through shared memory: a warp copies its next 8 rows in
 // whole 512-byte runs, each lane's 64 bytes to a place of its own, 80 bytes
 // apart (no bank conflicts); with plain loads the kernel waited for memory

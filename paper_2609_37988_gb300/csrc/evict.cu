@@ -10,14 +10,14 @@
 // with x = scale log2(e) <q_{w,h}, k_t> on the dequantised key and (M, L)
 // the row's maximum and sum over its causal range.  The budget - n_win
 // largest votes (ties: the smaller position) and the window become the
-// anchor's kept list for (b, j), sorted.  Four launches: scores and row
-// statistics per 128-position tile, the statistics merged per row, the votes
-// (streaming the stored scores), the selection.
+// anchor's kept list for (b, j), sorted.  Four launches: the rows' statistics,
+// merged per row, the votes, the selection.
 //
-// The scores run on the CUDA cores in fp32: the evictor runs once per
-// prefill, not per decode step, and fp32 dot products keep the votes within
-// ~1e-6 of the fp64 definition.  Storing the scores (R x 4 bytes per
-// position) costs less than computing them twice (R x D products).
+// head_dim 128 and at most 256 window rows score on the tensor cores, in bf16
+// hi and lo halves, and the vote pass scores again (second half of this
+// file).  Others score on the CUDA cores in fp32 and store the scores (R x 4
+// bytes per position) for the vote pass, which costs less there than scoring
+// twice (R x D products).  Votes are within ~1e-6 of the fp64 definition.
 #include <math.h>
 
 #include <algorithm>
@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) evict_tc_kernel(const EvictArgs
           x[0] = u0.x; x[1] = u0.y; x[2] = u0.z; x[3] = u0.w;
           x[4] = u1.x; x[5] = u1.y; x[6] = u1.z; x[7] = u1.w;
         }
-        put8(qh, ql, true, r, 8 * c8, box, x);
+        put8(qh, ql, r, 8 * c8, box, x);
       } else {
         cp_async16(qh + (c8 >> 3) * box + r * 128 + (((c8 & 7) ^ (r & 7)) << 4), static_cast<const uint16_t *>(a.q) + qi,
                    r < R);

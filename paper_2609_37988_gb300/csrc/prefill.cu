@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
     *abort_flag = 0;
     fence_mbar_init();
   }
-  pdl_wait();  // the expanded tiles, lengths and (output pass) statistics are complete
+  pdl_wait();  // the tiles, lengths and records of non-finite values are complete
   constexpr uint32_t kCols = 512;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(

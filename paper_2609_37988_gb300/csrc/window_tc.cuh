@@ -53,13 +53,12 @@ __device__ __forceinline__ void put_chunk(uint8_t *buf, int row, int ch0, int bo
   const int off = (ch0 >> 6) * box + row * 128 + ((((ch0 & 63) >> 3) ^ (row & 7)) << 4);
   *reinterpret_cast<uint4 *>(buf + off) = w;
 }
-__device__ __forceinline__ void put8(uint8_t *hi, uint8_t *lo, bool with_lo, int row, int ch0,
-                                     int box, const float (&x)[8]) {
+__device__ __forceinline__ void put8(uint8_t *hi, uint8_t *lo, int row, int ch0, int box, const float (&x)[8]) {
   uint32_t h[4], l[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) split2<true>(x[2 * i], x[2 * i + 1], h[i], l[i]);
   put_chunk(hi, row, ch0, box, make_uint4(h[0], h[1], h[2], h[3]));
-  if (with_lo) put_chunk(lo, row, ch0, box, make_uint4(l[0], l[1], l[2], l[3]));
+  put_chunk(lo, row, ch0, box, make_uint4(l[0], l[1], l[2], l[3]));
 }
 // The codes of a quarter's packed words as bytes: plane s of word i holds the
 // codes at bits 8 b + BITS s (byte b), so the code at bit 8 b + BITS s of word
