@@ -411,14 +411,14 @@ bool plan_runs(kvk_cache *c, int a, RunPlan *p) {
 // out equal, or nearly so, keep an even cut, at the cost of a reduction and
 // the counts (0.2-0.7 us), so the schedule is for splits of at least 4 tiles
 // (6 of the 64-position ones without per-channel keys; a CTA's tile takes
-// 1.2-2.5 us) and at least 4 sequences.  Decode and merge, 8 formats x 12
-// shapes of 4-40 sequences of 600-16000 positions, against the other plan:
-// equal lengths named by counts 0.94-1.06 (on average 1.01; a search in every
-// CTA and a merge of every slot: 0.95-1.23), lengths from half to all of the
-// longest 0.85-1.04 (0.98), from one position on 0.66-1.00 (0.93).  Instead
-// of the runs where whole splits fill 85 % of the wave (they fill all of it,
-// but by the longest length): 13 x 8 units of sym4, 5003 positions, equal
-// 0.96, ragged 0.90; 16 x 4 of sym8, 8192: 1.01 and 0.93.
+// 1.2-2.5 us) and at least 4 sequences.  Decode and merge, 8 formats x 14
+// shapes of 2-40 sequences of 600-32768 positions, against the other plan:
+// equal lengths named by counts 0.95-1.08 (on average 1.01; a search in every
+// CTA and a merge of every slot: 1.06, up to 1.27), lengths from half to all
+// of the longest 0.83-1.06 (0.98), from one position on 0.66-1.02 (0.93).
+// Instead of the runs where whole splits fill 85 % of the wave (they fill all
+// of it, but by the longest length): 13 x 8 units of sym4, 5003 positions,
+// equal 0.96, ragged 0.85; 16 x 4 of sym8, 8192: 1.03 and 0.90.
 struct BalPlan {
   int x = 0, n = 0;                  // CTAs per unit in the grid, CTAs of one wave per KV head
   int cap = 0, aim = 0;              // most slots per unit, most tiles of a balanced split
