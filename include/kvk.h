@@ -263,7 +263,9 @@ kvk_status kvk_evict_window(kvk_cache *cache, int32_t layer, const void *q_win, 
  *  scratch: device, 256-byte aligned, at least kvk_prefill_scratch_size
  *           bytes: the anchor's cache dequantised once into the products'
  *           operand layout (1 KB per position and KV head for quantised
- *           anchors, 512 B for bf16) and a job counter.
+ *           anchors, 512 B for bf16), 528 B per unit and a job counter.
+ * A stored value that is not finite gives NaN in its channel to the queries
+ * that see its position; the others do not depend on it.
  * Errors: UNSUPPORTED (MLA: see kvk_prefill_attention_mla; head_dim != 128),
  * INVALID_ARG (n_q outside [1, max_ctx], null or misaligned pointers,
  * scale not finite and positive, scratch too small). */

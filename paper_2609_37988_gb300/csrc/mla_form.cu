@@ -467,19 +467,21 @@ __global__ void __launch_bounds__(kFmThreads, 1)
             for (int c0 = 0; c0 < 128; c0 += 32) {
               float x[32];
               load(c0, x);
-              if (!odd_row) continue;
-              apply(c0, x, 1.f);
-              int *bad = a.bad + ((size_t)cur.b * a.nh + cur.h) * kPfBadStride;
-              const int at = (int)v.cap - (t0 + row);
+              if (odd_row) {
+                apply(c0, x, 1.f);
+                int *bad = a.bad + ((size_t)cur.b * a.nh + cur.h) * kPfBadStride;
+                const int at = (int)v.cap - (t0 + row);
 #pragma unroll
-              for (int k = 0; k < 32; ++k) {
-                if (fabsf(x[k]) < INFINITY) {
-                  top = fmaxf(top, fabsf(x[k]));
-                } else {
-                  atomicMax(bad + c0 + k, at);
-                  atomicMax(bad + 128, at);
+                for (int k = 0; k < 32; ++k) {
+                  if (fabsf(x[k]) < INFINITY) {
+                    top = fmaxf(top, fabsf(x[k]));
+                  } else {
+                    atomicMax(bad + c0 + k, at);
+                    atomicMax(bad + 128, at);
+                  }
                 }
               }
+              __syncwarp();  // the TMEM loads are warp-wide
             }
           }
           const uint32_t tb = __reduce_max_sync(0xffffffffu, __float_as_uint(top)) >> 23;
@@ -498,6 +500,7 @@ __global__ void __launch_bounds__(kFmThreads, 1)
               for (int k = 0; k < 32; ++k)
                 if (!(fabsf(x[k]) < INFINITY)) x[k] = 0.f;
             }
+            __syncwarp();
 #pragma unroll
             for (int k = 0; k < 16; ++k) split2<false>(x[2 * k], x[2 * k + 1], hw[k], lw[k]);
             store(c0, hw, lw);

@@ -782,6 +782,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
                   st8(dst, z, sector);
                   st8(dst + 8, z + 8, sector);
                 }
+                __syncwarp();  // the TMEM loads are warp-wide
               } else {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) zw[i] = __float_as_uint(z[i] * f);
@@ -877,6 +878,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
               for (int i = 0; i < 8; ++i) o[8 * c + i] = fmaf(x[i], f_old, o[8 * c + i]);
             }
           }
+          __syncwarp();
         }
       } else {
 #pragma unroll
@@ -897,6 +899,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const PfArgs a, 
           if (at <= x.w) o[4 * c + 3] = NAN;
         }
       }
+      __syncwarp();
       if (row_live) {
         float4 *dst = reinterpret_cast<float4 *>(out_row(J, rl));
 #pragma unroll
